@@ -9,6 +9,7 @@
 #include <new>
 #include <vector>
 
+#include "qng_frames.h"
 #include "qng_internal.h"
 #include "qng_large.h"
 
@@ -133,6 +134,26 @@ struct qng_ctx {
     size_t o_reg[large::kRegs] = {0, 0, 0, 0};
     size_t o_regscale = 0, o_partial = 0, o_slotfac = 0, o_pdesc = 0, o_pops = 0, o_red = 0, o_phases = 0;
     size_t o_queue = 0;
+    // diagonal-frame path (on-chip instances at default shapes; qng_frames.h)
+    bool frames = false;
+    int fkb = 4;  // index bits per thread
+    struct {
+        std::vector<frames::Inst> inst;
+        std::vector<frames::Run> run;
+        std::vector<frames::Member> member;
+        std::vector<frames::Ip> ip;
+        std::vector<frames::UOp> uop;
+        std::vector<frames::Perm> perm;
+        std::vector<DevTerm> term;
+        std::vector<frames::Item> item;
+        std::vector<int32_t> cols, order;
+        std::vector<frames::TabItem> tab;
+        std::vector<frames::HItem> hitem;
+        std::vector<frames::Class> cls;
+        int64_t amps_ad = 0, amps_v = 0;  // checkpoints or tables; final vectors or seeds
+    } f;
+    size_t of_inst = 0, of_run = 0, of_member = 0, of_ip = 0, of_uop = 0, of_perm = 0, of_term = 0, of_item = 0, of_cols = 0;
+    size_t of_order = 0, of_tab = 0, of_hitem = 0, of_badrun = 0, of_bad = 0, of_eacc = 0, of_etaexp = 0, of_a = 0, of_d = 0, of_v = 0, of_eta = 0;
     // mixed-precision solve: cluster size (0 = not used: P < 48 or its float32 matrix does not fit)
     int ir_C = 0;
     size_t o_irflag = 0;
@@ -215,6 +236,40 @@ struct qng_ctx {
         w.irflag = reinterpret_cast<int32_t *>(ws + o_irflag);
         w.ckpt = ws + o_ckpt;
         w.eta = ws + o_eta;
+        return w;
+    }
+    frames::FWork fwork(const double *theta) const {
+        frames::FWork w;
+        auto at = [&](size_t o) { return ws + o; };
+        w.inst = reinterpret_cast<const frames::Inst *>(at(of_inst));
+        w.run = reinterpret_cast<const frames::Run *>(at(of_run));
+        w.member = reinterpret_cast<const frames::Member *>(at(of_member));
+        w.ip = reinterpret_cast<const frames::Ip *>(at(of_ip));
+        w.uop = reinterpret_cast<const frames::UOp *>(at(of_uop));
+        w.perm = reinterpret_cast<const frames::Perm *>(at(of_perm));
+        w.term = reinterpret_cast<const DevTerm *>(at(of_term));
+        w.item = reinterpret_cast<const frames::Item *>(at(of_item));
+        w.cols = reinterpret_cast<const int32_t *>(at(of_cols));
+        w.order = reinterpret_cast<const int32_t *>(at(of_order));
+        w.tab = reinterpret_cast<const frames::TabItem *>(at(of_tab));
+        w.hitem = reinterpret_cast<const frames::HItem *>(at(of_hitem));
+        w.bad_run = reinterpret_cast<int32_t *>(at(of_badrun));
+        w.bad = reinterpret_cast<int32_t *>(at(of_bad));
+        w.eacc = reinterpret_cast<unsigned long long *>(at(of_eacc));
+        w.etaexp = reinterpret_cast<int32_t *>(at(of_etaexp));
+        w.a = at(of_a);
+        w.d = at(of_d);
+        w.v = at(of_v);
+        w.eta = at(of_eta);
+        w.theta = theta;
+        const Work g = work();
+        w.status = g.status;
+        w.pctrl = g.pctrl;
+        w.sigma = g.sigma;
+        w.L = g.L;
+        w.Lim = g.Lim;
+        w.gradraw = g.gradraw;
+        w.energy = g.energy;
         return w;
     }
 };
@@ -320,6 +375,163 @@ qng_status plan_streaming(qng_ctx *c, int64_t scale_n) {
     c->groups.clear();
     c->prepared = false;
     return QNG_OK;
+}
+
+// Index bits per thread of the diagonal-frame kernels. A single instance has few columns, and each one's
+// walk is a serial chain: 8 amplitudes a thread put twice the warps of 16 on it (11 qubits, general
+// circuit, complex128: columns 385 -> 233 us; 12 qubits, complex64: the same). A batch fills the GPU with
+// columns, where 16 need fewer exchanges (64 instances, complex64: 3.61 -> 1.84 ms). From 14 qubits on 16
+// keep the vector within 8 CTAs.
+int frames_kb(const qng_ctx *c) { return c->count == 1 && c->inst[0].n < 14 ? 3 : 4; }
+
+// CTAs per vector (log2): as many as it takes to hold it at 2^kb amplitudes a thread and 512 threads a
+// CTA. A single complex128 instance, bound by instruction issue, spreads its walks over up to 4 SMs
+// (12 qubits: sweep 117 -> 86 us, columns 165 -> 148 us); complex64 ones lose more to the exchanges
+// between SMs than they gain (columns 82 -> 91 us).
+int frames_cl(const qng_ctx *c, int n, int kb) {
+    const int need = std::max(0, n - (9 + kb));
+    return c->count == 1 && c->precision == QNG_C128 && n < 14 ? std::max(need, std::min(2, n - 10)) : need;
+}
+
+// Programs, work lists and launch classes of the diagonal-frame path. False when a class's shared
+// memory does not fit (then the gate-by-gate kernels run).
+bool plan_frames(qng_ctx *c) {
+    auto &f = c->f;
+    f = {};
+    const size_t ab = amp_bytes(c->precision);
+    std::vector<frames::Program> prog(c->count);
+    std::vector<std::array<int, 2>> key(c->count);
+    const int kb = c->fkb = frames_kb(c);
+    for (int b = 0; b < c->count; ++b) {
+        const HostInst &h = c->inst[b];
+        frames::Inst d = {};
+        d.cl = frames_cl(c, h.n, kb);
+        frames::Program &p = prog[b];
+        frames::build_program(h.gates, h.masks, h.terms, h.n, kb, d.cl, p);
+        d.n = h.n;
+        d.nE = p.nE;
+        d.R = (int32_t)p.runs.size();
+        d.P = h.P;
+        d.run_off = (int32_t)f.run.size();
+        d.fwd_off = (int32_t)f.uop.size();
+        d.fwd_cnt = (int32_t)p.fwd.size();
+        d.bwd_off = d.fwd_off + d.fwd_cnt;
+        d.bwd_cnt = (int32_t)p.bwd.size();
+        d.start0 = p.start0;
+        d.end_low = p.end_low;
+        d.term_off = (int32_t)f.term.size();
+        d.nterms = (int32_t)p.terms.size();
+        // |<E>| and the components of H psi are at most sum |c| (times 1 + rounding)
+        int ex = 0;
+        double cmax = 0.0;
+        for (const qng_pauli &t : h.terms) cmax = std::max(cmax, std::fabs(t.coeff));
+        if (cmax > 0.0) std::frexp(cmax, &ex);
+        d.eexp = ex + 1;
+        for (size_t k = 1; k < h.terms.size(); k *= 2) ++d.eexp;
+        const int N = 1 << p.nE, per = frames::kHThreads / frames::kHSplit;
+        d.hchunks = (N + per - 1) / per;
+        d.ip_off = (int32_t)f.ip.size();
+        d.a_off = d.d_off = f.amps_ad;
+        f.amps_ad += (int64_t)d.R << p.nE;
+        d.v_off = f.amps_v;
+        f.amps_v += N;
+        d.param_off = c->param_off[b];
+        d.metric_off = c->metric_off[b];
+        // tables, with indices into the instance's own ones moved to the shared ones
+        const int m0 = (int)f.member.size(), i0 = (int)f.ip.size(), p0 = (int)f.perm.size();
+        for (frames::Run r : p.runs) {
+            r.mem_begin += m0;
+            r.ip_begin += i0;
+            f.run.push_back(r);
+        }
+        f.member.insert(f.member.end(), p.members.begin(), p.members.end());
+        f.ip.insert(f.ip.end(), p.ips.begin(), p.ips.end());
+        f.perm.insert(f.perm.end(), p.perms.begin(), p.perms.end());
+        f.term.insert(f.term.end(), p.terms.begin(), p.terms.end());
+        for (auto *v : {&p.fwd, &p.bwd})
+            for (frames::UOp u : *v) {
+                u.perm = u.perm >= 0 ? u.perm + p0 : -1;
+                f.uop.push_back(u);
+            }
+        for (int r = 0; r < d.R; ++r)
+            for (int first = 0; first < N; first += frames::kTabThreads * frames::kTabAmps)
+                f.tab.push_back(frames::TabItem{b, r, first});
+        f.inst.push_back(d);
+        const int tpc = (N >> kb) >> d.cl;
+        // a batch packs small vectors into CTAs of 256 threads; one instance spreads over more CTAs
+        key[b] = {d.cl, std::max(tpc, c->count == 1 ? 64 : 256)};
+    }
+    std::vector<std::array<int, 2>> keys(key);
+    std::sort(keys.begin(), keys.end(), [](const std::array<int, 2> &x, const std::array<int, 2> &y) { return x > y; });
+    keys.erase(std::unique(keys.begin(), keys.end()), keys.end());
+    bool fits = keys.size() <= (size_t)kPipeMax;
+    for (const auto &k : keys) {
+        frames::Class cl;
+        cl.cl = k[0];
+        cl.threads = k[1];
+        cl.first_inst = (int)f.order.size();
+        cl.first_h = (int)f.hitem.size();
+        struct It { frames::Item it; double cost; bool grad; };
+        std::vector<It> items;
+        int tmax = 32;
+        size_t tabs = 0, ftabs = 0;
+        for (int b = 0; b < c->count; ++b) {
+            if (key[b] != k) continue;
+            const frames::Inst &d = f.inst[b];
+            const int tpc = (1 << (d.nE - kb)) >> d.cl, G = cl.threads / tpc;
+            tmax = std::max(tmax, tpc);
+            cl.max_P = std::max(cl.max_P, d.P);
+            tabs = std::max(tabs, sizeof(frames::Ip) * d.P + sizeof(frames::Run) * d.R + sizeof(frames::UOp) * d.bwd_cnt);
+            ftabs = std::max(ftabs, sizeof(frames::UOp) * d.fwd_cnt);
+            f.order.push_back(b);
+            for (int q = 0; q < d.hchunks; ++q) f.hitem.push_back(frames::HItem{b, q});
+            if (d.P > 0) items.push_back(It{frames::Item{b, d.R, 0, 0, 0, d.P, d.R, 0}, (d.R + 1.0), true});
+            for (int r = 0; r < d.R; ++r) {
+                const frames::Run &rn = f.run[d.run_off + r];
+                std::vector<int32_t> list;
+                for (int q = 0; q < rn.ip_count; ++q) {
+                    const int j = rn.ip_first + q;
+                    if (c->col_want.empty() || c->col_want[j]) list.push_back(j);
+                }
+                for (size_t q = 0; q < list.size(); q += G) {
+                    const int nc = (int)std::min<size_t>(G, list.size() - q);
+                    items.push_back(It{frames::Item{b, r, (int32_t)f.cols.size(), nc, prog[b].bwd_entry[r],
+                                                  rn.ip_first + rn.ip_count, r + 1, 0}, r + 1.0, false});
+                    f.cols.insert(f.cols.end(), list.begin() + q, list.begin() + q + nc);
+                }
+            }
+        }
+        std::stable_sort(items.begin(), items.end(), [](const It &x, const It &y) { return x.cost > y.cost; });
+        cl.num_inst = (int)f.order.size() - cl.first_inst;
+        cl.num_h = (int)f.hitem.size() - cl.first_h;
+        cl.first_item = (int)f.item.size();
+        for (const It &x : items) f.item.push_back(x.it);
+        cl.num_item = (int)items.size();
+        cl.first_grad = (int)f.item.size();
+        for (const It &x : items) if (x.grad) f.item.push_back(x.it);
+        cl.num_grad = (int)f.item.size() - cl.first_grad;
+        cl.first_met = (int)f.item.size();
+        for (const It &x : items) if (!x.grad) f.item.push_back(x.it);
+        cl.num_met = (int)f.item.size() - cl.first_met;
+        cl.fwd_threads = tmax;
+        cl.kb = kb;
+        cl.smem_fwd = ((size_t)tmax << kb) * ab + ftabs;
+        const size_t rows = sizeof(double) * (size_t)(cl.max_P + 1) * (cl.threads / 32);
+        cl.smem_col = ((size_t)cl.threads << kb) * ab + rows + tabs;
+        cl.smem_col_im = cl.smem_col + rows;
+        fits = fits && cl.smem_col_im <= kMaxSmem && cl.smem_fwd <= kMaxSmem;
+        f.cls.push_back(cl);
+    }
+    return fits;
+}
+
+// The default shapes of every qubit count of the context (no qng_set_tuning, qng_set_shape,
+// qng_set_forward_cluster and no shape kept by the autotuner).
+bool default_shapes(const qng_ctx *c) {
+    if (c->tune_cl >= 0 || c->tune_threads > 0) return false;
+    for (const HostInst &h : c->inst)
+        if (c->tuned_cl[h.n] >= 0 || c->tuned_threads[h.n] > 0 || c->tuned_fwd[h.n] > 0 || c->tuned_fcl[h.n] >= 0) return false;
+    return true;
 }
 
 // Build the device-table images, the launch groups and the workspace layout.
@@ -508,6 +720,11 @@ qng_status plan(qng_ctx *c) {
         c->groups.push_back(g);
     }
 
+    // The diagonal-frame kernels run at the default shapes; qng_set_shape and the like choose the
+    // gate-by-gate kernels. The workspace has room for either.
+    const bool frames_fit = plan_frames(c);
+    c->frames = frames_fit && default_shapes(c);
+
     // workspace layout
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = align256(off); off = o + std::max<size_t>(bytes, 1); return o; };
@@ -535,8 +752,36 @@ qng_status plan(qng_ctx *c) {
     c->o_io_energy = take(sizeof(double) * c->count);
     c->o_queue = take(256 * std::max<size_t>(c->groups.size(), 1));
     take_block_solve(c, take);
+    auto &f = c->f;
+    c->of_inst = take(sizeof(frames::Inst) * f.inst.size());
+    c->of_run = take(sizeof(frames::Run) * f.run.size());
+    c->of_member = take(sizeof(frames::Member) * f.member.size());
+    c->of_ip = take(sizeof(frames::Ip) * f.ip.size());
+    c->of_uop = take(sizeof(frames::UOp) * f.uop.size());
+    c->of_perm = take(sizeof(frames::Perm) * f.perm.size());
+    c->of_term = take(sizeof(DevTerm) * f.term.size());
+    c->of_item = take(sizeof(frames::Item) * f.item.size());
+    c->of_cols = take(sizeof(int32_t) * f.cols.size());
+    c->of_order = take(sizeof(int32_t) * f.order.size());
+    c->of_tab = take(sizeof(frames::TabItem) * f.tab.size());
+    c->of_hitem = take(sizeof(frames::HItem) * f.hitem.size());
+    c->of_badrun = take(sizeof(int32_t) * f.run.size());
+    c->of_bad = take(sizeof(int32_t) * c->count);
+    c->of_eacc = take(3 * sizeof(unsigned long long) * c->count);
+    c->of_etaexp = take(sizeof(int32_t) * c->count);
+    // checkpoints and seeds of the one path or the other, in the same place
+    const size_t big = off;
     c->o_ckpt = take(ab * (size_t)ckpt_amps);
     c->o_eta = take(ab * (size_t)eta_amps);
+    const size_t end = off;
+    if (frames_fit) {
+        off = big;
+        c->of_a = take(ab * (size_t)f.amps_ad);
+        c->of_d = take(ab * (size_t)f.amps_ad);
+        c->of_v = take(ab * (size_t)f.amps_v);
+        c->of_eta = take(ab * (size_t)f.amps_v);
+        off = std::max(off, end);
+    }
     c->ws_bytes = align256(off);
     c->prepared = false;
     return QNG_OK;
@@ -606,6 +851,26 @@ qng_status upload(qng_ctx *c) {
         if (c->ir_C > 0 && (e = prepare_solve_ir(c->max_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
         c->prepared = true;
         return QNG_OK;
+    }
+    if (c->frames) {
+        const auto &f = c->f;
+        auto putv = [&](size_t o, const auto &v) { return put(o, v.data(), sizeof(v[0]) * v.size()); };
+        if ((e = putv(c->of_inst, f.inst)) != cudaSuccess || (e = putv(c->of_run, f.run)) != cudaSuccess ||
+            (e = putv(c->of_member, f.member)) != cudaSuccess || (e = putv(c->of_ip, f.ip)) != cudaSuccess ||
+            (e = putv(c->of_uop, f.uop)) != cudaSuccess || (e = putv(c->of_perm, f.perm)) != cudaSuccess ||
+            (e = putv(c->of_term, f.term)) != cudaSuccess || (e = putv(c->of_item, f.item)) != cudaSuccess ||
+            (e = putv(c->of_cols, f.cols)) != cudaSuccess || (e = putv(c->of_order, f.order)) != cudaSuccess ||
+            (e = putv(c->of_tab, f.tab)) != cudaSuccess || (e = putv(c->of_hitem, f.hitem)) != cudaSuccess ||
+            (e = cudaMemsetAsync(c->ws + c->of_eacc, 0, 3 * sizeof(unsigned long long) * c->count, c->stream)) != cudaSuccess ||
+            (e = cudaMemsetAsync(c->ws + c->of_bad, 0, sizeof(int32_t) * c->count, c->stream)) != cudaSuccess)
+            return cuda_status(e);
+        size_t ff = 0, fc = 0, fci = 0;
+        for (const frames::Class &k : f.cls) {
+            ff = std::max(ff, k.smem_fwd);
+            fc = std::max(fc, k.smem_col);
+            fci = std::max(fci, k.smem_col_im);
+        }
+        if ((e = frames::prepare(c->precision, c->fkb, ff, fc, fci)) != cudaSuccess) return cuda_status(e);
     }
     size_t sf = 0, sc = 0, sci = 0;
     for (const Group &g : c->groups) {
@@ -783,6 +1048,46 @@ qng_status run_streaming(qng_ctx *c, int jobs, int64_t &launches) {
     return QNG_OK;
 }
 
+// The diagonal-frame launches up to the columns. A batch of several launch classes runs each class's
+// sweep and columns on a stream of its own, joined on the context's stream.
+qng_status run_frames(qng_ctx *c, int jobs, const double *theta, int64_t &launches) {
+    const frames::FWork w = c->fwork(theta);
+    const auto &f = c->f;
+    const bool wm = jobs & (kJobMetric | kJobSolve), wg = jobs & (kJobGradient | kJobSolve);
+    const bool wh = jobs & (kJobGradient | kJobEnergy | kJobSolve);
+    const int wim = (jobs & kJobMetricIm) ? 1 : 0;
+    cudaError_t e = timed(c, 0, [&] { return frames::launch_tables(w, (int)f.tab.size(), c->fkb, c->precision, c->stream); });
+    if (e != cudaSuccess) return cuda_status(e);
+    launches += f.tab.empty() ? 0 : 1;
+    const bool side = f.cls.size() > 1 && c->pipe_ready;
+    if (side && (e = cudaEventRecord(c->pipe_ev0, c->stream)) != cudaSuccess) return cuda_status(e);
+    for (size_t k = 0; k < f.cls.size(); ++k) {
+        const frames::Class &cl = f.cls[k];
+        cudaStream_t st = side && k > 0 ? c->pipe_col[k] : c->stream;
+        if (side && k > 0 && (e = cudaStreamWaitEvent(st, c->pipe_ev0, 0)) != cudaSuccess) return cuda_status(e);
+        e = timed_on(c, 1, st, [&] { return frames::launch_forward(w, cl, c->precision, st); });
+        if (e != cudaSuccess) return cuda_status(e);
+        ++launches;
+        if (wh) {
+            e = timed_on(c, 5, st, [&] { return frames::launch_hpsi(w, cl.first_h, cl.num_h, c->precision, st); });
+            if (e != cudaSuccess) return cuda_status(e);
+            ++launches;
+        }
+        const int first = wm && wg ? cl.first_item : (wm ? cl.first_met : cl.first_grad);
+        const int num = wm && wg ? cl.num_item : (wm ? cl.num_met : (wg ? cl.num_grad : 0));
+        if (num > 0) {
+            e = timed_on(c, 2, st, [&] { return frames::launch_columns(w, cl, c->precision, first, num, wim, st); });
+            if (e != cudaSuccess) return cuda_status(e);
+            ++launches;
+        }
+        if (side && k > 0) {
+            if ((e = cudaEventRecord(c->pipe_evc[k], st)) != cudaSuccess) return cuda_status(e);
+            if ((e = cudaStreamWaitEvent(c->stream, c->pipe_evc[k], 0)) != cudaSuccess) return cuda_status(e);
+        }
+    }
+    return QNG_OK;
+}
+
 qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
     if (!c) return QNG_ERR_ARG;
     if (!c->ws || !c->prepared) return QNG_ERR_WORKSPACE;
@@ -793,7 +1098,11 @@ qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
     const Work w = c->work();
     int64_t launches = 0;
     cudaError_t e = cudaSuccess;
-    if (c->total_params > 0) {
+    const bool frames = c->frames && !c->streaming && !(jobs & kJobFromParts);
+    if (frames) {
+        qng_status st = run_frames(c, jobs, args.theta, launches);
+        if (st != QNG_OK) return st;
+    } else if (c->total_params > 0) {
         e = timed(c, 0, [&] { return launch_coef(w, args.theta, c->total_params, c->stream); });
         if (e != cudaSuccess) return cuda_status(e);
         launches += 1;
@@ -808,7 +1117,7 @@ qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
             (e = cudaMemcpyAsync(w.gradraw, args.parts_grad, P1, cudaMemcpyDeviceToDevice, c->stream)) != cudaSuccess)
             return cuda_status(e);
     }
-    const bool need_cols = !(jobs & kJobFromParts) && (jobs & (kJobMetric | kJobGradient | kJobSolve));
+    const bool need_cols = !frames && !(jobs & kJobFromParts) && (jobs & (kJobMetric | kJobGradient | kJobSolve));
     const bool want_eta = jobs & (kJobGradient | kJobSolve);
     if (c->streaming && !(jobs & kJobFromParts)) {
         qng_status st = run_streaming(c, jobs, launches);
@@ -817,7 +1126,7 @@ qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
     const int wm = (jobs & (kJobMetric | kJobSolve)) ? 1 : 0;
     const int wg = (jobs & (kJobGradient | kJobSolve)) ? 1 : 0;
     const int wim = (jobs & kJobMetricIm) ? 1 : 0;
-    int S = (wm && !(jobs & kJobFromParts)) ? pipe_chunks(c) : 0;
+    int S = (wm && !frames && !(jobs & kJobFromParts)) ? pipe_chunks(c) : 0;
     std::vector<int> K;
     std::vector<std::array<int, 2>> rng;
     if (S) {
@@ -856,7 +1165,7 @@ qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
     // float64-bound groups leave the SMs room (batch256: 198 -> 172 ms per step); complex64 runs the
     // groups in turn, which measured as fast or faster (47.2 against 49.1 ms). qng_set_pipeline(ctx, 1)
     // runs them in turn, 2..8 side by side.
-    const bool side_by_side = !S && !(jobs & kJobFromParts) && !c->streaming && c->count > 1 && c->pipe_ready &&
+    const bool side_by_side = !S && !frames && !(jobs & kJobFromParts) && !c->streaming && c->count > 1 && c->pipe_ready &&
                               c->groups.size() > 1 && c->groups.size() <= (size_t)kPipeMax &&
                               (c->pipe_req >= 2 || (c->pipe_req == 0 && c->precision == QNG_C128));
     if (side_by_side) {
@@ -879,7 +1188,7 @@ qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
                 if ((e = cudaStreamWaitEvent(c->stream, c->pipe_evc[idx], 0)) != cudaSuccess) return cuda_status(e);
             }
         }
-    } else if (!S && !(jobs & kJobFromParts)) {
+    } else if (!S && !frames && !(jobs & kJobFromParts)) {
         for (const Group &g : c->groups) {
             if (g.num_inst == 0) continue;
             e = timed(c, 1, [&] { return launch_forward(w, g, c->precision, want_eta, c->stream); });
@@ -1349,6 +1658,12 @@ qng_status qng_autotune(qng_ctx *c, const double *theta, int reps, int64_t *repo
     ns.erase(std::unique(ns.begin(), ns.end()), ns.end());
     int64_t tried = 0;
     qng_status st = QNG_OK;
+    // the default first: the diagonal-frame kernels, which have no shape to choose
+    const bool frames_default = c->frames;
+    const int req0 = c->pipe_req;
+    float frames_ms = 0.f, shape_ms = 0.f;
+    if (frames_default && (st = time_step(frames_ms)) == QNG_OK) ++tried;
+    if (st != QNG_OK) ns.clear();
     for (int n : ns) {
         float best = 3.4e38f;
         int best_cl = c->tuned_cl[n], best_th = c->tuned_threads[n];
@@ -1416,10 +1731,19 @@ qng_status qng_autotune(qng_ctx *c, const double *theta, int reps, int64_t *repo
         }
         c->pipe_req = best_req;
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     qng_status s2 = plan(c);
     if (s2 == QNG_OK) s2 = upload(c);
+    if (st == QNG_OK && s2 == QNG_OK && frames_default && (st = time_step(shape_ms)) == QNG_OK && frames_ms <= shape_ms) {
+        for (int n : ns) {
+            c->tuned_cl[n] = c->tuned_fcl[n] = -1;
+            c->tuned_threads[n] = c->tuned_fwd[n] = 0;
+        }
+        c->pipe_req = req0;
+        s2 = plan(c);
+        if (s2 == QNG_OK) s2 = upload(c);
+    }
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
     if (report) *report = tried;
     return st != QNG_OK ? st : s2;
 }

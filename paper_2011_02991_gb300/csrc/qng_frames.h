@@ -1,0 +1,182 @@
+// Diagonal-frame path of the on-chip instances (n <= 16): tables shared by the host planner
+// (qng_frames_plan.cu), the host API and the kernels (qng_frames.cu).
+//
+// Every gate of this library is diagonal in some local Clifford frame: R_X is diagonal after a
+// Hadamard on its qubit, R_Y after H S^dag, a (controlled) Pauli-string rotation after one such
+// change per X or Y factor, CZ and Z as they stand. The planner therefore writes the circuit as
+//     psi = tau_R D_R tau_{R-1} ... D_1 tau_0 |0...0>
+// on a vector kept in a running local frame: a run D_r is a diagonal unitary (all of its rotations
+// and sign gates at once), and a transition tau_r is Hadamards on some qubits and linear index
+// permutations (CNOT networks). Pauli and phase gates, and the Hadamards of the circuit itself,
+// only change the frame and cost nothing.
+//
+// What that gives the recurrence of Algorithm 1: all parameters of a run commute, so with Psi_r
+// the vector after run r and b the column there, every inner product of the run is read off the one
+// product p_m = conj(Psi_r[m]) b[m], <Psi|K_i|b> = sum_m k_i(m) p_m with k_i(m) in {0, +1, -1}, and
+// one complex factor per amplitude takes b through all of the run's adjoint gates. A column costs two
+// multiplications per amplitude and run; everything else is additions.
+#pragma once
+
+#include <cstdint>
+#include <vector>
+
+#include "qng_internal.h"
+
+namespace qng {
+namespace frames {
+
+constexpr int kRegBitsMax = 4;  // a thread holds 2^kb amplitudes, kb index bits at a time (kb = 3 or 4)
+
+// A diagonal factor of a run. With par = parity(m & z) and on = ((m & ctrl) == cval):
+//   kind 0 (rotation):  on ? cos(theta/2) - i lam sin(theta/2) : 1,  lam = sgn (-1)^par
+//   kind 1 (sign gate): on ? lam : 1
+//   kind 2 (S^dag):     par ? -i : 1
+struct Member {
+    int32_t kind;
+    int32_t param;
+    uint32_t z, ctrl, cval;
+    int32_t sgn;
+};
+
+// A parameter of a run as the column kernel reads its inner product off the thread's 16 products:
+// index bits split into the thread's own (zreg, sign16, incl16) and the others (z, ctrl, cval over
+// the thread index).
+struct Ip {
+    uint16_t z, ctrl, cval;
+    uint16_t zreg;     // parity mask over the thread's bits
+    uint16_t incl16;   // the products that the controls include (all: no control)
+    uint16_t sign16;   // the products whose sign flips
+    int16_t sgn;
+    uint16_t all16;    // every product of a thread
+};
+
+struct Run {
+    int32_t mem_begin, mem_count;  // Member table
+    int32_t ip_begin, ip_count;    // Ip table; parameters ip_first .. ip_first + ip_count - 1 in order
+    int32_t ip_first;
+    int32_t low;                   // lowest of the index bits a thread holds at this run
+    int32_t khalf;                 // Hadamards since the run before (each is sqrt 2 times an isometry)
+    int32_t simple;                // every parameter: no control, at most one of the thread's bits
+};
+
+// One step of the vector: exchange into arrangement `low` (through permutation perm >= 0), Hadamards
+// on the thread's bits hm followed by `shift` halvings (fixed point), then run `run` (>= 0).
+struct UOp {
+    int16_t low;    // -1: no exchange
+    int16_t hm;
+    int16_t shift;
+    int16_t pad;
+    int32_t perm;   // -1: none
+    int32_t run;
+};
+
+struct Perm {
+    uint32_t img[16];  // gather: new[m] = old[xor of img[b] over the bits b of m]
+};
+
+// Per-instance descriptor.
+struct Inst {
+    int32_t n, nE;            // qubits; index bits (at least kb)
+    int32_t R, P;
+    int32_t run_off;          // first Run
+    int32_t fwd_off, fwd_cnt; // forward UOps
+    int32_t bwd_off, bwd_cnt; // walk UOps (from the last run down to run 0)
+    int32_t start0, end_low;  // arrangement before the first forward step / after the last
+    int32_t cl;               // log2 CTAs per vector
+    int32_t term_off, nterms; // Hamiltonian terms in the final frame
+    int32_t eexp;             // <E> is summed in fixed point, units of 2^(eexp - 60)
+    int32_t hchunks;          // CTAs of the H psi kernel for this instance
+    int32_t ip_off;           // first Ip
+    int32_t pad;
+    int64_t a_off, d_off;     // checkpoints / factor tables, amplitude units (R << nE each)
+    int64_t v_off;            // final vector and eta (1 << nE each)
+    int64_t param_off, metric_off;
+};
+
+// A work item of the column kernel: ncol columns (cols[list..]) of run `run`, or the gradient column
+// (ncol = 0).
+struct Item {
+    int32_t inst, run;
+    int32_t list, ncol;
+    int32_t entry;      // first step of the walk, index into the instance's walk UOps
+    int32_t nip, nruns;  // parameters and runs the walk meets: the first ones, up to its own run
+    int32_t pad;
+};
+
+struct TabItem {        // 512 entries of one run's factor table
+    int32_t inst, run, first;
+};
+
+struct HItem {          // a CTA of the H psi kernel
+    int32_t inst, chunk;
+};
+
+// One launch class: instances whose vectors use one CTA shape.
+struct Class {
+    int cl = 0;
+    int kb = 4;                          // index bits per thread
+    int threads = 0;                     // CTA size of the column kernel
+    int fwd_threads = 0;                 // CTA size of the forward sweep
+    int max_P = 0;
+    int first_inst = 0, num_inst = 0;    // into order
+    int first_item = 0, num_item = 0;    // metric and gradient columns, longest first
+    int first_met = 0, num_met = 0;
+    int first_grad = 0, num_grad = 0;
+    int first_h = 0, num_h = 0;
+    size_t smem_fwd = 0, smem_col = 0, smem_col_im = 0;
+};
+
+// Device pointers of the path (the workspace's tables and arrays).
+struct FWork {
+    const Inst *inst;
+    const Run *run;
+    const Member *member;
+    const Ip *ip;
+    const UOp *uop;
+    const Perm *perm;
+    const DevTerm *term;
+    const Item *item;
+    const int32_t *cols;
+    const int32_t *order;     // instances by class
+    const TabItem *tab;
+    const HItem *hitem;
+    int32_t *bad_run;         // per run: an angle is not finite
+    int32_t *bad;             // per instance
+    unsigned long long *eacc; // per instance: <E> and |H psi|^2 in fixed point, the count of finished
+    int32_t *etaexp;          //   CTAs; |H psi| <= 2^etaexp
+    void *a, *d, *v, *eta;
+    const double *theta;
+    int32_t *status;
+    double *pctrl, *sigma, *L, *Lim, *gradraw, *energy;
+};
+
+constexpr int kTabThreads = 128, kTabBits = 2, kTabAmps = 1 << kTabBits;
+constexpr int kHThreads = 64, kHSplit = 4;  // H psi: threads per CTA, threads per amplitude
+
+cudaError_t prepare(int precision, int kb, size_t smem_fwd, size_t smem_col, size_t smem_col_im);
+cudaError_t launch_tables(const FWork &w, int ntab, int kb, int precision, cudaStream_t st);
+cudaError_t launch_forward(const FWork &w, const Class &c, int precision, cudaStream_t st);
+cudaError_t launch_hpsi(const FWork &w, int first, int num, int precision, cudaStream_t st);
+cudaError_t launch_columns(const FWork &w, const Class &c, int precision, int first, int num, int metric_im,
+                           cudaStream_t st);
+
+struct Program {  // one instance, host side
+    int n = 0, nE = 4, kb = 4;
+    std::vector<Run> runs;
+    std::vector<Member> members;
+    std::vector<Ip> ips;
+    std::vector<UOp> fwd, bwd;
+    std::vector<int32_t> bwd_entry;  // index of run r's step in bwd
+    std::vector<Perm> perms;
+    std::vector<DevTerm> terms;
+    int start0 = 0, end_low = 0;
+};
+
+// Build the program of one circuit on index bits [0, nE), kb of them per thread and the top cl
+// distributed over CTAs.
+// Indices in the program (members, perms) are relative to its own tables.
+void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks,
+                   const std::vector<qng_pauli> &terms, int n, int kb, int cl, Program &out);
+
+}  // namespace frames
+}  // namespace qng

@@ -1,0 +1,384 @@
+// Host planner of the diagonal-frame path: one circuit -> runs of diagonal gates, the transitions
+// between them, and the steps a CTA takes through them (qng_frames.h).
+//
+// The frame of qubit q is a one-qubit Clifford C_q with psi = (C_1 x C_2 x ...) v for the stored vector
+// v. It is kept as the signed Paulis C_q^dag X C_q and C_q^dag Z C_q: a gate's generator on qubit q
+// acts on v through these images.
+#include <algorithm>
+#include <cstring>
+
+#include "qng_frames.h"
+
+namespace qng {
+namespace frames {
+
+namespace {
+
+enum { PX = 1, PY = 2, PZ = 3 };  // Pauli labels
+struct SP { int p, s; };          // signed Pauli
+
+struct Frame {
+    SP x{PX, 1}, z{PZ, 1};
+    SP y() const {  // Y = i X Z: the product of the images, i P Q = (+-) R for P != Q
+        // i X Z = Y, i Z Y = X, i Y X = Z; the other order gives a minus sign
+        const int a = x.p, b = z.p;
+        const int r = 6 - a - b;  // the third label
+        const bool pos = (a == PX && b == PZ) || (a == PZ && b == PY) || (a == PY && b == PX);
+        return SP{r, x.s * z.s * (pos ? 1 : -1)};
+    }
+    SP image(int axis) const { return axis == kAxisX ? x : (axis == kAxisY ? y() : z); }
+};
+
+SP conj_h(SP a) { return a.p == PY ? SP{PY, -a.s} : SP{a.p == PX ? PZ : PX, a.s}; }             // H P H
+SP conj_sdg(SP a) { return a.p == PX ? SP{PY, -a.s} : (a.p == PY ? SP{PX, a.s} : a); }          // S^dag P S
+
+// Linear map of index bits, as the images of the basis vectors.
+struct Lin {
+    uint32_t img[16];
+    Lin() { for (int b = 0; b < 16; ++b) img[b] = 1u << b; }
+    uint32_t operator()(uint32_t m) const {
+        uint32_t r = 0;
+        for (int b = 0; b < 16; ++b) if ((m >> b) & 1) r ^= img[b];
+        return r;
+    }
+    // mask z' with parity(m & z') = parity(A m & z)
+    uint32_t pull(uint32_t z) const {
+        uint32_t r = 0;
+        for (int b = 0; b < 16; ++b) r |= (uint32_t)(__builtin_popcount(img[b] & z) & 1) << b;
+        return r;
+    }
+    Lin inverse() const {
+        uint32_t a[16];
+        Lin inv;
+        for (int b = 0; b < 16; ++b) a[b] = img[b];
+        // column operations: reduce a to the identity, the same operations on inv
+        for (int b = 0; b < 16; ++b) {
+            int p = b;
+            while (!((a[p] >> b) & 1)) ++p;
+            std::swap(a[p], a[b]);
+            std::swap(inv.img[p], inv.img[b]);
+            for (int k = 0; k < 16; ++k)
+                if (k != b && ((a[k] >> b) & 1)) { a[k] ^= a[b]; inv.img[k] ^= inv.img[b]; }
+        }
+        return inv;
+    }
+};
+
+struct Stage {
+    bool perm = false;
+    uint32_t h = 0;  // Hadamards (perm = false)
+    Lin map;         // new index of old index m is map(m) (perm = true)
+};
+
+struct Builder {
+    std::vector<Frame> fr;
+    std::vector<std::vector<Member>> run_members;  // closed runs and, last, the open one
+    std::vector<std::vector<Stage>> tau;           // tau[r]: the transition before run r
+
+    explicit Builder(int n) : fr(n), run_members(1), tau(1) {}
+
+    std::vector<Member> &open() { return run_members.back(); }
+    std::vector<Stage> &otau() { return tau.back(); }
+    void close() {
+        run_members.emplace_back();
+        tau.emplace_back();
+    }
+    bool open_touches(uint32_t mask) {
+        for (const Member &m : open()) if ((m.z | m.ctrl) & mask) return true;
+        return false;
+    }
+    // S^dag on qubit q of the vector as it is at the end of the open transition: into the run before
+    // it, as a parity of that run's index. False if a Hadamard in between does not commute with it.
+    bool sdg_before_open(int q) {
+        uint32_t z = 1u << q;
+        for (int s = (int)otau().size() - 1; s >= 0; --s) {
+            const Stage &st = otau()[s];
+            if (st.perm) z = st.map.pull(z);
+            else if (st.h & z) return false;
+        }
+        if (run_members.size() == 1) return true;  // |0...0>: parity 0
+        run_members[run_members.size() - 2].push_back(Member{2, -1, z, 0, 0, 1});
+        return true;
+    }
+    // Make the images of (qubit, axis) requirements Z-type.
+    void diagonalise(const std::vector<std::pair<int, int>> &req) {
+        uint32_t need = 0;
+        for (auto &r : req) if (fr[r.first].image(r.second).p != PZ) need |= 1u << r.first;
+        if (!need) return;
+        if (open_touches(need)) close();
+        for (auto &r : req) {
+            const int q = r.first;
+            if (!((need >> q) & 1)) continue;
+            if (fr[q].image(r.second).p == PY) {
+                if (!sdg_before_open(q)) {
+                    // the S^dag has to come between two Hadamards of this transition: a run of its own
+                    close();
+                    run_members[run_members.size() - 2].push_back(Member{2, -1, 1u << q, 0, 0, 1});
+                }
+                fr[q].x = conj_sdg(fr[q].x);
+                fr[q].z = conj_sdg(fr[q].z);
+            }
+            if (otau().empty() || otau().back().perm) otau().emplace_back();
+            otau().back().h ^= 1u << q;
+            fr[q].x = conj_h(fr[q].x);
+            fr[q].z = conj_h(fr[q].z);
+        }
+    }
+    void rotation(int param, const std::vector<std::pair<int, int>> &req, int control) {
+        std::vector<std::pair<int, int>> all(req);
+        if (control >= 0) all.push_back({control, kAxisZ});
+        diagonalise(all);
+        Member m{0, param, 0, 0, 0, 1};
+        for (auto &r : req) {
+            m.z |= 1u << r.first;
+            m.sgn *= fr[r.first].image(r.second).s;
+        }
+        if (control >= 0) {  // acts where the control is 1: the Z image's eigenvalue -1
+            m.ctrl = 1u << control;
+            m.cval = fr[control].z.s > 0 ? m.ctrl : 0;
+        }
+        open().push_back(m);
+    }
+    // controlled Pauli (axis on the target) as a diagonal sign
+    void controlled_sign(int c, int t, int axis) {
+        Member m{1, -1, 1u << t, 1u << c, 0, fr[t].image(axis).s};
+        m.cval = fr[c].z.s > 0 ? m.ctrl : 0;
+        open().push_back(m);
+    }
+    void cnot(int c, int t) {
+        if (fr[c].z.p == PZ && fr[t].x.p == PZ) { controlled_sign(c, t, kAxisX); return; }
+        diagonalise({{c, kAxisZ}, {t, kAxisZ}});
+        for (int q : {c, t})
+            if (fr[q].x.p == PY) {  // a diagonal S^dag of the open run turns the X image back to X
+                open().push_back(Member{2, -1, 1u << q, 0, 0, 1});
+                fr[q].x = conj_sdg(fr[q].x);
+                fr[q].z = conj_sdg(fr[q].z);
+            }
+        if (!open().empty()) close();
+        if (otau().empty() || !otau().back().perm) { otau().emplace_back(); otau().back().perm = true; }
+        Lin &A = otau().back().map;
+        for (int b = 0; b < 16; ++b) A.img[b] ^= ((A.img[b] >> c) & 1u) << t;
+        // the frames of c and t are Paulis X^a Z^b: X_c -> X_c X_t, Z_t -> Z_c Z_t
+        fr[t].z.s *= fr[c].z.s;
+        fr[c].x.s *= fr[t].x.s;
+    }
+};
+
+std::vector<std::pair<int, int>> string_req(uint64_t x, uint64_t z, int n) {
+    std::vector<std::pair<int, int>> r;
+    for (int q = 0; q < n; ++q) {
+        const int hx = (int)((x >> q) & 1), hz = (int)((z >> q) & 1);
+        if (hx || hz) r.push_back({q, hx ? (hz ? kAxisY : kAxisX) : kAxisZ});
+    }
+    return r;
+}
+
+}  // namespace
+
+void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks,
+                   const std::vector<qng_pauli> &terms, int n, int kb, int cl, Program &out) {
+    out = Program();
+    out.n = n;
+    out.kb = kb;
+    const int nE = out.nE = std::max(n, kb);
+    Builder B(n);
+    for (size_t gi = 0; gi < gates.size(); ++gi) {
+        const qng_gate &g = gates[gi];
+        Frame *f = (g.q0 >= 0 && g.q0 < n) ? &B.fr[g.q0] : nullptr;
+        switch (g.kind) {
+        case QNG_GATE_RX: B.rotation(g.param, {{g.q0, kAxisX}}, -1); break;
+        case QNG_GATE_RY: B.rotation(g.param, {{g.q0, kAxisY}}, -1); break;
+        case QNG_GATE_RZ: B.rotation(g.param, {{g.q0, kAxisZ}}, -1); break;
+        case QNG_GATE_CRX: B.rotation(g.param, {{g.q1, kAxisX}}, g.q0); break;
+        case QNG_GATE_CRY: B.rotation(g.param, {{g.q1, kAxisY}}, g.q0); break;
+        case QNG_GATE_CRZ: B.rotation(g.param, {{g.q1, kAxisZ}}, g.q0); break;
+        case QNG_GATE_RP: B.rotation(g.param, string_req(masks[2 * gi], masks[2 * gi + 1], n), -1); break;
+        case QNG_GATE_CRP: B.rotation(g.param, string_req(masks[2 * gi], masks[2 * gi + 1], n), g.q0); break;
+        case QNG_GATE_X: f->z.s = -f->z.s; break;
+        case QNG_GATE_Y: f->x.s = -f->x.s; f->z.s = -f->z.s; break;
+        case QNG_GATE_Z: f->x.s = -f->x.s; break;
+        case QNG_GATE_H: std::swap(f->x, f->z); break;
+        case QNG_GATE_CZ:
+            B.diagonalise({{g.q0, kAxisZ}, {g.q1, kAxisZ}});
+            B.controlled_sign(g.q0, g.q1, kAxisZ);
+            break;
+        case QNG_GATE_CNOT: B.cnot(g.q0, g.q1); break;
+        default: break;
+        }
+    }
+    // Without members left, a last transition that holds Hadamards still needs a run to carry their
+    // normalisation; one of permutations alone, or an empty one, does not.
+    bool last_h = false;
+    for (const Stage &s : B.otau()) last_h = last_h || (!s.perm && s.h);
+    std::vector<Stage> tail;
+    if (B.open().empty() && !last_h) {
+        tail = B.otau();
+        B.run_members.pop_back();
+        B.tau.pop_back();
+    }
+    const int R = (int)B.run_members.size();
+
+    // arrangements: kb consecutive index bits; blocks within a CTA's own bits, the last one flush with
+    // their top, and one at the very top for the distributed bits (local or not, nl >= kb)
+    const int nl = nE - cl;
+    std::vector<int> lows;
+    for (int lo = 0; lo + kb <= nl; lo += kb) lows.push_back(lo);
+    if (nl % kb) lows.push_back(nl - kb);
+    if (cl > 0) lows.push_back(nE - kb);
+    auto block_of = [&](int q) {
+        for (int lo : lows) if (q >= lo && q < lo + kb) return lo;
+        return lows.back();
+    };
+
+    // elementary steps in circuit order
+    struct Step { int kind, low0, low1, perm; uint32_t h; int run; };
+    std::vector<Step> el;
+    std::vector<Lin> maps;
+    int cur = -1;  // arrangement (decided by the first step that needs one)
+    auto blocks_in = [&](uint32_t h) {
+        std::vector<int> b;
+        for (int q = 0; q < nE; ++q) if ((h >> q) & 1) { int lo = block_of(q); if (std::find(b.begin(), b.end(), lo) == b.end()) b.push_back(lo); }
+        std::sort(b.begin(), b.end());
+        return b;
+    };
+    auto first_need = [&](const std::vector<Stage> &t, size_t s, int dflt) {
+        for (; s < t.size(); ++s)
+            if (!t[s].perm && t[s].h) {
+                auto b = blocks_in(t[s].h);
+                return (std::find(b.begin(), b.end(), dflt) != b.end()) ? dflt : b.front();
+            }
+        return dflt;
+    };
+    auto emit_tau = [&](const std::vector<Stage> &t) {
+        for (size_t s = 0; s < t.size(); ++s) {
+            if (t[s].perm) {
+                maps.push_back(t[s].map);
+                const int to = first_need(t, s + 1, cur);
+                el.push_back(Step{0, cur, to, (int)maps.size() - 1, 0, -1});
+                cur = to;
+            } else if (t[s].h) {
+                std::vector<int> b = blocks_in(t[s].h);
+                // the current arrangement first, then away from it in order
+                if (cur != b.front() && (cur == b.back() || std::abs(cur - b.back()) < std::abs(cur - b.front())))
+                    std::reverse(b.begin(), b.end());
+                auto it = std::find(b.begin(), b.end(), cur);
+                if (it != b.end()) std::rotate(b.begin(), it, it + 1);
+                for (int lo : b) {
+                    if (lo != cur) { el.push_back(Step{0, cur, lo, -1, 0, -1}); cur = lo; }
+                    uint32_t h = 0;
+                    for (int q = 0; q < nE; ++q) if (((t[s].h >> q) & 1) && block_of(q) == lo) h |= 1u << (q - lo);
+                    el.push_back(Step{1, lo, lo, -1, h, -1});
+                }
+            }
+        }
+    };
+    const int dflt = cl > 0 ? lows.front() : lows.back();
+    cur = R > 0 ? first_need(B.tau[0], 0, dflt) : first_need(tail, 0, dflt);
+    out.start0 = cur;
+    for (int r = 0; r < R; ++r) {
+        emit_tau(B.tau[r]);
+        el.push_back(Step{2, cur, cur, -1, 0, r});
+        Run run = {};
+        run.low = cur;
+        run.mem_begin = (int)out.members.size();
+        run.mem_count = (int)B.run_members[r].size();
+        run.ip_begin = (int)out.ips.size();
+        run.ip_first = -1;
+        run.simple = 1;
+        for (const Stage &s : B.tau[r]) if (!s.perm) run.khalf += __builtin_popcount(s.h);
+        const int L = cur;
+        auto thr = [&](uint32_t m) { return (m & ((1u << L) - 1u)) | ((m >> (L + kb)) << L); };
+        auto reg = [&](uint32_t m) { return (m >> L) & ((1u << kb) - 1u); };
+        for (const Member &m : B.run_members[r]) {
+            out.members.push_back(m);
+            if (m.kind != 0) continue;
+            if (run.ip_first < 0) run.ip_first = m.param;
+            Ip ip = {};
+            ip.z = (uint16_t)thr(m.z);
+            ip.ctrl = (uint16_t)thr(m.ctrl);
+            ip.cval = (uint16_t)thr(m.cval);
+            ip.sgn = (int16_t)m.sgn;
+            ip.zreg = (uint16_t)reg(m.z);
+            ip.all16 = (uint16_t)((1u << (1 << kb)) - 1u);
+            for (uint32_t k = 0; k < (1u << kb); ++k) {
+                if ((k & reg(m.ctrl)) == reg(m.cval)) ip.incl16 |= (uint16_t)(1u << k);
+                if (__builtin_popcount(k & reg(m.z)) & 1) ip.sign16 |= (uint16_t)(1u << k);
+            }
+            if (m.ctrl || (ip.zreg & (ip.zreg - 1))) run.simple = 0;
+            out.ips.push_back(ip);
+        }
+        run.ip_count = (int)out.ips.size() - run.ip_begin;
+        if (run.ip_first < 0) run.ip_first = 0;
+        out.runs.push_back(run);
+    }
+    emit_tau(tail);
+    out.end_low = cur;
+
+    // fuse into steps: exchange, then Hadamards, then a run. Halvings keep the fixed-point vector
+    // within sqrt 2 of unit norm: floor(k / 2) after k Hadamards of a transition, the odd sqrt 2 is in
+    // the run's factor table.
+    auto fuse = [&](const std::vector<Step> &v, bool back, std::vector<UOp> &ops) {
+        int k = 0;
+        UOp u{-1, 0, 0, 0, -1, -1};
+        int stage = 0;  // 0 nothing yet, 1 exchange, 2 Hadamards
+        auto flush = [&]() { ops.push_back(u); u = UOp{-1, 0, 0, 0, -1, -1}; stage = 0; };
+        for (const Step &s : v) {
+            if (s.kind == 0) {
+                if (stage > 0) flush();
+                u.low = (int16_t)(back ? s.low0 : s.low1);
+                if (s.perm >= 0) {
+                    // gather: forward new[m] = old[A^-1 m], adjoint new[m] = old[A m]
+                    const Lin A = back ? maps[s.perm] : maps[s.perm].inverse();
+                    Perm p;
+                    std::memcpy(p.img, A.img, sizeof(p.img));
+                    u.perm = (int32_t)out.perms.size();
+                    out.perms.push_back(p);
+                }
+                stage = 1;
+            } else if (s.kind == 1) {
+                if (stage > 1) flush();
+                u.hm = (int16_t)s.h;
+                const int k1 = k + __builtin_popcount(s.h);
+                u.shift = (int16_t)(k1 / 2 - k / 2);
+                k = k1;
+                stage = 2;
+            } else {
+                u.run = s.run;
+                if (back) out.bwd_entry[s.run] = (int32_t)ops.size();
+                flush();
+                k = 0;
+            }
+        }
+        if (stage > 0) flush();
+    };
+    out.bwd_entry.assign(R, -1);
+    fuse(el, false, out.fwd);
+    std::vector<Step> rel(el.rbegin(), el.rend());
+    // the walk ends at run 0 (what precedes it is never needed)
+    std::vector<Step> cut;
+    for (const Step &s : rel) {
+        cut.push_back(s);
+        if (s.kind == 2 && s.run == 0) break;
+    }
+    if (R > 0) fuse(cut, true, out.bwd);
+
+    // the Hamiltonian in the final frame
+    for (const qng_pauli &t : terms) {
+        DevTerm d = {};
+        d.coeff = t.coeff;
+        for (int q = 0; q < n; ++q) {
+            const int hx = (int)((t.xmask >> q) & 1), hz = (int)((t.zmask >> q) & 1);
+            if (!hx && !hz) continue;
+            const SP im = B.fr[q].image(hx ? (hz ? kAxisY : kAxisX) : kAxisZ);
+            if (im.s < 0) d.coeff = -d.coeff;
+            if (im.p != PZ) d.x |= 1ull << q;
+            if (im.p != PX) d.z |= 1ull << q;
+        }
+        d.ny = __builtin_popcountll(d.x & d.z) & 3;
+        out.terms.push_back(d);
+    }
+    std::stable_sort(out.terms.begin(), out.terms.end(), [](const DevTerm &a, const DevTerm &b) { return a.x < b.x; });
+}
+
+}  // namespace frames
+}  // namespace qng

@@ -1,0 +1,97 @@
+"""Host checks of the diagonal-frame planner (no GPU): the program that the on-chip kernels run is
+executed in float64 by a host-only probe (tests/frames_probe.cu, linking the library's planner) and
+compared with the oracle: metric, its imaginary part, <sigma_j>, control probabilities, gradient and
+energy. Circuits of every gate kind in every order, so that frames of every kind meet rotations,
+CNOT networks, controlled and string rotations; 1 to 9 qubits, one to eight CTAs per vector."""
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2011_02991_gb300 import workloads as W
+
+ROOT = __import__("pathlib").Path(__file__).resolve().parents[1]
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not shutil.which(nvcc):
+        pytest.skip("nvcc not found")
+    exe = tmp_path_factory.mktemp("probe") / "frames_probe"
+    src = ROOT / "paper_2011_02991_gb300" / "csrc"
+    r = subprocess.run([nvcc, "-std=c++17", "-O1", "-I", str(ROOT / "include"), "-I", str(src), "-o", str(exe),
+                        str(ROOT / "tests" / "frames_probe.cu"), str(src / "qng_frames_plan.cu")],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return exe
+
+
+def run_probe(exe, p, kb=4, cl=0):
+    c, h = p.circuit, p.hamiltonian
+    lines = [f"{c.n} {c.num_params} {len(c.gates)} {h.num_terms} {kb} {cl}"]
+    for row, m in zip(c.gates, c.gate_masks()):
+        lines.append(" ".join(str(int(v)) for v in row) + f" {int(m[0])} {int(m[1])}")
+    lines += [f"{float(a)!r} {int(x)} {int(z)}" for a, x, z in zip(h.coeffs, h.xmask, h.zmask)]
+    lines += [repr(float(t)) for t in p.theta]
+    r = subprocess.run([str(exe)], input="\n".join(lines) + "\n", capture_output=True, text=True)
+    out = r.stdout.strip().split("\n")
+    assert r.returncode == 0 and out[-1] == "ok", f"probe: {out[-3:]} {r.stderr}"
+    return {x.split()[0]: np.array([float(v) for v in x.split()[1:]]) for x in out if " " in x or x in ("L", "grad")}
+
+
+def check(exe, oracle, p, kb=4, cl=0):
+    d = run_probe(exe, p, kb, cl)
+    ref = oracle.qng_step(p)
+    P = p.P
+    tol = 1e-11
+    assert abs(d["E"][0] - ref["E"]) <= tol * max(1.0, np.abs(p.hamiltonian.coeffs).sum())
+    if P == 0:
+        return d
+    assert np.abs(d["grad"] - ref["grad"]).max() <= tol * max(1.0, np.abs(p.hamiltonian.coeffs).sum())
+    assert np.abs(d["sigma"] + 2 * ref["T"].imag).max() <= tol
+    g = np.zeros((P, P), dtype=complex)
+    iu = [(i, j) for j in range(P) for i in range(j)]
+    for (i, j), v in zip(iu, d["L"].reshape(-1, 2)):
+        g[i, j] = complex(v[0], v[1]) - 0.25 * d["sigma"][i] * d["sigma"][j]
+        g[j, i] = np.conj(g[i, j])
+    for j in range(P):
+        g[j, j] = 0.25 * (d["ctrl"][j] - d["sigma"][j] ** 2)
+    assert np.abs(g - ref["G"]).max() <= tol
+    return d
+
+
+@pytest.mark.parametrize("kb", [3, 4])
+@pytest.mark.parametrize("seed", range(18))
+def test_random_circuits(probe, oracle, seed, kb):
+    """Every simple gate kind at random places, 1 to 9 qubits, 8 and 16 amplitudes per thread."""
+    check(probe, oracle, W.random_problem(1 + seed % 9, 70, 6, 4000 + seed), kb)
+
+
+@pytest.mark.parametrize("seed", range(8))
+def test_generalised(probe, oracle, seed):
+    """Controlled and Pauli-string rotations in frames of every kind."""
+    check(probe, oracle, W.general_problem(3 + seed % 5, 50, 90 + seed), 3 + seed % 2)
+
+
+@pytest.mark.parametrize("cl", [0, 1, 2, 3])
+@pytest.mark.parametrize("kinds,ent", [((W.RY, W.RZ), W.CZ), ((W.RY, W.RX, W.RZ), W.CNOT), ((W.RX, W.RY), W.CNOT)])
+def test_layered(probe, oracle, kinds, ent, cl):
+    """Layered ansätze; every layer's rotations of one axis are one run (a CNOT ladder
+    right after rotations of another axis than Z is cut into more)."""
+    n = 7
+    c = W.layered_ansatz(n, 3, kinds, ent)
+    rng = np.random.Generator(np.random.PCG64(3))
+    p = W.Problem("l", c, W.random_pauli_hamiltonian(n, 9, rng), W.uniform_theta(c.num_params, rng))
+    d = check(probe, oracle, p, 4, cl)
+    check(probe, oracle, p, 3, cl)
+    if kinds[-1] == W.RZ:
+        assert d["runs"][0] <= 3 * len(kinds) + 1
+
+
+def test_z_runs_and_no_parameters(probe, oracle):
+    check(probe, oracle, W.z_run_problem(6, 80, 3))
+    c = W.Circuit(3, np.array([[W.H, 0, -1, -1], [W.CNOT, 0, 2, -1], [W.Y, 1, -1, -1], [W.CZ, 0, 1, -1]], dtype=np.int32))
+    h = W.hamiltonian_from_terms([(0.5, {0: "X", 2: "X"}), (0.25, {1: "Z"}), (-1.5, {0: "Y", 2: "Y"})])
+    check(probe, oracle, W.Problem("fixed", c, h, np.zeros(0)))
