@@ -154,6 +154,13 @@ struct qng_ctx {
     } f;
     size_t of_inst = 0, of_run = 0, of_member = 0, of_ip = 0, of_uop = 0, of_perm = 0, of_term = 0, of_item = 0, of_cols = 0;
     size_t of_order = 0, of_tab = 0, of_hitem = 0, of_badrun = 0, of_bad = 0, of_eacc = 0, of_etaexp = 0, of_a = 0, of_d = 0, of_v = 0, of_eta = 0;
+    // streaming instances on the same path (qng_frames.h, StreamProgram)
+    bool sframes = false;
+    frames::StreamProgram sp;
+    std::vector<frames::SCol> scol;  // the gradient column, then the metric columns by decreasing run
+    int sslots = 0, seexp = 0;
+    size_t os_run = 0, os_member = 0, os_ip = 0, os_perm = 0, os_uop = 0, os_entry = 0, os_col = 0, os_term = 0, os_lo = 0;
+    size_t os_hi = 0, os_mask = 0, os_a = 0, os_b = 0, os_acc = 0, os_sacc = 0, os_eacc = 0, os_etaexp = 0, os_bad = 0;
     // mixed-precision solve: cluster size (0 = not used: P < 48 or its float32 matrix does not fit)
     int ir_C = 0;
     size_t o_irflag = 0;
@@ -326,15 +333,70 @@ template <class Take> void take_block_solve(qng_ctx *c, Take &take) {
     c->o_sdinv = take(sizeof(double) * nblk * kSolveBlock * kSolveBlock);
 }
 
-// Streaming path: schedule of passes and the workspace layout (no checkpoints).
+// |<E>| and the components of H psi are at most sum |c|: a power of two above it (coefficients near the
+// largest double: above the largest one times their number).
+int energy_exponent(const std::vector<qng_pauli> &terms) {
+    int ex = 0;
+    double sum = 0.0, cmax = 0.0;
+    for (const qng_pauli &t : terms) {
+        sum += std::fabs(t.coeff);
+        cmax = std::max(cmax, std::fabs(t.coeff));
+    }
+    if (cmax == 0.0) return 1;
+    if (std::isfinite(sum)) {
+        std::frexp(sum * (1.0 + 1e-12), &ex);
+        return ex + 1;
+    }
+    std::frexp(cmax, &ex);
+    ++ex;
+    for (size_t k = 1; k < terms.size(); k *= 2) ++ex;
+    return ex;
+}
+
+constexpr int64_t kStreamFramesMax = 96ll << 30;  // bytes of checkpoints and columns at most
+
+// Plan of the diagonal-frame passes; false when the vector is smaller than a tile or the checkpoints
+// (one vector per run) take more memory than they are worth.
+bool plan_sframes(qng_ctx *c) {
+    const HostInst &h = c->inst[0];
+    const int pi = c->precision == QNG_C128 ? 1 : 0, tb = frames::kStreamTileBits[pi], kb = frames::kStreamRegBits[pi];
+    if (h.n < tb) return false;
+    // contiguous low bits: at most a thread's block (its bits in any other block are then consecutive index
+    // bits), fewer where two windows still cover the index bits (rows of 32 bytes at least), else rows of
+    // 128 bytes. Byte offsets into a vector are 32 bits wide.
+    const int64_t reg = (int64_t)amp_bytes(c->precision) << h.n;
+    if (reg > (4ll << 30)) return false;
+    int low = std::min(2 * tb - h.n, kb);
+    if (low < (pi ? 1 : 2)) low = pi ? 3 : 4;
+    frames::build_stream(h.gates, h.terms, h.n, kb, tb, low, c->sp);
+    const int R = (int)c->sp.runs.size();
+    // column slots: what a launch walks together. Up to 20 qubits 32 MiB of them (enough CTAs, and L2 holds
+    // them between passes), beyond that four, which share each checkpoint read
+    c->sslots = h.n <= 20 ? (int)std::max<int64_t>(2, std::min<int64_t>(32, (32ll << 20) / reg)) : 4;
+    if ((R + c->sslots) * reg > kStreamFramesMax) return false;
+    c->seexp = energy_exponent(h.terms);
+    c->scol.clear();
+    if (h.P > 0) c->scol.push_back(frames::SCol{h.P, R});
+    for (int r = R - 1; r >= 0; --r)
+        for (int q = 0; q < c->sp.runs[r].ip_count; ++q) {
+            const int j = c->sp.runs[r].ip_first + q;
+            if (c->col_want.empty() || c->col_want[j]) c->scol.push_back(frames::SCol{j, r});
+        }
+    return true;
+}
+
+// Streaming path: schedule of passes and the workspace layout.
 qng_status plan_streaming(qng_ctx *c, int64_t scale_n) {
     const HostInst &h = c->inst[0];
     const size_t ab = amp_bytes(c->precision);
     c->sched = large::Schedule();
-    large::build_schedule(h.gates, h.n, h.P, c->precision, c->sched, c->col_want.empty() ? nullptr : &c->col_want);
-    const int64_t ntiles = 1ll << (h.n - c->sched.t);
-    // k_pass: two CTAs per SM; the register-phase kernel: one persistent CTA per SM (152 on GB300)
-    c->l_grid = (int)std::min<int64_t>(ntiles, c->sched.phased ? 152 : 152 * 2);
+    c->sframes = plan_sframes(c);
+    if (!c->sframes) {
+        large::build_schedule(h.gates, h.n, h.P, c->precision, c->sched, c->col_want.empty() ? nullptr : &c->col_want);
+        const int64_t ntiles = 1ll << (h.n - c->sched.t);
+        // k_pass: two CTAs per SM; the register-phase kernel: one persistent CTA per SM (152 on GB300)
+        c->l_grid = (int)std::min<int64_t>(ntiles, c->sched.phased ? 152 : 152 * 2);
+    }
     c->t_inst[0].cl = 0;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = align256(off); off = o + std::max<size_t>(bytes, 1); return o; };
@@ -361,6 +423,33 @@ qng_status plan_streaming(qng_ctx *c, int64_t scale_n) {
     c->o_io_grad = take(sizeof(double) * c->total_params);
     c->o_io_energy = take(sizeof(double) * c->count);
     take_block_solve(c, take);
+    if (c->sframes) {
+        const frames::StreamProgram &p = c->sp;
+        const size_t R = p.runs.size(), P = h.P, nlo = size_t(1) << p.hl, nhi = size_t(1) << (h.n - p.hl);
+        c->os_run = take(sizeof(frames::Run) * R);
+        c->os_member = take(sizeof(frames::Member) * p.members.size());
+        c->os_ip = take(sizeof(frames::SIp) * p.ips.size());
+        c->os_perm = take(sizeof(frames::SPerm) * p.perms.size());
+        c->os_uop = take(sizeof(frames::UOp) * p.ops.size());
+        c->os_entry = take(sizeof(frames::SEntry) * R);
+        c->os_col = take(sizeof(frames::SCol) * c->scol.size());
+        c->os_term = take(sizeof(DevTerm) * p.terms.size());
+        c->os_lo = take(ab * R * nlo);
+        c->os_hi = take(ab * R * nhi);
+        c->os_mask = take(sizeof(uint32_t) * R * nhi);
+        c->os_acc = take(2 * sizeof(int64_t) * P * P);
+        c->os_sacc = take(2 * sizeof(int64_t) * P);  // <sigma>, gradient
+        c->os_eacc = take(3 * sizeof(unsigned long long));
+        c->os_etaexp = take(sizeof(int32_t));
+        c->os_bad = take(sizeof(int32_t));
+        c->os_a = take((ab << h.n) * R);
+        c->os_b = take((ab << h.n) * c->sslots);
+        c->o_ckpt = c->o_eta = 0;
+        c->ws_bytes = align256(off);
+        c->groups.clear();
+        c->prepared = false;
+        return QNG_OK;
+    }
     c->o_regscale = take(sizeof(double) * 2 * large::kRegs);
     c->o_partial = take(sizeof(double) * (size_t)c->sched.max_slots * c->l_grid);
     c->o_slotfac = take(sizeof(double) * (size_t)c->sched.max_slots);
@@ -421,13 +510,7 @@ bool plan_frames(qng_ctx *c) {
         d.end_low = p.end_low;
         d.term_off = (int32_t)f.term.size();
         d.nterms = (int32_t)p.terms.size();
-        // |<E>| and the components of H psi are at most sum |c| (times 1 + rounding)
-        int ex = 0;
-        double cmax = 0.0;
-        for (const qng_pauli &t : h.terms) cmax = std::max(cmax, std::fabs(t.coeff));
-        if (cmax > 0.0) std::frexp(cmax, &ex);
-        d.eexp = ex + 1;
-        for (size_t k = 1; k < h.terms.size(); k *= 2) ++d.eexp;
+        d.eexp = energy_exponent(h.terms);
         const int N = 1 << p.nE, per = frames::kHThreads / frames::kHSplit;
         d.hchunks = (N + per - 1) / per;
         d.ip_off = (int32_t)f.ip.size();
@@ -819,6 +902,24 @@ qng_status upload(qng_ctx *c) {
         return cuda_status(e);
     // host tables must stay valid until the copies ran: pageable-memory copies are staged
     // synchronously with respect to the host, so returning here is safe
+    if (c->streaming && c->sframes) {
+        const frames::StreamProgram &p = c->sp;
+        auto putv = [&](size_t o, const auto &v) { return put(o, v.data(), sizeof(v[0]) * v.size()); };
+        if ((e = putv(c->os_run, p.runs)) != cudaSuccess || (e = putv(c->os_member, p.members)) != cudaSuccess ||
+            (e = putv(c->os_ip, p.ips)) != cudaSuccess || (e = putv(c->os_perm, p.perms)) != cudaSuccess ||
+            (e = putv(c->os_uop, p.ops)) != cudaSuccess || (e = putv(c->os_entry, p.entry)) != cudaSuccess ||
+            (e = putv(c->os_col, c->scol)) != cudaSuccess || (e = putv(c->os_term, p.terms)) != cudaSuccess ||
+            (e = cudaMemsetAsync(c->ws + c->os_eacc, 0, 3 * sizeof(unsigned long long), c->stream)) != cudaSuccess ||
+            (e = cudaMemsetAsync(c->ws + c->os_etaexp, 0, sizeof(int32_t), c->stream)) != cudaSuccess ||
+            (e = frames::prepare_stream(c->precision)) != cudaSuccess)
+            return cuda_status(e);
+        const int scl = solve_cluster_log2(c->max_P);
+        if (scl >= 0 && (e = prepare_solve(solve_smem_bytes(c->max_P, scl))) != cudaSuccess) return cuda_status(e);
+        if (c->bsolve && (e = prepare_sblock(c->inst[0].P, c->bs_C)) != cudaSuccess) return cuda_status(e);
+        if (c->ir_C > 0 && (e = prepare_solve_ir(c->max_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
+        c->prepared = true;
+        return QNG_OK;
+    }
     if (c->streaming) {
         const large::Schedule &S = c->sched;
         if ((e = put(c->o_pdesc, S.passes.data(), sizeof(large::PassDesc) * S.passes.size())) != cudaSuccess) return cuda_status(e);
@@ -991,6 +1092,149 @@ int stream_class(const large::Launch &L) {
     }
 }
 
+// One launch of the walk: pass `pass` over columns [col0, col0 + ncol) of scol in slots 0..ncol-1.
+struct SLaunch { int pass, col0, ncol; bool store; };
+
+// The walk's launches over columns [first, end) of scol: batches of sslots columns, each through the
+// passes from the first one that a column of it starts in.
+std::vector<SLaunch> walk_launches(const qng_ctx *c, int first, int end) {
+    std::vector<SLaunch> out;
+    const int np = (int)c->sp.bwd.size(), R = (int)c->sp.runs.size();
+    auto start = [&](int k) { return c->scol[k].run == R ? 0 : c->sp.entry[c->scol[k].run].pass; };
+    for (int c0 = first; c0 < end; c0 += c->sslots) {
+        const int c1 = std::min(end, c0 + c->sslots);
+        for (int p = start(c0); p < np; ++p) {
+            int n = 0;
+            while (c0 + n < c1 && start(c0 + n) <= p) ++n;
+            out.push_back(SLaunch{p, c0, n, p + 1 < np});
+        }
+    }
+    return out;
+}
+
+// Work ranges of scol for the requested jobs: the gradient column comes first.
+void stream_range(const qng_ctx *c, int jobs, int &first, int &end) {
+    const bool metric = jobs & (kJobMetric | kJobSolve), grad = jobs & (kJobGradient | kJobSolve);
+    first = grad ? 0 : 1;
+    end = metric ? (int)c->scol.size() : std::min<int>(1, (int)c->scol.size());
+    if (first > end) first = end;
+}
+
+// The streaming instance on the diagonal-frame path.
+qng_status run_sframes(qng_ctx *c, int jobs, const double *theta, int64_t &launches) {
+    const HostInst &h = c->inst[0];
+    const frames::StreamProgram &p = c->sp;
+    const bool energy = jobs & (kJobEnergy | kJobGradient | kJobSolve);
+    const bool grad = jobs & (kJobGradient | kJobSolve), metric = jobs & (kJobMetric | kJobSolve);
+    const int im = (jobs & kJobMetricIm) ? 1 : 0;
+    const Work g = c->work();
+    frames::SWork w;
+    auto at = [&](size_t o) { return c->ws + o; };
+    w.run = reinterpret_cast<const frames::Run *>(at(c->os_run));
+    w.member = reinterpret_cast<const frames::Member *>(at(c->os_member));
+    w.ip = reinterpret_cast<const frames::SIp *>(at(c->os_ip));
+    w.perm = reinterpret_cast<const frames::SPerm *>(at(c->os_perm));
+    w.uop = reinterpret_cast<const frames::UOp *>(at(c->os_uop));
+    w.entry = reinterpret_cast<const frames::SEntry *>(at(c->os_entry));
+    w.col = reinterpret_cast<const frames::SCol *>(at(c->os_col));
+    w.term = reinterpret_cast<const DevTerm *>(at(c->os_term));
+    w.lo = at(c->os_lo);
+    w.hi = at(c->os_hi);
+    w.mask = reinterpret_cast<uint32_t *>(at(c->os_mask));
+    w.a = at(c->os_a);
+    w.b = at(c->os_b);
+    w.acc = reinterpret_cast<long long *>(at(c->os_acc));
+    w.sacc = reinterpret_cast<long long *>(at(c->os_sacc));
+    w.gacc = w.sacc + h.P;
+    w.eacc = reinterpret_cast<unsigned long long *>(at(c->os_eacc));
+    w.etaexp = reinterpret_cast<int32_t *>(at(c->os_etaexp));
+    w.bad = reinterpret_cast<int32_t *>(at(c->os_bad));
+    w.theta = theta;
+    w.status = g.status;
+    w.pctrl = g.pctrl;
+    w.sigma = g.sigma;
+    w.L = g.L;
+    w.Lim = g.Lim;
+    w.gradraw = g.gradraw;
+    w.energy = g.energy;
+    w.n = h.n;
+    w.P = h.P;
+    w.R = (int32_t)p.runs.size();
+    w.kb = p.kb;
+    w.tb = p.tb;
+    w.low = p.low;
+    w.hl = p.hl;
+    w.nterms = (int32_t)p.terms.size();
+    w.eexp = c->seexp;
+    w.hblocks = (int32_t)std::min<int64_t>((1ll << h.n) / 1024, 152 * 8);
+    cudaError_t e = timed(c, 0, [&] { return frames::launch_stream_tables(w, c->precision, c->stream); });
+    if (e != cudaSuccess) return cuda_status(e);
+    launches += 1;
+    const int vslot = c->sslots - 1;  // the forward vector; H psi goes to slot 0, the gradient column's
+    for (size_t k = 0; k < p.fwd.size(); ++k) {
+        e = timed(c, 1, [&] { return frames::launch_stream_forward(w, p.fwd[k], k == 0, vslot, c->precision, c->stream); });
+        if (e != cudaSuccess) return cuda_status(e);
+        ++launches;
+    }
+    if (energy) {
+        e = timed(c, 5, [&] { return frames::launch_stream_hpsi(w, vslot, 0, c->precision, c->stream); });
+        if (e != cudaSuccess) return cuda_status(e);
+        ++launches;
+    }
+    if (!metric && !grad) return QNG_OK;
+    const size_t PP = (size_t)h.P * h.P;
+    if ((metric && (e = cudaMemsetAsync(w.acc, 0, sizeof(int64_t) * PP * (im ? 2 : 1), c->stream)) != cudaSuccess) ||
+        (e = cudaMemsetAsync(w.sacc, 0, 2 * sizeof(int64_t) * (size_t)h.P, c->stream)) != cudaSuccess)
+        return cuda_status(e);
+    int first, end;
+    stream_range(c, jobs, first, end);
+    for (const SLaunch &L : walk_launches(c, first, end)) {
+        e = timed(c, metric ? 2 : 6, [&] {
+            return frames::launch_stream_walk(w, p.bwd[L.pass], L.pass, L.col0, L.ncol, L.store, c->precision, im, c->stream);
+        });
+        if (e != cudaSuccess) return cuda_status(e);
+        ++launches;
+    }
+    e = timed(c, 7, [&] {
+        return frames::launch_stream_finish(w, (metric ? 1 : 0) | (grad ? 2 : 0) | (im ? 4 : 0), c->precision, c->stream);
+    });
+    if (e != cudaSuccess) return cuda_status(e);
+    ++launches;
+    return QNG_OK;
+}
+
+// Per kernel class, the bytes one qng_step moves on that path: vectors loaded and stored and checkpoints
+// written by the passes, each launch of the walk reading a run's checkpoint once.
+void sframes_bytes(const qng_ctx *c, int64_t *b, int64_t *n) {
+    const int64_t reg = (int64_t)amp_bytes(c->precision) << c->inst[0].n;
+    auto runs_in = [&](const frames::SPass &ps) {
+        int64_t r = 0;
+        for (int o = 0; o < ps.nops; ++o) r += c->sp.ops[ps.op_begin + o].run >= 0;
+        return r;
+    };
+    b[0] += 0;
+    ++n[0];
+    for (size_t k = 0; k < c->sp.fwd.size(); ++k) {
+        b[1] += reg * ((k > 0) + 1 + runs_in(c->sp.fwd[k]));
+        ++n[1];
+    }
+    b[5] += 2 * reg;
+    ++n[5];
+    int first, end;
+    stream_range(c, kJobSolve, first, end);
+    const int R = (int)c->sp.runs.size();
+    for (const SLaunch &L : walk_launches(c, first, end)) {
+        int64_t loads = 0;
+        for (int k = 0; k < L.ncol; ++k) {
+            const int r = c->scol[L.col0 + k].run;
+            loads += r == R || c->sp.entry[r].pass < L.pass;
+        }
+        b[2] += reg * (loads + (L.store ? L.ncol : 0) + runs_in(c->sp.bwd[L.pass]));
+        ++n[2];
+    }
+    ++n[7];
+}
+
 // The streaming schedule's launches for the requested jobs.
 qng_status run_streaming(qng_ctx *c, int jobs, int64_t &launches) {
     const large::Schedule &S = c->sched;
@@ -1099,8 +1343,12 @@ qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
     int64_t launches = 0;
     cudaError_t e = cudaSuccess;
     const bool frames = c->frames && !c->streaming && !(jobs & kJobFromParts);
+    const bool sframes = c->streaming && c->sframes && !(jobs & kJobFromParts);
     if (frames) {
         qng_status st = run_frames(c, jobs, args.theta, launches);
+        if (st != QNG_OK) return st;
+    } else if (sframes) {
+        qng_status st = run_sframes(c, jobs, args.theta, launches);
         if (st != QNG_OK) return st;
     } else if (c->total_params > 0) {
         e = timed(c, 0, [&] { return launch_coef(w, args.theta, c->total_params, c->stream); });
@@ -1117,16 +1365,16 @@ qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
             (e = cudaMemcpyAsync(w.gradraw, args.parts_grad, P1, cudaMemcpyDeviceToDevice, c->stream)) != cudaSuccess)
             return cuda_status(e);
     }
-    const bool need_cols = !frames && !(jobs & kJobFromParts) && (jobs & (kJobMetric | kJobGradient | kJobSolve));
+    const bool need_cols = !frames && !sframes && !(jobs & kJobFromParts) && (jobs & (kJobMetric | kJobGradient | kJobSolve));
     const bool want_eta = jobs & (kJobGradient | kJobSolve);
-    if (c->streaming && !(jobs & kJobFromParts)) {
+    if (c->streaming && !sframes && !(jobs & kJobFromParts)) {
         qng_status st = run_streaming(c, jobs, launches);
         if (st != QNG_OK) return st;
     }
     const int wm = (jobs & (kJobMetric | kJobSolve)) ? 1 : 0;
     const int wg = (jobs & (kJobGradient | kJobSolve)) ? 1 : 0;
     const int wim = (jobs & kJobMetricIm) ? 1 : 0;
-    int S = (wm && !frames && !(jobs & kJobFromParts)) ? pipe_chunks(c) : 0;
+    int S = (wm && !frames && !sframes && !(jobs & kJobFromParts)) ? pipe_chunks(c) : 0;
     std::vector<int> K;
     std::vector<std::array<int, 2>> rng;
     if (S) {
@@ -1813,7 +2061,13 @@ qng_status qng_get_forward_cluster(const qng_ctx *c, int n_qubits, int *cluster_
 qng_status qng_stream_traffic(const qng_ctx *c, int64_t *metric_bytes, int64_t *other_bytes, int64_t *metric_passes) {
     if (!c) return QNG_ERR_ARG;
     int64_t mb = 0, ob = 0, mp = 0;
-    if (c->streaming) {
+    if (c->streaming && c->sframes) {
+        int64_t b[QNG_KERNEL_CLASSES] = {}, n[QNG_KERNEL_CLASSES] = {};
+        sframes_bytes(c, b, n);
+        mb = b[2];
+        mp = n[2];
+        for (int k = 0; k < QNG_KERNEL_CLASSES; ++k) ob += k == 2 ? 0 : b[k];
+    } else if (c->streaming) {
         const int64_t reg = (int64_t)amp_bytes(c->precision) << c->inst[0].n;
         for (const large::Launch &L : c->sched.launches) {
             if (L.kind != large::Launch::Pass) continue;
@@ -1832,7 +2086,9 @@ qng_status qng_stream_traffic(const qng_ctx *c, int64_t *metric_bytes, int64_t *
 qng_status qng_stream_segments(const qng_ctx *c, int64_t *bytes, int64_t *launches) {
     if (!c) return QNG_ERR_ARG;
     int64_t b[QNG_KERNEL_CLASSES] = {}, n[QNG_KERNEL_CLASSES] = {};
-    if (c->streaming) {
+    if (c->streaming && c->sframes) {
+        sframes_bytes(c, b, n);
+    } else if (c->streaming) {
         const int64_t reg = (int64_t)amp_bytes(c->precision) << c->inst[0].n;
         for (const large::Launch &L : c->sched.launches) {
             if (L.segment == large::kSegMetricIm) continue;  // a complex-metric call's, not a step's

@@ -1,0 +1,182 @@
+// Arithmetic of the diagonal-frame kernels, shared by the on-chip (qng_frames.cu) and streaming
+// (qng_frames_stream.cu) ones: the two amplitude types, their products and sums.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "qng_frames.h"
+
+namespace qng {
+namespace frames {
+
+typedef long long ll;
+
+struct Fix {  // complex128: fixed point
+    using A = longlong2;  // amplitude, 2^60 = 1
+    using S = int4;       // stored: (re hi, re lo, im hi, im lo), value = hi 2^32 + lo, lo signed
+    using Acc = ll;       // inner products, 2^60 = 1
+    using Red = ll;
+    using Eta = double2;  // H psi
+    static constexpr uint32_t kSwz = 7;  // eight 16-byte banks
+};
+struct Flt {  // complex64
+    using A = float2;
+    using S = float2;
+    using Acc = float;
+    using Red = double;
+    using Eta = float2;
+    static constexpr uint32_t kSwz = 15;  // sixteen 8-byte banks
+};
+
+__device__ __forceinline__ int hi_of(ll x) { return (int)((x + 0x80000000ll) >> 32); }
+__device__ __forceinline__ int lo_of(ll x) { return (int)x; }
+__device__ __forceinline__ ll join(int hi, int lo) { return ((ll)hi << 32) + lo; }
+__device__ __forceinline__ ll wide(int a, int b) { return (ll)a * (ll)b; }
+
+__device__ __forceinline__ int4 pack(longlong2 x) { return int4{hi_of(x.x), lo_of(x.x), hi_of(x.y), lo_of(x.y)}; }
+__device__ __forceinline__ float2 pack(float2 x) { return x; }
+__device__ __forceinline__ longlong2 unpack(int4 s) { return longlong2{join(s.x, s.y), join(s.z, s.w)}; }
+__device__ __forceinline__ float2 unpack(float2 s) { return s; }
+
+// c 2^-30 to nearest, halves away from zero: x d and (-x) d are negatives of each other, so states that
+// are symmetric stay exactly so (ties are common where x is a power of two)
+__device__ __forceinline__ ll round30(ll c) { return (c + ((1ll << 29) + (c >> 63))) >> 30; }
+
+// x d (CONJ = 0) or x conj(d); d is stored with 2^62 = 1
+template <int CONJ> __device__ __forceinline__ longlong2 mul(longlong2 x, int4 d, uint32_t dither = 0) {
+    const int rh = hi_of(x.x), rl = lo_of(x.x), ih = hi_of(x.y), il = lo_of(x.y);
+    // y_r = x_r c + x_i m, y_i = x_i c + x_r p with (m, p) = (-s, s), conjugate (s, -s)
+    const int mh = CONJ ? d.z : -d.z, ml = CONJ ? d.w : -d.w, ph = -mh, pl = -ml;
+    const ll h0 = wide(rh, d.x) + wide(ih, mh), h1 = wide(ih, d.x) + wide(rh, ph);
+    const ll c0 = wide(rh, d.y) + wide(rl, d.x) + wide(ih, ml) + wide(il, mh);
+    const ll c1 = wide(ih, d.y) + wide(il, d.x) + wide(rh, pl) + wide(rl, ph);
+    if (dither) {
+        const ll l0 = wide(rl, d.y) + wide(il, ml), l1 = wide(il, d.y) + wide(rl, pl);
+        return longlong2{(h0 << 2) + ((c0 + (l0 >> 32) + (ll)(dither >> 2)) >> 30),
+                         (h1 << 2) + ((c1 + (l1 >> 32) + (ll)((dither * 5u) >> 2)) >> 30)};
+    }
+    return longlong2{(h0 << 2) + round30(c0), (h1 << 2) + round30(c1)};
+}
+template <int CONJ> __device__ __forceinline__ float2 mul(float2 x, float2 d, uint32_t = 0) {
+    const float s = CONJ ? -d.y : d.y;
+    return float2{fmaf(x.x, d.x, -x.y * s), fmaf(x.x, s, x.y * d.x)};
+}
+
+// Re (IM = 0) or Im (IM = 1) of conj(a) b, lo lo included: at 2^12 amplitudes and more a product is
+// 2^-12 and less, and float64 would round it at 2^-65
+// UP: the operands' unit is 2^-(60 - UP), the product's 2^-60
+template <int IM, int UP = 0> __device__ __forceinline__ ll prod(int4 a, longlong2 b, uint32_t dither = 0) {
+    const int rh = hi_of(b.x), rl = lo_of(b.x), ih = hi_of(b.y), il = lo_of(b.y);
+    const ll rnd = dither ? (ll)(dither >> (4 + 2 * UP)) : 1ll << (27 - 2 * UP), half = 1ll << 31;  // to nearest: a product and its negative round alike
+    if constexpr (IM == 0) {
+        const ll h = wide(a.x, rh) + wide(a.z, ih);
+        const ll l = wide(a.y, rl) + wide(a.w, il) + half;
+        const ll c = wide(a.x, rl) + wide(a.y, rh) + wide(a.z, il) + wide(a.w, ih) + rnd + (l >> 32);
+        return (h << (4 + 2 * UP)) + (c >> (28 - 2 * UP));
+    } else {
+        const ll h = wide(a.x, ih) - wide(a.z, rh);
+        const ll l = wide(a.y, il) - wide(a.w, rl) + half;
+        const ll c = wide(a.x, il) + wide(a.y, ih) - wide(a.z, rl) - wide(a.w, rh) + rnd + (l >> 32);
+        return (h << (4 + 2 * UP)) + (c >> (28 - 2 * UP));
+    }
+}
+template <int IM, int UP = 0> __device__ __forceinline__ float prod(float2 a, float2 b, uint32_t = 0) {
+    return IM ? fmaf(a.x, b.y, -a.y * b.x) : fmaf(a.x, b.x, a.y * b.y);
+}
+
+__device__ __forceinline__ longlong2 operator+(longlong2 a, longlong2 b) { return longlong2{a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ longlong2 operator-(longlong2 a, longlong2 b) { return longlong2{a.x - b.x, a.y - b.y}; }
+// both components of a complex64 amplitude in one instruction
+__device__ __forceinline__ float2 operator+(float2 a, float2 b) {
+    float2 r;
+    asm("{.reg .b64 x, y;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 x, x, y;\n mov.b64 {%0, %1}, x;}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 operator-(float2 a, float2 b) {  // fma(b, -1, a) rounds once, as a - b does
+    float2 r;
+    asm("{.reg .b64 x, y, m;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mov.b64 m, 0xbf800000bf800000;\n"
+        " fma.rn.f32x2 x, y, m, x;\n mov.b64 {%0, %1}, x;}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
+// x 2^-s to nearest, ties to even. Rounding down instead would put the same -1/2 unit on every component:
+// a constant vector, and states can overlap with that one (22 qubits: g off by 6e-13 instead of 1e-15).
+__device__ __forceinline__ void halve(longlong2 &x, int s) {
+    const ll h = (1ll << (s - 1)) - 1;
+    x.x = (x.x + (h + (((int)x.x >> s) & 1))) >> s;
+    x.y = (x.y + (h + (((int)x.y >> s) & 1))) >> s;
+}
+
+__device__ __forceinline__ ll shfl(ll v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ float shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+
+// Warp sums of 8 values: the lane returns the sum of a[(lane >> 2) & 7].
+template <typename T> __device__ __forceinline__ T warp8(const T (&a)[8], int lane) {
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+    T t[4], u[2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t[k] = (b4 ? a[4 + k] : a[k]) + shfl(b4 ? a[k] : a[4 + k], 16);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) u[k] = (b3 ? t[2 + k] : t[k]) + shfl(b3 ? t[k] : t[2 + k], 8);
+    T v = (b2 ? u[1] : u[0]) + shfl(b2 ? u[0] : u[1], 4);
+    v += shfl(v, 2);
+    v += shfl(v, 1);
+    return v;
+}
+
+// Hadamards (unnormalised) on the thread's bits hm, then `shift` halvings in fixed point.
+template <class T, int KB> __device__ __forceinline__ void hadamards(typename T::A (&b)[1 << KB], int hm, int shift) {
+#pragma unroll
+    for (int j = 0; j < KB; ++j)
+        if ((hm >> j) & 1) {
+#pragma unroll
+            for (int k = 0; k < (1 << KB); ++k)
+                if (!((k >> j) & 1)) {
+                    const typename T::A x = b[k], y = b[k | (1 << j)];
+                    b[k] = x + y;
+                    b[k | (1 << j)] = x - y;
+                }
+        }
+    if constexpr (sizeof(typename T::A) == 16) {
+        if (shift) {
+#pragma unroll
+            for (int k = 0; k < (1 << KB); ++k) halve(b[k], shift);
+        }
+    }
+}
+
+__device__ __forceinline__ void store_factor(int4 *d, longlong2 f) {
+    ll y = f.y << 1;
+    // the low half of the sine is negated by the product: keep it off -2^31
+    if ((int)y == INT32_MIN) ++y;
+    *d = pack(longlong2{f.x << 1, y});
+}
+__device__ __forceinline__ void store_factor(float2 *d, longlong2 f) {
+    *d = float2{(float)f.x * 0x1p-61f, (float)f.y * 0x1p-61f};
+}
+
+__device__ __forceinline__ double2 amp_of(longlong2 x) { return double2{(double)x.x * 0x1p-60, (double)x.y * 0x1p-60}; }
+__device__ __forceinline__ double2 amp_of(float2 x) { return double2{(double)x.x, (double)x.y}; }
+
+__device__ __forceinline__ longlong2 seed(double2 e, double up) {  // -i eta
+    return longlong2{__double2ll_rn(e.y * up), __double2ll_rn(-e.x * up)};
+}
+__device__ __forceinline__ float2 seed(float2 e, double) { return float2{e.y, -e.x}; }
+
+template <class T, int KB> struct Sums {  // of the thread's products: all, and signed by each of its bits
+    typename T::Acc all, bit[KB];
+};
+
+template <class T, int KB> __device__ __forceinline__ typename T::Acc pick(const Sums<T, KB> &s, int z) {
+    typename T::Acc v = s.all;
+#pragma unroll
+    for (int j = 0; j < KB; ++j) if (z == (1 << j)) v = s.bit[j];
+    return v;
+}
+
+}  // namespace frames
+}  // namespace qng

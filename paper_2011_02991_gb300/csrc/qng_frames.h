@@ -65,7 +65,7 @@ struct UOp {
     int16_t low;    // -1: no exchange
     int16_t hm;
     int16_t shift;
-    int16_t pad;
+    int16_t rshift; // halvings right before the run (streaming)
     int32_t perm;   // -1: none
     int32_t run;
 };
@@ -177,6 +177,89 @@ struct Program {  // one instance, host side
 // Indices in the program (members, perms) are relative to its own tables.
 void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks,
                    const std::vector<qng_pauli> &terms, int n, int kb, int cl, Program &out);
+
+// ------------------------------------------------------------------------------------------
+// Streaming: one instance whose vectors lie in global memory. A pass loads tiles of 2^tb amplitudes (the
+// low bits and a window of tb - low consecutive others), runs its steps on each and stores them.
+// A run's factor on amplitude m is lo[m mod 2^hl] hi[m >> hl] (-1)^parity(m & mask[m >> hl]).
+struct SIp {
+    uint32_t zall, z;  // the qubit's bit; the same unless a warp's own sums resolve it
+    int16_t sgn;
+    int16_t src;       // which warp sum of the products: 0 all, 1 + j signed by the thread's bit j,
+                       // 8 + j signed by lane bit j
+};
+
+struct SPerm {         // gather within a tile: local source index
+    uint32_t limg[16]; // image of each local bit
+    uint32_t oimg[32]; // what a set bit outside the tile adds
+};
+
+struct SPass {
+    int32_t s;         // first bit of the window
+    int32_t load_low;  // arrangement the tile is loaded in
+    int32_t op_begin, nops;
+    int32_t run0;      // its first run, -1 without one
+    int32_t shift;     // halvings of the fixed-point vector when it is stored
+};
+
+struct SEntry {        // where the walk's columns of a run start
+    int32_t pass, op, low, pad;
+};
+
+struct SCol {          // a column: its parameter (P: the gradient column) and its run (R: the gradient's)
+    int32_t col, run;
+};
+
+struct StreamProgram {
+    int n = 0, kb = 4, tb = 12, low = 2, hl = 0;
+    std::vector<Run> runs;
+    std::vector<Member> members;
+    std::vector<SIp> ips;
+    std::vector<SPerm> perms;
+    std::vector<UOp> ops;
+    std::vector<SPass> fwd, bwd;
+    std::vector<SEntry> entry;
+    std::vector<DevTerm> terms;
+};
+
+constexpr int kStreamTileBits[2] = {13, 12};  // complex64, complex128: 64 KiB
+constexpr int kStreamRegBits[2] = {5, 4};
+void build_stream(const std::vector<qng_gate> &gates, const std::vector<qng_pauli> &terms, int n, int kb, int tb, int low,
+                  StreamProgram &out);
+
+struct SWork {
+    const Run *run;
+    const Member *member;
+    const SIp *ip;
+    const SPerm *perm;
+    const UOp *uop;
+    const SEntry *entry;
+    const SCol *col;
+    const DevTerm *term;
+    void *lo, *hi;            // factor tables, 2^hl and 2^(n-hl) entries per run
+    uint32_t *mask;           // 2^(n-hl) per run
+    void *a;                  // checkpoints, natural order, 2^n per run
+    void *b;                  // column slots, 2^n each
+    long long *acc;           // (P x P) sums of the metric, twice that with Im, in units of 2^-60
+    long long *sacc, *gacc;   // <sigma_j>; the gradient, units of 2^(etaexp - 60)
+    unsigned long long *eacc; // as in FWork
+    int32_t *etaexp;
+    const double *theta;
+    int32_t *status, *bad;
+    double *pctrl, *sigma, *L, *Lim, *gradraw, *energy;
+    int32_t n, P, R, kb, tb, low, hl, nterms, eexp, hblocks;
+};
+
+cudaError_t prepare_stream(int precision);
+cudaError_t launch_stream_tables(const SWork &w, int precision, cudaStream_t st);
+cudaError_t launch_stream_forward(const SWork &w, const SPass &p, int first, int slot, int precision, cudaStream_t st);
+// Pass p of the walk over ncol columns col[col0 ..], column k in slot k.
+cudaError_t launch_stream_walk(const SWork &w, const SPass &p, int pass, int col0, int ncol, int store, int precision,
+                               int metric_im, cudaStream_t st);
+// H psi: slot `in` -> slot `out`, and <E>.
+cudaError_t launch_stream_hpsi(const SWork &w, int in, int out, int precision, cudaStream_t st);
+// Sums to float64: what = 1 metric, 2 gradient (bits), 4 with Im.
+cudaError_t launch_stream_finish(const SWork &w, int what, int precision, cudaStream_t st);
 
 }  // namespace frames
 }  // namespace qng

@@ -5,7 +5,7 @@
 // v. It is kept as the signed Paulis C_q^dag X C_q and C_q^dag Z C_q: a gate's generator on qubit q
 // acts on v through these images.
 #include <algorithm>
-#include <cstring>
+#include <cstdlib>
 
 #include "qng_frames.h"
 
@@ -34,30 +34,30 @@ SP conj_sdg(SP a) { return a.p == PX ? SP{PY, -a.s} : (a.p == PY ? SP{PX, a.s} :
 
 // Linear map of index bits, as the images of the basis vectors.
 struct Lin {
-    uint32_t img[16];
-    Lin() { for (int b = 0; b < 16; ++b) img[b] = 1u << b; }
+    uint32_t img[kMaxQubits];
+    Lin() { for (int b = 0; b < kMaxQubits; ++b) img[b] = 1u << b; }
     uint32_t operator()(uint32_t m) const {
         uint32_t r = 0;
-        for (int b = 0; b < 16; ++b) if ((m >> b) & 1) r ^= img[b];
+        for (int b = 0; b < kMaxQubits; ++b) if ((m >> b) & 1) r ^= img[b];
         return r;
     }
     // mask z' with parity(m & z') = parity(A m & z)
     uint32_t pull(uint32_t z) const {
         uint32_t r = 0;
-        for (int b = 0; b < 16; ++b) r |= (uint32_t)(__builtin_popcount(img[b] & z) & 1) << b;
+        for (int b = 0; b < kMaxQubits; ++b) r |= (uint32_t)(__builtin_popcount(img[b] & z) & 1) << b;
         return r;
     }
     Lin inverse() const {
-        uint32_t a[16];
+        uint32_t a[kMaxQubits];
         Lin inv;
-        for (int b = 0; b < 16; ++b) a[b] = img[b];
+        for (int b = 0; b < kMaxQubits; ++b) a[b] = img[b];
         // column operations: reduce a to the identity, the same operations on inv
-        for (int b = 0; b < 16; ++b) {
+        for (int b = 0; b < kMaxQubits; ++b) {
             int p = b;
             while (!((a[p] >> b) & 1)) ++p;
             std::swap(a[p], a[b]);
             std::swap(inv.img[p], inv.img[b]);
-            for (int k = 0; k < 16; ++k)
+            for (int k = 0; k < kMaxQubits; ++k)
                 if (k != b && ((a[k] >> b) & 1)) { a[k] ^= a[b]; inv.img[k] ^= inv.img[b]; }
         }
         return inv;
@@ -68,6 +68,7 @@ struct Stage {
     bool perm = false;
     uint32_t h = 0;  // Hadamards (perm = false)
     Lin map;         // new index of old index m is map(m) (perm = true)
+    std::vector<std::pair<int, int>> cnots;  // the gates of the map, (control, target)
 };
 
 struct Builder {
@@ -157,7 +158,8 @@ struct Builder {
         if (!open().empty()) close();
         if (otau().empty() || !otau().back().perm) { otau().emplace_back(); otau().back().perm = true; }
         Lin &A = otau().back().map;
-        for (int b = 0; b < 16; ++b) A.img[b] ^= ((A.img[b] >> c) & 1u) << t;
+        for (int b = 0; b < kMaxQubits; ++b) A.img[b] ^= ((A.img[b] >> c) & 1u) << t;
+        otau().back().cnots.push_back({c, t});
         // the frames of c and t are Paulis X^a Z^b: X_c -> X_c X_t, Z_t -> Z_c Z_t
         fr[t].z.s *= fr[c].z.s;
         fr[c].x.s *= fr[t].x.s;
@@ -173,15 +175,8 @@ std::vector<std::pair<int, int>> string_req(uint64_t x, uint64_t z, int n) {
     return r;
 }
 
-}  // namespace
-
-void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks,
-                   const std::vector<qng_pauli> &terms, int n, int kb, int cl, Program &out) {
-    out = Program();
-    out.n = n;
-    out.kb = kb;
-    const int nE = out.nE = std::max(n, kb);
-    Builder B(n);
+// The circuit's gates, in order, into runs and transitions.
+void walk_gates(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks, int n, Builder &B) {
     for (size_t gi = 0; gi < gates.size(); ++gi) {
         const qng_gate &g = gates[gi];
         Frame *f = (g.q0 >= 0 && g.q0 < n) ? &B.fr[g.q0] : nullptr;
@@ -206,6 +201,39 @@ void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_
         default: break;
         }
     }
+}
+
+// The Hamiltonian in the final frame, terms grouped by X mask.
+std::vector<DevTerm> final_terms(const std::vector<qng_pauli> &terms, int n, const Builder &B) {
+    std::vector<DevTerm> out;
+    for (const qng_pauli &t : terms) {
+        DevTerm d = {};
+        d.coeff = t.coeff;
+        for (int q = 0; q < n; ++q) {
+            const int hx = (int)((t.xmask >> q) & 1), hz = (int)((t.zmask >> q) & 1);
+            if (!hx && !hz) continue;
+            const SP im = B.fr[q].image(hx ? (hz ? kAxisY : kAxisX) : kAxisZ);
+            if (im.s < 0) d.coeff = -d.coeff;
+            if (im.p != PZ) d.x |= 1ull << q;
+            if (im.p != PX) d.z |= 1ull << q;
+        }
+        d.ny = __builtin_popcountll(d.x & d.z) & 3;
+        out.push_back(d);
+    }
+    std::stable_sort(out.begin(), out.end(), [](const DevTerm &a, const DevTerm &b) { return a.x < b.x; });
+    return out;
+}
+
+}  // namespace
+
+void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks,
+                   const std::vector<qng_pauli> &terms, int n, int kb, int cl, Program &out) {
+    out = Program();
+    out.n = n;
+    out.kb = kb;
+    const int nE = out.nE = std::max(n, kb);
+    Builder B(n);
+    walk_gates(gates, masks, n, B);
     // Without members left, a last transition that holds Hadamards still needs a run to carry their
     // normalisation; one of permutations alone, or an empty one, does not.
     bool last_h = false;
@@ -330,7 +358,7 @@ void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_
                     // gather: forward new[m] = old[A^-1 m], adjoint new[m] = old[A m]
                     const Lin A = back ? maps[s.perm] : maps[s.perm].inverse();
                     Perm p;
-                    std::memcpy(p.img, A.img, sizeof(p.img));
+                    std::copy(A.img, A.img + 16, p.img);
                     u.perm = (int32_t)out.perms.size();
                     out.perms.push_back(p);
                 }
@@ -362,22 +390,225 @@ void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_
     }
     if (R > 0) fuse(cut, true, out.bwd);
 
-    // the Hamiltonian in the final frame
-    for (const qng_pauli &t : terms) {
-        DevTerm d = {};
-        d.coeff = t.coeff;
-        for (int q = 0; q < n; ++q) {
-            const int hx = (int)((t.xmask >> q) & 1), hz = (int)((t.zmask >> q) & 1);
-            if (!hx && !hz) continue;
-            const SP im = B.fr[q].image(hx ? (hz ? kAxisY : kAxisX) : kAxisZ);
-            if (im.s < 0) d.coeff = -d.coeff;
-            if (im.p != PZ) d.x |= 1ull << q;
-            if (im.p != PX) d.z |= 1ull << q;
+    out.terms = final_terms(terms, n, B);
+}
+
+// ------------------------------------------------------------------------------------------
+// Streaming: vectors in global memory, passes over tiles of 2^tb amplitudes.
+namespace {
+
+struct Atom { int kind, q, c, run; };  // 0 Hadamard on q; 1 CNOT c -> q; 2 run
+
+struct Window { int low, s, w; };
+bool holds(const Window &W, int q) { return q < W.low || (q >= W.s && q < W.s + W.w); }
+
+// The atoms of the list (those not done) that a pass over window W can execute: in order, each one
+// whose pair qubit the window holds and that no skipped atom shares a qubit with.
+std::vector<int> executable(const std::vector<Atom> &at, const std::vector<uint8_t> &done, size_t from, const Window &W) {
+    std::vector<int> ex;
+    uint32_t blocked = 0;
+    for (size_t k = from; k < at.size(); ++k) {
+        if (done[k]) continue;
+        const Atom &a = at[k];
+        if (a.kind == 2) {
+            if (blocked) break;
+            ex.push_back((int)k);
+            continue;
         }
-        d.ny = __builtin_popcountll(d.x & d.z) & 3;
-        out.terms.push_back(d);
+        const uint32_t m = (1u << a.q) | (a.kind == 1 ? 1u << a.c : 0u);
+        if (!(m & blocked) && holds(W, a.q)) ex.push_back((int)k);
+        else blocked |= m;
     }
-    std::stable_sort(out.terms.begin(), out.terms.end(), [](const DevTerm &a, const DevTerm &b) { return a.x < b.x; });
+    return ex;
+}
+
+void pack_passes(const std::vector<Atom> &at, bool back, StreamProgram &P, std::vector<SPass> &out) {
+    const int n = P.n, kb = P.kb, tb = P.tb;
+    std::vector<Window> wins;
+    wins.push_back(Window{P.low, P.low, tb - P.low});  // the lowest tb bits
+    for (int s = tb; s < n; s += tb - P.low) wins.push_back(Window{P.low, std::min(s, n - (tb - P.low)), tb - P.low});
+    std::vector<int> lows;
+    for (int lo = 0; lo + kb <= tb; lo += kb) lows.push_back(lo);
+    if (tb % kb) lows.push_back(tb - kb);
+    auto block_of = [&](int b) {
+        for (int lo : lows) if (b >= lo && b < lo + kb) return lo;
+        return lows.back();
+    };
+    std::vector<uint8_t> done(at.size(), 0);
+    size_t from = 0;
+    // Hadamards since the last run, and halvings of the fixed-point vector (once three are due, at a run and at
+    // the end of a pass): floor(k / 2) in all, the odd sqrt 1/2 is in the run's factor. Between them the
+    // vector grows to 2^4.5 of its norm at most (two halvings due, an odd Hadamard, a block of four more)
+    int k = 0, halved = 0;
+    while (from < at.size()) {
+        std::vector<int> best;
+        Window W = wins[0];
+        for (const Window &w : wins) {
+            std::vector<int> ex = executable(at, done, from, w);
+            if (ex.size() > best.size()) { best = ex; W = w; }
+        }
+        SPass ps = {};
+        ps.run0 = -1;
+        ps.s = W.s;
+        ps.op_begin = (int32_t)P.ops.size();
+        auto local = [&](int q) { return q < W.low ? q : q - W.s + W.low; };
+        int cur = -1;
+        UOp u{-1, 0, 0, 0, -1, -1};
+        int stage = 0;
+        auto flush = [&]() { if (stage) { P.ops.push_back(u); u = UOp{-1, 0, 0, 0, -1, -1}; stage = 0; } };
+        auto goto_low = [&](int lo, int perm) {
+            if (cur < 0 && perm < 0) { cur = lo; ps.load_low = lo; return; }
+            if (cur < 0) { cur = lows.back(); ps.load_low = cur; }
+            if (cur == lo && perm < 0) return;
+            flush();
+            u.low = (int16_t)lo;
+            u.perm = perm;
+            stage = 1;
+            cur = lo;
+        };
+        for (size_t i = 0; i < best.size();) {
+            const Atom &a = at[best[i]];
+            if (a.kind == 0) {
+                uint32_t h = 0;  // over local bits
+                while (i < best.size() && at[best[i]].kind == 0) h ^= 1u << local(at[best[i++]].q);
+                std::vector<int> bl;
+                for (int b = 0; b < tb; ++b) if ((h >> b) & 1) { const int lo = block_of(b); if (!std::count(bl.begin(), bl.end(), lo)) bl.push_back(lo); }
+                // the current block first, block 0 next, the others last: runs, loads and stores want their
+                // low bits on the threads
+                std::vector<int> ord;
+                if (cur < 0) { if (*std::max_element(bl.begin(), bl.end()) > 0) ord.push_back(*std::max_element(bl.begin(), bl.end())); }
+                else if (std::count(bl.begin(), bl.end(), cur)) ord.push_back(cur);
+                if (std::count(bl.begin(), bl.end(), 0) && !std::count(ord.begin(), ord.end(), 0)) ord.push_back(0);
+                for (int lo : bl) if (!std::count(ord.begin(), ord.end(), lo)) ord.push_back(lo);
+                for (int lo : ord) {
+                    if (cur < 0 && lo == 0) goto_low(lows.back(), -1);
+                    goto_low(lo, -1);
+                    uint32_t m = 0;
+                    for (int b = 0; b < tb; ++b) if (((h >> b) & 1) && block_of(b) == lo) m |= 1u << (b - lo);
+                    if (stage > 1) flush();
+                    u.hm = (int16_t)m;
+                    k += __builtin_popcount(m);
+                    if (k / 2 - halved >= 3) {
+                        u.shift = (int16_t)(k / 2 - halved);
+                        halved = k / 2;
+                    }
+                    stage = 2;
+                }
+            } else if (a.kind == 1) {
+                Lin A;  // new index of old index m is A(m): the pass's CNOTs in the order they run
+                while (i < best.size() && at[best[i]].kind == 1) {
+                    const Atom &c = at[best[i++]];
+                    for (int b = 0; b < kMaxQubits; ++b) A.img[b] ^= ((A.img[b] >> c.c) & 1u) << c.q;
+                }
+                const Lin inv = A.inverse();  // gather: new[m] = old[A^-1 m]
+                SPerm p = {};
+                for (int b = 0; b < n; ++b) {
+                    uint32_t l = 0;
+                    for (int q = 0; q < n; ++q) if (((inv.img[b] >> q) & 1) && holds(W, q)) l |= 1u << local(q);
+                    if (holds(W, b)) p.limg[local(b)] = l;
+                    else p.oimg[b] = l;
+                }
+                P.perms.push_back(p);
+                goto_low(cur > 0 ? cur : lows.back(), (int)P.perms.size() - 1);
+            } else {
+                if (cur <= 0 && lows.back() > 0) goto_low(lows.back(), -1);
+                else if (cur < 0) goto_low(lows.back(), -1);
+                u.run = a.run;
+                if (ps.run0 < 0) ps.run0 = a.run;
+                stage = 3;
+                if (back) {
+                    P.entry[a.run] = SEntry{(int32_t)out.size(), (int32_t)P.ops.size() - ps.op_begin, cur, 0};
+                    // parameters of the run: which of the thread's bits, if any, each one's qubit is here
+                    Run &rn = P.runs[a.run];
+                    rn.low = cur;
+                    for (int x = 0; x < rn.ip_count; ++x) {
+                        SIp &ip = P.ips[rn.ip_begin + x];
+                        const int q = __builtin_ctz(ip.zall), lb = holds(W, q) ? local(q) : -1;
+                        const int th = lb < cur ? lb : lb - kb;  // its bit of the thread index
+                        ip.src = 0;
+                        if (lb >= cur && lb < cur + kb) ip.src = (int16_t)(1 + lb - cur);
+                        else if (lb >= 0 && th < 5 && th < tb - kb) ip.src = (int16_t)(8 + th);
+                        ip.z = ip.src ? 0u : ip.zall;
+                    }
+                }
+                u.rshift = (int16_t)(k / 2 - halved);
+                flush();
+                k = halved = 0;
+                ++i;
+            }
+        }
+        if (cur <= 0 && lows.back() > 0) goto_low(lows.back(), -1);
+        flush();
+        ps.shift = k / 2 - halved;
+        halved = k / 2;
+        ps.nops = (int32_t)P.ops.size() - ps.op_begin;
+        out.push_back(ps);
+        for (int x : best) done[x] = 1;
+        while (from < at.size() && done[from]) ++from;
+    }
+}
+
+}  // namespace
+
+void build_stream(const std::vector<qng_gate> &gates, const std::vector<qng_pauli> &terms, int n, int kb, int tb, int low,
+                  StreamProgram &out) {
+    out = StreamProgram();
+    out.n = n;
+    out.kb = kb;
+    out.tb = tb;
+    out.low = low;
+    // halves of the factor tables: the second window's first bit, so that (but for narrow windows) the thread's
+    // bits at a run lie in one half
+    out.hl = std::min(tb, n - 1);
+    if (n > tb && n - (tb - low) < tb) out.hl = n - (tb - low);
+    Builder B(n);
+    walk_gates(gates, {}, n, B);
+    bool last_h = false;
+    for (const Stage &s : B.otau()) last_h = last_h || (!s.perm && s.h);
+    std::vector<Stage> tail;
+    if (B.open().empty() && !last_h) {
+        tail = B.otau();
+        B.run_members.pop_back();
+        B.tau.pop_back();
+    }
+    const int R = (int)B.run_members.size();
+    std::vector<Atom> fwd;
+    auto add_tau = [&](const std::vector<Stage> &t) {
+        for (const Stage &s : t) {
+            if (s.perm) for (auto &c : s.cnots) fwd.push_back(Atom{1, c.second, c.first, -1});
+            else for (int q = 0; q < n; ++q) if ((s.h >> q) & 1) fwd.push_back(Atom{0, q, -1, -1});
+        }
+    };
+    for (int r = 0; r < R; ++r) {
+        add_tau(B.tau[r]);
+        fwd.push_back(Atom{2, -1, -1, r});
+        Run run = {};
+        run.mem_begin = (int)out.members.size();
+        run.mem_count = (int)B.run_members[r].size();
+        run.ip_begin = (int)out.ips.size();
+        run.ip_first = -1;
+        for (const Stage &s : B.tau[r]) if (!s.perm) run.khalf += __builtin_popcount(s.h);
+        for (const Member &m : B.run_members[r]) {
+            out.members.push_back(m);
+            if (m.kind != 0) continue;
+            if (run.ip_first < 0) run.ip_first = m.param;
+            out.ips.push_back(SIp{m.z, m.z, (int16_t)m.sgn, 0});
+        }
+        run.ip_count = (int)out.ips.size() - run.ip_begin;
+        if (run.ip_first < 0) run.ip_first = 0;
+        out.runs.push_back(run);
+    }
+    add_tau(tail);
+    std::vector<Atom> bwd;
+    for (auto it = fwd.rbegin(); it != fwd.rend(); ++it) {
+        bwd.push_back(*it);
+        if (it->kind == 2 && it->run == 0) break;
+    }
+    out.entry.assign(R, SEntry{0, 0, 0, 0});
+    pack_passes(fwd, false, out, out.fwd);
+    if (out.fwd.empty()) out.fwd.push_back(SPass{low, tb - kb, 0, 0, -1, 0});  // no gate that moves |0...0>
+    if (R > 0) pack_passes(bwd, true, out, out.bwd);
+    out.terms = final_terms(terms, n, B);
 }
 
 }  // namespace frames

@@ -4,7 +4,8 @@
 // Hadamards on a thread's own bits, runs), and prints
 //   E <energy>, grad <P values>, L <re im> for i < j, sigma <P values>, ctrl <P values>
 // Structural invariants are checked on the way ("bad <what>", exit 1).
-// Input (stdin): n P G T kb cl, G lines "kind q0 q1 param xmask zmask", T lines "coeff x z", P angles.
+// The same for the streaming program (tiles of 2^tb amplitudes, `low` contiguous low bits) when tb > 0.
+// Input (stdin): n P G T kb cl tb low, G lines "kind q0 q1 param xmask zmask", T lines "coeff x z", P angles.
 #include <cmath>
 #include <complex>
 #include <cstdio>
@@ -22,9 +23,153 @@ static void bad(const char *what, long a, long b) {
     std::exit(1);
 }
 
+static cd member_factor(const std::vector<Member> &mem, const Run &rn, const std::vector<double> &th, uint32_t m) {
+    cd f = std::pow(0.5, 0.5 * rn.khalf);
+    for (int k = 0; k < rn.mem_count; ++k) {
+        const Member &e = mem[rn.mem_begin + k];
+        const int par = __builtin_popcount(m & e.z) & 1;
+        const double lam = par ? -e.sgn : e.sgn;
+        if (e.kind == 2) { if (par) f *= cd(0, -1); continue; }
+        if ((m & e.ctrl) != e.cval) continue;
+        f *= e.kind == 1 ? cd(lam) : cd(std::cos(th[e.param] / 2), -lam * std::sin(th[e.param] / 2));
+    }
+    return f;
+}
+
+static void print_all(double E, const std::vector<double> &grad, const std::vector<double> &sig, const std::vector<double> &ctrl,
+                      const std::vector<cd> &Lm, int P, int R) {
+    std::printf("E %.17g\nruns %d\n", E, R);
+    auto vec = [&](const char *nm, const std::vector<double> &x) {
+        std::printf("%s", nm);
+        for (double t : x) std::printf(" %.17g", t);
+        std::printf("\n");
+    };
+    vec("grad", grad);
+    vec("sigma", sig);
+    vec("ctrl", ctrl);
+    std::printf("L");
+    for (int j = 0; j < P; ++j) for (int i = 0; i < j; ++i) std::printf(" %.17g %.17g", Lm[(size_t)i * P + j].real(), Lm[(size_t)i * P + j].imag());
+    std::printf("\nok\n");
+}
+
+static int stream(const std::vector<qng_gate> &gates, const std::vector<qng_pauli> &terms, const std::vector<double> &th, int n,
+                  int P, int kb, int tb, int lowbits) {
+    StreamProgram pr;
+    build_stream(gates, terms, n, kb, tb, lowbits, pr);
+    const uint32_t N = 1u << n;
+    const int R = (int)pr.runs.size(), w = tb - lowbits;
+    int low = -1;
+    auto local = [&](const SPass &ps, uint32_t m) { return (m & ((1u << lowbits) - 1)) | (((m >> ps.s) & ((1u << w) - 1)) << lowbits); };
+    auto global = [&](const SPass &ps, uint32_t l) { return (l & ((1u << lowbits) - 1)) | ((l >> lowbits) << ps.s); };
+    auto move = [&](std::vector<cd> &v, const SPass &ps, const UOp &u) {
+        if (u.low >= 0) {
+            low = u.low;
+            if (u.perm >= 0) {
+                std::vector<cd> x(N);
+                for (uint32_t m = 0; m < N; ++m) {
+                    const uint32_t l = local(ps, m), out = m & ~global(ps, (1u << tb) - 1);
+                    uint32_t s = 0;
+                    for (int b = 0; b < tb; ++b) if ((l >> b) & 1) s ^= pr.perms[u.perm].limg[b];
+                    for (int b = 0; b < n; ++b) if ((out >> b) & 1) s ^= pr.perms[u.perm].oimg[b];
+                    if (s >> tb) bad("perm", m, s);
+                    x[m] = v[out | global(ps, s)];
+                }
+                v.swap(x);
+            }
+        }
+        if (low < 0 || low + kb > tb || ps.s + w > n || (ps.s > lowbits && ps.s < tb && ps.s + w != n)) bad("arrangement", low, ps.s);
+        for (int b = 0; b < kb; ++b)
+            if ((u.hm >> b) & 1) {
+                const uint32_t bit = global(ps, 1u << (low + b));
+                for (uint32_t m = 0; m < N; ++m)
+                    if (!(m & bit)) {
+                        const cd x = v[m], y = v[m | bit];
+                        v[m] = x + y;
+                        v[m | bit] = x - y;
+                    }
+            }
+    };
+    std::vector<std::vector<cd>> psi(R);
+    std::vector<cd> v(N, 0.0);
+    v[0] = 1;
+    int last = -1;
+    for (const SPass &ps : pr.fwd) {
+        low = ps.load_low;
+        if (low == 0 && tb > kb) bad("load", low, 0);
+        for (int o = 0; o < ps.nops; ++o) {
+            const UOp &u = pr.ops[ps.op_begin + o];
+            move(v, ps, u);
+            if (u.run < 0) continue;
+            if (u.run != last + 1) bad("run order", u.run, last);
+            last = u.run;
+            double nrm = 0;
+            for (uint32_t m = 0; m < N; ++m) nrm += std::norm(v[m] *= member_factor(pr.members, pr.runs[u.run], th, m));
+            if (std::fabs(nrm - 1) > 1e-9) bad("norm", u.run, (long)(nrm * 1e6));
+            psi[u.run] = v;
+        }
+    }
+    if (last != R - 1) bad("forward end", last, R);
+    std::vector<cd> eta(N, 0.0);
+    double E = 0;
+    for (const DevTerm &t : pr.terms)
+        for (uint32_t m = 0; m < N; ++m) {
+            const uint32_t s = m ^ (uint32_t)t.x;
+            eta[m] += t.coeff * std::pow(cd(0, 1), (t.ny + 2 * (__builtin_popcount(s & (uint32_t)t.z) & 1)) & 3) * v[s];
+        }
+    for (uint32_t m = 0; m < N; ++m) E += std::real(std::conj(v[m]) * eta[m]);
+    std::vector<cd> Lm((size_t)P * P, 0.0), p(N);
+    std::vector<double> sig(P, 0.0), ctrl(P, 1.0), grad(P, 0.0);
+    auto ip_of = [&](const SPass &ps, const SIp &ip) {  // the kernel's split: the thread's own bit, or an index bit
+        const int th = ip.src >= 8 ? ip.src - 8 : -1;
+        const uint32_t own = ip.src == 0 ? 0u : global(ps, 1u << (th < 0 ? low + ip.src - 1 : (th < low ? th : th + kb)));
+        if ((own | ip.z) != ip.zall || (own && ip.z)) bad("parameter bits", ip.zall, own);
+        cd s = 0;
+        for (uint32_t m = 0; m < N; ++m) s += ((m & (own | ip.z)) != 0) != (ip.sgn < 0) ? -p[m] : p[m];
+        return s;
+    };
+    auto walk = [&](std::vector<cd> b, int col, int run) {
+        const size_t p0 = run == R ? 0 : pr.entry[run].pass;
+        for (size_t k = p0; k < pr.bwd.size(); ++k) {
+            const SPass &ps = pr.bwd[k];
+            low = ps.load_low;
+            const bool st = run < R && k == p0;
+            for (int o = st ? pr.entry[run].op : 0; o < ps.nops; ++o) {
+                const UOp &u = pr.ops[ps.op_begin + o];
+                const bool own = st && o == pr.entry[run].op;
+                if (own) low = pr.entry[run].low;
+                else move(b, ps, u);
+                if (own && u.run != run) bad("entry", run, u.run);
+                if (u.run < 0) continue;
+                if (low == 0 && tb > kb) bad("run in block 0", u.run, 0);
+                const Run &rn = pr.runs[u.run];
+                for (uint32_t m = 0; m < N; ++m) p[m] = std::conj(psi[u.run][m]) * b[m];
+                for (int q = 0; q < rn.ip_count; ++q) {
+                    const cd x = ip_of(ps, pr.ips[rn.ip_begin + q]);
+                    const int i = rn.ip_first + q;
+                    if (run == R) grad[i] = -std::imag(x);
+                    else if (i < col) Lm[(size_t)i * P + col] = 0.25 * x;
+                }
+                if (own) { cd s = 0; for (const cd &x : p) s += x; sig[col] = std::real(s); }
+                for (uint32_t m = 0; m < N; ++m) b[m] *= std::conj(member_factor(pr.members, rn, th, m));
+            }
+        }
+    };
+    for (int r = 0; r < R; ++r)
+        for (int c = 0; c < pr.runs[r].ip_count; ++c) {
+            const SIp &ip = pr.ips[pr.runs[r].ip_begin + c];
+            std::vector<cd> b(N);
+            for (uint32_t m = 0; m < N; ++m) b[m] = ((m & ip.zall) != 0) != (ip.sgn < 0) ? -psi[r][m] : psi[r][m];
+            walk(b, pr.runs[r].ip_first + c, r);
+        }
+    walk(eta, P, R);
+    std::printf("passes %d %d\n", (int)pr.fwd.size(), (int)pr.bwd.size());
+    print_all(E, grad, sig, ctrl, Lm, P, R);
+    return 0;
+}
+
 int main() {
-    int n, P, G, T, kb, cl;
-    if (std::scanf("%d %d %d %d %d %d", &n, &P, &G, &T, &kb, &cl) != 6) return 2;
+    int n, P, G, T, kb, cl, tb, lowbits;
+    if (std::scanf("%d %d %d %d %d %d %d %d", &n, &P, &G, &T, &kb, &cl, &tb, &lowbits) != 8) return 2;
     std::vector<qng_gate> gates(G);
     std::vector<uint64_t> masks(2 * G);
     for (int g = 0; g < G; ++g) {
@@ -42,6 +187,7 @@ int main() {
     }
     std::vector<double> th(P);
     for (double &t : th) if (std::scanf("%lf", &t) != 1) return 2;
+    if (tb > 0) return stream(gates, terms, th, n, P, kb, tb, lowbits);
     Program pr;
     build_program(gates, masks, terms, n, kb, cl, pr);
     const uint32_t N = 1u << pr.nE;
@@ -108,7 +254,6 @@ int main() {
             eta[m] += t.coeff * f * v[s];
         }
     for (uint32_t m = 0; m < N; ++m) E += std::real(std::conj(v[m]) * eta[m]);
-    std::printf("E %.17g\n", E);
     // a parameter's inner product read off p as the column kernel does: thread index and own bits
     auto ip_of = [&](const Ip &ip, int L, const std::vector<cd> &p) {
         cd s = 0;
@@ -171,17 +316,6 @@ int main() {
         }
         for (uint32_t m = 0; m < N; ++m) eta[m] *= std::conj(factor(u.run, m));
     }
-    std::printf("runs %d\n", R);
-    auto vec = [&](const char *nm, const std::vector<double> &x) {
-        std::printf("%s", nm);
-        for (double t : x) std::printf(" %.17g", t);
-        std::printf("\n");
-    };
-    vec("grad", grad);
-    vec("sigma", sig);
-    vec("ctrl", ctrl);
-    std::printf("L");
-    for (int j = 0; j < P; ++j) for (int i = 0; i < j; ++i) std::printf(" %.17g %.17g", Lm[(size_t)i * P + j].real(), Lm[(size_t)i * P + j].imag());
-    std::printf("\nok\n");
+    print_all(E, grad, sig, ctrl, Lm, P, R);
     return 0;
 }

@@ -28,9 +28,9 @@ def probe(tmp_path_factory):
     return exe
 
 
-def run_probe(exe, p, kb=4, cl=0):
+def run_probe(exe, p, kb=4, cl=0, tb=0, low=0):
     c, h = p.circuit, p.hamiltonian
-    lines = [f"{c.n} {c.num_params} {len(c.gates)} {h.num_terms} {kb} {cl}"]
+    lines = [f"{c.n} {c.num_params} {len(c.gates)} {h.num_terms} {kb} {cl} {tb} {low}"]
     for row, m in zip(c.gates, c.gate_masks()):
         lines.append(" ".join(str(int(v)) for v in row) + f" {int(m[0])} {int(m[1])}")
     lines += [f"{float(a)!r} {int(x)} {int(z)}" for a, x, z in zip(h.coeffs, h.xmask, h.zmask)]
@@ -41,8 +41,8 @@ def run_probe(exe, p, kb=4, cl=0):
     return {x.split()[0]: np.array([float(v) for v in x.split()[1:]]) for x in out if " " in x or x in ("L", "grad")}
 
 
-def check(exe, oracle, p, kb=4, cl=0):
-    d = run_probe(exe, p, kb, cl)
+def check(exe, oracle, p, kb=4, cl=0, tb=0, low=0):
+    d = run_probe(exe, p, kb, cl, tb, low)
     ref = oracle.qng_step(p)
     P = p.P
     tol = 1e-11
@@ -95,3 +95,24 @@ def test_z_runs_and_no_parameters(probe, oracle):
     c = W.Circuit(3, np.array([[W.H, 0, -1, -1], [W.CNOT, 0, 2, -1], [W.Y, 1, -1, -1], [W.CZ, 0, 1, -1]], dtype=np.int32))
     h = W.hamiltonian_from_terms([(0.5, {0: "X", 2: "X"}), (0.25, {1: "Z"}), (-1.5, {0: "Y", 2: "Y"})])
     check(probe, oracle, W.Problem("fixed", c, h, np.zeros(0)))
+
+
+@pytest.mark.parametrize("n,kb,tb,low", [(7, 3, 5, 2), (9, 3, 6, 3), (8, 3, 7, 3), (9, 4, 6, 1), (10, 3, 6, 3), (6, 4, 6, 2)])
+@pytest.mark.parametrize("seed", range(4))
+def test_streaming_passes(probe, oracle, n, kb, tb, low, seed):
+    """Passes over tiles: one to four windows over the index bits, CNOTs whose control lies outside the
+    tile, runs that start in the middle of a pass."""
+    check(probe, oracle, W.random_problem(n, 60, 6, 5000 + seed), kb, 0, tb, low)
+
+
+@pytest.mark.parametrize("kinds,ent", [((W.RY, W.RZ), W.CZ), ((W.RY, W.RX, W.RZ), W.CNOT)])
+def test_streaming_layered(probe, oracle, kinds, ent):
+    """Two windows over the index bits: one pass per run, and one more per CNOT ladder."""
+    n = 9
+    c = W.layered_ansatz(n, 2, kinds, ent)
+    rng = np.random.Generator(np.random.PCG64(4))
+    p = W.Problem("l", c, W.random_pauli_hamiltonian(n, 9, rng), W.uniform_theta(c.num_params, rng))
+    d = check(probe, oracle, p, 3, 0, 6, 3)
+    assert d["passes"][1] <= d["runs"][0] + (2 if ent == W.CNOT else 0)
+    fixed = W.Circuit(6, np.array([[W.H, 0, -1, -1], [W.Z, 2, -1, -1]], dtype=np.int32))
+    check(probe, oracle, W.Problem("fixed", fixed, W.tfim_chain(6, 1.0, 0.3), np.zeros(0)), 3, 0, 5, 2)
