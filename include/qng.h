@@ -349,7 +349,8 @@ qng_status qng_step_from_parts(qng_ctx *ctx, const double *theta, const double *
  *   QNG_SOLVE_CLUSTER  one thread-block cluster per instance, float64 Cholesky
  *   QNG_SOLVE_MIXED    float32 Cholesky and float64 iterative refinement; an instance whose
  *                      float32 factorisation breaks down, or whose refinement does not reach
- *                      1e-10 of |dtheta|, is handed over to the float64 cluster solve
+ *                      1e-10 of |dtheta|, is handed over to the float64 cluster solve; instances
+ *                      of a batch too large for it go there directly (not counted)
  *   QNG_SOLVE_BLOCK    one instance with P beyond the cluster solve, blocked float64 Cholesky
  * *handed_over counts the instances the mixed-precision solve handed over (0 for the others).
  * After a mixed-precision solve it waits for the context's stream (one 4-byte-per-instance

@@ -163,6 +163,7 @@ struct qng_ctx {
     size_t os_hi = 0, os_mask = 0, os_a = 0, os_b = 0, os_acc = 0, os_sacc = 0, os_eacc = 0, os_etaexp = 0, os_bad = 0;
     // mixed-precision solve: cluster size (0 = not used: P < 48 or its float32 matrix does not fit)
     int ir_C = 0;
+    int ir_P = 0;  // the largest P it takes
     size_t o_irflag = 0;
     // block solve (one instance whose P is beyond the cluster solve's shared memory)
     bool bsolve = false;
@@ -728,11 +729,19 @@ qng_status plan(qng_ctx *c) {
     c->total_metric = c->metric_off[c->count];
     c->streaming = c->count == 1 && (c->path == 2 || (c->path == 0 && c->inst[0].n > kMaxQubitsSmall));
     if (c->streaming && c->inst[0].general) return QNG_ERR_UNSUPPORTED;  // generalised rotations: on-chip only
-    // mixed-precision solve where the cluster solve is there to take over
-    c->ir_C = 0;
+    // Mixed-precision solve where the cluster solve is there to take over: for every instance of a batch
+    // that it fits, on 4 CTAs each (CTA 0 does the serial part; fewer CTAs per instance leave room for
+    // more instances at once), the others go to the cluster solve. Beyond 222 parameters, where only the
+    // packed triangle fits, batches alone take it (they wait for the slowest instance: 64 instances of
+    // 6 to 14 qubits 0.86 ms with the float64 solve for their largest, 0.33 ms with this one).
+    c->ir_C = c->ir_P = 0;
     if (c->max_P >= kBlockSolveMinP && solve_cluster_log2(c->max_P) >= 0) {
-        const int C = c->max_P >= 128 ? 8 : 4;
-        if (solve_ir_smem_bytes(c->max_P, C) <= kMaxSmem) c->ir_C = C;
+        const int C = c->count == 1 && c->max_P >= 128 ? 8 : 4;
+        for (const HostInst &h : c->inst)
+            if (h.P >= kBlockSolveMinP &&
+                (c->count > 1 || !solve_ir_packed(h.P, C)) && solve_ir_smem_bytes(h.P, C) + 1200 <= kMaxSmem)  // and 1168 static
+                c->ir_P = std::max(c->ir_P, h.P);
+        if (c->ir_P > 0) c->ir_C = C;
     }
     // the block solve takes over where the cluster solve's rows no longer fit in shared memory
     c->bsolve = false;
@@ -916,7 +925,7 @@ qng_status upload(qng_ctx *c) {
         const int scl = solve_cluster_log2(c->max_P);
         if (scl >= 0 && (e = prepare_solve(solve_smem_bytes(c->max_P, scl))) != cudaSuccess) return cuda_status(e);
         if (c->bsolve && (e = prepare_sblock(c->inst[0].P, c->bs_C)) != cudaSuccess) return cuda_status(e);
-        if (c->ir_C > 0 && (e = prepare_solve_ir(c->max_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
+        if (c->ir_C > 0 && (e = prepare_solve_ir(c->ir_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
         c->prepared = true;
         return QNG_OK;
     }
@@ -949,7 +958,7 @@ qng_status upload(qng_ctx *c) {
         const int scl = solve_cluster_log2(c->max_P);
         if (scl >= 0 && (e = prepare_solve(solve_smem_bytes(c->max_P, scl))) != cudaSuccess) return cuda_status(e);
         if (c->bsolve && (e = prepare_sblock(c->inst[0].P, c->bs_C)) != cudaSuccess) return cuda_status(e);
-        if (c->ir_C > 0 && (e = prepare_solve_ir(c->max_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
+        if (c->ir_C > 0 && (e = prepare_solve_ir(c->ir_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
         c->prepared = true;
         return QNG_OK;
     }
@@ -983,7 +992,7 @@ qng_status upload(qng_ctx *c) {
     const int scl = solve_cluster_log2(c->max_P);
     if (scl >= 0 && (e = prepare_solve(solve_smem_bytes(c->max_P, scl))) != cudaSuccess) return cuda_status(e);
     if (c->bsolve && (e = prepare_sblock(c->inst[0].P, c->bs_C)) != cudaSuccess) return cuda_status(e);
-    if (c->ir_C > 0 && (e = prepare_solve_ir(c->max_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
+    if (c->ir_C > 0 && (e = prepare_solve_ir(c->ir_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
     // streams and events of the pipelined sweep (single instance) and of the launch groups side by
     // side (batches), made here so that no stream is created inside a graph capture
     if (!c->pipe_ready) {
@@ -1481,7 +1490,7 @@ qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
     } else if ((jobs & kJobSolve) && scl >= 0 && c->ir_C > 0) {
         // mixed precision first; the float64 cluster solve takes any instance it hands over
         e = timed(c, 3, [&] {
-            cudaError_t r = launch_solve_ir(w, c->count, c->max_P, c->ir_C, a, c->stream);
+            cudaError_t r = launch_solve_ir(w, c->count, c->ir_P, c->ir_C, a, c->stream);
             if (r != cudaSuccess) return r;
             LaunchArgs ag = a;
             ag.ir_gate = 1;
@@ -2167,7 +2176,7 @@ qng_status qng_solve_report(qng_ctx *c, int *path, int32_t *handed_over) {
                                     cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_status(e);
-    for (int32_t f : flag) *handed_over += f != 0;
+    for (int32_t f : flag) *handed_over += f == 1;  // (2: beyond its size, never tried)
     return QNG_OK;
 }
 

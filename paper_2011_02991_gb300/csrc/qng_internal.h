@@ -223,6 +223,7 @@ cudaError_t launch_sblock(const Work &w, const LaunchArgs &a, int P, int C, int 
 cudaError_t launch_sback(const Work &w, const LaunchArgs &a, int P, cudaStream_t st);
 // mixed-precision solve (qng_solve_ir.cu): one cluster of C CTAs per instance
 size_t solve_ir_smem_bytes(int P, int C);
+bool solve_ir_packed(int P, int C);  // only the lower triangle of the float32 matrix is kept
 cudaError_t prepare_solve_ir(int P, int C);
 cudaError_t launch_solve_ir(const Work &w, int count, int max_P, int C, const LaunchArgs &a, cudaStream_t st);
 cudaError_t launch_solve(const Work &w, int count, int max_P, int cl, const LaunchArgs &a, cudaStream_t st);

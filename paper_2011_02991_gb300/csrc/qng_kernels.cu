@@ -1297,7 +1297,126 @@ __device__ __forceinline__ void column_item(const Work &w, const DevWork wk, int
 }
 
 // ------------------------------------------------------------------------------------------
-// k_finish: one CTA per instance. Assembly of g (Eq. g_t_L_def with L_ii = 1/4 and
+// k_assemble: the outputs of calls without a solve. G_ij = L_ij - T_i^* T_j (Eq. g_t_L_def) with L_ii = <C_i>/4
+// and T_k = -(i/2) sigma_k; Im G = Im L (T_i^* T_j is real). One CTA per 32 x 32 tile of the upper triangle:
+// L is read along its rows and both g tiles are written along theirs (one CTA per instance, reading the
+// lower half down the columns, took 58 us for P = 99 against 7 us here).
+__global__ void __launch_bounds__(256) k_assemble(Work w, LaunchArgs a) {
+    __shared__ double tr[32][33], ti[32][33];
+    const int b = blockIdx.x, tile = blockIdx.y;  // instances along x, which has no 16-bit limit
+    const DevInst &in = w.inst[b];
+    const int P = in.P, T = (P + 31) / 32;
+    const double *sg = w.sigma + in.param_off;
+    const bool metric = a.jobs & kJobMetric, im = (a.jobs & kJobMetricIm) && a.gim_out;
+    const int tid = threadIdx.x;
+    if (tile == 0) {
+        if (metric && a.sigma_out)
+            for (int k = tid; k < P; k += 256) a.sigma_out[in.param_off + k] = sg[k];
+        if ((a.jobs & kJobGradient) && a.grad_out) {
+            const double gs = a.grad_scale ? a.grad_scale[b] : 1.0;
+            for (int k = tid; k < P; k += 256) a.grad_out[in.param_off + k] = gs * w.gradraw[in.param_off + k];
+        }
+        if ((a.jobs & (kJobGradient | kJobEnergy)) && a.energy_out && tid == 0) a.energy_out[b] = w.energy[b];
+    }
+    if (!metric || tile >= T * (T + 1) / 2) return;
+    int bi = 0, rest = tile;  // tile row bi, tile column bj >= bi
+    while (rest >= T - bi) { rest -= T - bi; ++bi; }
+    const int bj = bi + rest, i0 = bi * 32, j0 = bj * 32;
+    const double *L = w.L + in.metric_off, *Li = w.Lim + in.metric_off, *pc = w.pctrl + in.param_off;
+    for (int y = tid >> 5; y < 32; y += 8) {
+        const int x = tid & 31, i = i0 + y, j = j0 + x;
+        double v = 0.0, u = 0.0;
+        if (i < P && j < P) {
+            if (i < j) {
+                v = L[(int64_t)i * P + j] - 0.25 * sg[i] * sg[j];
+                if (im) u = Li[(int64_t)i * P + j];
+            } else if (i == j) {
+                v = 0.25 * (pc[i] - sg[i] * sg[i]);
+            }
+            if (i <= j) {
+                if (a.g_out) a.g_out[in.metric_off + (int64_t)i * P + j] = v;
+                if (im) a.gim_out[in.metric_off + (int64_t)i * P + j] = i < j ? u : 0.0;
+            }
+        }
+        tr[y][x] = v;
+        ti[y][x] = u;
+    }
+    __syncthreads();
+    for (int y = tid >> 5; y < 32; y += 8) {  // the mirrored tile, row j0 + y
+        const int x = tid & 31, j = j0 + y, i = i0 + x;
+        if (j < P && i < j && i < P) {
+            if (a.g_out) a.g_out[in.metric_off + (int64_t)j * P + i] = tr[x][y];
+            if (im) a.gim_out[in.metric_off + (int64_t)j * P + i] = -ti[x][y];
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------
+// k_small: assembly and solve of instances with P < 48, one CTA each, everything in shared memory. A = g +
+// lambda I is factored as L D L^T by right-looking updates with the right-hand side as one more row, so the
+// forward substitution comes with it; every thread takes the pivot's reciprocal itself, and a pivot costs
+// one barrier. Latency-bound: a reciprocal (about 370 cycles) and two dependent float64 operations per
+// pivot (P = 16: 40 us with the matrix in device memory and five barriers a pivot, 11 us here).
+constexpr int kSmallP = 48;
+__global__ void __launch_bounds__(128) k_small(Work w, LaunchArgs a) {
+    __shared__ double A[kSmallP + 1][kSmallP + 1];  // row P: the right-hand side
+    __shared__ double inv[kSmallP];
+    const int b = blockIdx.x, tid = threadIdx.x;
+    const DevInst &in = w.inst[b];
+    const int P = in.P;
+    const double *sg = w.sigma + in.param_off;
+    const double *pc = w.pctrl + in.param_off;
+    const double *L = w.L + in.metric_off;
+    const double *gr = w.gradraw + in.param_off;
+    for (int t = tid; t < P * P; t += 128) {
+        const int i = t / P, j = t % P;
+        double v;
+        if (i == j) v = 0.25 * (pc[i] - sg[i] * sg[i]);
+        else v = L[i < j ? i * P + j : j * P + i] - 0.25 * sg[i] * sg[j];
+        if (a.g_out) a.g_out[in.metric_off + t] = v;
+        A[i][j] = v + (i == j ? a.lambda : 0.0);
+    }
+    for (int k = tid; k < P; k += 128) {
+        A[P][k] = -a.dt * gr[k];
+        if (a.sigma_out) a.sigma_out[in.param_off + k] = sg[k];
+        if (a.grad_out) a.grad_out[in.param_off + k] = (a.grad_scale ? a.grad_scale[b] : 1.0) * gr[k];
+    }
+    if (a.energy_out && tid == 0) a.energy_out[b] = w.energy[b];
+    __syncthreads();
+    const int tx = tid & 15, ty = tid >> 4;
+    for (int k = 0; k < P; ++k) {
+        const double d = A[k][k];
+        if (!(d > 0.0)) {  // the same value in every thread
+            if (tid == 0) atomicCAS(w.status, 0, (int)QNG_ERR_NOT_SPD);
+            return;
+        }
+        const double iv = 1.0 / d;
+        if (tid == 0) inv[k] = iv;
+        for (int j = k + 1 + tx; j < P; j += 16) {
+            const double lj = A[j][k] * iv;
+            for (int i = k + 1 + ty; i <= P; i += 8)
+                if (i >= j) A[i][j] = fma(-A[i][k], lj, A[i][j]);
+        }
+        __syncthreads();
+    }
+    if (tid >= 32) return;
+    // x_k = (y_k - sum_{i > k} A_ik x_i) / d_k, last row first: lane l holds y_l and y_{l + 32}
+    double y0 = tid < P ? A[P][tid] : 0.0, y1 = tid + 32 < P ? A[P][tid + 32] : 0.0;
+    for (int k = P - 1; k >= 0; --k) {
+        const double xk = __shfl_sync(0xffffffffu, k < 32 ? y0 : y1, k & 31) * inv[k];
+        if (tid == (k & 31)) {
+            if (k < 32) y0 = xk;
+            else y1 = xk;
+        }
+        if (tid < k) y0 = fma(-A[k][tid], xk, y0);
+        if (tid + 32 < k) y1 = fma(-A[k][tid + 32], xk, y1);
+    }
+    if (tid < P) a.dtheta_out[in.param_off + tid] = y0;
+    if (tid + 32 < P) a.dtheta_out[in.param_off + tid + 32] = y1;
+}
+
+// ------------------------------------------------------------------------------------------
+// k_finish: one CTA per instance, P beyond the cluster solve. Assembly of g (Eq. g_t_L_def with L_ii = <C_i>/4 and
 // T_k = -(i/2) sigma_k), outputs, and the Cholesky solve of (g + lambda I) dtheta = -dt grad.
 __global__ void __launch_bounds__(512) k_finish(Work w, LaunchArgs a) {
     __shared__ double sh[2];
@@ -1308,35 +1427,22 @@ __global__ void __launch_bounds__(512) k_finish(Work w, LaunchArgs a) {
     const double *sg = w.sigma + in.param_off;
     const double *pc = w.pctrl + in.param_off;  // <C_i>: the diagonal L_ii = <C_i>/4 (Sec. 2)
     const double *L = w.L + in.metric_off;
-    const bool metric = a.jobs & (kJobMetric | kJobSolve);
     double *A = w.chol + in.metric_off;
-    if (metric) {
-        for (int64_t idx = threadIdx.x; idx < (int64_t)P * P; idx += blockDim.x) {
-            const int i = (int)(idx / P), j = (int)(idx % P);
-            double v;
-            if (i == j) v = 0.25 * (pc[i] - sg[i] * sg[i]);
-            else if (i < j) v = L[(int64_t)i * P + j] - 0.25 * sg[i] * sg[j];
-            else v = L[(int64_t)j * P + i] - 0.25 * sg[i] * sg[j];
-            if (a.g_out) a.g_out[in.metric_off + idx] = v;
-            if (a.jobs & kJobSolve) A[idx] = v + (i == j ? a.lambda : 0.0);
-        }
-        if ((a.jobs & kJobMetricIm) && a.gim_out) {  // Im G = Im L: T_i^* T_j is real; Hermitian
-            const double *Li = w.Lim + in.metric_off;
-            for (int64_t idx = threadIdx.x; idx < (int64_t)P * P; idx += blockDim.x) {
-                const int i = (int)(idx / P), j = (int)(idx % P);
-                a.gim_out[in.metric_off + idx] = i < j ? Li[(int64_t)i * P + j] : (i > j ? -Li[(int64_t)j * P + i] : 0.0);
-            }
-        }
-        if (a.sigma_out)
-            for (int k = threadIdx.x; k < P; k += blockDim.x) a.sigma_out[in.param_off + k] = sg[k];
+    for (int64_t idx = threadIdx.x; idx < (int64_t)P * P; idx += blockDim.x) {
+        const int i = (int)(idx / P), j = (int)(idx % P);
+        double v;
+        if (i == j) v = 0.25 * (pc[i] - sg[i] * sg[i]);
+        else if (i < j) v = L[(int64_t)i * P + j] - 0.25 * sg[i] * sg[j];
+        else v = L[(int64_t)j * P + i] - 0.25 * sg[i] * sg[j];
+        if (a.g_out) a.g_out[in.metric_off + idx] = v;
+        A[idx] = v + (i == j ? a.lambda : 0.0);
     }
-    if (a.jobs & kJobGradient) {
-        const double gs = a.grad_scale ? a.grad_scale[b] : 1.0;
-        if (a.grad_out)
-            for (int k = threadIdx.x; k < P; k += blockDim.x) a.grad_out[in.param_off + k] = gs * w.gradraw[in.param_off + k];
+    for (int k = threadIdx.x; k < P; k += blockDim.x) {
+        if (a.sigma_out) a.sigma_out[in.param_off + k] = sg[k];
+        if (a.grad_out) a.grad_out[in.param_off + k] = (a.grad_scale ? a.grad_scale[b] : 1.0) * w.gradraw[in.param_off + k];
     }
-    if ((a.jobs & (kJobGradient | kJobEnergy)) && a.energy_out && threadIdx.x == 0) a.energy_out[b] = w.energy[b];
-    if (!(a.jobs & kJobSolve) || P == 0) return;
+    if (a.energy_out && threadIdx.x == 0) a.energy_out[b] = w.energy[b];
+    if (P == 0) return;
     __syncthreads();
     // right-looking Cholesky, lower triangle, in place
     if (threadIdx.x == 0) bad = 0;
@@ -1785,8 +1891,14 @@ cudaError_t launch_solve(const Work &w, int count, int max_P, int cl, const Laun
 }
 
 cudaError_t launch_finish(const Work &w, int count, int max_P, const LaunchArgs &a, cudaStream_t st) {
-    const int t = max_P >= 128 ? 512 : 128;
-    k_finish<<<count, t, 0, st>>>(w, a);
+    if (!(a.jobs & kJobSolve)) {
+        const int T = (max_P + 31) / 32, tiles = (a.jobs & kJobMetric) ? T * (T + 1) / 2 : 1;
+        k_assemble<<<dim3(count, tiles > 0 ? tiles : 1), 256, 0, st>>>(w, a);
+    } else if (max_P < kSmallP) {
+        k_small<<<count, 128, 0, st>>>(w, a);
+    } else {
+        k_finish<<<count, max_P >= 128 ? 512 : 128, 0, st>>>(w, a);
+    }
     return cudaGetLastError();
 }
 

@@ -38,7 +38,7 @@ constexpr int kIrMaxIter = 12; // refinement steps at most
 
 struct IrGeom {
     int P, C, R;     // rows of A per CTA of rank >= 1
-    int ld;          // row stride of the float32 matrix
+    int ld;          // row stride of the float32 matrix; 0: its lower triangle packed by rows
     int Pp;          // P rounded up to 16 (row length of the transposed panel)
     size_t o_xt, o_di, o_y, o_x;  // float offsets in CTA 0's shared memory
     size_t smem;
@@ -46,15 +46,17 @@ struct IrGeom {
 
 __host__ __device__ inline size_t up4(size_t x) { return (x + 3) & ~(size_t)3; }
 
-__host__ __device__ inline IrGeom ir_geom(int P, int C) {
+// packed = 1 keeps the lower triangle of the float32 matrix only. For a given form the bytes grow with
+// P; every instance of a launch uses the same form, so the launch's largest P sizes its shared memory.
+__host__ __device__ inline IrGeom ir_geom(int P, int C, int packed) {
     IrGeom g;
     g.P = P;
     g.C = C;
     g.R = (P + C - 2) / (C - 1);
-    g.ld = P + 1;
+    g.ld = packed ? 0 : P + 1;
     g.Pp = (P + kIb - 1) / kIb * kIb;
     const int nblk = (P + kIb - 1) / kIb;
-    g.o_xt = up4((size_t)P * g.ld);                  // Lm [P][ld]
+    g.o_xt = up4(packed ? (size_t)P * (P + 1) / 2 : (size_t)P * g.ld);  // Lm
     g.o_di = g.o_xt + (size_t)kIb * g.Pp;             // Xt [16][Pp], 16-byte aligned rows
     g.o_y = g.o_di + (size_t)nblk * kIb * kIb;        // Di [nblk][16][16]
     g.o_x = up4(g.o_y + (size_t)P);                   // yv [P]; then float64 x, r
@@ -64,16 +66,19 @@ __host__ __device__ inline IrGeom ir_geom(int P, int C) {
     return g;
 }
 
-// One warp: the diagonal block at (k0, k0) of the float32 matrix (row stride ld), already updated
+// Offset of row i of the float32 matrix.
+__device__ __forceinline__ size_t ir_row(int i, int ld) { return ld ? (size_t)i * ld : (size_t)i * (i + 1) / 2; }
+
+// One warp: a diagonal block of the float32 matrix (rowp: the lane's row of it), already updated
 // by every earlier panel, with nb <= 16 real rows (the rest padded with the identity) -> its
 // Cholesky factor L_K in place and L_K^-1 in D (16 x 16, zero past nb). Lane r holds row r; a
 // column takes one rsqrt, and 1/L_cc = rsqrt(d) also serves the inverse. False if a pivot is not
 // positive.
-__device__ __noinline__ bool chol_diag16(float *Lm, int ld, int k0, int nb, float *D, int lane) {
+__device__ __noinline__ bool chol_diag16(float *rowp, int nb, float *D, int lane) {
     float row[kIb], rdiag[kIb];
 #pragma unroll
     for (int c = 0; c < kIb; ++c)
-        row[c] = (lane < nb) ? (c <= lane ? Lm[(size_t)(k0 + lane) * ld + k0 + c] : 0.0f) : (lane == c ? 1.0f : 0.0f);
+        row[c] = (lane < nb) ? (c <= lane ? rowp[c] : 0.0f) : (lane == c ? 1.0f : 0.0f);
     bool bad = false;
 #pragma unroll
     for (int c = 0; c < kIb; ++c) {
@@ -92,7 +97,7 @@ __device__ __noinline__ bool chol_diag16(float *Lm, int ld, int k0, int nb, floa
     if (lane < nb) {
 #pragma unroll
         for (int c = 0; c < kIb; ++c)
-            if (c <= lane) Lm[(size_t)(k0 + lane) * ld + k0 + c] = row[c];
+            if (c <= lane) rowp[c] = row[c];
     }
     // lane c (mod 16) forms column c of L_K^-1 by forward substitution, rows taken from the warp
     const int c = lane & (kIb - 1);
@@ -113,9 +118,10 @@ __device__ __noinline__ bool chol_diag16(float *Lm, int ld, int k0, int nb, floa
 
 }  // namespace
 
-size_t solve_ir_smem_bytes(int P, int C) { return ir_geom(P, C).smem + 64; }
+bool solve_ir_packed(int P, int C) { return ir_geom(P, C, 0).smem + 64 > kMaxSmem; }
+size_t solve_ir_smem_bytes(int P, int C) { return ir_geom(P, C, solve_ir_packed(P, C)).smem + 64; }
 
-__global__ void __launch_bounds__(512, 1) k_solve_ir(Work w, LaunchArgs a) {
+__global__ void __launch_bounds__(512, 1) k_solve_ir(Work w, LaunchArgs a, int max_P, int packed) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_fail, s_done;
     __shared__ double s_est;
@@ -126,7 +132,11 @@ __global__ void __launch_bounds__(512, 1) k_solve_ir(Work w, LaunchArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nwarp = blockDim.x >> 5, nt = blockDim.x;
     const DevInst in = w.inst[b];
     const int P = in.P;
-    const IrGeom G = ir_geom(P, C);
+    if (P > max_P) {  // an instance of a batch whose float32 matrix does not fit: the float64 solve's
+        if (rank == 0 && tid == 0) w.irflag[b] = 2;
+        return;
+    }
+    const IrGeom G = ir_geom(P, C, packed);
     const int nblk = (P + kIb - 1) / kIb;
     const double *sg = w.sigma + in.param_off;
     const double *pc = w.pctrl + in.param_off;
@@ -150,19 +160,19 @@ __global__ void __launch_bounds__(512, 1) k_solve_ir(Work w, LaunchArgs a) {
     cl.sync();  // every CTA runs before the first distributed shared memory store
 
     // (A) assembly (Eq. g_t_L_def): float64 rows in CTAs >= 1, g for those rows, and the float32
-    // lower triangle pushed to CTA 0
+    // lower triangle pushed to CTA 0; four reads of L in flight
     if (rank > 0) {
         float *L0 = cl.map_shared_rank(Lm, 0);
-        for (int t = tid; t < (r1 - r0) * P; t += nt) {
+        const int n = (r1 - r0) * P;
+#pragma unroll 4
+        for (int t = tid; t < n; t += nt) {
             const int il = t / P, j = t % P, i = r0 + il;
-            double v;
-            if (i == j) v = 0.25 * (pc[i] - sg[i] * sg[i]);
-            else if (i < j) v = L[(int64_t)i * P + j] - 0.25 * sg[i] * sg[j];
-            else v = L[(int64_t)j * P + i] - 0.25 * sg[i] * sg[j];
+            const double l = L[(int64_t)min(i, j) * P + max(i, j)];  // (the diagonal's value is not used)
+            double v = (i == j ? 0.25 * pc[i] : l) - 0.25 * sg[i] * sg[j];
             if (a.g_out) a.g_out[in.metric_off + (int64_t)i * P + j] = v;
             v += (i == j ? a.lambda : 0.0);
             Arow[t] = v;
-            if (j <= i) L0[(size_t)i * G.ld + j] = (float)v;
+            if (j <= i) L0[ir_row(i, G.ld) + j] = (float)v;
         }
     }
     cl.sync();
@@ -182,7 +192,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_ir(Work w, LaunchArgs a) {
                 float x[kIb];
                 if (i < P) {
                     float av[kIb];
-                    float *rowp = Lm + (size_t)i * G.ld + k0;
+                    float *rowp = Lm + ir_row(i, G.ld) + k0;
 #pragma unroll
                     for (int mm = 0; mm < kIb; ++mm) av[mm] = (mm < nb) ? rowp[mm] : 0.0f;
 #pragma unroll
@@ -231,13 +241,13 @@ __global__ void __launch_bounds__(512, 1) k_solve_ir(Work w, LaunchArgs a) {
                         acc[6] = fmaf(xr, v.z, acc[6]);
                         acc[7] = fmaf(xr, v.w, acc[7]);
                     }
-                    float *arow = Lm + (size_t)(k1 + r) * G.ld + k1 + jh;
+                    float *arow = Lm + ir_row(k1 + r, G.ld) + k1 + jh;
 #pragma unroll
                     for (int q = 0; q < 8; ++q)
                         if (jh + q <= r) arow[q] -= acc[q];
                 }
                 __syncwarp();
-                const bool ok = chol_diag16(Lm, G.ld, k1, min(kIb, P - k1), Di + (size_t)(kb + 1) * kIb * kIb, lane);
+                const bool ok = chol_diag16(Lm + ir_row(k1 + lane, G.ld) + k1, min(kIb, P - k1), Di + (size_t)(kb + 1) * kIb * kIb, lane);
                 if (!ok && lane == 0) s_fail = 1;
             } else if (kb >= 0) {
                 for (int t = skip + tid - 32; t < ntile; t += nt - 32) {
@@ -266,7 +276,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_ir(Work w, LaunchArgs a) {
 #pragma unroll
                         for (int v = 0; v < 4; ++v) {
                             const int i = i0 + u, j = j0 + v;
-                            if (i < P && j <= i) Lm[(size_t)i * G.ld + j] -= acc[u][v];
+                            if (i < P && j <= i) Lm[ir_row(i, G.ld) + j] -= acc[u][v];
                         }
                 }
             }
@@ -305,7 +315,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_ir(Work w, LaunchArgs a) {
                 __syncthreads();
                 if (tid < nb) yv[k0 + tid] = s_blk[tid];
                 for (int i = k1 + tid; i < P; i += nt) {  // rows below K exist only when K is full
-                    const float *row = Lm + (size_t)i * G.ld + k0;
+                    const float *row = Lm + ir_row(i, G.ld) + k0;
                     float s0 = yv[i], s1 = 0.0f;
 #pragma unroll
                     for (int m = 0; m < kIb; m += 2) {
@@ -322,7 +332,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_ir(Work w, LaunchArgs a) {
                 const int k0 = kb * kIb, nb = min(kIb, P - k0), k1 = k0 + nb;
                 if (wid < nb) {
                     float sacc = 0.0f;
-                    for (int i = k1 + lane; i < P; i += 32) sacc = fmaf(Lm[(size_t)i * G.ld + k0 + wid], yv[i], sacc);
+                    for (int i = k1 + lane; i < P; i += 32) sacc = fmaf(Lm[ir_row(i, G.ld) + k0 + wid], yv[i], sacc);
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, o);
                     if (lane == 0) s_blk[wid] = yv[k0 + wid] - sacc;
@@ -471,7 +481,7 @@ cudaError_t launch_solve_ir(const Work &w, int count, int max_P, int C, const La
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_solve_ir, w, a);
+    return cudaLaunchKernelEx(&cfg, k_solve_ir, w, a, max_P, (int)solve_ir_packed(max_P, C));
 }
 
 }  // namespace qng
