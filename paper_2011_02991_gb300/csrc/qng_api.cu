@@ -360,8 +360,8 @@ constexpr int64_t kStreamFramesMax = 96ll << 30;  // bytes of checkpoints and co
 // (one vector per run) take more memory than they are worth.
 bool plan_sframes(qng_ctx *c) {
     const HostInst &h = c->inst[0];
-    const int pi = c->precision == QNG_C128 ? 1 : 0, tb = frames::kStreamTileBits[pi], kb = frames::kStreamRegBits[pi];
-    if (h.n < tb) return false;
+    const int pi = c->precision == QNG_C128 ? 1 : 0, tb = frames::stream_tile_bits(c->precision, h.n), kb = frames::stream_reg_bits(tb);
+    if (h.n < (pi ? 12 : 13)) return false;
     // contiguous low bits: at most a thread's block (its bits in any other block are then consecutive index
     // bits), fewer where two windows still cover the index bits (rows of 32 bytes at least), else rows of
     // 128 bytes. Byte offsets into a vector are 32 bits wide.
@@ -622,6 +622,7 @@ bool default_shapes(const qng_ctx *c) {
 qng_status plan(qng_ctx *c) {
     c->t_inst.clear(); c->t_param.clear(); c->t_gen.clear(); c->t_fixed.clear(); c->t_diag.clear(); c->t_term.clear();
     c->t_work.clear(); c->t_group_inst.clear(); c->groups.clear();
+    c->frames = c->sframes = false;  // decided below, for this plan's path
     c->param_off.assign(c->count + 1, 0);
     c->metric_off.assign(c->count + 1, 0);
     const size_t ab = amp_bytes(c->precision);
@@ -893,6 +894,72 @@ qng_status cuda_status(cudaError_t e) {
     return QNG_ERR_CUDA;
 }
 
+// Streams and events of the pipelined sweep (single instance) and of launch groups or classes side by side
+// (batches), made here so that no stream is created inside a graph capture.
+qng_status make_streams(qng_ctx *c) {
+    if (c->pipe_ready) return QNG_OK;
+    cudaError_t e;
+    int lo = 0, hi = 0;
+    if ((e = cudaDeviceGetStreamPriorityRange(&lo, &hi)) != cudaSuccess) return cuda_status(e);
+    if ((e = cudaStreamCreateWithPriority(&c->pipe_fwd, cudaStreamNonBlocking, hi)) != cudaSuccess) return cuda_status(e);
+    if ((e = cudaEventCreateWithFlags(&c->pipe_ev0, cudaEventDisableTiming)) != cudaSuccess) return cuda_status(e);
+    for (int k = 0; k < kPipeMax; ++k) {
+        if ((e = cudaStreamCreateWithPriority(&c->pipe_col[k], cudaStreamNonBlocking, lo)) != cudaSuccess ||
+            (e = cudaEventCreateWithFlags(&c->pipe_evf[k], cudaEventDisableTiming)) != cudaSuccess ||
+            (e = cudaEventCreateWithFlags(&c->pipe_evc[k], cudaEventDisableTiming)) != cudaSuccess)
+            return cuda_status(e);
+    }
+    c->pipe_ready = true;
+    return QNG_OK;
+}
+
+qng_status prepare_solves(qng_ctx *c) {
+    cudaError_t e;
+    const int scl = solve_cluster_log2(c->max_P);
+    if (scl >= 0 && (e = prepare_solve(solve_smem_bytes(c->max_P, scl))) != cudaSuccess) return cuda_status(e);
+    if (c->bsolve && (e = prepare_sblock(c->inst[0].P, c->bs_C)) != cudaSuccess) return cuda_status(e);
+    if (c->ir_C > 0 && (e = prepare_solve_ir(c->ir_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
+    return QNG_OK;
+}
+
+// The diagonal-frame path reads its own tables and the instance descriptors: they are gathered into one
+// host image and go up in one copy (from pageable memory, so it is staged before the call returns).
+qng_status upload_frames(qng_ctx *c) {
+    const auto &f = c->f;
+    cudaError_t e;
+    if ((e = cudaMemcpyAsync(c->ws + c->o_inst, c->t_inst.data(), sizeof(DevInst) * c->t_inst.size(), cudaMemcpyHostToDevice,
+                             c->stream)) != cudaSuccess)
+        return cuda_status(e);
+    const size_t first = c->of_inst, end = align256(c->of_etaexp + sizeof(int32_t) * c->count);
+    std::vector<unsigned char> image(end - first, 0);  // zeros: flags, energy sums and their counts
+    auto put = [&](size_t o, const auto &v) { if (!v.empty()) std::memcpy(image.data() + (o - first), v.data(), sizeof(v[0]) * v.size()); };
+    put(c->of_inst, f.inst);
+    put(c->of_run, f.run);
+    put(c->of_member, f.member);
+    put(c->of_ip, f.ip);
+    put(c->of_uop, f.uop);
+    put(c->of_perm, f.perm);
+    put(c->of_term, f.term);
+    put(c->of_item, f.item);
+    put(c->of_cols, f.cols);
+    put(c->of_order, f.order);
+    put(c->of_tab, f.tab);
+    put(c->of_hitem, f.hitem);
+    if ((e = cudaMemcpyAsync(c->ws + first, image.data(), image.size(), cudaMemcpyHostToDevice, c->stream)) != cudaSuccess)
+        return cuda_status(e);
+    size_t ff = 0, fc = 0, fci = 0;
+    for (const frames::Class &k : f.cls) {
+        ff = std::max(ff, k.smem_fwd);
+        fc = std::max(fc, k.smem_col);
+        fci = std::max(fci, k.smem_col_im);
+    }
+    if ((e = frames::prepare(c->precision, c->fkb, ff, fc, fci)) != cudaSuccess) return cuda_status(e);
+    qng_status st = prepare_solves(c);
+    if (st == QNG_OK && f.cls.size() > 1) st = make_streams(c);
+    if (st == QNG_OK) c->prepared = true;
+    return st;
+}
+
 qng_status upload(qng_ctx *c) {
     auto put = [&](size_t o, const void *src, size_t bytes) -> cudaError_t {
         if (bytes == 0) return cudaSuccess;
@@ -900,6 +967,7 @@ qng_status upload(qng_ctx *c) {
     };
     cudaError_t e;
     if ((e = cudaMemsetAsync(c->ws + c->o_status, 0, 256, c->stream)) != cudaSuccess) return cuda_status(e);
+    if (c->frames && !c->streaming) return upload_frames(c);
     if ((e = put(c->o_inst, c->t_inst.data(), sizeof(DevInst) * c->t_inst.size())) != cudaSuccess) return cuda_status(e);
     if ((e = put(c->o_param, c->t_param.data(), sizeof(DevParam) * c->t_param.size())) != cudaSuccess) return cuda_status(e);
     if ((e = put(c->o_gen, c->t_gen.data(), sizeof(DevGen) * c->t_gen.size())) != cudaSuccess) return cuda_status(e);
@@ -920,14 +988,11 @@ qng_status upload(qng_ctx *c) {
             (e = putv(c->os_col, c->scol)) != cudaSuccess || (e = putv(c->os_term, p.terms)) != cudaSuccess ||
             (e = cudaMemsetAsync(c->ws + c->os_eacc, 0, 3 * sizeof(unsigned long long), c->stream)) != cudaSuccess ||
             (e = cudaMemsetAsync(c->ws + c->os_etaexp, 0, sizeof(int32_t), c->stream)) != cudaSuccess ||
-            (e = frames::prepare_stream(c->precision)) != cudaSuccess)
+            (e = frames::prepare_stream(c->precision, p.tb)) != cudaSuccess)
             return cuda_status(e);
-        const int scl = solve_cluster_log2(c->max_P);
-        if (scl >= 0 && (e = prepare_solve(solve_smem_bytes(c->max_P, scl))) != cudaSuccess) return cuda_status(e);
-        if (c->bsolve && (e = prepare_sblock(c->inst[0].P, c->bs_C)) != cudaSuccess) return cuda_status(e);
-        if (c->ir_C > 0 && (e = prepare_solve_ir(c->ir_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
-        c->prepared = true;
-        return QNG_OK;
+        const qng_status st = prepare_solves(c);
+        if (st == QNG_OK) c->prepared = true;
+        return st;
     }
     if (c->streaming) {
         const large::Schedule &S = c->sched;
@@ -955,32 +1020,9 @@ qng_status upload(qng_ctx *c) {
             pass_smem = std::max(pass_smem, (size_t)__builtin_popcount(pd.regmask) * (amp_bytes(c->precision) << pd.t));
         if ((e = large::prepare_pass(c->precision, std::max<size_t>(pass_smem, 1))) != cudaSuccess) return cuda_status(e);
         if (S.phased && (e = large::prepare_pass_phased()) != cudaSuccess) return cuda_status(e);
-        const int scl = solve_cluster_log2(c->max_P);
-        if (scl >= 0 && (e = prepare_solve(solve_smem_bytes(c->max_P, scl))) != cudaSuccess) return cuda_status(e);
-        if (c->bsolve && (e = prepare_sblock(c->inst[0].P, c->bs_C)) != cudaSuccess) return cuda_status(e);
-        if (c->ir_C > 0 && (e = prepare_solve_ir(c->ir_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
-        c->prepared = true;
-        return QNG_OK;
-    }
-    if (c->frames) {
-        const auto &f = c->f;
-        auto putv = [&](size_t o, const auto &v) { return put(o, v.data(), sizeof(v[0]) * v.size()); };
-        if ((e = putv(c->of_inst, f.inst)) != cudaSuccess || (e = putv(c->of_run, f.run)) != cudaSuccess ||
-            (e = putv(c->of_member, f.member)) != cudaSuccess || (e = putv(c->of_ip, f.ip)) != cudaSuccess ||
-            (e = putv(c->of_uop, f.uop)) != cudaSuccess || (e = putv(c->of_perm, f.perm)) != cudaSuccess ||
-            (e = putv(c->of_term, f.term)) != cudaSuccess || (e = putv(c->of_item, f.item)) != cudaSuccess ||
-            (e = putv(c->of_cols, f.cols)) != cudaSuccess || (e = putv(c->of_order, f.order)) != cudaSuccess ||
-            (e = putv(c->of_tab, f.tab)) != cudaSuccess || (e = putv(c->of_hitem, f.hitem)) != cudaSuccess ||
-            (e = cudaMemsetAsync(c->ws + c->of_eacc, 0, 3 * sizeof(unsigned long long) * c->count, c->stream)) != cudaSuccess ||
-            (e = cudaMemsetAsync(c->ws + c->of_bad, 0, sizeof(int32_t) * c->count, c->stream)) != cudaSuccess)
-            return cuda_status(e);
-        size_t ff = 0, fc = 0, fci = 0;
-        for (const frames::Class &k : f.cls) {
-            ff = std::max(ff, k.smem_fwd);
-            fc = std::max(fc, k.smem_col);
-            fci = std::max(fci, k.smem_col_im);
-        }
-        if ((e = frames::prepare(c->precision, c->fkb, ff, fc, fci)) != cudaSuccess) return cuda_status(e);
+        const qng_status st = prepare_solves(c);
+        if (st == QNG_OK) c->prepared = true;
+        return st;
     }
     size_t sf = 0, sc = 0, sci = 0;
     for (const Group &g : c->groups) {
@@ -989,25 +1031,9 @@ qng_status upload(qng_ctx *c) {
         sci = std::max(sci, std::min(g.smem_col_im, kMaxSmem));
     }
     if ((e = prepare_kernels(c->precision, sf, sc, sci)) != cudaSuccess) return cuda_status(e);
-    const int scl = solve_cluster_log2(c->max_P);
-    if (scl >= 0 && (e = prepare_solve(solve_smem_bytes(c->max_P, scl))) != cudaSuccess) return cuda_status(e);
-    if (c->bsolve && (e = prepare_sblock(c->inst[0].P, c->bs_C)) != cudaSuccess) return cuda_status(e);
-    if (c->ir_C > 0 && (e = prepare_solve_ir(c->ir_P, c->ir_C)) != cudaSuccess) return cuda_status(e);
-    // streams and events of the pipelined sweep (single instance) and of the launch groups side by
-    // side (batches), made here so that no stream is created inside a graph capture
-    if (!c->pipe_ready) {
-        int lo = 0, hi = 0;
-        if ((e = cudaDeviceGetStreamPriorityRange(&lo, &hi)) != cudaSuccess) return cuda_status(e);
-        if ((e = cudaStreamCreateWithPriority(&c->pipe_fwd, cudaStreamNonBlocking, hi)) != cudaSuccess) return cuda_status(e);
-        if ((e = cudaEventCreateWithFlags(&c->pipe_ev0, cudaEventDisableTiming)) != cudaSuccess) return cuda_status(e);
-        for (int k = 0; k < kPipeMax; ++k) {
-            if ((e = cudaStreamCreateWithPriority(&c->pipe_col[k], cudaStreamNonBlocking, lo)) != cudaSuccess ||
-                (e = cudaEventCreateWithFlags(&c->pipe_evf[k], cudaEventDisableTiming)) != cudaSuccess ||
-                (e = cudaEventCreateWithFlags(&c->pipe_evc[k], cudaEventDisableTiming)) != cudaSuccess)
-                return cuda_status(e);
-        }
-        c->pipe_ready = true;
-    }
+    qng_status ready = prepare_solves(c);
+    if (ready == QNG_OK) ready = make_streams(c);
+    if (ready != QNG_OK) return ready;
     // launch groups, most work first (they run side by side on their own streams)
     c->group_order.resize(c->groups.size());
     for (size_t k = 0; k < c->groups.size(); ++k) c->group_order[k] = (int)k;
@@ -1052,7 +1078,7 @@ template <class F> cudaError_t timed(qng_ctx *c, int cls, F &&launch) { return t
 
 // Chunks of the pipelined sweep for this call (0: one sweep, then one column launch).
 int pipe_chunks(const qng_ctx *c) {
-    if (!c->pipe_ready || c->streaming || c->count != 1 || c->groups.size() != 1 || !c->col_want.empty()) return 0;
+    if (!c->ws || c->streaming || c->count != 1 || c->groups.size() != 1 || !c->col_want.empty()) return 0;
     const int P = c->inst[0].P;
     // automatic: only for circuits with generalised rotations (measured faster there; with plain
     // rotations the column phase ends on the latency of its longest items, which cannot start

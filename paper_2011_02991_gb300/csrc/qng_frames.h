@@ -222,8 +222,13 @@ struct StreamProgram {
     std::vector<DevTerm> terms;
 };
 
-constexpr int kStreamTileBits[2] = {13, 12};  // complex64, complex128: 64 KiB
-constexpr int kStreamRegBits[2] = {5, 4};
+// Tile bits for n qubits, and index bits per thread for that tile: 64 KiB for large vectors, smaller tiles where
+// those would leave SMs idle (20 qubits complex64, energy and backward: 548 -> 470 us).
+inline int stream_tile_bits(int precision, int n) {
+    if (precision == QNG_C128) return n <= 19 ? 11 : 12;
+    return n <= 19 ? 11 : (n == 20 ? 12 : 13);
+}
+inline int stream_reg_bits(int tb) { return tb == 13 ? 5 : 4; }
 void build_stream(const std::vector<qng_gate> &gates, const std::vector<qng_pauli> &terms, int n, int kb, int tb, int low,
                   StreamProgram &out);
 
@@ -250,7 +255,7 @@ struct SWork {
     int32_t n, P, R, kb, tb, low, hl, nterms, eexp, hblocks;
 };
 
-cudaError_t prepare_stream(int precision);
+cudaError_t prepare_stream(int precision, int tb);
 cudaError_t launch_stream_tables(const SWork &w, int precision, cudaStream_t st);
 cudaError_t launch_stream_forward(const SWork &w, const SPass &p, int first, int slot, int precision, cudaStream_t st);
 // Pass p of the walk over ncol columns col[col0 ..], column k in slot k.

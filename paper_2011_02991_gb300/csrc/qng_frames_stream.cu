@@ -26,14 +26,16 @@ namespace frames {
 // the vector by 2^4), and as every rounding is unbiased (see hash) a unit of 2^-58 on each component moves an
 // inner product with a unit vector by no more.
 constexpr int kUnit = 58;
-constexpr int kSThreads = 256;
 constexpr int kHalfThreads = 128;
 constexpr int kRows = 32;  // parameters of a run kept in shared memory
 
-// tile bits and amplitudes per thread: 64 KiB of tile, two CTAs per SM
-template <class T> struct STile;
-template <> struct STile<Fix> { static constexpr int kb = 4; };
-template <> struct STile<Flt> { static constexpr int kb = 5; };
+// CTAs of NT threads with 2^KB amplitudes each per SM, that the registers are held to. complex64 vectors of 21
+// qubits and more: 32 amplitudes a thread and 16 warps (24 qubits: 67 ms against 78 ms with 16 amplitudes
+// and 32 warps, which exchange more often); smaller ones 16 amplitudes and 32 warps. complex128: 16 amplitudes,
+// 16 warps.
+template <class T> constexpr int ctas_per_sm(int kb, int nt) {
+    return (sizeof(typename T::A) == 16 || kb == 5 ? 512 : 1024) / nt;
+}
 
 // ------------------------------------------------------------------------------------------
 // One entry of a half table per thread. Members on one half's bits multiply its factor; a CZ across the
@@ -163,22 +165,22 @@ __device__ __forceinline__ longlong2 seed_dithered(double2 e, double up, uint32_
 __device__ __forceinline__ float2 seed_dithered(float2 e, double, uint32_t) { return float2{e.y, -e.x}; }
 
 // MIM: both parts of the metric's inner products. FWD: the forward sweep (one vector, checkpoints out).
-template <class T, int MIM, int FWD>
-__global__ void __launch_bounds__(kSThreads, 2) k_stream(SWork w, SPass ps, int pass, int col0, int ncol, int flag) {
-    constexpr int KB = STile<T>::kb, NA = 1 << KB;
+template <class T, int MIM, int FWD, int KB, int NT>
+__global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, SPass ps, int pass, int col0, int ncol, int flag) {
+    constexpr int NA = 1 << KB;
     using A = typename T::A;
     using S = typename T::S;
     using Acc = typename T::Acc;
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ Acc red[16][kSThreads / 32][MIM ? 2 : 1];
+    __shared__ Acc red[16][NT / 32][MIM ? 2 : 1];
     // the pass's steps and the parameters of its (first) run: read once, or each would wait on L2
     constexpr int kOpsMax = 48;
     __shared__ UOp ops_sh[kOpsMax];
     __shared__ SIp ips_sh[kRows];
-    for (int x = threadIdx.x; x < min(ps.nops, kOpsMax); x += kSThreads) ops_sh[x] = w.uop[ps.op_begin + x];
+    for (int x = threadIdx.x; x < min(ps.nops, kOpsMax); x += NT) ops_sh[x] = w.uop[ps.op_begin + x];
     if (!FWD && ps.run0 >= 0) {
         const Run &rn = w.run[ps.run0];
-        for (int x = threadIdx.x; x < min(rn.ip_count, kRows); x += kSThreads) ips_sh[x] = w.ip[rn.ip_begin + x];
+        for (int x = threadIdx.x; x < min(rn.ip_count, kRows); x += NT) ips_sh[x] = w.ip[rn.ip_begin + x];
     }
     const int slot = FWD ? col0 : (int)(blockIdx.x % (unsigned)ncol);
     const uint32_t tile = FWD ? blockIdx.x : blockIdx.x / (unsigned)ncol;
@@ -202,7 +204,7 @@ __global__ void __launch_bounds__(kSThreads, 2) k_stream(SWork w, SPass ps, int 
         gsh = low - w.low + ps.s;
     };
     auto gidx = [&](int k) { return g0 + ((uint32_t)k << gsh); };
-    const uint32_t h0 = sizeof(A) == 16 ? hash(tile * kSThreads + t) : 0u;
+    const uint32_t h0 = sizeof(A) == 16 ? hash(tile * NT + t) : 0u;
     auto dith = [&](int k) { return sizeof(A) == 16 ? (h0 ^ salt(k)) | 64u : 0u; };
     bool start = false;
     if (FWD) {
@@ -265,8 +267,8 @@ __global__ void __launch_bounds__(kSThreads, 2) k_stream(SWork w, SPass ps, int 
                 uint32_t b0 = tbase<KB>(t, low);
                 if (u.perm >= 0) {
                     const SPerm &pm = w.perm[u.perm];
-                    uint32_t x = 0;
-                    for (int q = 0; q < w.n; ++q) x ^= ((gtile >> q) & 1u) ? pm.oimg[q] : 0u;
+                    const int q0 = (int)(t & 31u);
+                    uint32_t x = __reduce_xor_sync(0xffffffffu, ((gtile >> q0) & 1u) ? pm.oimg[q0] : 0u);
                     for (int q = 0; q < w.tb; ++q) x ^= ((b0 >> q) & 1u) ? pm.limg[q] : 0u;
                     b0 = x;
 #pragma unroll
@@ -314,7 +316,7 @@ __global__ void __launch_bounds__(kSThreads, 2) k_stream(SWork w, SPass ps, int 
                 // in one half of the index (else, in narrow windows: `both`): the other half's factor is the same
                 // for all of its amplitudes, and the sign, bilinear in the halves, is linear in k: par0 ^ bit k
                 // of sgnw.
-                constexpr int U = sizeof(A) == 16 ? 4 : 8, LU = sizeof(A) == 16 ? 2 : 3;
+                constexpr int U = KB == 5 ? 8 : 4, LU = KB == 5 ? 3 : 2;
                 constexpr uint32_t kWalsh[5] = {0xaaaaaaaau, 0xccccccccu, 0xf0f0f0f0u, 0xff00ff00u, 0xffff0000u};
                 const bool hi_var = gsh + KB > w.hl, both = hi_var && gsh < w.hl;
                 const uint32_t l0 = g0 & (nlo - 1u), hh = g0 >> w.hl;
@@ -421,12 +423,12 @@ __global__ void __launch_bounds__(kSThreads, 2) k_stream(SWork w, SPass ps, int 
                     }
                 }
                 __syncthreads();
-                for (int x = t; x < nrow * (MIM ? 2 : 1); x += kSThreads) {
+                for (int x = t; x < nrow * (MIM ? 2 : 1); x += NT) {
                     const int q = MIM ? x >> 1 : x, part = MIM ? x & 1 : 0, row = ipf + q;
                     SIp ip = {0, 0, 1, 0};
                     if (q < ipc) ip = r == ps.run0 && q < kRows ? ips_sh[q] : w.ip[rn.ip_begin + q];
                     typename std::conditional<sizeof(A) == 16, ll, double>::type d = 0;
-                    for (int k = 0; k < kSThreads / 32; ++k) {
+                    for (int k = 0; k < NT / 32; ++k) {
                         const uint32_t g = gtile | spread(tbase<KB>(k * 32, low));
                         const auto y = (typename std::conditional<sizeof(A) == 16, ll, double>::type)red[ip.src][k][part];
                         d += ((g & ip.z) != 0) != (ip.sgn < 0) ? -y : y;
@@ -601,17 +603,23 @@ __global__ void k_sfinish(SWork w, int what) {
 // ------------------------------------------------------------------------------------------
 static size_t tile_bytes(int precision, int tb) { return (size_t)(precision == QNG_C128 ? 16 : 8) << tb; }
 
-cudaError_t prepare_stream(int precision) {
-    const size_t sm = 64 * 1024;
-    cudaError_t e;
-#define QNG_P(T)                                                                                         \
-    if ((e = raise_smem_limit(reinterpret_cast<const void *>(k_stream<T, 0, 0>), sm)) != cudaSuccess ||  \
-        (e = raise_smem_limit(reinterpret_cast<const void *>(k_stream<T, 1, 0>), sm)) != cudaSuccess)    \
-        return e;                                                                                        \
-    return raise_smem_limit(reinterpret_cast<const void *>(k_stream<T, 0, 1>), sm);
-    if (precision == QNG_C128) { QNG_P(Fix) }
-    QNG_P(Flt)
-#undef QNG_P
+template <class T, int KB, int NT> static cudaError_t prepare_nt(size_t sm) {
+    cudaError_t e = raise_smem_limit(reinterpret_cast<const void *>(k_stream<T, 0, 0, KB, NT>), sm);
+    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void *>(k_stream<T, 1, 0, KB, NT>), sm);
+    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void *>(k_stream<T, 0, 1, KB, NT>), sm);
+    return e;
+}
+
+// the kernel of a precision and tile of 2^tb amplitudes
+#define QNG_STREAM(F, tb)                                                                                     \
+    (precision == QNG_C128 ? (tb == 11 ? F(Fix, 4, 128) : F(Fix, 4, 256))                                     \
+                           : (tb == 11 ? F(Flt, 4, 128) : tb == 12 ? F(Flt, 4, 256) : F(Flt, 5, 256)))
+
+cudaError_t prepare_stream(int precision, int tb) {
+    const size_t sm = tile_bytes(precision, tb);
+#define QNG_F(T, KB, NT) prepare_nt<T, KB, NT>(sm)
+    return QNG_STREAM(QNG_F, tb);
+#undef QNG_F
 }
 
 cudaError_t launch_stream_tables(const SWork &w, int precision, cudaStream_t st) {
@@ -625,20 +633,21 @@ cudaError_t launch_stream_tables(const SWork &w, int precision, cudaStream_t st)
 cudaError_t launch_stream_forward(const SWork &w, const SPass &p, int first, int slot, int precision, cudaStream_t st) {
     const unsigned tiles = 1u << (w.n - w.tb);
     const size_t sm = tile_bytes(precision, w.tb);
-    if (precision == QNG_C128) k_stream<Fix, 0, 1><<<tiles, kSThreads, sm, st>>>(w, p, 0, slot, 1, first);
-    else k_stream<Flt, 0, 1><<<tiles, kSThreads, sm, st>>>(w, p, 0, slot, 1, first);
-    return cudaGetLastError();
+#define QNG_F(T, KB, NT) (k_stream<T, 0, 1, KB, NT><<<tiles, NT, sm, st>>>(w, p, 0, slot, 1, first), cudaGetLastError())
+    return QNG_STREAM(QNG_F, w.tb);
+#undef QNG_F
 }
 
 cudaError_t launch_stream_walk(const SWork &w, const SPass &p, int pass, int col0, int ncol, int store, int precision,
                                int metric_im, cudaStream_t st) {
     const unsigned grid = (1u << (w.n - w.tb)) * (unsigned)ncol;
     const size_t sm = tile_bytes(precision, w.tb);
-#define QNG_W(T, M) k_stream<T, M, 0><<<grid, kSThreads, sm, st>>>(w, p, pass, col0, ncol, store)
-    if (precision == QNG_C128) { if (metric_im) QNG_W(Fix, 1); else QNG_W(Fix, 0); }
-    else { if (metric_im) QNG_W(Flt, 1); else QNG_W(Flt, 0); }
-#undef QNG_W
-    return cudaGetLastError();
+#define QNG_F(T, KB, NT)                                                                                      \
+    ((metric_im ? k_stream<T, 1, 0, KB, NT><<<grid, NT, sm, st>>>(w, p, pass, col0, ncol, store)                  \
+                : k_stream<T, 0, 0, KB, NT><<<grid, NT, sm, st>>>(w, p, pass, col0, ncol, store)),                \
+     cudaGetLastError())
+    return QNG_STREAM(QNG_F, w.tb);
+#undef QNG_F
 }
 
 cudaError_t launch_stream_hpsi(const SWork &w, int in, int out, int precision, cudaStream_t st) {
