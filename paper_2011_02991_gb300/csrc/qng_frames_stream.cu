@@ -462,11 +462,14 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
 // combine to one factor per amplitude first (for TFIM the n - 1 ZZ terms are one real factor of psi[m]).
 // complex64 sums in float32, the precision it is stored in. complex128 in fixed point: coefficients as
 // multiples of 2^(eexp - 62), sums as multiples of 2^(eexp - 61); the float64 pipe would take four times as
-// long (22 qubits, 43 terms: 3.4 ms). <E> and |eta|^2 in float64 over a thread's amplitudes and then fixed
-// point (as the on-chip kernel).
+// long (22 qubits, 43 terms: 3.4 ms). <E> and |eta|^2 in float64 and then fixed point (as the on-chip
+// kernel), complex64 in float32 over a thread's four amplitudes first. The next mask's
+// loads go out before a mask's products (20 qubits, 41 masks, complex64: 56 to 45 us, 344 MB of gathers from L2;
+// and float64 conversions and warp sums taken to once per thread and CTA).
 template <class T> struct Coef;
 template <> struct Coef<Fix> {
     using C = ll;
+    using S = double;  // a thread's share of <E> and |eta|^2
     static __device__ __forceinline__ C of(double c, int eexp) { return __double2ll_rn(scalbn(c, 62 - eexp)); }
     static __device__ __forceinline__ ll mul(ll c, ll x) {
         const int ch = hi_of(c), cl = lo_of(c), xh = hi_of(x), xl = lo_of(x);
@@ -479,15 +482,16 @@ template <> struct Coef<Fix> {
 };
 template <> struct Coef<Flt> {
     using C = float;
+    using S = float;
     static __device__ __forceinline__ C of(double c, int) { return (float)c; }
     static __device__ __forceinline__ float mul(float c, float x) { return c * x; }
-    static __device__ __forceinline__ double value(float h, int) { return (double)h; }
+    static __device__ __forceinline__ float value(float h, int) { return h; }
 };
 
 __device__ __forceinline__ double2 amp_at(longlong2 x) {
     return double2{scalbn((double)x.x, -kUnit), scalbn((double)x.y, -kUnit)};
 }
-__device__ __forceinline__ double2 amp_at(float2 x) { return amp_of(x); }
+__device__ __forceinline__ float2 amp_at(float2 x) { return x; }
 
 template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int in, int out) {
     using A = typename T::A;
@@ -498,10 +502,13 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
     __shared__ C coef[kTerms];
     __shared__ uint32_t tx[kTerms], tz[kTerms];
     __shared__ int tny[kTerms];
-    __shared__ double red[8][2];
+    using S = typename K::S;
+    __shared__ double red[256][2];
     const A *v = reinterpret_cast<const A *>(w.b) + ((size_t)in << w.n);
     E *eta = reinterpret_cast<E *>(reinterpret_cast<A *>(w.b) + ((size_t)out << w.n));
     const uint64_t N = 1ull << w.n;
+    const int sc = sizeof(S) == 4 ? max(-120, min(120, -w.eexp)) : 0;  // float32 squares stay in range
+    const S fs = (S)scalbnf(1.0f, sc);
     double e = 0.0, n2 = 0.0;
     for (uint64_t m0 = (uint64_t)blockIdx.x * (256 * NA); m0 < N; m0 += (uint64_t)gridDim.x * (256 * NA)) {
         const uint32_t m = (uint32_t)m0 + threadIdx.x;  // and m + 256, ..
@@ -509,14 +516,17 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
         C cr[NA], ci[NA];
 #pragma unroll
         for (int k = 0; k < NA; ++k) { h[k] = A{0, 0}; cr[k] = ci[k] = 0; }
-        uint32_t x = 0;
         int kinds = 0;  // parts of the factor that the mask's terms have: 1 real, 2 imaginary
-        auto add = [&]() {
+        A y[NA];        // psi at the mask's sources
+        auto load = [&](uint32_t x) {
+#pragma unroll
+            for (int k = 0; k < NA; ++k) y[k] = v[(m + 256 * k) ^ x];
+        };
+        auto add = [&](const A *y) {
 #pragma unroll
             for (int k = 0; k < NA; ++k) {
-                const A y = v[(m + 256 * k) ^ x];
-                if (kinds & 1) { h[k].x += K::mul(cr[k], y.x); h[k].y += K::mul(cr[k], y.y); }
-                if (kinds & 2) { h[k].x -= K::mul(ci[k], y.y); h[k].y += K::mul(ci[k], y.x); }
+                if (kinds & 1) { h[k].x += K::mul(cr[k], y[k].x); h[k].y += K::mul(cr[k], y[k].y); }
+                if (kinds & 2) { h[k].x -= K::mul(ci[k], y[k].y); h[k].y += K::mul(ci[k], y[k].x); }
                 cr[k] = ci[k] = 0;
             }
             kinds = 0;
@@ -534,9 +544,9 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
                 }
                 __syncthreads();
             }
+            load(tx[0]);
             for (int t = 0; t < nt; ++t) {
-                if (kinds && tx[t] != x) add();
-                x = tx[t];
+                const uint32_t x = tx[t];
                 const C c = coef[t];
                 const uint32_t z = tz[t];
                 if (tny[t]) {
@@ -548,37 +558,51 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
 #pragma unroll
                     for (int k = 0; k < NA; ++k) cr[k] += (__popc(((m + 256 * k) ^ x) & z) & 1) ? -c : c;
                 }
+                const bool last = t + 1 == nt;
+                if (last || tx[t + 1] != x) {  // the mask's last term: the next mask's loads go out first
+                    A u[NA];
+#pragma unroll
+                    for (int k = 0; k < NA; ++k) u[k] = y[k];
+                    if (!last) load(tx[t + 1]);
+                    add(u);
+                }
             }
         }
-        if (kinds) add();
+        S e4 = 0, n4 = 0;  // a thread's four amplitudes
 #pragma unroll
         for (int k = 0; k < NA; ++k) {
-            const double2 y = amp_at(v[m + 256 * k]);
+            const auto y = amp_at(v[m + 256 * k]);
             E o;
-            const double hr = K::value(h[k].x, w.eexp), hi = K::value(h[k].y, w.eexp);
+            const S hr = K::value(h[k].x, w.eexp), hi = K::value(h[k].y, w.eexp);
             o.x = hr;
             o.y = hi;
             eta[m + 256 * k] = o;
-            e += y.x * hr + y.y * hi;
-            n2 += hr * hr + hi * hi;
+            e4 += y.x * hr + y.y * hi;
+            const S ar = hr * fs, ai = hi * fs;
+            n4 += ar * ar + ai * ai;
         }
+        e += e4;
+        n2 += n4;
     }
+    red[threadIdx.x][0] = e;
+    red[threadIdx.x][1] = n2;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double s = 0.0, s2 = 0.0;
+    for (int k = 0; k < 8; ++k) { s += red[32 * k + threadIdx.x][0]; s2 += red[32 * k + threadIdx.x][1]; }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        e += __shfl_xor_sync(0xffffffffu, e, o);
-        n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
     }
-    if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = e; red[threadIdx.x >> 5][1] = n2; }
-    __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0.0, s2 = 0.0;
-        for (int k = 0; k < 8; ++k) { s += red[k][0]; s2 += red[k][1]; }
+        s2 = scalbn(s2, -2 * sc);
         atomicAdd(w.eacc, (unsigned long long)__double2ll_rn(scalbn(s, 60 - w.eexp)));
         atomicAdd(w.eacc + 1, (unsigned long long)__double2ll_ru(scalbn(s2, -w.eexp) * scalbn(1.0, 60 - w.eexp)) + 1ull);
         __threadfence();
         if (atomicAdd(w.eacc + 2, 1ull) == (unsigned long long)(gridDim.x - 1)) {
             const double en = scalbn((double)(ll)atomicExch(w.eacc, 0ull), w.eexp - 60);
-            const double nrm = sqrt((double)atomicExch(w.eacc + 1, 0ull)) * 0x1p-30 * (1.0 + 0x1p-40);
+            const double nrm = sqrt((double)atomicExch(w.eacc + 1, 0ull)) * 0x1p-30 * (1.0 + (sizeof(S) == 4 ? 0x1p-20 : 0x1p-40));
             atomicExch(w.eacc + 2, 0ull);
             *w.etaexp = w.eexp + ilogb(nrm) + 1;
             *w.energy = *w.bad ? __longlong_as_double(0x7ff8000000000000ll) : en;
