@@ -82,7 +82,8 @@ enum {
 /* amplitude precisions */
 enum {
     QNG_C64 = 0,  /* complex64 amplitudes; float64 accumulation of inner products, assembly and solve */
-    QNG_C128 = 1  /* complex128 amplitudes, float64 arithmetic throughout                            */
+    QNG_C128 = 1  /* complex128 amplitudes, carried as float64 or as 64-bit fixed point with a resolution
+                     of 2^-58 or finer of the unit-norm state; float64 inner products, assembly and solve */
 };
 
 /* One gate: param is the index of its angle in theta for the rotations (RX..RZ, CRX..CRP), which
@@ -216,15 +217,20 @@ qng_status qng_graph_capture(qng_ctx *ctx, const double *theta, double dt, doubl
 qng_status qng_graph_launch(qng_ctx *ctx);
 
 /* Autotuner of the on-chip path: for every qubit count present in the context, times qng_step
- * (reps repetitions after one warm-up, CUDA events) for every cluster size (1..8 CTAs) and CTA size
- * (64, 128, 256 threads) that fits, and keeps the fastest; then the checkpoint sweep's cluster and
- * CTA size; then, for a single instance, the pipelined sweep's chunk count (1..4), or, for a batch
- * of several launch groups, the groups in turn or side by side (qng_set_pipeline 1 or 2). theta is
- * a device array of the context's parameters. report (may be NULL) receives the number of shapes
+ * (reps repetitions after one warm-up, CUDA events) as the context runs it by default (the
+ * diagonal-frame kernels, which have one shape per size) and then for every cluster size (1..8 CTAs)
+ * and CTA size (64, 128, 256 threads) of the gate-by-gate kernels that fits, and keeps the fastest; if
+ * that is a gate-by-gate shape, then the checkpoint sweep's cluster and CTA size and, for a single
+ * instance, the pipelined sweep's chunk count (1..4), or, for a batch of several launch groups, the
+ * groups in turn or side by side (qng_set_pipeline 1 or 2). theta is a device array of the context's
+ * parameters. report (may be NULL) receives the number of shapes
  * timed. Shapes needing more workspace than the one set are skipped. Drops a captured graph. */
 qng_status qng_autotune(qng_ctx *ctx, const double *theta, int reps, int64_t *report);
 
-/* Launch shape used for instances of n_qubits qubits (after defaults, autotuning and qng_set_shape):
+/* Launch shape of the gate-by-gate kernels for instances of n_qubits qubits (after defaults,
+ * autotuning and qng_set_shape). An explicit shape, here, through qng_set_tuning or through
+ * qng_set_forward_cluster, makes instances of that size run those kernels instead of the
+ * diagonal-frame ones; restoring the defaults restores the diagonal-frame ones.
  * cluster_log2 = log2 of CTAs per state, threads = CTA size of the column kernel (64..256),
  * forward_threads = CTA size of the checkpoint sweep (64..512); any output pointer may be NULL.
  * qng_set_shape is the manual override (cluster_log2 -1, threads 0 and forward_threads 0 restore
@@ -252,15 +258,19 @@ qng_status qng_set_tuning(qng_ctx *ctx, int min_qubits, int cluster_log2, int th
 
 /* Execution path: 0 automatic (on-chip for n <= 16 qubits, streaming above), 1 on-chip (every
  * state of an instance in the shared memory of one thread-block cluster, O(P) checkpoints in HBM),
- * 2 streaming (single instance only: four registers of 2^n amplitudes in HBM, psi, a and b of
- * Algorithm 1 and a second b, since the metric columns walk in pairs that share a; tiled passes). A
- * change re-plans the context; if the workspace already set is then too small the call returns
+ * 2 streaming (single instance only, states in HBM, tiled passes). By default the streaming path
+ * keeps one checkpoint per run of commuting rotations (about P / n of them) plus as many column
+ * slots as fill 32 MiB (at least 4), vectors of 2^n amplitudes, and every pass takes one run for
+ * several columns. Vectors beyond 4 GiB, instances whose checkpoints and slots would pass 96 GiB,
+ * and n < 13 (complex64) or n < 12 (complex128) run on four registers instead: psi, a and b of
+ * Algorithm 1 and a second b, the metric columns walking in pairs that share a. A change re-plans the context; if the workspace already set is then too small the call returns
  * QNG_ERR_WORKSPACE and keeps the old path (query qng_workspace_size before setting a workspace). */
 qng_status qng_set_path(qng_ctx *ctx, int path);
 
-/* Streaming path only: HBM bytes one qng_step moves through the pass schedule (registers loaded
- * and stored by every pass), split into the metric columns and the rest (forward, energy, adjoint),
- * and the number of inner-product steps (elements) of the metric. Zeros on the on-chip path. */
+/* Streaming path only: HBM bytes one qng_step moves through the pass schedule (vectors loaded and
+ * stored and checkpoints read by every pass), split into the metric walk and the rest, and the number
+ * of launches of that walk. With checkpoints the gradient column walks with the metric columns and
+ * counts there. Zeros on the on-chip path. */
 qng_status qng_stream_traffic(const qng_ctx *ctx, int64_t *metric_bytes, int64_t *other_bytes, int64_t *metric_passes);
 
 /* Streaming path only: per kernel class of qng_profile_read (QNG_KERNEL_CLASSES entries each, may be
@@ -273,10 +283,11 @@ qng_status qng_stream_segments(const qng_ctx *ctx, int64_t *bytes, int64_t *laun
 /* Kernel timing with CUDA events recorded on the context's stream around every launch.
  * qng_profile(ctx, 1) starts recording, qng_profile(ctx, 0) stops. qng_profile_read waits for the
  * stream, then returns per kernel class the summed milliseconds and the launch counts since the
- * last read (arrays of QNG_KERNEL_CLASSES entries). Classes: 0 coefficients; 1 the checkpoint sweep
- * (on-chip) or the forward passes (streaming); 2 the recurrence columns (on-chip) or the metric
- * passes (streaming); 3 assembly and solve; streaming only: 4 energy passes (W, W^dag), 5 the Pauli
- * sum H psi, 6 adjoint passes, 7 the inner-product reductions of every segment. */
+ * last read (arrays of QNG_KERNEL_CLASSES entries). Classes: 0 coefficients and factor tables; 1 the
+ * checkpoint sweep (on-chip) or the forward passes (streaming); 2 the column walk, the gradient
+ * column with it; 3 assembly and solve; 5 the Pauli sum H psi; 7 the inner-product reductions of the
+ * streaming path. The gate-by-gate streaming passes also use 4, energy passes (W, W^dag), and 6,
+ * adjoint passes; the gate-by-gate on-chip sweep counts H psi in class 1. */
 #define QNG_KERNEL_CLASSES 8
 qng_status qng_profile(qng_ctx *ctx, int enable);
 qng_status qng_profile_read(qng_ctx *ctx, double *ms, int64_t *launches);
@@ -284,21 +295,23 @@ qng_status qng_profile_read(qng_ctx *ctx, double *ms, int64_t *launches);
 /* Number of kernel launches the last compute call issued (for accounting). */
 qng_status qng_last_launch_count(const qng_ctx *ctx, int64_t *launches);
 
-/* Pipelined sweep (one instance on the on-chip path). Column j of the recurrence (Algorithm 1's
+/* Pipelined sweep (one instance on the on-chip path, gate-by-gate kernels: explicit shapes). Column j of the recurrence (Algorithm 1's
  * inner loop from parameter j down) reads only the checkpoints psi_0..psi_j, so the checkpoint
  * sweep runs in chunks of consecutive parameters on a high-priority stream, and the columns each
  * chunk makes ready run on streams of their own while the sweep goes on, on the SMs the sweep
  * leaves idle. The calling stream forks into these streams and joins them before the solve (graph
  * capture included). Results are bit-identical to the unchunked sweep.
- * Batched contexts can run each launch group's sweep and columns on a stream of its own, most work
- * first, so that the groups fill one another's tails (joined before the solve, graph capture
- * included). For batches qng_set_pipeline(ctx, 0) does this for complex128 and runs complex64 groups
- * one after another; 1 runs them one after another, 2..8 side by side.
+ * The diagonal-frame kernels ignore the chunk count; batches on them run each launch class (one per
+ * cluster size) on a stream of its own, whatever the setting.
+ * Batched contexts on gate-by-gate shapes can run each launch group's sweep and columns on a stream of
+ * its own, most work first, so that the groups fill one another's tails (joined before the solve,
+ * graph capture included). For those qng_set_pipeline(ctx, 0) does this for complex128 and runs
+ * complex64 groups one after another; 1 runs them one after another, 2..8 side by side.
  * qng_set_pipeline: chunks = 0 automatic, 1 off, 2..8 that many. Automatic is 3 chunks for a
  * circuit with generalised rotations and P >= 64, else off: with plain rotations the column phase
  * ends on the latency of its longest columns, which start only when the sweep has ended, so the
  * extra launches do not pay (measured at 12 qubits). qng_autotune picks the count per context.
- * qng_get_pipeline: the chunk count the next call will use (0: none). */
+ * qng_get_pipeline: the chunk count the next call on gate-by-gate shapes will use (0: none). */
 qng_status qng_set_pipeline(qng_ctx *ctx, int chunks);
 qng_status qng_get_pipeline(const qng_ctx *ctx, int *chunks);
 

@@ -734,7 +734,7 @@ qng_status plan(qng_ctx *c) {
     // that it fits, on 4 CTAs each (CTA 0 does the serial part; fewer CTAs per instance leave room for
     // more instances at once), the others go to the cluster solve. Beyond 222 parameters, where only the
     // packed triangle fits, batches alone take it (they wait for the slowest instance: 64 instances of
-    // 6 to 14 qubits 0.86 ms with the float64 solve for their largest, 0.33 ms with this one).
+    // 6 to 14 qubits 0.86 ms with the float64 solve for their largest, 0.29 ms with this one).
     c->ir_C = c->ir_P = 0;
     if (c->max_P >= kBlockSolveMinP && solve_cluster_log2(c->max_P) >= 0) {
         const int C = c->count == 1 && c->max_P >= 128 ? 8 : 4;
@@ -1205,6 +1205,7 @@ qng_status run_sframes(qng_ctx *c, int jobs, const double *theta, int64_t &launc
     cudaError_t e = timed(c, 0, [&] { return frames::launch_stream_tables(w, c->precision, c->stream); });
     if (e != cudaSuccess) return cuda_status(e);
     launches += 1;
+    w.chain = true;
     const int vslot = c->sslots - 1;  // the forward vector; H psi goes to slot 0, the gradient column's
     for (size_t k = 0; k < p.fwd.size(); ++k) {
         e = timed(c, 1, [&] { return frames::launch_stream_forward(w, p.fwd[k], k == 0, vslot, c->precision, c->stream); });
@@ -1223,12 +1224,14 @@ qng_status run_sframes(qng_ctx *c, int jobs, const double *theta, int64_t &launc
         return cuda_status(e);
     int first, end;
     stream_range(c, jobs, first, end);
+    w.chain = false;  // the first one follows a fill, not a kernel
     for (const SLaunch &L : walk_launches(c, first, end)) {
         e = timed(c, metric ? 2 : 6, [&] {
             return frames::launch_stream_walk(w, p.bwd[L.pass], L.pass, L.col0, L.ncol, L.store, c->precision, im, c->stream);
         });
         if (e != cudaSuccess) return cuda_status(e);
         ++launches;
+        w.chain = true;
     }
     e = timed(c, 7, [&] {
         return frames::launch_stream_finish(w, (metric ? 1 : 0) | (grad ? 2 : 0) | (im ? 4 : 0), c->precision, c->stream);
@@ -1330,7 +1333,7 @@ qng_status run_streaming(qng_ctx *c, int jobs, int64_t &launches) {
 // The diagonal-frame launches up to the columns. A batch of several launch classes runs each class's
 // sweep and columns on a stream of its own, joined on the context's stream.
 qng_status run_frames(qng_ctx *c, int jobs, const double *theta, int64_t &launches) {
-    const frames::FWork w = c->fwork(theta);
+    frames::FWork w = c->fwork(theta);
     const auto &f = c->f;
     const bool wm = jobs & (kJobMetric | kJobSolve), wg = jobs & (kJobGradient | kJobSolve);
     const bool wh = jobs & (kJobGradient | kJobEnergy | kJobSolve);
@@ -1339,6 +1342,7 @@ qng_status run_frames(qng_ctx *c, int jobs, const double *theta, int64_t &launch
     if (e != cudaSuccess) return cuda_status(e);
     launches += f.tab.empty() ? 0 : 1;
     const bool side = f.cls.size() > 1 && c->pipe_ready;
+    w.chain = !side;  // classes side by side: a waiting kernel would take another class's room
     if (side && (e = cudaEventRecord(c->pipe_ev0, c->stream)) != cudaSuccess) return cuda_status(e);
     for (size_t k = 0; k < f.cls.size(); ++k) {
         const frames::Class &cl = f.cls[k];
@@ -1481,6 +1485,7 @@ qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
     }
     LaunchArgs a = args;
     a.jobs = jobs;
+    a.chain = (frames && !(c->f.cls.size() > 1 && c->pipe_ready)) || sframes;
     if (need_cols && !S && !side_by_side) {
         for (const Group &g : c->groups) {
             if ((wm && wg ? g.num_work : (wm ? g.num_met : g.num_grad)) == 0) continue;
@@ -1722,7 +1727,7 @@ qng_status qng_optimize(qng_ctx *c, double *theta, double dt, double lambda, int
         const qng_status s = run(c, kJobSolve | kJobGradient | kJobEnergy | kJobMetric, a);
         if (s != QNG_OK) return s;
         launches += c->last_launches + 1;
-        const cudaError_t e = timed(c, 0, [&] { return launch_theta_update(c->work(), theta, dth, c->total_params, c->stream); });
+        const cudaError_t e = timed(c, 0, [&] { return launch_theta_update(c->work(), theta, dth, c->total_params, c->stream, c->count == 1); });
         if (e != cudaSuccess) return cuda_status(e);
     }
     c->last_launches = launches;

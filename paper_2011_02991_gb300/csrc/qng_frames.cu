@@ -122,6 +122,7 @@ template <class T> __global__ void __launch_bounds__(kTabThreads) k_tables(FWork
     __shared__ int4 cs[kTabThreads];    // cos, sin of a member, 2^62 = 1
     __shared__ Member mem[kTabThreads];
     __shared__ int any_bad;
+    grid_ready();
     const TabItem it = w.tab[blockIdx.x];
     const Inst &in = w.inst[it.inst];
     const Run &rn = w.run[in.run_off + it.run];
@@ -213,11 +214,6 @@ template <class T, int KB> __global__ void __launch_bounds__(512) k_fwd(FWork w,
     if (cl) cg::this_cluster().sync();  // every CTA runs before its shared memory is touched
     const bool on = threadIdx.x < tpc;
     const Place<KB> p{on ? rank * tpc + threadIdx.x : 0u, in.nE - cl, cl};
-    if (rank == 0 && threadIdx.x == 0) {
-        int bad = 0;
-        for (int r = 0; r < in.R; ++r) bad |= w.bad_run[in.run_off + r];
-        w.bad[inst] = bad;
-    }
     A b[NA];
 #pragma unroll
     for (int k = 0; k < (1 << KB); ++k) b[k] = A{0, 0};
@@ -230,6 +226,12 @@ template <class T, int KB> __global__ void __launch_bounds__(512) k_fwd(FWork w,
     const int nE = in.nE, nops = in.fwd_cnt;
     UOp *ops = reinterpret_cast<UOp *>(smem + ((size_t)blockDim.x << KB) * sizeof(A));
     for (int x = threadIdx.x; x < nops; x += blockDim.x) ops[x] = w.uop[in.fwd_off + x];
+    grid_ready();
+    if (rank == 0 && threadIdx.x == 0) {
+        int bad = 0;
+        for (int r = 0; r < in.R; ++r) bad |= w.bad_run[in.run_off + r];
+        w.bad[inst] = bad;
+    }
     const S *dall = reinterpret_cast<const S *>(w.d) + in.d_off;
     S *aall = reinterpret_cast<S *>(w.a) + in.a_off;
     __syncthreads();
@@ -274,6 +276,7 @@ template <class T> __global__ void __launch_bounds__(kHThreads) k_heff(FWork w, 
     constexpr int kTerms = 64;
     __shared__ DevTerm terms[kTerms];
     __shared__ double red[kHThreads / 32][2];
+    grid_ready();
     const HItem it = w.hitem[first + blockIdx.x];
     const Inst &in = w.inst[it.inst];
     // 8 consecutive amplitudes and 4 shares of the terms per warp
@@ -404,7 +407,6 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
     const bool grad = it.ncol == 0;
     const bool live = grad ? sl == 0 : sl < it.ncol;
     const int col = grad ? P : (live ? w.cols[it.list + sl] : -1);
-    const bool bad = w.bad[it.inst] != 0;
     const double unit = sizeof(A) == 16 ? 0x1p-60 : 1.0;
 
     // the walk's tables in shared memory: steps, runs and parameters (a table read per run would wait on
@@ -416,6 +418,8 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
     for (int x = threadIdx.x; x < it.nip; x += blockDim.x) ips[x] = w.ip[in.ip_off + x];
     for (int x = threadIdx.x; x < it.nruns; x += blockDim.x) runs[x] = w.run[in.run_off + x];
     for (int x = threadIdx.x; x < nops; x += blockDim.x) ops[x] = w.uop[in.bwd_off + it.entry + x];
+    grid_ready();
+    const bool bad = w.bad[it.inst] != 0;
     __syncthreads();
 
     // a finished sum of the column c's row: a parameter below c, c itself (its control probability), or P
@@ -562,25 +566,6 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
 }
 
 // ------------------------------------------------------------------------------------------
-template <typename K, typename... Args>
-static cudaError_t launch(K kern, int grid, int threads, size_t smem, int cl, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    if (cl > 0) {
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 1u << cl;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-    }
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 #define QNG_FRAMES(F)                                                                       \
     (precision == QNG_C128 ? (kb == 3 ? F(Fix, 3) : F(Fix, 4)) : (kb == 3 ? F(Flt, 3) : F(Flt, 4)))
 
@@ -599,33 +584,29 @@ cudaError_t prepare(int precision, int kb, size_t smem_fwd, size_t smem_col, siz
 
 cudaError_t launch_tables(const FWork &w, int ntab, int kb, int precision, cudaStream_t st) {
     if (ntab == 0) return cudaSuccess;
-    if (precision == QNG_C128) k_tables<Fix><<<ntab, kTabThreads, 0, st>>>(w, kb);
-    else k_tables<Flt><<<ntab, kTabThreads, 0, st>>>(w, kb);
-    return cudaGetLastError();
+    return launch_next(false, precision == QNG_C128 ? k_tables<Fix> : k_tables<Flt>, ntab, kTabThreads, 0, 1, st, w, kb);
 }
 
 cudaError_t launch_forward(const FWork &w, const Class &c, int precision, cudaStream_t st) {
     if (c.num_inst == 0) return cudaSuccess;
     const int kb = c.kb;
-#define QNG_F(T, KB) launch(k_fwd<T, KB>, c.num_inst << c.cl, c.fwd_threads, c.smem_fwd, c.cl, st, w, c.first_inst, c.cl)
+#define QNG_F(T, KB) launch_next(w.chain, k_fwd<T, KB>, c.num_inst << c.cl, c.fwd_threads, c.smem_fwd, 1u << c.cl, st, w, c.first_inst, c.cl)
     return QNG_FRAMES(QNG_F);
 #undef QNG_F
 }
 
 cudaError_t launch_hpsi(const FWork &w, int first, int num, int precision, cudaStream_t st) {
     if (num == 0) return cudaSuccess;
-    if (precision == QNG_C128) k_heff<Fix><<<num, kHThreads, 0, st>>>(w, first);
-    else k_heff<Flt><<<num, kHThreads, 0, st>>>(w, first);
-    return cudaGetLastError();
+    return launch_next(w.chain, precision == QNG_C128 ? k_heff<Fix> : k_heff<Flt>, num, kHThreads, 0, 1, st, w, first);
 }
 
 cudaError_t launch_columns(const FWork &w, const Class &c, int precision, int first, int num, int metric_im,
                            cudaStream_t st) {
     if (num == 0) return cudaSuccess;
     const int kb = c.kb;
-#define QNG_F(T, KB)                                                                                                 \
-    (metric_im ? launch(k_cols<T, KB, 1>, num << c.cl, c.threads, c.smem_col_im, c.cl, st, w, first, c.cl, c.max_P)  \
-               : launch(k_cols<T, KB, 0>, num << c.cl, c.threads, c.smem_col, c.cl, st, w, first, c.cl, c.max_P))
+#define QNG_F(T, KB)                                                                                             \
+    launch_next(w.chain, metric_im ? k_cols<T, KB, 1> : k_cols<T, KB, 0>, num << c.cl, c.threads,               \
+                metric_im ? c.smem_col_im : c.smem_col, 1u << c.cl, st, w, first, c.cl, c.max_P)
     return QNG_FRAMES(QNG_F);
 #undef QNG_F
 }

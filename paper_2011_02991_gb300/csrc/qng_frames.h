@@ -128,6 +128,7 @@ struct Class {
 
 // Device pointers of the path (the workspace's tables and arrays).
 struct FWork {
+    bool chain = false;  // launches after the tables' follow on as a chain (launch_next)
     const Inst *inst;
     const Run *run;
     const Member *member;
@@ -233,6 +234,7 @@ void build_stream(const std::vector<qng_gate> &gates, const std::vector<qng_paul
                   StreamProgram &out);
 
 struct SWork {
+    bool chain = false;  // as FWork's
     const Run *run;
     const Member *member;
     const SIp *ip;

@@ -44,6 +44,7 @@ template <class T> constexpr int ctas_per_sm(int kb, int nt) {
 __global__ void __launch_bounds__(kHalfThreads) k_half(SWork w, int fix) {
     __shared__ int4 cs[kHalfThreads];
     __shared__ Member mem[kHalfThreads];
+    grid_ready();
     const int r = blockIdx.y;
     const Run &rn = w.run[r];
     const uint32_t nlo = 1u << w.hl, nhi = 1u << (w.n - w.hl);
@@ -182,6 +183,7 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
         const Run &rn = w.run[ps.run0];
         for (int x = threadIdx.x; x < min(rn.ip_count, kRows); x += NT) ips_sh[x] = w.ip[rn.ip_begin + x];
     }
+    grid_ready();
     const int slot = FWD ? col0 : (int)(blockIdx.x % (unsigned)ncol);
     const uint32_t tile = FWD ? blockIdx.x : blockIdx.x / (unsigned)ncol;
     const int wn = w.tb - w.low;  // window bits
@@ -504,6 +506,7 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
     __shared__ int tny[kTerms];
     using S = typename K::S;
     __shared__ double red[256][2];
+    grid_ready();
     const A *v = reinterpret_cast<const A *>(w.b) + ((size_t)in << w.n);
     E *eta = reinterpret_cast<E *>(reinterpret_cast<A *>(w.b) + ((size_t)out << w.n));
     const uint64_t N = 1ull << w.n;
@@ -611,6 +614,7 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
 }
 
 __global__ void k_sfinish(SWork w, int what) {
+    grid_ready();
     const size_t PP = (size_t)w.P * w.P, x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     const bool bad = *w.bad != 0;
@@ -650,14 +654,14 @@ cudaError_t launch_stream_tables(const SWork &w, int precision, cudaStream_t st)
     cudaError_t e = cudaMemsetAsync(w.bad, 0, sizeof(int32_t), st);
     if (e != cudaSuccess || w.R == 0) return e;
     const unsigned n = (1u << w.hl) + (1u << (w.n - w.hl));
-    k_half<<<dim3((n + kHalfThreads - 1) / kHalfThreads, w.R), kHalfThreads, 0, st>>>(w, precision == QNG_C128);
-    return cudaGetLastError();
+    return launch_next(false, k_half, dim3((n + kHalfThreads - 1) / kHalfThreads, w.R), kHalfThreads, 0, 1, st, w,
+                       (int)(precision == QNG_C128));
 }
 
 cudaError_t launch_stream_forward(const SWork &w, const SPass &p, int first, int slot, int precision, cudaStream_t st) {
     const unsigned tiles = 1u << (w.n - w.tb);
     const size_t sm = tile_bytes(precision, w.tb);
-#define QNG_F(T, KB, NT) (k_stream<T, 0, 1, KB, NT><<<tiles, NT, sm, st>>>(w, p, 0, slot, 1, first), cudaGetLastError())
+#define QNG_F(T, KB, NT) launch_next(w.chain, k_stream<T, 0, 1, KB, NT>, tiles, NT, sm, 1, st, w, p, 0, slot, 1, (int)first)
     return QNG_STREAM(QNG_F, w.tb);
 #undef QNG_F
 }
@@ -666,26 +670,22 @@ cudaError_t launch_stream_walk(const SWork &w, const SPass &p, int pass, int col
                                int metric_im, cudaStream_t st) {
     const unsigned grid = (1u << (w.n - w.tb)) * (unsigned)ncol;
     const size_t sm = tile_bytes(precision, w.tb);
-#define QNG_F(T, KB, NT)                                                                                      \
-    ((metric_im ? k_stream<T, 1, 0, KB, NT><<<grid, NT, sm, st>>>(w, p, pass, col0, ncol, store)                  \
-                : k_stream<T, 0, 0, KB, NT><<<grid, NT, sm, st>>>(w, p, pass, col0, ncol, store)),                \
-     cudaGetLastError())
+#define QNG_F(T, KB, NT)                                                                                            \
+    launch_next(w.chain, metric_im ? k_stream<T, 1, 0, KB, NT> : k_stream<T, 0, 0, KB, NT>, grid, NT, sm, 1, st, w, p, pass, \
+                col0, ncol, (int)store)
     return QNG_STREAM(QNG_F, w.tb);
 #undef QNG_F
 }
 
 cudaError_t launch_stream_hpsi(const SWork &w, int in, int out, int precision, cudaStream_t st) {
-    if (precision == QNG_C128) k_sheff<Fix><<<w.hblocks, 256, 0, st>>>(w, in, out);
-    else k_sheff<Flt><<<w.hblocks, 256, 0, st>>>(w, in, out);
-    return cudaGetLastError();
+    return launch_next(w.chain, precision == QNG_C128 ? k_sheff<Fix> : k_sheff<Flt>, w.hblocks, 256, 0, 1, st, w, in, out);
 }
 
 cudaError_t launch_stream_finish(const SWork &w, int what, int precision, cudaStream_t st) {
     (void)precision;
     if (w.P == 0) return cudaSuccess;
     const size_t n = (what & 1) ? (size_t)w.P * w.P : (size_t)w.P;
-    k_sfinish<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(w, what);
-    return cudaGetLastError();
+    return launch_next(w.chain, k_sfinish, (unsigned)((n + 255) / 256), 256, 0, 1, st, w, what);
 }
 
 }  // namespace frames

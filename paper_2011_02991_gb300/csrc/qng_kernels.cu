@@ -1,4 +1,6 @@
-// sm_103a kernels of the on-chip path: every state vector of an instance lives in the shared
+// Assembly and solve of every path, and the gate-by-gate kernels of the on-chip path (explicit launch
+// shapes, the allocation-free metric, instances that the diagonal-frame kernels do not fit; the default
+// is qng_frames.cu). In the latter every state vector of an instance lives in the shared
 // memory of one thread-block cluster (2^cl CTAs, each holding 2^(n-cl) amplitudes), so the
 // O(P^2) recurrence of Algorithm 1 runs without touching HBM except to read checkpoints.
 //
@@ -9,8 +11,9 @@
 //              gate per element, L_ij = prod[dU_i psi_{i-1}, phi_{i+1,j}] (Eq. L_recurrent_def,
 //              the inner loop of Algorithm 1); the extra column P walks eta down the same way
 //              and yields d<E>/d theta_i (reverse sweep)
-//   k_finish   G_ij = L_ij - T_i^* T_j (Eq. g_t_L_def), g = Re G, and the float64 Cholesky solve
-//              of (g + lambda I) dtheta = -dt grad<E> (Eq. 3)
+//   k_assemble G_ij = L_ij - T_i^* T_j (Eq. g_t_L_def), g = Re G, and Im G
+//   k_small    the float64 solve of (g + lambda I) dtheta = -dt grad<E> (Eq. 3) for P < 48;
+//              k_solve the cluster Cholesky, k_finish the one for what no cluster holds
 //
 // Notation used throughout (0-based parameters k = 0..P-1):
 //   Psi[k]    the state after U_{k-1} (Psi[0] = |0>), stored as a checkpoint;
@@ -1303,6 +1306,7 @@ __device__ __forceinline__ void column_item(const Work &w, const DevWork wk, int
 // lower half down the columns, took 58 us for P = 99 against 7 us here).
 __global__ void __launch_bounds__(256) k_assemble(Work w, LaunchArgs a) {
     __shared__ double tr[32][33], ti[32][33];
+    grid_ready();
     const int b = blockIdx.x, tile = blockIdx.y;  // instances along x, which has no 16-bit limit
     const DevInst &in = w.inst[b];
     const int P = in.P, T = (P + 31) / 32;
@@ -1361,6 +1365,7 @@ constexpr int kSmallP = 48;
 __global__ void __launch_bounds__(128) k_small(Work w, LaunchArgs a) {
     __shared__ double A[kSmallP + 1][kSmallP + 1];  // row P: the right-hand side
     __shared__ double inv[kSmallP];
+    grid_ready();
     const int b = blockIdx.x, tid = threadIdx.x;
     const DevInst &in = w.inst[b];
     const int P = in.P;
@@ -1537,6 +1542,7 @@ __global__ void __launch_bounds__(256) k_solve(Work w, LaunchArgs a, int cl) {
     const int C = 1 << cl;
     const int b = blockIdx.x >> cl;
     const int rank = cl ? (int)cg::this_cluster().block_rank() : 0;
+    grid_ready();
     // after the mixed-precision solve: only the instances it handed over (same word in every CTA)
     if (a.ir_gate && w.irflag[b] == 0) return;
     const DevInst in = w.inst[b];
@@ -1776,16 +1782,17 @@ cudaError_t prepare_kernels(int precision, size_t smem_fwd, size_t smem_col, siz
 // theta <- theta + dtheta (the parameter update of Eq. 3), skipped once the device status word
 // holds an error so that a failed solve leaves theta at its last good value.
 __global__ void k_theta_update(double *theta, const double *dtheta, int64_t total, const int32_t *status) {
+    grid_ready();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= total || *status != 0) return;
     theta[k] += dtheta[k];
 }
 
-cudaError_t launch_theta_update(const Work &w, double *theta, const double *dtheta, int64_t total, cudaStream_t st) {
+cudaError_t launch_theta_update(const Work &w, double *theta, const double *dtheta, int64_t total, cudaStream_t st, bool chain) {
     if (total <= 0) return cudaSuccess;
     const int t = 256;
-    k_theta_update<<<(unsigned)((total + t - 1) / t), t, 0, st>>>(theta, dtheta, total, w.status);
-    return cudaGetLastError();
+    return launch_next(chain, k_theta_update, (unsigned)((total + t - 1) / t), t, 0, 1, st, theta, dtheta, total,
+                       (const int32_t *)w.status);
 }
 
 cudaError_t launch_coef(const Work &w, const double *theta, int64_t total, cudaStream_t st) {
@@ -1872,33 +1879,16 @@ cudaError_t prepare_solve(size_t smem) {
 }
 
 cudaError_t launch_solve(const Work &w, int count, int max_P, int cl, const LaunchArgs &a, cudaStream_t st) {
-    const size_t smem = solve_smem_bytes(max_P, cl);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)count << cl);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    if (cl > 0) {
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 1u << cl;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-    }
-    return cudaLaunchKernelEx(&cfg, k_solve, w, a, cl);
+    return launch_next(a.chain, k_solve, (unsigned)count << cl, 256, solve_smem_bytes(max_P, cl), 1u << cl, st, w, a, cl);
 }
 
 cudaError_t launch_finish(const Work &w, int count, int max_P, const LaunchArgs &a, cudaStream_t st) {
     if (!(a.jobs & kJobSolve)) {
         const int T = (max_P + 31) / 32, tiles = (a.jobs & kJobMetric) ? T * (T + 1) / 2 : 1;
-        k_assemble<<<dim3(count, tiles > 0 ? tiles : 1), 256, 0, st>>>(w, a);
-    } else if (max_P < kSmallP) {
-        k_small<<<count, 128, 0, st>>>(w, a);
-    } else {
-        k_finish<<<count, max_P >= 128 ? 512 : 128, 0, st>>>(w, a);
+        return launch_next(a.chain, k_assemble, dim3(count, tiles > 0 ? tiles : 1), 256, 0, 1, st, w, a);
     }
+    if (max_P < kSmallP) return launch_next(a.chain, k_small, count, 128, 0, 1, st, w, a);
+    k_finish<<<count, max_P >= 128 ? 512 : 128, 0, st>>>(w, a);
     return cudaGetLastError();
 }
 

@@ -1,5 +1,6 @@
-// sm_103a kernels of the streaming path, for one instance whose state vectors live in HBM
-// (n > 16 qubits, 2^n amplitudes per register). Algorithm 1 keeps O(1) registers (Sec. 3): the
+// sm_103a kernels of the streaming path's register form, for one instance whose state vectors live in
+// HBM (2^n amplitudes per register): vectors too large or too many for checkpoints, and the smallest
+// sizes when streaming is asked for; the others take qng_frames_stream.cu. Algorithm 1 keeps O(1) registers (Sec. 3): the
 // rolling state psi, the prefix lambda (here "a") and phi (here "b"). Every kernel launch is one
 // pass over the registers it touches: the state is cut into tiles of 2^t amplitudes (the low
 // kLow qubits, contiguous in memory, plus a window of up to kMaxWin other qubits); a CTA loads a

@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_ir(Work w, LaunchArgs a, int m
     __shared__ int s_fail, s_done;
     __shared__ double s_est;
     __shared__ float s_red[2][16];
+    grid_ready();
     const int C = (int)cg::this_cluster().num_blocks();
     const int b = blockIdx.x / C;
     const int rank = (int)cg::this_cluster().block_rank();
@@ -469,19 +470,8 @@ cudaError_t prepare_solve_ir(int P, int C) {
 }
 
 cudaError_t launch_solve_ir(const Work &w, int count, int max_P, int C, const LaunchArgs &a, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(count * C));
-    cfg.blockDim = dim3(512);
-    cfg.dynamicSmemBytes = solve_ir_smem_bytes(max_P, C);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_solve_ir, w, a, max_P, (int)solve_ir_packed(max_P, C));
+    return launch_next(a.chain, k_solve_ir, (unsigned)(count * C), 512, solve_ir_smem_bytes(max_P, C), (unsigned)C, st, w, a,
+                       max_P, (int)solve_ir_packed(max_P, C));
 }
 
 }  // namespace qng
