@@ -37,12 +37,9 @@ METRIC = "QNG steps/s (g,∇E,Δθ) per config; HBM GB/s vs GB300 peak; max err 
 FP64_PEAK_TFLOPS = 2 * 2 * 152 * 2.07e9 / 1e12
 FP32_PEAK_TFLOPS = 128 * 2 * 152 * 2.07e9 / 1e12
 HBM_PEAK_GBS = 6669.2  # measured copy bandwidth of this GPU pool
-# DRAM bytes (read + write) per launch of the timed kernel, from one ncu capture of this build's
-# kernel on the workload; None where no capture of the current kernel exists. 12 qubits
-# (profiles/rand12_p192_c128_step.md): only the first read of the checkpoints reaches DRAM. 28 qubits
-# (profiles/rand28_p252_c64_step.md): mean over 30 consecutive metric passes, each reading the
-# registers it loads and writing the ones it stores.
-TRAFFIC = {"rand12_p192_c128": 12894976, "rand28_p252_c64": 11972552388}
+# DRAM bytes (read + write) per launch of the timed kernel, from an ncu capture of this build's kernel on
+# the workload; empty while no capture of the current kernels at these sizes exists.
+TRAFFIC: dict[str, float] = {}
 
 
 def workloads():
@@ -88,6 +85,13 @@ DESCRIPTION = {
     "vqe_tfim12_p144_c128": "natural-gradient descent (qng_optimize, one iteration per step: step + theta update) "
                             "on the open TFIM chain, 12 qubits, 6 x [Ry, Rz, CZ ladder] (P=144), complex128",
 }
+
+
+# What the flop counts below are: the work of the recurrence taken gate by gate, the same for every
+# implementation. The diagonal-frame kernels do less (two products per amplitude and run of commuting
+# gates) and run complex128 on the integer pipes, so this rate can exceed the float64 pipe's peak.
+GATE_WORK = ("flops of the gate-by-gate recurrence, against the pipe of its precision; the kernel takes runs of "
+             "commuting gates at once, complex128 in fixed point on the integer pipes, so frac can exceed 1")
 
 
 # ------------------------------------------------------------------------------------------
@@ -461,7 +465,7 @@ def measure(name, steps, warmup, dev, rank, world, local_rank, check=True, shard
 
 
 def roofline(res, steps):
-    """Roofline of the step's dominant kernel class (see DESIGN: algorithmic work per unit)."""
+    """Roofline of the step's dominant kernel class, on the algorithmic work per unit."""
     from paper_2011_02991_gb300 import workloads as W
     problems, kind, prof, name = res["problems"], res["kind"], res["prof"], res["name"]
     prec64 = problems[0].precision == W.C128
@@ -475,14 +479,14 @@ def roofline(res, steps):
             achieved = flops / met_s / 1e12
             return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                     "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
-                    "kernel": "k_pass metric passes", "kernel_avg_ms": met_s * 1e3 * steps / max(col_n, 1),
+                    "kernel": "k_stream walk", "note": GATE_WORK, "kernel_avg_ms": met_s * 1e3 * steps / max(col_n, 1),
                     "flops_per_step": flops, "launches_per_step": col_n / steps,
                     "peak_source": "derived: float64 2 FMA/clk/SM x 152 SMs x 2.07 GHz"}
         achieved = mb / met_s / 1e9
         traffic = TRAFFIC.get(name)
         return {"bound": "hbm", "achieved": achieved, "peak": HBM_PEAK_GBS, "unit": "GB/s",
                 "frac": achieved / HBM_PEAK_GBS, "traffic": traffic,
-                "kernel": "k_pass_phased metric passes (registers loaded and stored per pass)",
+                "kernel": "k_stream walk (columns loaded and stored and checkpoints read per pass)",
                 "kernel_avg_ms": col_ms / max(col_n, 1), "bytes_per_launch": mb / max(mp, 1),
                 "bytes_per_step": mb, "launches_per_step": mp, "peak_source": "measured copy bandwidth (of measured)"}
     col_avg_s = col_ms / max(col_n, 1) / 1e3
@@ -491,22 +495,19 @@ def roofline(res, steps):
     flops = flops_step / max(launches_per_step, 1)                # per launch, averaged
     peak = FP64_PEAK_TFLOPS if prec64 else FP32_PEAK_TFLOPS
     achieved = flops_step * steps / (col_ms / 1e3) / 1e12 if col_ms > 0 else 0.0
-    # complex128 batches run their launch groups side by side: the column launches overlap, and the
-    # sum of their durations overstates the time; the whole step's time bounds it from above
-    overlap = kind == "batch" and prec64
+    # batches run their launch classes side by side: the column launches overlap, and the sum of their
+    # durations overstates the time; the whole step's time bounds it from above
+    overlap = kind == "batch"
     if overlap:
         achieved = flops_step * steps / (res["ms_total"] / 1e3) / 1e12
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": TRAFFIC.get(name), "kernel": "k_columns (recurrence + gradient sweep)",
+            "traffic": TRAFFIC.get(name), "kernel": "k_cols (column walk, gradient column included)", "note": GATE_WORK,
             "peak_source": "derived: float64 2 FMA/clk/SM x 152 SMs x 2.07 GHz" if prec64 else
                            "derived: float32 128 FMA/clk/SM x 152 SMs x 2.07 GHz",
             "kernel_avg_ms": col_avg_s * 1e3, "flops_per_launch": flops, "launches_per_step": launches_per_step}
     if overlap:
-        roof["note"] = ("launch groups side by side: achieved divides the step's column flops by the whole "
-                        "step's time (sweep and solve included), a lower bound")
-    if res["pipeline"]:
-        roof["note"] = ("pipelined sweep: the column launches overlap one another and the sweep; achieved divides "
-                        "the step's column flops by the sum of their durations, a lower bound")
+        roof["note"] += ("; launch classes side by side: achieved divides the step's column flops by the whole "
+                         "step's time (sweep and solve included), a lower bound")
     return roof
 
 
