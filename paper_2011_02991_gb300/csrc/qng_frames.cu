@@ -14,8 +14,9 @@
 // unit norm, so no component ever exceeds sqrt 2 between transitions (4 sqrt 2 inside one), additions
 // are exact and a product rounds at 2^-60, where float64 would round at 2^-53 of the component.
 // Products come from 32-bit halves in signed (balanced) form, x = hi 2^32 + lo: hi hi and the two
-// cross terms, six IMAD.WIDE for a sum of two products; lo lo (below 2^-62) is left out. Inner
-// products sum 2^-60 units exactly in 64-bit integers, whatever the order.
+// cross terms, six IMAD.WIDE for a sum of two products; lo lo (below 2^-62) is left out of the factors'
+// products and taken into the inner products'. Those sum 2^-60 units exactly in 64-bit integers, whatever
+// the order.
 // complex64 runs the same steps on float32 amplitudes.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>

@@ -103,7 +103,7 @@ struct DevWork {
     int32_t col;  // 0..P-1: metric column; P: gradient (adjoint) column
 };
 constexpr int kSolveBlock = 16;      // block width of the block solve
-constexpr int kBlockSolveMinP = 48;  // smaller instances use k_finish
+constexpr int kBlockSolveMinP = 48;  // smaller instances use k_small
 
 // Coefficients of parameter k (float64): c = cos(theta/2), s = sin(theta/2), and the scaled
 // form of the adjoint rotation R^dag = c I + i s sigma = f (I + i t sigma) (|c| >= |s|) or
