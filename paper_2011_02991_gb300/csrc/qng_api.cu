@@ -369,7 +369,7 @@ bool plan_sframes(qng_ctx *c) {
     if (reg > (4ll << 30)) return false;
     int low = std::min(2 * tb - h.n, kb);
     if (low < (pi ? 1 : 2)) low = pi ? 3 : 4;
-    frames::build_stream(h.gates, h.terms, h.n, kb, tb, low, c->sp);
+    frames::build_stream(h.gates, h.terms, h.n, kb, tb, low, pi == 1, c->sp);
     const int R = (int)c->sp.runs.size();
     // column slots: what a launch walks together. Up to 20 qubits 32 MiB of them (enough CTAs, and L2 holds
     // them between passes), beyond that four, which share each checkpoint read
@@ -497,7 +497,7 @@ bool plan_frames(qng_ctx *c) {
         frames::Inst d = {};
         d.cl = frames_cl(c, h.n, kb);
         frames::Program &p = prog[b];
-        frames::build_program(h.gates, h.masks, h.terms, h.n, kb, d.cl, p);
+        frames::build_program(h.gates, h.masks, h.terms, h.n, kb, d.cl, c->precision == QNG_C128, p);
         d.n = h.n;
         d.nE = p.nE;
         d.R = (int32_t)p.runs.size();

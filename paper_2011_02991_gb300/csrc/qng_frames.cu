@@ -115,8 +115,7 @@ __device__ __forceinline__ void exchange(typename T::A (&b)[1 << KB], unsigned c
 
 // ------------------------------------------------------------------------------------------
 // Factor tables: entry k * 2^(nE-kb) + t of run r is the factor of amplitude (t, k) in the run's
-// arrangement, times 2^(-khalf/2) of the transition before it (fixed point: only the odd sqrt 1/2, the
-// rest is halved away inside the transition). The products are taken in fixed point for both
+// arrangement, times 2^(-khalf/2) of the transition before it (table_half). The products are taken in fixed point for both
 // precisions (2^61 = 1, cos and sin of float64): members that do not touch the thread's own two index
 // bits multiply one common factor, the others each of the four.
 template <class T> __global__ void __launch_bounds__(kTabThreads) k_tables(FWork w, int kb) {
@@ -135,7 +134,7 @@ template <class T> __global__ void __launch_bounds__(kTabThreads) k_tables(FWork
     const uint32_t t = u & (TC - 1u), kq = (u / TC) * kTabAmps;
     const uint32_t base = ((t >> low) << (low + kb)) | (t & ((1u << low) - 1u)) | (kq << low);
     const uint32_t own = (uint32_t)(kTabAmps - 1) << low;
-    const int half = sizeof(typename T::A) == 16 ? (rn.khalf & 1) : rn.khalf;
+    const int half = rn.khalf;
     longlong2 com = {__double2ll_rn(((half & 1) ? 0.70710678118654752440 : 1.0) * exp2((double)(61 - (half >> 1)))), 0};
     longlong2 f[kTabAmps];
     bool any_own = false;  // uniform over the block

@@ -111,6 +111,12 @@ __device__ __forceinline__ void halve(longlong2 &x, int s) {
     x.y = (x.y + (h + (((int)x.y >> s) & 1))) >> s;
 }
 
+__device__ __forceinline__ void halve(float2 &x, int s) {
+    const float h = __int_as_float((127 - s) << 23);
+    x.x *= h;
+    x.y *= h;
+}
+
 __device__ __forceinline__ ll shfl(ll v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ float shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 
@@ -128,7 +134,7 @@ template <typename T> __device__ __forceinline__ T warp8(const T (&a)[8], int la
     return v;
 }
 
-// Hadamards (unnormalised) on the thread's bits hm, then `shift` halvings in fixed point.
+// Hadamards (unnormalised) on the thread's bits hm, then `shift` halvings.
 template <class T, int KB> __device__ __forceinline__ void hadamards(typename T::A (&b)[1 << KB], int hm, int shift) {
 #pragma unroll
     for (int j = 0; j < KB; ++j)
@@ -141,11 +147,9 @@ template <class T, int KB> __device__ __forceinline__ void hadamards(typename T:
                     b[k | (1 << j)] = x - y;
                 }
         }
-    if constexpr (sizeof(typename T::A) == 16) {
-        if (shift) {
+    if (shift) {
 #pragma unroll
-            for (int k = 0; k < (1 << KB); ++k) halve(b[k], shift);
-        }
+        for (int k = 0; k < (1 << KB); ++k) halve(b[k], shift);
     }
 }
 

@@ -27,6 +27,14 @@ namespace frames {
 
 constexpr int kRegBitsMax = 4;  // a thread holds 2^kb amplitudes, kb index bits at a time (kb = 3 or 4)
 
+// A transition of k Hadamards (unnormalised, sqrt 2 times an isometry each) and the run after it. Fixed point
+// halves floor(k / 2) times inside the transition and leaves the odd sqrt 1/2 to the run's factor. float32 has the
+// range to leave all of 2^(-k/2) to the factor, which costs nothing, but only to a bound: the table's products are
+// multiples of 2^-61, so 2^-24 relative needs 2^(-k/2) well above 2^-37, and circuits of H and CNOT alone put any
+// number of Hadamards into one transition. Longer transitions are halved inside as in fixed point.
+constexpr int kTableHalf = 48;
+inline int table_half(int k, bool fixed) { return fixed || k > kTableHalf ? (k & 1) : k; }
+
 // A diagonal factor of a run. With par = parity(m & z) and on = ((m & ctrl) == cval):
 //   kind 0 (rotation):  on ? cos(theta/2) - i lam sin(theta/2) : 1,  lam = sgn (-1)^par
 //   kind 1 (sign gate): on ? lam : 1
@@ -55,17 +63,18 @@ struct Run {
     int32_t ip_begin, ip_count;    // Ip table; parameters ip_first .. ip_first + ip_count - 1 in order
     int32_t ip_first;
     int32_t low;                   // lowest of the index bits a thread holds at this run
-    int32_t khalf;                 // Hadamards since the run before (each is sqrt 2 times an isometry)
+    int32_t khalf;                 // Hadamards since the run before (each is sqrt 2 times an isometry) that its
+                                   // factor normalises; the others are halved away inside the transition
     int32_t simple;                // every parameter: no control, at most one of the thread's bits
 };
 
 // One step of the vector: exchange into arrangement `low` (through permutation perm >= 0), Hadamards
-// on the thread's bits hm followed by `shift` halvings (fixed point), then run `run` (>= 0).
+// on the thread's bits hm followed by `shift` halvings, then run `run` (>= 0).
 struct UOp {
     int16_t low;    // -1: no exchange
     int16_t hm;
-    int16_t shift;
-    int16_t rshift; // halvings right before the run (streaming)
+    int16_t shift;  // halvings after the Hadamards (float32: of long transitions only)
+    int16_t rshift; // halvings right before the run (streaming, fixed point)
     int32_t perm;   // -1: none
     int32_t run;
 };
@@ -174,10 +183,10 @@ struct Program {  // one instance, host side
 };
 
 // Build the program of one circuit on index bits [0, nE), kb of them per thread and the top cl
-// distributed over CTAs.
+// distributed over CTAs; fixed: for fixed-point vectors, else for float32 ones.
 // Indices in the program (members, perms) are relative to its own tables.
 void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks,
-                   const std::vector<qng_pauli> &terms, int n, int kb, int cl, Program &out);
+                   const std::vector<qng_pauli> &terms, int n, int kb, int cl, bool fixed, Program &out);
 
 // ------------------------------------------------------------------------------------------
 // Streaming: one instance whose vectors lie in global memory. A pass loads tiles of 2^tb amplitudes (the
@@ -231,7 +240,7 @@ inline int stream_tile_bits(int precision, int n) {
 }
 inline int stream_reg_bits(int tb) { return tb == 13 ? 5 : 4; }
 void build_stream(const std::vector<qng_gate> &gates, const std::vector<qng_pauli> &terms, int n, int kb, int tb, int low,
-                  StreamProgram &out);
+                  bool fixed, StreamProgram &out);
 
 struct SWork {
     bool chain = false;  // as FWork's

@@ -227,7 +227,7 @@ std::vector<DevTerm> final_terms(const std::vector<qng_pauli> &terms, int n, con
 }  // namespace
 
 void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks,
-                   const std::vector<qng_pauli> &terms, int n, int kb, int cl, Program &out) {
+                   const std::vector<qng_pauli> &terms, int n, int kb, int cl, bool fixed, Program &out) {
     out = Program();
     out.n = n;
     out.kb = kb;
@@ -300,6 +300,9 @@ void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_
             }
         }
     };
+    std::vector<int> had(R + 1, 0);  // Hadamards of the transition before run r (none after the last)
+    for (int r = 0; r < R; ++r)
+        for (const Stage &s : B.tau[r]) if (!s.perm) had[r] += __builtin_popcount(s.h);
     const int dflt = cl > 0 ? lows.front() : lows.back();
     cur = R > 0 ? first_need(B.tau[0], 0, dflt) : first_need(tail, 0, dflt);
     out.start0 = cur;
@@ -313,7 +316,7 @@ void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_
         run.ip_begin = (int)out.ips.size();
         run.ip_first = -1;
         run.simple = 1;
-        for (const Stage &s : B.tau[r]) if (!s.perm) run.khalf += __builtin_popcount(s.h);
+        run.khalf = table_half(had[r], fixed);
         const int L = cur;
         auto thr = [&](uint32_t m) { return (m & ((1u << L) - 1u)) | ((m >> (L + kb)) << L); };
         auto reg = [&](uint32_t m) { return (m >> L) & ((1u << kb) - 1u); };
@@ -342,11 +345,10 @@ void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_
     emit_tau(tail);
     out.end_low = cur;
 
-    // fuse into steps: exchange, then Hadamards, then a run. Halvings keep the fixed-point vector
-    // within sqrt 2 of unit norm: floor(k / 2) after k Hadamards of a transition, the odd sqrt 2 is in
-    // the run's factor table.
+    // fuse into steps: exchange, then Hadamards, then a run. Halvings keep the vector within sqrt 2 of unit
+    // norm: floor(k / 2) after k Hadamards of a transition, unless its run's factor takes all of them.
     auto fuse = [&](const std::vector<Step> &v, bool back, std::vector<UOp> &ops) {
-        int k = 0;
+        int k = 0, tr = back ? R : 0;  // the transition that the next steps belong to
         UOp u{-1, 0, 0, 0, -1, -1};
         int stage = 0;  // 0 nothing yet, 1 exchange, 2 Hadamards
         auto flush = [&]() { ops.push_back(u); u = UOp{-1, 0, 0, 0, -1, -1}; stage = 0; };
@@ -367,7 +369,7 @@ void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_
                 if (stage > 1) flush();
                 u.hm = (int16_t)s.h;
                 const int k1 = k + __builtin_popcount(s.h);
-                u.shift = (int16_t)(k1 / 2 - k / 2);
+                u.shift = (int16_t)(table_half(had[tr], fixed) == had[tr] ? 0 : k1 / 2 - k / 2);
                 k = k1;
                 stage = 2;
             } else {
@@ -375,6 +377,7 @@ void build_program(const std::vector<qng_gate> &gates, const std::vector<uint64_
                 if (back) out.bwd_entry[s.run] = (int32_t)ops.size();
                 flush();
                 k = 0;
+                tr = back ? s.run : s.run + 1;
             }
         }
         if (stage > 0) flush();
@@ -422,7 +425,8 @@ std::vector<int> executable(const std::vector<Atom> &at, const std::vector<uint8
     return ex;
 }
 
-void pack_passes(const std::vector<Atom> &at, bool back, StreamProgram &P, std::vector<SPass> &out) {
+void pack_passes(const std::vector<Atom> &at, bool back, bool fixed, const std::vector<int> &had, StreamProgram &P,
+                 std::vector<SPass> &out) {
     const int n = P.n, kb = P.kb, tb = P.tb;
     std::vector<Window> wins;
     wins.push_back(Window{P.low, P.low, tb - P.low});  // the lowest tb bits
@@ -436,10 +440,12 @@ void pack_passes(const std::vector<Atom> &at, bool back, StreamProgram &P, std::
     };
     std::vector<uint8_t> done(at.size(), 0);
     size_t from = 0;
-    // Hadamards since the last run, and halvings of the fixed-point vector (once three are due, at a run and at
-    // the end of a pass): floor(k / 2) in all, the odd sqrt 1/2 is in the run's factor. Between them the
-    // vector grows to 2^4.5 of its norm at most (two halvings due, an odd Hadamard, a block of four more)
-    int k = 0, halved = 0;
+    // Hadamards since the last run, and halvings (fixed point: once three are due, at a run and at the end of a
+    // pass): floor(k / 2) in all, the odd sqrt 1/2 is in the run's factor. Between them the vector grows to
+    // 2^4.5 of its norm at most (two halvings due, an odd Hadamard, a block of four more). float32 halves after
+    // each step of the transitions whose factor does not take it all
+    int k = 0, halved = 0, tr = back ? (int)P.runs.size() : 0;
+    auto due = [&]() { return table_half(had[tr], fixed) == had[tr] ? 0 : k / 2 - halved; };
     while (from < at.size()) {
         std::vector<int> best;
         Window W = wins[0];
@@ -488,8 +494,8 @@ void pack_passes(const std::vector<Atom> &at, bool back, StreamProgram &P, std::
                     if (stage > 1) flush();
                     u.hm = (int16_t)m;
                     k += __builtin_popcount(m);
-                    if (k / 2 - halved >= 3) {
-                        u.shift = (int16_t)(k / 2 - halved);
+                    if (due() >= (fixed ? 3 : 1)) {
+                        u.shift = (int16_t)due();
                         halved = k / 2;
                     }
                     stage = 2;
@@ -531,15 +537,16 @@ void pack_passes(const std::vector<Atom> &at, bool back, StreamProgram &P, std::
                         ip.z = ip.src ? 0u : ip.zall;
                     }
                 }
-                u.rshift = (int16_t)(k / 2 - halved);
+                u.rshift = (int16_t)due();
                 flush();
                 k = halved = 0;
+                tr = back ? a.run : a.run + 1;
                 ++i;
             }
         }
         if (cur <= 0 && lows.back() > 0) goto_low(lows.back(), -1);
         flush();
-        ps.shift = k / 2 - halved;
+        ps.shift = due();
         halved = k / 2;
         ps.nops = (int32_t)P.ops.size() - ps.op_begin;
         out.push_back(ps);
@@ -551,7 +558,7 @@ void pack_passes(const std::vector<Atom> &at, bool back, StreamProgram &P, std::
 }  // namespace
 
 void build_stream(const std::vector<qng_gate> &gates, const std::vector<qng_pauli> &terms, int n, int kb, int tb, int low,
-                  StreamProgram &out) {
+                  bool fixed, StreamProgram &out) {
     out = StreamProgram();
     out.n = n;
     out.kb = kb;
@@ -572,6 +579,7 @@ void build_stream(const std::vector<qng_gate> &gates, const std::vector<qng_paul
         B.tau.pop_back();
     }
     const int R = (int)B.run_members.size();
+    std::vector<int> had(R + 1, 0);
     std::vector<Atom> fwd;
     auto add_tau = [&](const std::vector<Stage> &t) {
         for (const Stage &s : t) {
@@ -587,7 +595,8 @@ void build_stream(const std::vector<qng_gate> &gates, const std::vector<qng_paul
         run.mem_count = (int)B.run_members[r].size();
         run.ip_begin = (int)out.ips.size();
         run.ip_first = -1;
-        for (const Stage &s : B.tau[r]) if (!s.perm) run.khalf += __builtin_popcount(s.h);
+        for (const Stage &s : B.tau[r]) if (!s.perm) had[r] += __builtin_popcount(s.h);
+        run.khalf = table_half(had[r], fixed);
         for (const Member &m : B.run_members[r]) {
             out.members.push_back(m);
             if (m.kind != 0) continue;
@@ -605,9 +614,9 @@ void build_stream(const std::vector<qng_gate> &gates, const std::vector<qng_paul
         if (it->kind == 2 && it->run == 0) break;
     }
     out.entry.assign(R, SEntry{0, 0, 0, 0});
-    pack_passes(fwd, false, out, out.fwd);
+    pack_passes(fwd, false, fixed, had, out, out.fwd);
     if (out.fwd.empty()) out.fwd.push_back(SPass{low, tb - kb, 0, 0, -1, 0});  // no gate that moves |0...0>
-    if (R > 0) pack_passes(bwd, true, out, out.bwd);
+    if (R > 0) pack_passes(bwd, true, fixed, had, out, out.bwd);
     out.terms = final_terms(terms, n, B);
 }
 

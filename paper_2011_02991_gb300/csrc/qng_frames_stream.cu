@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_half(SWork w, int fix) {
     const uint32_t own = lo ? nlo - 1u : ~(nlo - 1u);       // this half's bits
     const uint32_t m = lo ? e : (e - nlo) << w.hl;          // index with the other half 0
     const int mem_count = rn.mem_count, mem_begin = rn.mem_begin;
-    const int half = fix ? (rn.khalf & 1) : rn.khalf;
+    const int half = rn.khalf;
     longlong2 f = {1ll << 61, 0};
     if (lo) f.x = __double2ll_rn(((half & 1) ? 0.70710678118654752440 : 1.0) * exp2((double)(61 - (half >> 1))));
     uint32_t mask = 0;
@@ -287,9 +287,12 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
                 if (u.perm >= 0) __syncthreads();  // others still read what this thread writes next
             }
             if (u.hm) hadamards<T, KB>(b, u.hm, 0);
-            if (sizeof(A) == 16 && u.shift) {
+            if (u.shift) {
 #pragma unroll
-                for (int k = 0; k < NA; ++k) scale_down(b[k], u.shift, dith(k + 384));
+                for (int k = 0; k < NA; ++k) {
+                    if constexpr (sizeof(A) == 16) scale_down(b[k], u.shift, dith(k + 384));
+                    else halve(b[k], u.shift);
+                }
             }
         }
         if (u.run >= 0) {

@@ -3,7 +3,8 @@
 // executes it in float64 on the host, step by step as the kernels do (exchanges, permutations,
 // Hadamards on a thread's own bits, runs), and prints
 //   E <energy>, grad <P values>, L <re im> for i < j, sigma <P values>, ctrl <P values>
-// Structural invariants are checked on the way ("bad <what>", exit 1).
+// Structural invariants are checked on the way ("bad <what>", exit 1). Both forms of a program, for float32 and
+// for fixed-point vectors, are executed and have to agree; halvings are where the kernels have them.
 // The same for the streaming program (tiles of 2^tb amplitudes, `low` contiguous low bits) when tb > 0.
 // Input (stdin): n P G T kb cl tb low, G lines "kind q0 q1 param xmask zmask", T lines "coeff x z", P angles.
 #include <cmath>
@@ -23,6 +24,15 @@ static void bad(const char *what, long a, long b) {
     std::exit(1);
 }
 
+// Halvings. Fixed-point vectors have room for 2^4.5 of their norm, float32 ones are left to grow to 2^(kTableHalf / 2).
+static void scale(std::vector<cd> &v, int shift, bool fixed) {
+    double nrm = 0, f = std::ldexp(1.0, -shift);
+    for (const cd &x : v) nrm += std::norm(x);
+    if (std::sqrt(nrm) > std::ldexp(1.0001, fixed ? 5 : kTableHalf / 2)) bad("growth", (long)std::log2(nrm), shift);
+    if (shift < 0 || shift > 32) bad("shift", shift, 0);
+    for (cd &x : v) x *= f;
+}
+
 static cd member_factor(const std::vector<Member> &mem, const Run &rn, const std::vector<double> &th, uint32_t m) {
     cd f = std::pow(0.5, 0.5 * rn.khalf);
     for (int k = 0; k < rn.mem_count; ++k) {
@@ -36,8 +46,19 @@ static cd member_factor(const std::vector<Member> &mem, const Run &rn, const std
     return f;
 }
 
+// Prints the first form's results and holds the second's against them.
 static void print_all(double E, const std::vector<double> &grad, const std::vector<double> &sig, const std::vector<double> &ctrl,
                       const std::vector<cd> &Lm, int P, int R) {
+    static std::vector<double> first;
+    std::vector<double> all{E};
+    for (const auto *x : {&grad, &sig, &ctrl}) all.insert(all.end(), x->begin(), x->end());
+    for (int j = 0; j < P; ++j) for (int i = 0; i < j; ++i) { all.push_back(Lm[(size_t)i * P + j].real()); all.push_back(Lm[(size_t)i * P + j].imag()); }
+    if (!first.empty()) {
+        for (size_t k = 0; k < all.size(); ++k)
+            if (!(std::fabs(all[k] - first[k]) <= 1e-11 * (1 + std::fabs(first[k])))) bad("forms differ", (long)k, P);
+        return;
+    }
+    first = all;
     std::printf("E %.17g\nruns %d\n", E, R);
     auto vec = [&](const char *nm, const std::vector<double> &x) {
         std::printf("%s", nm);
@@ -49,13 +70,14 @@ static void print_all(double E, const std::vector<double> &grad, const std::vect
     vec("ctrl", ctrl);
     std::printf("L");
     for (int j = 0; j < P; ++j) for (int i = 0; i < j; ++i) std::printf(" %.17g %.17g", Lm[(size_t)i * P + j].real(), Lm[(size_t)i * P + j].imag());
-    std::printf("\nok\n");
+    std::printf("\n");
 }
 
 static int stream(const std::vector<qng_gate> &gates, const std::vector<qng_pauli> &terms, const std::vector<double> &th, int n,
-                  int P, int kb, int tb, int lowbits) {
+                  int P, int kb, int tb, int lowbits, bool fixed) {
     StreamProgram pr;
-    build_stream(gates, terms, n, kb, tb, lowbits, pr);
+    build_stream(gates, terms, n, kb, tb, lowbits, fixed, pr);
+    for (const Run &r : pr.runs) if (r.khalf > kTableHalf) bad("factor", r.khalf, 0);
     const uint32_t N = 1u << n;
     const int R = (int)pr.runs.size(), w = tb - lowbits;
     int low = -1;
@@ -88,6 +110,7 @@ static int stream(const std::vector<qng_gate> &gates, const std::vector<qng_paul
                         v[m | bit] = x - y;
                     }
             }
+        scale(v, u.shift, fixed);
     };
     std::vector<std::vector<cd>> psi(R);
     std::vector<cd> v(N, 0.0);
@@ -102,11 +125,13 @@ static int stream(const std::vector<qng_gate> &gates, const std::vector<qng_paul
             if (u.run < 0) continue;
             if (u.run != last + 1) bad("run order", u.run, last);
             last = u.run;
+            scale(v, u.rshift, fixed);
             double nrm = 0;
             for (uint32_t m = 0; m < N; ++m) nrm += std::norm(v[m] *= member_factor(pr.members, pr.runs[u.run], th, m));
             if (std::fabs(nrm - 1) > 1e-9) bad("norm", u.run, (long)(nrm * 1e6));
             psi[u.run] = v;
         }
+        scale(v, ps.shift, fixed);
     }
     if (last != R - 1) bad("forward end", last, R);
     std::vector<cd> eta(N, 0.0);
@@ -141,6 +166,7 @@ static int stream(const std::vector<qng_gate> &gates, const std::vector<qng_paul
                 if (own && u.run != run) bad("entry", run, u.run);
                 if (u.run < 0) continue;
                 if (low == 0 && tb > kb) bad("run in block 0", u.run, 0);
+                if (!own) scale(b, u.rshift, fixed);
                 const Run &rn = pr.runs[u.run];
                 for (uint32_t m = 0; m < N; ++m) p[m] = std::conj(psi[u.run][m]) * b[m];
                 for (int q = 0; q < rn.ip_count; ++q) {
@@ -152,6 +178,7 @@ static int stream(const std::vector<qng_gate> &gates, const std::vector<qng_paul
                 if (own) { cd s = 0; for (const cd &x : p) s += x; sig[col] = std::real(s); }
                 for (uint32_t m = 0; m < N; ++m) b[m] *= std::conj(member_factor(pr.members, rn, th, m));
             }
+            scale(b, ps.shift, fixed);
         }
     };
     for (int r = 0; r < R; ++r)
@@ -167,29 +194,11 @@ static int stream(const std::vector<qng_gate> &gates, const std::vector<qng_paul
     return 0;
 }
 
-int main() {
-    int n, P, G, T, kb, cl, tb, lowbits;
-    if (std::scanf("%d %d %d %d %d %d %d %d", &n, &P, &G, &T, &kb, &cl, &tb, &lowbits) != 8) return 2;
-    std::vector<qng_gate> gates(G);
-    std::vector<uint64_t> masks(2 * G);
-    for (int g = 0; g < G; ++g) {
-        unsigned long long x, z;
-        if (std::scanf("%d %d %d %d %llu %llu", &gates[g].kind, &gates[g].q0, &gates[g].q1, &gates[g].param, &x, &z) != 6) return 2;
-        masks[2 * g] = x;
-        masks[2 * g + 1] = z;
-    }
-    std::vector<qng_pauli> terms(T);
-    for (qng_pauli &t : terms) {
-        unsigned long long x, z;
-        if (std::scanf("%lf %llu %llu", &t.coeff, &x, &z) != 3) return 2;
-        t.xmask = x;
-        t.zmask = z;
-    }
-    std::vector<double> th(P);
-    for (double &t : th) if (std::scanf("%lf", &t) != 1) return 2;
-    if (tb > 0) return stream(gates, terms, th, n, P, kb, tb, lowbits);
+static int onchip(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks, const std::vector<qng_pauli> &terms,
+                  const std::vector<double> &th, int n, int P, int kb, int cl, bool fixed) {
     Program pr;
-    build_program(gates, masks, terms, n, kb, cl, pr);
+    build_program(gates, masks, terms, n, kb, cl, fixed, pr);
+    for (const Run &r : pr.runs) if (r.khalf > kTableHalf) bad("factor", r.khalf, 0);
     const uint32_t N = 1u << pr.nE;
     const int R = (int)pr.runs.size();
     auto factor = [&](int r, uint32_t m) {
@@ -228,6 +237,7 @@ int main() {
                         v[m] = x + y;
                         v[m | (1u << (low + b))] = x - y;
                     }
+        scale(v, u.shift, fixed);
     };
     std::vector<std::vector<cd>> psi(R);
     std::vector<cd> v(N, 0.0);
@@ -317,5 +327,33 @@ int main() {
         for (uint32_t m = 0; m < N; ++m) eta[m] *= std::conj(factor(u.run, m));
     }
     print_all(E, grad, sig, ctrl, Lm, P, R);
+    return 0;
+}
+
+int main() {
+    int n, P, G, T, kb, cl, tb, lowbits;
+    if (std::scanf("%d %d %d %d %d %d %d %d", &n, &P, &G, &T, &kb, &cl, &tb, &lowbits) != 8) return 2;
+    std::vector<qng_gate> gates(G);
+    std::vector<uint64_t> masks(2 * G);
+    for (int g = 0; g < G; ++g) {
+        unsigned long long x, z;
+        if (std::scanf("%d %d %d %d %llu %llu", &gates[g].kind, &gates[g].q0, &gates[g].q1, &gates[g].param, &x, &z) != 6) return 2;
+        masks[2 * g] = x;
+        masks[2 * g + 1] = z;
+    }
+    std::vector<qng_pauli> terms(T);
+    for (qng_pauli &t : terms) {
+        unsigned long long x, z;
+        if (std::scanf("%lf %llu %llu", &t.coeff, &x, &z) != 3) return 2;
+        t.xmask = x;
+        t.zmask = z;
+    }
+    std::vector<double> th(P);
+    for (double &t : th) if (std::scanf("%lf", &t) != 1) return 2;
+    for (const bool fixed : {false, true}) {
+        const int rc = tb > 0 ? stream(gates, terms, th, n, P, kb, tb, lowbits, fixed) : onchip(gates, masks, terms, th, n, P, kb, cl, fixed);
+        if (rc) return rc;
+    }
+    std::printf("ok\n");
     return 0;
 }

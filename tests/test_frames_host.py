@@ -97,6 +97,26 @@ def test_z_runs_and_no_parameters(probe, oracle):
     check(probe, oracle, W.Problem("fixed", c, h, np.zeros(0)))
 
 
+def brickwork(n, layers, seed=0):
+    """Layers of H on the even qubits and a CNOT from each to its neighbour, then one layer of RY: all of the Hadamards lie
+    in one transition (the frame does not absorb one behind a CNOT)."""
+    rows = []
+    for k in range(layers):
+        rows += [[W.H, q, -1, -1] for q in range(0, n, 2)] + [[W.CNOT, q, q + 1, -1] for q in range(0, n - 1, 2)]
+    rows += [[W.RY, q, -1, q] for q in range(n)]
+    rng = np.random.Generator(np.random.PCG64([n, layers, seed]))
+    return W.Problem("brickwork", W.Circuit(n, np.array(rows, dtype=np.int32)), W.random_pauli_hamiltonian(n, 12, rng),
+                     W.uniform_theta(n, rng))
+
+
+@pytest.mark.parametrize("n,layers", [(5, 3), (6, 16), (7, 30), (9, 60)])
+def test_long_transitions(probe, oracle, n, layers):
+    """More Hadamards in one transition than a factor table can normalise (its entries are multiples of 2^-61)."""
+    p = brickwork(n, layers)
+    check(probe, oracle, p, 3)
+    check(probe, oracle, p, 3, 0, 5, 2)
+
+
 @pytest.mark.parametrize("n,kb,tb,low", [(7, 3, 5, 2), (9, 3, 6, 3), (8, 3, 7, 3), (9, 4, 6, 1), (10, 3, 6, 3), (6, 4, 6, 2)])
 @pytest.mark.parametrize("seed", range(4))
 def test_streaming_passes(probe, oracle, n, kb, tb, low, seed):

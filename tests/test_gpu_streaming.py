@@ -201,3 +201,27 @@ def test_launch_chain(qng, n, layers, path, precision):
             ctx.sync()
             for k in out:
                 assert torch.equal(out[k], ref[t][k]), (t, k)
+
+
+@pytest.mark.parametrize("precision", [W.C64, W.C128])
+@pytest.mark.parametrize("n,path", [(9, 1), (12, 1), (14, 2)])
+def test_long_transitions(qng, oracle, n, path, precision):
+    """Circuits of H and CNOT before the first rotation: 32 layers put 16 n Hadamards into one transition, whose
+    2^(-8 n) is below what a factor table or a float32 amplitude holds."""
+    rows = []
+    for k in range(32):
+        rows += [[W.H, q, -1, -1] for q in range(0, n, 2)] + [[W.CNOT, q, q + 1, -1] for q in range(0, n - 1, 2)]
+    rows += [[W.RY, q, -1, q] for q in range(n)]
+    rng = np.random.Generator(np.random.PCG64([n, path]))
+    p = W.Problem("long", W.Circuit(n, np.array(rows, dtype=np.int32)), W.random_pauli_hamiltonian(n, 3 * n, rng),
+                  W.uniform_theta(n, rng), precision=precision)
+    ctx = qng.Context(p, precision=precision, path=path)
+    g, sig = ctx.metric(ctx.theta0(), want_sigma=True)
+    gr, en = ctx.gradient(ctx.theta0())
+    ctx.sync()
+    ref = oracle.qng_step(p)
+    scale = np.abs(p.hamiltonian.coeffs).sum()  # <E> and its gradient can vanish on these states
+    assert np.abs(g.cpu().numpy().reshape(n, n) - ref["g"]).max() <= TOL[precision] / 4
+    assert np.abs(sig.cpu().numpy() + 2.0 * ref["T"].imag).max() <= TOL[precision]
+    assert np.abs(gr.cpu().numpy() - ref["grad"]).max() <= TOL[precision] * scale
+    assert abs(float(en[0]) - ref["E"]) <= TOL[precision] * scale
