@@ -311,7 +311,11 @@ template <class T> __global__ void __launch_bounds__(kHThreads) k_heff(FWork w, 
     if (m < N && share == 0) {
         const double2 x = amp_of(v[m]);
         e = fma(x.x, hr, x.y * hi);
-        n2 = fma(hr, hr, hi * hi);
+        // |eta| / 2^eexp <= 1 before it is squared (coefficients beyond 1e154 or below 1e-154 would leave float64's
+        // range squared); two factors, as 2^-eexp alone can leave it too
+        const double f0 = scalbn(1.0, -(in.eexp / 2)), f1 = scalbn(1.0, in.eexp / 2 - in.eexp);
+        const double sr = hr * f0 * f1, si = hi * f0 * f1;
+        n2 = fma(sr, sr, si * si);
         E *eta = reinterpret_cast<E *>(w.eta) + in.v_off;
         E h;
         h.x = hr;
@@ -331,7 +335,7 @@ template <class T> __global__ void __launch_bounds__(kHThreads) k_heff(FWork w, 
         unsigned long long *acc = w.eacc + 3 * it.inst;
         atomicAdd(acc, (unsigned long long)__double2ll_rn(scalbn(s, 60 - in.eexp)));
         // rounded up, so that the sum never falls below the true one
-        atomicAdd(acc + 1, (unsigned long long)__double2ll_ru(scalbn(s2, -in.eexp) * scalbn(1.0, 60 - in.eexp)) + 1ull);
+        atomicAdd(acc + 1, (unsigned long long)__double2ll_ru(s2 * 0x1p60) + 1ull);
         __threadfence();
         if (atomicAdd(acc + 2, 1ull) == (unsigned long long)(in.hchunks - 1)) {
             const double en = scalbn((double)(ll)atomicExch(acc, 0ull), in.eexp - 60);
@@ -426,7 +430,7 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
     auto put = [&](int c, int row, double re, double im) {
         if (bad) re = im = __longlong_as_double(0x7ff8000000000000ll);
         if (grad) {
-            w.gradraw[in.param_off + row] = -re * (sizeof(A) == 16 ? scalbn(1.0, w.etaexp[it.inst] - 60) : 1.0);
+            w.gradraw[in.param_off + row] = sizeof(A) == 16 ? -scalbn(re, w.etaexp[it.inst] - 60) : -re;
         } else if (row == P) {
             w.sigma[in.param_off + c] = re * unit;
         } else if (row < c) {
@@ -444,7 +448,7 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
         low = in.end_low;
         const typename T::Eta *eta = reinterpret_cast<const typename T::Eta *>(w.eta) + in.v_off;
         const uint32_t mb = p.base(low);
-        const double up = sizeof(A) == 16 ? scalbn(1.0, 60 - w.etaexp[it.inst]) : 1.0;
+        const SeedScale up(sizeof(A) == 16 ? 60 - w.etaexp[it.inst] : 0);
 #pragma unroll
         for (int k = 0; k < NA; ++k) b[k] = seed(eta[mb | (k << low)], up);
     } else {  // column j of run r starts as K_j Psi_r

@@ -166,10 +166,16 @@ __device__ __forceinline__ void store_factor(float2 *d, longlong2 f) {
 __device__ __forceinline__ double2 amp_of(longlong2 x) { return double2{(double)x.x * 0x1p-60, (double)x.y * 0x1p-60}; }
 __device__ __forceinline__ double2 amp_of(float2 x) { return double2{(double)x.x, (double)x.y}; }
 
-__device__ __forceinline__ longlong2 seed(double2 e, double up) {  // -i eta
-    return longlong2{__double2ll_rn(e.y * up), __double2ll_rn(-e.x * up)};
+// A factor 2^k. Only for Hamiltonians below 1e-280 or so does it take more than one float64 (the same in every thread).
+struct SeedScale {
+    double f, g;
+    __device__ __forceinline__ explicit SeedScale(int k) : f(scalbn(1.0, min(k, 1000))), g(k > 1000 ? scalbn(1.0, k - 1000) : 0.0) {}
+    __device__ __forceinline__ double operator()(double x) const { return g != 0.0 ? x * f * g : x * f; }
+};
+__device__ __forceinline__ longlong2 seed(double2 e, const SeedScale &up) {  // -i eta
+    return longlong2{__double2ll_rn(up(e.y)), __double2ll_rn(-up(e.x))};
 }
-__device__ __forceinline__ float2 seed(float2 e, double) { return float2{e.y, -e.x}; }
+__device__ __forceinline__ float2 seed(float2 e, const SeedScale &) { return float2{e.y, -e.x}; }
 
 template <class T, int KB> struct Sums {  // of the thread's products: all, and signed by each of its bits
     typename T::Acc all, bit[KB];

@@ -164,10 +164,10 @@ __device__ __forceinline__ void scale_down(float2 &, int, uint32_t) {}
 __host__ __device__ constexpr uint32_t salt(int k) { return 0x9e3779b9u * (uint32_t)(2 * k + 1); }
 
 // -i eta, rounded by the dither
-__device__ __forceinline__ longlong2 seed_dithered(double2 e, double up, uint32_t d) {
-    return longlong2{__double2ll_rd(e.y * up + (double)d * 0x1p-32), __double2ll_rd(-e.x * up + (double)(d * 5u) * 0x1p-32)};
+__device__ __forceinline__ longlong2 seed_dithered(double2 e, const SeedScale &up, uint32_t d) {
+    return longlong2{__double2ll_rd(up(e.y) + (double)d * 0x1p-32), __double2ll_rd(-up(e.x) + (double)(d * 5u) * 0x1p-32)};
 }
-__device__ __forceinline__ float2 seed_dithered(float2 e, double, uint32_t) { return float2{e.y, -e.x}; }
+__device__ __forceinline__ float2 seed_dithered(float2 e, const SeedScale &, uint32_t) { return float2{e.y, -e.x}; }
 
 // MIM: both parts of the metric's inner products. FWD: the forward sweep (one vector, checkpoints out).
 template <class T, int MIM, int FWD, int KB, int NT>
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
             set_g();
             if (grad && pass == 0) {
                 const typename T::Eta *eta = reinterpret_cast<const typename T::Eta *>(buf);
-                const double up = sizeof(A) == 16 ? scalbn(1.0, kUnit - *w.etaexp) : 1.0;
+                const SeedScale up(sizeof(A) == 16 ? kUnit - *w.etaexp : 0);
 #pragma unroll
                 for (int k = 0; k < NA; ++k) b[k] = seed_dithered(at(eta, gidx(k)), up, dith(k + 320));
             } else {
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
                     }
                     ll v;
                     if constexpr (sizeof(A) == 16) v = d;
-                    else v = __double2ll_rn(d * scalbn(1.0, kSumUnit - (grad ? *w.etaexp : 0)));
+                    else v = __double2ll_rn(scalbn(d, kSumUnit - (grad ? *w.etaexp : 0)));
                     ll *dst = nullptr;
                     if (q == ipc) dst = part ? nullptr : w.sacc + me.col;
                     else if (grad) dst = w.gacc + row;
@@ -488,6 +488,8 @@ template <> struct Coef<Fix> {
         return (wide(ch, xh) << (32 - S)) + ((m + (1ll << (S - 1))) >> S);
     }
     static __device__ __forceinline__ double value(ll h, int eexp) { return scalbn((double)h, eexp - 61); }
+    // h / 2^eexp: at most 1, so that its square stays in range
+    static __device__ __forceinline__ double scaled(ll h, float) { return (double)h * 0x1p-61; }
 };
 template <> struct Coef<Flt> {
     using C = float;
@@ -495,6 +497,7 @@ template <> struct Coef<Flt> {
     static __device__ __forceinline__ C of(double c, int) { return (float)c; }
     static __device__ __forceinline__ float mul(float c, float x) { return c * x; }
     static __device__ __forceinline__ float value(float h, int) { return h; }
+    static __device__ __forceinline__ float scaled(float h, float fs) { return h * fs; }
 };
 
 __device__ __forceinline__ double2 amp_at(longlong2 x) {
@@ -517,8 +520,8 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
     const A *v = reinterpret_cast<const A *>(w.b) + ((size_t)in << w.n);
     E *eta = reinterpret_cast<E *>(reinterpret_cast<A *>(w.b) + ((size_t)out << w.n));
     const uint64_t N = 1ull << w.n;
-    const int sc = sizeof(S) == 4 ? max(-120, min(120, -w.eexp)) : 0;  // float32 squares stay in range
-    const S fs = (S)scalbnf(1.0f, sc);
+    const int sc = max(-120, min(120, -w.eexp));  // complex64: eta / 2^eexp, within float32's range
+    const float fs = scalbnf(1.0f, sc);
     double e = 0.0, n2 = 0.0;
     for (uint64_t m0 = (uint64_t)blockIdx.x * (256 * NA); m0 < N; m0 += (uint64_t)gridDim.x * (256 * NA)) {
         const uint32_t m = (uint32_t)m0 + threadIdx.x;  // and m + 256, ..
@@ -588,7 +591,7 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
             o.y = hi;
             eta[m + 256 * k] = o;
             e4 += y.x * hr + y.y * hi;
-            const S ar = hr * fs, ai = hi * fs;
+            const S ar = K::scaled(h[k].x, fs), ai = K::scaled(h[k].y, fs);
             n4 += ar * ar + ai * ai;
         }
         e += e4;
@@ -606,9 +609,9 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
         s2 += __shfl_xor_sync(0xffffffffu, s2, o);
     }
     if (threadIdx.x == 0) {
-        s2 = scalbn(s2, -2 * sc);
+        if (sizeof(S) == 4) s2 = scalbn(s2, -2 * (sc + w.eexp));  // of (eta / 2^eexp)^2
         atomicAdd(w.eacc, (unsigned long long)__double2ll_rn(scalbn(s, 60 - w.eexp)));
-        atomicAdd(w.eacc + 1, (unsigned long long)__double2ll_ru(scalbn(s2, -w.eexp) * scalbn(1.0, 60 - w.eexp)) + 1ull);
+        atomicAdd(w.eacc + 1, (unsigned long long)__double2ll_ru(s2 * 0x1p60) + 1ull);
         __threadfence();
         if (atomicAdd(w.eacc + 2, 1ull) == (unsigned long long)(gridDim.x - 1)) {
             const double en = scalbn((double)(ll)atomicExch(w.eacc, 0ull), w.eexp - 60);
@@ -632,7 +635,7 @@ __global__ void k_sfinish(SWork w, int what) {
     }
     if (x < (size_t)w.P) {
         if (what & 1) w.sigma[x] = bad ? nan : unit * (double)w.sacc[x];
-        if (what & 2) w.gradraw[x] = bad ? nan : -(double)w.gacc[x] * scalbn(1.0, *w.etaexp - kSumUnit);
+        if (what & 2) w.gradraw[x] = bad ? nan : -scalbn((double)w.gacc[x], *w.etaexp - kSumUnit);
     }
 }
 
