@@ -49,10 +49,10 @@ __global__ void __launch_bounds__(kHalfThreads) k_half(SWork w, int fix) {
     __shared__ int4 cs[kHalfThreads];
     __shared__ Member mem[kHalfThreads];
     grid_ready();
-    const int r = blockIdx.y;
+    const int r = blockIdx.x;
     const Run &rn = w.run[r];
     const uint32_t nlo = 1u << w.hl, nhi = 1u << (w.n - w.hl);
-    const uint32_t e = blockIdx.x * kHalfThreads + threadIdx.x;
+    const uint32_t e = blockIdx.y * kHalfThreads + threadIdx.x;
     const bool lo = e < nlo;
     const bool on = e < nlo + nhi;
     const uint32_t own = lo ? nlo - 1u : ~(nlo - 1u);       // this half's bits
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_half(SWork w, int fix) {
                 double s, c;
                 if (!isfinite(th)) { *w.bad = 1; atomicCAS(w.status, 0, (int)QNG_ERR_ARG); }
                 sincos(0.5 * th, &s, &c);
-                if (blockIdx.x == 0) w.pctrl[x.param] = 1.0;
+                if (blockIdx.y == 0) w.pctrl[x.param] = 1.0;
                 ll y = __double2ll_rn((x.sgn > 0 ? -s : s) * 0x1p62);
                 if ((int)y == INT32_MIN) ++y;
                 cs[threadIdx.x] = pack(longlong2{__double2ll_rn(c * 0x1p62), y});
@@ -665,7 +665,7 @@ cudaError_t launch_stream_tables(const SWork &w, int precision, cudaStream_t st)
     cudaError_t e = cudaMemsetAsync(w.bad, 0, sizeof(int32_t), st);
     if (e != cudaSuccess || w.R == 0) return e;
     const unsigned n = (1u << w.hl) + (1u << (w.n - w.hl));
-    return launch_next(false, k_half, dim3((n + kHalfThreads - 1) / kHalfThreads, w.R), kHalfThreads, 0, 1, st, w,
+    return launch_next(false, k_half, dim3(w.R, (n + kHalfThreads - 1) / kHalfThreads), kHalfThreads, 0, 1, st, w,
                        (int)(precision == QNG_C128));
 }
 

@@ -26,6 +26,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -1304,10 +1305,10 @@ __device__ __forceinline__ void column_item(const Work &w, const DevWork wk, int
 // and T_k = -(i/2) sigma_k; Im G = Im L (T_i^* T_j is real). One CTA per 32 x 32 tile of the upper triangle:
 // L is read along its rows and both g tiles are written along theirs (one CTA per instance, reading the
 // lower half down the columns, took 58 us for P = 99 against 7 us here).
-__global__ void __launch_bounds__(256) k_assemble(Work w, LaunchArgs a) {
+__global__ void __launch_bounds__(256) k_assemble(Work w, LaunchArgs a, int tiles) {
     __shared__ double tr[32][33], ti[32][33];
     grid_ready();
-    const int b = blockIdx.x, tile = blockIdx.y;  // instances along x, which has no 16-bit limit
+    const int b = blockIdx.x / tiles, tile = blockIdx.x % tiles;  // all along x: y ends at 65535, 361 x 361 tiles
     const DevInst &in = w.inst[b];
     const int P = in.P, T = (P + 31) / 32;
     const double *sg = w.sigma + in.param_off;
@@ -1885,7 +1886,7 @@ cudaError_t launch_solve(const Work &w, int count, int max_P, int cl, const Laun
 cudaError_t launch_finish(const Work &w, int count, int max_P, const LaunchArgs &a, cudaStream_t st) {
     if (!(a.jobs & kJobSolve)) {
         const int T = (max_P + 31) / 32, tiles = (a.jobs & kJobMetric) ? T * (T + 1) / 2 : 1;
-        return launch_next(a.chain, k_assemble, dim3(count, tiles > 0 ? tiles : 1), 256, 0, 1, st, w, a);
+        return launch_next(a.chain, k_assemble, (unsigned)(count * std::max(tiles, 1)), 256, 0, 1, st, w, a, std::max(tiles, 1));
     }
     if (max_P < kSmallP) return launch_next(a.chain, k_small, count, 128, 0, 1, st, w, a);
     k_finish<<<count, max_P >= 128 ? 512 : 128, 0, st>>>(w, a);

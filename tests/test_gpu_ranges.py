@@ -1,4 +1,5 @@
-"""Inputs at the ends of what the entry points take: Hamiltonian coefficients near the ends of float64's range."""
+"""Inputs at the ends of what the entry points take: Hamiltonian coefficients near the ends of float64's range, more
+parameters than a launch grid's y dimension has tiles of the metric, more runs than it has blocks."""
 import numpy as np
 import pytest
 import torch
@@ -36,3 +37,42 @@ def test_hamiltonian_scale(qng, n, path, scale):
         out.append((grad.cpu().numpy() / s, float(energy[0]) / s))
     assert np.abs(out[1][0] - out[0][0]).max() <= 1e-12 * np.abs(out[0][0]).max()
     assert abs(out[1][1] - out[0][1]) <= 1e-12 * np.abs(h.coeffs).sum()
+
+
+def test_metric_of_many_parameters(qng):
+    """P = 11 617 on 17 qubits, an RY on each and then RZ on one after the other: 66 066 tiles of the metric. RY
+    entries are 1/4 on the diagonal, RZ ones <Z_a Z_b> - <Z_a><Z_b> over 4 (a product state: sin^2 / 4 on one
+    qubit), and the real part of <Y_a Z_b> vanishes."""
+    n, P = 17, 11617
+    rows = [[W.RY, q, -1, q] for q in range(n)] + [[W.RZ, k % n, -1, k] for k in range(n, P)]
+    rng = np.random.Generator(np.random.PCG64(5))
+    theta = W.uniform_theta(P, rng)
+    p = W.Problem("many", W.Circuit(n, np.array(rows, dtype=np.int32)), W.tfim_chain(n, 1.0, 0.5), theta, precision=W.C64)
+    ctx = qng.Context(p)
+    g = ctx.metric(ctx.theta0()).view(P, P)
+    ctx.sync()
+    q = torch.arange(n, P, device=g.device) % n
+    s2 = 0.25 * torch.sin(torch.as_tensor(theta[:n], device=g.device)) ** 2
+    ref = torch.zeros_like(g)
+    ref[:n, :n] = 0.25 * torch.eye(n, dtype=g.dtype, device=g.device)
+    ref[n:, n:] = torch.where(q[:, None] == q[None, :], s2[q][:, None], torch.zeros((), dtype=g.dtype, device=g.device))
+    assert float((g - ref).abs().max()) <= 1e-6
+
+
+def test_streaming_many_runs(qng):
+    """70 000 runs (a CZ between Hadamards each) on the streaming path, against the on-chip path's <E>."""
+    n, runs = 13, 70000
+    rows = [[W.RY, q, -1, q] for q in range(n)]
+    for k in range(runs):
+        rows += [[W.H, 0, -1, -1], [W.CZ, 0, 1 + k % (n - 1), -1]]
+    rng = np.random.Generator(np.random.PCG64(6))
+    p = W.Problem("runs", W.Circuit(n, np.array(rows, dtype=np.int32)), W.random_pauli_hamiltonian(n, 10, rng),
+                  W.uniform_theta(n, rng), precision=W.C64)
+    e = []
+    for path in (1, 2):
+        ctx = qng.Context(p, path=path)
+        v = ctx.energy(ctx.theta0())
+        ctx.sync()
+        e.append(float(v[0]))
+        ctx.close()
+    assert abs(e[0] - e[1]) <= 2e-4 * np.abs(p.hamiltonian.coeffs).sum()
