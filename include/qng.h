@@ -139,10 +139,16 @@ qng_status qng_get_sizes(const qng_ctx *ctx, int32_t *count, int64_t *total_para
  * Either pointer may be NULL. */
 qng_status qng_get_offsets(const qng_ctx *ctx, int64_t *param_offset, int64_t *metric_offset);
 
-/* Bytes of device workspace the context needs (a multiple of 256). */
+/* Bytes of device workspace the context runs fastest with (a multiple of 256). */
 qng_status qng_workspace_size(const qng_ctx *ctx, size_t *bytes);
 
-/* Hand the context a device workspace (256-byte aligned, >= qng_workspace_size bytes, owned by
+/* The least workspace qng_set_workspace takes (a multiple of 256, at most qng_workspace_size). With less than
+ * qng_workspace_size the gate-by-gate kernels run, which keep no checkpoint per run: four vectors of
+ * 2^n amplitudes for a streaming instance (Algorithm 1's O(1) registers), however long its circuit; the
+ * results differ by rounding. */
+qng_status qng_workspace_min(const qng_ctx *ctx, size_t *bytes);
+
+/* Hand the context a device workspace (256-byte aligned, >= qng_workspace_min bytes, owned by
  * the caller and kept alive while the context uses it) and the CUDA stream (cudaStream_t, may be
  * NULL for the legacy default stream) every later call is ordered on. Uploads the circuit tables
  * into the workspace with asynchronous copies on that stream. */
@@ -263,8 +269,10 @@ qng_status qng_set_tuning(qng_ctx *ctx, int min_qubits, int cluster_log2, int th
  * slots as fill 32 MiB (at least 4), vectors of 2^n amplitudes, and every pass takes one run for
  * several columns. Vectors beyond 4 GiB, instances whose checkpoints and slots would pass 96 GiB,
  * and n < 13 (complex64) or n < 12 (complex128) run on four registers instead: psi, a and b of
- * Algorithm 1 and a second b, the metric columns walking in pairs that share a. A change re-plans the context; if the workspace already set is then too small the call returns
- * QNG_ERR_WORKSPACE and keeps the old path (query qng_workspace_size before setting a workspace). */
+ * Algorithm 1 and a second b, the metric columns walking in pairs that share a; so do contexts whose
+ * workspace is smaller than qng_workspace_size. A change re-plans the context; if the workspace already set is
+ * below qng_workspace_min for it the call returns QNG_ERR_WORKSPACE and keeps the old path (query the sizes
+ * before setting a workspace). */
 qng_status qng_set_path(qng_ctx *ctx, int path);
 
 /* Streaming path only: HBM bytes one qng_step moves through the pass schedule (vectors loaded and

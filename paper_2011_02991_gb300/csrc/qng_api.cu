@@ -118,6 +118,8 @@ struct qng_ctx {
     size_t o_coef = 0, o_sigma = 0, o_scale = 0, o_L = 0, o_grad = 0, o_energy = 0, o_chol = 0, o_ckpt = 0, o_eta = 0;
     size_t o_io_theta = 0, o_io_dtheta = 0, o_io_g = 0, o_io_grad = 0, o_io_energy = 0;
     size_t ws_bytes = 0;      // bytes the current plan needs
+    size_t ws_want = 0;       // bytes that the plan without a workspace limit needs
+    bool compact = false;     // planned without checkpoints of runs: the workspace is smaller than ws_want
     size_t ws_cap = 0;        // bytes of the workspace the caller set
     unsigned char *ws = nullptr;
     cudaStream_t stream = nullptr;
@@ -354,7 +356,7 @@ int energy_exponent(const std::vector<qng_pauli> &terms) {
     return ex;
 }
 
-constexpr int64_t kStreamFramesMax = 96ll << 30;  // bytes of checkpoints and columns at most
+constexpr int64_t kFramesMax = 96ll << 30;  // bytes of checkpoints, tables and columns at most
 
 // Plan of the diagonal-frame passes; false when the vector is smaller than a tile or the checkpoints
 // (one vector per run) take more memory than they are worth.
@@ -374,7 +376,7 @@ bool plan_sframes(qng_ctx *c) {
     // column slots: what a launch walks together. Up to 20 qubits 32 MiB of them (enough CTAs, and L2 holds
     // them between passes), beyond that four, which share each checkpoint read
     c->sslots = h.n <= 20 ? (int)std::max<int64_t>(2, std::min<int64_t>(32, (32ll << 20) / reg)) : 4;
-    if ((R + c->sslots) * reg > kStreamFramesMax) return false;
+    if ((R + c->sslots) * reg > kFramesMax) return false;
     c->seexp = energy_exponent(h.terms);
     c->scol.clear();
     if (h.P > 0) c->scol.push_back(frames::SCol{h.P, R});
@@ -391,7 +393,7 @@ qng_status plan_streaming(qng_ctx *c, int64_t scale_n) {
     const HostInst &h = c->inst[0];
     const size_t ab = amp_bytes(c->precision);
     c->sched = large::Schedule();
-    c->sframes = plan_sframes(c);
+    c->sframes = !c->compact && plan_sframes(c);
     if (!c->sframes) {
         large::build_schedule(h.gates, h.n, h.P, c->precision, c->sched, c->col_want.empty() ? nullptr : &c->col_want);
         const int64_t ntiles = 1ll << (h.n - c->sched.t);
@@ -487,7 +489,6 @@ int frames_cl(const qng_ctx *c, int n, int kb) {
 // memory does not fit (then the gate-by-gate kernels run).
 bool plan_frames(qng_ctx *c) {
     auto &f = c->f;
-    f = {};
     const size_t ab = amp_bytes(c->precision);
     std::vector<frames::Program> prog(c->count);
     std::vector<std::array<int, 2>> key(c->count);
@@ -606,7 +607,7 @@ bool plan_frames(qng_ctx *c) {
         fits = fits && cl.smem_col_im <= kMaxSmem && cl.smem_fwd <= kMaxSmem;
         f.cls.push_back(cl);
     }
-    return fits;
+    return fits && 2 * (f.amps_ad + f.amps_v) * (int64_t)ab <= kFramesMax;
 }
 
 // The default shapes of every qubit count of the context (no qng_set_tuning, qng_set_shape,
@@ -619,7 +620,7 @@ bool default_shapes(const qng_ctx *c) {
 }
 
 // Build the device-table images, the launch groups and the workspace layout.
-qng_status plan(qng_ctx *c) {
+qng_status plan_as(qng_ctx *c) {
     c->t_inst.clear(); c->t_param.clear(); c->t_gen.clear(); c->t_fixed.clear(); c->t_diag.clear(); c->t_term.clear();
     c->t_work.clear(); c->t_group_inst.clear(); c->groups.clear();
     c->frames = c->sframes = false;  // decided below, for this plan's path
@@ -815,7 +816,8 @@ qng_status plan(qng_ctx *c) {
 
     // The diagonal-frame kernels run at the default shapes; qng_set_shape and the like choose the
     // gate-by-gate kernels. The workspace has room for either.
-    const bool frames_fit = plan_frames(c);
+    c->f = {};
+    const bool frames_fit = !c->compact && plan_frames(c);
     c->frames = frames_fit && default_shapes(c);
 
     // workspace layout
@@ -886,6 +888,19 @@ int solve_cluster_log2(int max_P) {
     for (int cl = 3; cl >= 0; --cl)
         if (solve_smem_bytes(max_P, cl) <= 200 * 1024) return cl;
     return -1;
+}
+
+// The plan, and, where a workspace is set that its checkpoints of runs do not fit, the plan of the gate-by-gate
+// kernels: four registers of a streaming instance, one checkpoint per parameter on chip.
+qng_status plan(qng_ctx *c) {
+    c->compact = false;
+    qng_status s = plan_as(c);
+    c->ws_want = c->ws_bytes;
+    if (s == QNG_OK && c->ws && c->ws_bytes > c->ws_cap) {
+        c->compact = true;
+        s = plan_as(c);
+    }
+    return s;
 }
 
 qng_status cuda_status(cudaError_t e) {
@@ -1611,15 +1626,50 @@ qng_status qng_get_offsets(const qng_ctx *c, int64_t *param_offset, int64_t *met
 
 qng_status qng_workspace_size(const qng_ctx *c, size_t *bytes) {
     if (!c || !bytes) return QNG_ERR_ARG;
-    *bytes = c->ws_bytes;
+    *bytes = c->ws_want;
     return QNG_OK;
+}
+
+qng_status qng_workspace_min(const qng_ctx *c, size_t *bytes) {
+    if (!c || !bytes) return QNG_ERR_ARG;
+    *bytes = c->ws_bytes;
+    if (c->compact) return QNG_OK;
+    qng_ctx t;  // the settings alone, planned without checkpoints of runs
+    t.precision = c->precision;
+    t.count = c->count;
+    t.inst = c->inst;
+    t.path = c->path;
+    t.col_want = c->col_want;
+    t.tune_min_qubits = c->tune_min_qubits;
+    t.tune_cl = c->tune_cl;
+    t.tune_threads = c->tune_threads;
+    std::copy(c->tuned_cl, c->tuned_cl + kMaxQubits + 1, t.tuned_cl);
+    std::copy(c->tuned_threads, c->tuned_threads + kMaxQubits + 1, t.tuned_threads);
+    std::copy(c->tuned_fwd, c->tuned_fwd + kMaxQubits + 1, t.tuned_fwd);
+    std::copy(c->tuned_fcl, c->tuned_fcl + kMaxQubits + 1, t.tuned_fcl);
+    t.compact = true;
+    const qng_status s = plan_as(&t);
+    if (s == QNG_OK) *bytes = std::min(t.ws_bytes, c->ws_bytes);
+    return s;
 }
 
 qng_status qng_set_workspace(qng_ctx *c, void *workspace, size_t bytes, void *stream) {
     if (!c) return QNG_ERR_ARG;
-    if (!workspace || bytes < c->ws_bytes || (reinterpret_cast<uintptr_t>(workspace) & 255)) return QNG_ERR_WORKSPACE;
+    if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255)) return QNG_ERR_WORKSPACE;
+    unsigned char *const old_ws = c->ws;
+    const size_t old_cap = c->ws_cap;
     c->ws = static_cast<unsigned char *>(workspace);
     c->ws_cap = bytes;
+    if (bytes < c->ws_bytes || c->compact) {  // another size may choose another plan
+        const qng_status s = plan(c);
+        if (s != QNG_OK || c->ws_bytes > bytes) {
+            c->ws = old_ws;
+            c->ws_cap = old_cap;
+            plan(c);
+            if (c->ws) upload(c);
+            return s != QNG_OK ? s : QNG_ERR_WORKSPACE;
+        }
+    }
     c->stream = static_cast<cudaStream_t>(stream);
     return upload(c);
 }

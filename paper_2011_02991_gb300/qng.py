@@ -57,6 +57,7 @@ SYMBOLS = {
     "qng_get_sizes": [_vp, _i32p, _i64p, _i64p],
     "qng_get_offsets": [_vp, _i64p, _i64p],
     "qng_workspace_size": [_vp, ctypes.POINTER(ctypes.c_size_t)],
+    "qng_workspace_min": [_vp, ctypes.POINTER(ctypes.c_size_t)],
     "qng_set_workspace": [_vp, _vp, ctypes.c_size_t, _vp],
     "qng_set_stream": [_vp, _vp],
     "qng_metric": [_vp, _vp, _vp, _vp],
@@ -162,10 +163,13 @@ class Context:
 
     ``problems`` is a Problem or a list of Problems (a batch). theta and the per-parameter outputs
     are concatenated over instances; metrics are concatenated P_b x P_b blocks.
+
+    The workspace is what the context runs fastest with; where the device has no room for that, or it is more
+    than ``workspace_limit`` bytes, the least one (qng_workspace_min), on which the gate-by-gate kernels run.
     """
 
     def __init__(self, problems, precision: int | None = None, device=None, stream: torch.cuda.Stream | None = None,
-                 path: int = 0):
+                 path: int = 0, workspace_limit: int | None = None):
         L = load()
         if not torch.cuda.is_available():
             raise RuntimeError("libqng needs a CUDA device")
@@ -212,6 +216,7 @@ class Context:
         _chk(L.qng_get_offsets(self._h, po.ctypes.data_as(_i64p), mo.ctypes.data_as(_i64p)), "qng_get_offsets")
         self.param_offsets, self.metric_offsets = po, mo
         self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
+        self.workspace_limit = workspace_limit
         if path:
             _chk(L.qng_set_path(self._h, int(path)), "qng_set_path")
         self._alloc_workspace()
@@ -220,7 +225,16 @@ class Context:
         L = load()
         nb = ctypes.c_size_t()
         _chk(L.qng_workspace_size(self._h, ctypes.byref(nb)), "qng_workspace_size")
-        self.workspace = torch.empty(max(int(nb.value), 256), dtype=torch.uint8, device=self.device)
+        want, limit = max(int(nb.value), 256), self.workspace_limit
+        self.workspace = None
+        if limit is None or want <= limit:
+            try:
+                self.workspace = torch.empty(want, dtype=torch.uint8, device=self.device)
+            except torch.cuda.OutOfMemoryError:
+                pass
+        if self.workspace is None:
+            _chk(L.qng_workspace_min(self._h, ctypes.byref(nb)), "qng_workspace_min")
+            self.workspace = torch.empty(max(int(nb.value), 256), dtype=torch.uint8, device=self.device)
         _chk(L.qng_set_workspace(self._h, _ptr(self.workspace), self.workspace.numel(),
                                  ctypes.c_void_p(self.stream.cuda_stream)), "qng_set_workspace")
 
@@ -368,12 +382,18 @@ class Context:
             self._alloc_workspace_for_new_plan(path)
             return
         _chk(st, "qng_set_path")
+        nb = ctypes.c_size_t()
+        _chk(L.qng_workspace_size(self._h, ctypes.byref(nb)), "qng_workspace_size")
+        # a smaller workspace runs it gate by gate: the new path's own size where that is allowed
+        if nb.value > self.workspace.numel() and (self.workspace_limit is None or nb.value <= self.workspace_limit):
+            self._alloc_workspace_for_new_plan(path)
 
     def _alloc_workspace_for_new_plan(self, path: int):
         # release the workspace binding, re-plan without one, then allocate the new size
         L = load()
         self.close()
-        self.__init__(self.problems, self.precision, self.device, self.stream, path=path)
+        self.__init__(self.problems, self.precision, self.device, self.stream, path=path,
+                      workspace_limit=self.workspace_limit)
 
     def set_tuning(self, min_qubits: int, cluster_log2: int, threads: int):
         _chk(load().qng_set_tuning(self._h, min_qubits, cluster_log2, threads), "qng_set_tuning")

@@ -164,6 +164,29 @@ def test_streaming_workspace(lib):
                                 W.C128, ctypes.byref(h)) == 7
 
 
+@pytest.mark.parametrize("n,layers,precision", [(28, 3, W.C64), (20, 2, W.C128), (14, 2, W.C64)])
+def test_least_workspace(lib, n, layers, precision):
+    """Four registers are enough for a streaming instance, however many runs its circuit has, and what holds an
+    on-chip one gate by gate; anything below is refused."""
+    c = W.layered_ansatz(n, layers, (W.RY, W.RX, W.RZ), W.CNOT)
+    st, h = _create(lib, n, [tuple(int(v) for v in r) for r in c.gates], [(1.0, 1, 0)], precision)
+    assert st == 0
+    nb, least = ctypes.c_size_t(), ctypes.c_size_t()
+    amp = 8 if precision == W.C64 else 16
+    for path in (0, 2):
+        assert lib.qng_set_path(h, path) == 0
+        assert lib.qng_workspace_size(h, ctypes.byref(nb)) == 0
+        assert lib.qng_workspace_min(h, ctypes.byref(least)) == 0
+        assert least.value <= nb.value and least.value % 256 == 0
+        if n > 16 or path == 2:
+            regs = 4 * (amp << n)
+            assert regs <= least.value < regs + 64 * 1024 * 1024 and least.value < nb.value
+        assert lib.qng_set_workspace(h, ctypes.c_void_p(0x1000), least.value - 256, None) == 6
+        again = ctypes.c_size_t()
+        assert lib.qng_workspace_size(h, ctypes.byref(again)) == 0 and again.value == nb.value
+    lib.qng_destroy(h)
+
+
 def test_status_strings(lib):
     for s in range(8):
         assert lib.qng_status_string(s)

@@ -31,8 +31,8 @@ def qng():
     return Q
 
 
-def run_streaming(qng, oracle, p, precision):
-    ctx = qng.Context(p, precision=precision, path=2)
+def run_streaming(qng, oracle, p, precision, limit=None):
+    ctx = qng.Context(p, precision=precision, path=2, workspace_limit=limit)
     out = ctx.step(ctx.theta0(), p.dt, p.lam)
     g2, sig = ctx.metric(ctx.theta0(), want_sigma=True)
     gr, en = ctx.gradient(ctx.theta0())
@@ -225,3 +225,73 @@ def test_long_transitions(qng, oracle, n, path, precision):
     assert np.abs(sig.cpu().numpy() + 2.0 * ref["T"].imag).max() <= TOL[precision]
     assert np.abs(gr.cpu().numpy() - ref["grad"]).max() <= TOL[precision] * scale
     assert abs(float(en[0]) - ref["E"]) <= TOL[precision] * scale
+
+
+LEAST = 1  # a workspace limit that leaves the four registers
+
+
+@pytest.mark.parametrize("precision", [W.C128, W.C64])
+@pytest.mark.parametrize("n,seed", [(13, 3), (15, 4), (17, 6)])
+def test_register_form_random_circuits(qng, oracle, n, seed, precision):
+    """The least workspace: registers instead of checkpoints, the gate-by-gate passes over 2 to 64 tiles (the
+    register-phase kernel in complex64). Every gate kind."""
+    p = W.random_problem(n, 50 + 4 * n, 10, 3000 + seed, precision)
+    run_streaming(qng, oracle, p, precision, LEAST)
+
+
+@pytest.mark.parametrize("precision", [W.C128, W.C64])
+@pytest.mark.parametrize("kinds,ent", [((W.RY, W.RZ), W.CZ), ((W.RY, W.RX, W.RZ), W.CNOT)])
+def test_register_form_layered_14(qng, oracle, kinds, ent, precision):
+    rng = np.random.Generator(np.random.PCG64(78))
+    c = W.layered_ansatz(14, 2, kinds, ent)
+    p = W.Problem("layered14", c, W.random_pauli_hamiltonian(14, 20, rng), W.uniform_theta(c.num_params, rng),
+                  precision=precision)
+    run_streaming(qng, oracle, p, precision, LEAST)
+
+
+def test_register_form_c64_diagonal_runs(qng, oracle):
+    """Runs of 1-24 RZ steps over four tiles: inner products on a run's starting registers, one composed
+    factor per amplitude; real step and complex metric."""
+    p = W.z_run_problem(14, 160, 22, W.C64)
+    run_streaming(qng, oracle, p, W.C64, LEAST)
+    ctx = qng.Context(p, precision=W.C64, path=2, workspace_limit=LEAST)
+    G = ctx.metric_complex(ctx.theta0()).reshape(p.P, p.P).cpu().numpy()
+    ctx.sync()
+    ref = oracle.qng_step(p)["G"]
+    assert float(np.abs(G - ref).max() / np.abs(ref).max()) <= TOL[W.C64]
+    assert np.all(G.imag == -G.imag.T)
+
+
+@pytest.mark.parametrize("n,precision", [(18, W.C64), (14, W.C128), (6, W.C128)])
+def test_workspace_limit(qng, n, precision):
+    """A context takes what it is given: the full workspace, the least one, and a larger one after that; all
+    agree, the first and the last to the bit. A path change keeps the limit."""
+    rng = np.random.Generator(np.random.PCG64(n))
+    c = W.layered_ansatz(n, 2, (W.RY, W.RZ), W.CZ)
+    p = W.Problem("limit", c, W.random_pauli_hamiltonian(n, 8, rng), W.uniform_theta(c.num_params, rng), precision=precision)
+    path = 2 if n > 12 else 1
+    full, least = qng.Context(p, path=path), qng.Context(p, path=path, workspace_limit=LEAST)
+    assert least.workspace.numel() <= full.workspace.numel()
+    if path == 2:
+        assert least.workspace.numel() < full.workspace.numel()
+    out = []
+    for ctx in (full, least):
+        g = ctx.metric(ctx.theta0())
+        gr, en = ctx.gradient(ctx.theta0())
+        ctx.sync()
+        out.append((g.clone(), gr.clone(), en.clone()))
+    least.workspace_limit = None
+    least._alloc_workspace()
+    assert least.workspace.numel() == full.workspace.numel()
+    g = least.metric(least.theta0())
+    gr, en = least.gradient(least.theta0())
+    least.sync()
+    for a, b, c2 in zip(out[0], out[1], (g, gr, en)):
+        assert rel(b.cpu(), a.cpu()) <= (1e-11 if precision == W.C128 else TOL[precision])
+        assert torch.equal(a, c2)
+    if n <= 16:
+        least.workspace_limit = LEAST
+        least.set_path(3 - path)
+        g = least.metric(least.theta0())
+        least.sync()
+        assert rel(g.cpu(), out[0][0].cpu()) <= 1e-11
