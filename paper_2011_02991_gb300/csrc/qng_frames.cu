@@ -135,7 +135,7 @@ template <class T> __global__ void __launch_bounds__(kTabThreads) k_tables(FWork
     const uint32_t base = ((t >> low) << (low + kb)) | (t & ((1u << low) - 1u)) | (kq << low);
     const uint32_t own = (uint32_t)(kTabAmps - 1) << low;
     const int half = rn.khalf;
-    longlong2 com = {__double2ll_rn(((half & 1) ? 0.70710678118654752440 : 1.0) * exp2((double)(61 - (half >> 1)))), 0};
+    longlong2 com = {root_half(half), 0};
     longlong2 f[kTabAmps];
     bool any_own = false;  // uniform over the block
     if (threadIdx.x == 0) any_bad = 0;
@@ -159,9 +159,7 @@ template <class T> __global__ void __launch_bounds__(kTabThreads) k_tables(FWork
                         if (!isfinite(th)) { any_bad = 1; atomicCAS(w.status, 0, (int)QNG_ERR_ARG); }
                         sincos(0.5 * th, &s, &c);
                         if (it.first == 0) w.pctrl[in.param_off + e.param] = 1.0;  // controlled ones: their column
-                        ll y = __double2ll_rn((e.sgn > 0 ? -s : s) * 0x1p62);  // c - i lam s
-                        if ((int)y == INT32_MIN) ++y;
-                        cs[threadIdx.x] = pack(longlong2{__double2ll_rn(c * 0x1p62), y});
+                        cs[threadIdx.x] = rotation_pair(c, e.sgn > 0 ? -s : s);  // c - i lam s
                     }
                 }
                 __syncthreads();

@@ -153,6 +153,37 @@ template <class T, int KB> __device__ __forceinline__ void hadamards(typename T:
     }
 }
 
+// 2^(-half / 2), 2^61 = 1: sqrt(1/2) to all of its bits. The float64 one is 1.4e-16 of its square short, and as
+// every transition with an odd number of Hadamards multiplies by it, the norm drifted by that much each time (11 qubits,
+// 21 such transitions: <E> 2.5e-15 off, 0.6e-15 now).
+__host__ __device__ __forceinline__ ll root_half(int half) {
+    const ll r = (half & 1) ? 1630477228166597777ll : 1ll << 61;
+    const int s = half >> 1;
+    return s ? (r + (1ll << (s - 1))) >> s : r;
+}
+
+// (c, s) of a rotation, 2^62 = 1, brought to c^2 + s^2 = 1: float64 rounds each of them at 2^-54, which leaves the
+// norm of every rotation off by about 1e-16, and a circuit's by the sum of that.
+__host__ __device__ __forceinline__ longlong2 unit_pair(ll c, ll s) {
+#ifdef __CUDA_ARCH__
+    const unsigned long long ch = __umul64hi(c < 0 ? -c : c, c < 0 ? -c : c), sh = __umul64hi(s < 0 ? -s : s, s < 0 ? -s : s);
+#else
+    const unsigned long long ch = (unsigned long long)(((__int128)c * c) >> 64), sh = (unsigned long long)(((__int128)s * s) >> 64);
+#endif
+    const unsigned long long cl = (unsigned long long)c * (unsigned long long)c, sl = (unsigned long long)s * (unsigned long long)s;
+    const unsigned long long lo = cl + sl, hi = ch + sh + (lo < cl);  // c^2 + s^2, 2^124 = 1
+    // e = 1 - c^2 - s^2, 2^62 = 1; c (1 + e / 2)
+    const ll e = (ll)((((1ull << 60) - hi - (lo != 0)) << 2) | ((0ull - lo) >> 62));
+    return longlong2{c + (((c >> 20) * e + (1ll << 42)) >> 43), s + (((s >> 20) * e + (1ll << 42)) >> 43)};
+}
+
+// (cos, lam sin) of theta / 2 as the factor tables multiply by it, 2^62 = 1; sin's low half is negated there: off -2^31
+__device__ __forceinline__ int4 rotation_pair(double c, double s) {
+    longlong2 p = unit_pair(__double2ll_rn(c * 0x1p62), __double2ll_rn(s * 0x1p62));
+    if ((int)p.y == INT32_MIN) ++p.y;
+    return pack(p);
+}
+
 __device__ __forceinline__ void store_factor(int4 *d, longlong2 f) {
     ll y = f.y << 1;
     // the low half of the sine is negated by the product: keep it off -2^31

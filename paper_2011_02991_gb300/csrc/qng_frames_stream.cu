@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_half(SWork w, int fix) {
     const int mem_count = rn.mem_count, mem_begin = rn.mem_begin;
     const int half = rn.khalf;
     longlong2 f = {1ll << 61, 0};
-    if (lo) f.x = __double2ll_rn(((half & 1) ? 0.70710678118654752440 : 1.0) * exp2((double)(61 - (half >> 1))));
+    if (lo) f.x = root_half(half);
     uint32_t mask = 0;
     for (int e0 = 0; e0 < mem_count; e0 += kHalfThreads) {
         __syncthreads();
@@ -73,9 +73,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_half(SWork w, int fix) {
                 if (!isfinite(th)) { *w.bad = 1; atomicCAS(w.status, 0, (int)QNG_ERR_ARG); }
                 sincos(0.5 * th, &s, &c);
                 if (blockIdx.y == 0) w.pctrl[x.param] = 1.0;
-                ll y = __double2ll_rn((x.sgn > 0 ? -s : s) * 0x1p62);
-                if ((int)y == INT32_MIN) ++y;
-                cs[threadIdx.x] = pack(longlong2{__double2ll_rn(c * 0x1p62), y});
+                cs[threadIdx.x] = rotation_pair(c, x.sgn > 0 ? -s : s);
             }
         }
         __syncthreads();

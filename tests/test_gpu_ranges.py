@@ -76,3 +76,17 @@ def test_streaming_many_runs(qng):
         e.append(float(v[0]))
         ctx.close()
     assert abs(e[0] - e[1]) <= 2e-4 * np.abs(p.hamiltonian.coeffs).sum()
+
+
+@pytest.mark.parametrize("n,path", [(9, 1), (13, 2)])
+def test_norm_is_kept(qng, n, path):
+    """H = 1: <E> is the state's squared norm after 80 layers, 80 n rotations and as many transitions with an odd
+    number of Hadamards. Factors are unitary to 2^-61 each, so what is left is the float64 sum of <E>."""
+    c = W.layered_ansatz(n, 40)
+    zero = np.zeros(1, dtype=np.uint64)
+    rng = np.random.Generator(np.random.PCG64(n))
+    p = W.Problem("norm", c, W.Hamiltonian(np.ones(1), zero, zero), W.uniform_theta(c.num_params, rng), precision=W.C128)
+    ctx = qng.Context(p, path=path)
+    e = ctx.energy(ctx.theta0())
+    ctx.sync()
+    assert abs(float(e[0]) - 1.0) <= 2e-15
