@@ -347,12 +347,16 @@ template <class T> __global__ void __launch_bounds__(kHThreads) k_heff(FWork w, 
 
 // ------------------------------------------------------------------------------------------
 // Column walk. MIM = 1: metric columns take Im L_ij as well.
+// Inner products are sums of 2^-62 (vectors: 2^-60); each product is rounded by pseudo-random bits, as rounding to
+// nearest is the same for the equal amplitudes of a structured state and adds up over them.
+constexpr int kSumUp = 1;
+
 // One run of the walk: products with the checkpoint, then (mult) the run's adjoint factors. scratch
 // (runs that are not simple): the products go to shared memory, stride apart.
 template <class T, int KB, int MIM>
 __device__ __forceinline__ void run_step(typename T::A (&b)[1 << KB], const typename T::S *a, const typename T::S *d,
                                          uint32_t TC, bool mult, Sums<T, KB> &sr, Sums<T, KB> &si, typename T::A *scratch,
-                                         int stride) {
+                                         int stride, uint32_t h0) {
     constexpr int B = 4;  // loads in flight
     sr.all = si.all = 0;
 #pragma unroll
@@ -367,8 +371,8 @@ __device__ __forceinline__ void run_step(typename T::A (&b)[1 << KB], const type
         }
 #pragma unroll
         for (int k = 0; k < B; ++k) {
-            const typename T::Acc p = prod<0>(av[k], b[k0 + k]);
-            const typename T::Acc q = MIM ? prod<1>(av[k], b[k0 + k]) : typename T::Acc(0);
+            const typename T::Acc p = prod<0, kSumUp>(av[k], b[k0 + k], h0 ^ salt(k0 + k));
+            const typename T::Acc q = MIM ? prod<1, kSumUp>(av[k], b[k0 + k], h0 ^ salt(64 + k0 + k)) : typename T::Acc(0);
             if (scratch) scratch[(k0 + k) * stride] = typename T::A{p, q};
             sr.all += p;
             if (MIM) si.all += q;
@@ -409,7 +413,8 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
     const bool grad = it.ncol == 0;
     const bool live = grad ? sl == 0 : sl < it.ncol;
     const int col = grad ? P : (live ? w.cols[it.list + sl] : -1);
-    const double unit = sizeof(A) == 16 ? 0x1p-60 : 1.0;
+    const double unit = sizeof(A) == 16 ? 0x1p-62 : 1.0;
+    const uint32_t h0 = sizeof(A) == 16 ? hash(p.t) : 0u;
 
     // the walk's tables in shared memory: steps, runs and parameters (a table read per run would wait on
     // L2 each time)
@@ -428,7 +433,7 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
     auto put = [&](int c, int row, double re, double im) {
         if (bad) re = im = __longlong_as_double(0x7ff8000000000000ll);
         if (grad) {
-            w.gradraw[in.param_off + row] = sizeof(A) == 16 ? -scalbn(re, w.etaexp[it.inst] - 60) : -re;
+            w.gradraw[in.param_off + row] = sizeof(A) == 16 ? -scalbn(re, w.etaexp[it.inst] - 62) : -re;
         } else if (row == P) {
             w.sigma[in.param_off + c] = re * unit;
         } else if (row < c) {
@@ -478,7 +483,7 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
             Sums<T, KB> sr, si;
             run_step<T, KB, MIM>(b, reinterpret_cast<const S *>(w.a) + in.a_off + off,
                              reinterpret_cast<const S *>(w.d) + in.d_off + off, TC, u.run > 0, sr, si,
-                             simple ? nullptr : buf + tin, tpc);
+                             simple ? nullptr : buf + tin, tpc, h0);
             const int ipc = rn.ip_count, ipf = rn.ip_first;
             const int nrow = ipc + (start ? 1 : 0);  // the column's own run: <sigma_j> as one more row
             for (int q0 = 0; q0 < nrow; q0 += 8) {

@@ -13,10 +13,12 @@ namespace frames {
 
 typedef long long ll;
 
+struct Part;
 struct Fix {  // complex128: fixed point
     using A = longlong2;  // amplitude, 2^60 = 1
     using S = int4;       // stored: (re hi, re lo, im hi, im lo), value = hi 2^32 + lo, lo signed
-    using Acc = ll;       // inner products, 2^60 = 1
+    using Acc = ll;       // inner products
+    using Part = frames::Part;
     using Red = ll;
     using Eta = double2;  // H psi
     static constexpr uint32_t kSwz = 7;  // eight 16-byte banks
@@ -25,6 +27,7 @@ struct Flt {  // complex64
     using A = float2;
     using S = float2;
     using Acc = float;
+    using Part = float;
     using Red = double;
     using Eta = float2;
     static constexpr uint32_t kSwz = 15;  // sixteen 8-byte banks
@@ -64,27 +67,57 @@ template <int CONJ> __device__ __forceinline__ float2 mul(float2 x, float2 d, ui
     return float2{fmaf(x.x, d.x, -x.y * s), fmaf(x.x, s, x.y * d.x)};
 }
 
-// Re (IM = 0) or Im (IM = 1) of conj(a) b, lo lo included: at 2^12 amplitudes and more a product is
-// 2^-12 and less, and float64 would round it at 2^-65
-// UP: the operands' unit is 2^-(60 - UP), the product's 2^-60
-template <int IM, int UP = 0> __device__ __forceinline__ ll prod(int4 a, longlong2 b, uint32_t dither = 0) {
+// Re (IM = 0) or Im (IM = 1) of conj(a) b for fixed-point vectors of unit 2^-(60 - UP), as a multiple of 2^-60 (v)
+// and what is left below it (f, kFracBits bits, never negative). Inner products are between vectors of norm 1 at
+// most, so sums stay within 1 in magnitude.
+struct Part {
+    ll v;
+    int f;
+};
+template <int UP> constexpr int kFracBits = 28 - 2 * UP;
+template <int IM, int UP> __device__ __forceinline__ Part prod_part(int4 a, longlong2 b) {
     const int rh = hi_of(b.x), rl = lo_of(b.x), ih = hi_of(b.y), il = lo_of(b.y);
-    const ll rnd = dither ? (ll)(dither >> (4 + 2 * UP)) : 1ll << (27 - 2 * UP), half = 1ll << 31;  // to nearest: a product and its negative round alike
+    constexpr int F = kFracBits<UP>;
+    const ll half = 1ll << 31;
+    ll h, c;
     if constexpr (IM == 0) {
-        const ll h = wide(a.x, rh) + wide(a.z, ih);
+        h = wide(a.x, rh) + wide(a.z, ih);
         const ll l = wide(a.y, rl) + wide(a.w, il) + half;
-        const ll c = wide(a.x, rl) + wide(a.y, rh) + wide(a.z, il) + wide(a.w, ih) + rnd + (l >> 32);
-        return (h << (4 + 2 * UP)) + (c >> (28 - 2 * UP));
+        c = wide(a.x, rl) + wide(a.y, rh) + wide(a.z, il) + wide(a.w, ih) + (l >> 32);
     } else {
-        const ll h = wide(a.x, ih) - wide(a.z, rh);
+        h = wide(a.x, ih) - wide(a.z, rh);
         const ll l = wide(a.y, il) - wide(a.w, rl) + half;
-        const ll c = wide(a.x, il) + wide(a.y, ih) - wide(a.z, rl) - wide(a.w, rh) + rnd + (l >> 32);
-        return (h << (4 + 2 * UP)) + (c >> (28 - 2 * UP));
+        c = wide(a.x, il) + wide(a.y, ih) - wide(a.z, rl) - wide(a.w, rh) + (l >> 32);
     }
+    return Part{(h << (32 - F)) + (c >> F), (int)((unsigned)c & ((1u << F) - 1u))};
 }
-template <int IM, int UP = 0> __device__ __forceinline__ float prod(float2 a, float2 b, uint32_t = 0) {
+template <int IM, int UP> __device__ __forceinline__ float prod_part(float2 a, float2 b) {
     return IM ? fmaf(a.x, b.y, -a.y * b.x) : fmaf(a.x, b.x, a.y * b.y);
 }
+__device__ __forceinline__ void add(Part &s, Part p, bool neg) {
+    s.v += neg ? -p.v : p.v;
+    s.f += neg ? -p.f : p.f;
+}
+__device__ __forceinline__ void add(float &s, float p, bool neg) { s += neg ? -p : p; }
+// A thread's sum rounded by rnd, uniform below one unit.
+template <int UP> __device__ __forceinline__ ll rounded(Part s, uint32_t rnd) {
+    constexpr int F = kFracBits<UP>;
+    return s.v + ((s.f + (int)(rnd >> (32 - F))) >> F);
+}
+template <int UP> __device__ __forceinline__ float rounded(float s, uint32_t) { return s; }
+// One product, rounded by rnd.
+template <int IM, int UP> __device__ __forceinline__ ll prod(int4 a, longlong2 b, uint32_t rnd) {
+    return rounded<UP>(prod_part<IM, UP>(a, b), rnd);
+}
+template <int IM, int UP> __device__ __forceinline__ float prod(float2 a, float2 b, uint32_t) { return prod_part<IM, UP>(a, b); }
+
+// Pseudo-random bits over the amplitudes: a thread's (hash of its index), xor a constant per amplitude.
+__device__ __forceinline__ uint32_t hash(uint32_t x) {
+    x = (x ^ (x >> 16)) * 0x7feb352du;
+    x = (x ^ (x >> 15)) * 0x846ca68bu;
+    return x ^ (x >> 16);
+}
+__host__ __device__ constexpr uint32_t salt(int k) { return 0x9e3779b9u * (uint32_t)(2 * k + 1); }
 
 __device__ __forceinline__ longlong2 operator+(longlong2 a, longlong2 b) { return longlong2{a.x + b.x, a.y + b.y}; }
 __device__ __forceinline__ longlong2 operator-(longlong2 a, longlong2 b) { return longlong2{a.x - b.x, a.y - b.y}; }

@@ -146,11 +146,6 @@ __device__ __forceinline__ void slots_of(unsigned char *smem, uint32_t b0, const
 // xor a constant per amplitude), uniform below one unit. Rounding to nearest would not do at these
 // sizes: shallow circuits leave the state with few distinct values, each of which is rounded alike on
 // all of its amplitudes, and the errors of 2^22 products add up instead of cancelling.
-__device__ __forceinline__ uint32_t hash(uint32_t x) {
-    x = (x ^ (x >> 16)) * 0x7feb352du;
-    x = (x ^ (x >> 15)) * 0x846ca68bu;
-    return x ^ (x >> 16);
-}
 // x 2^-s, rounded by the dither's bits; s uniform over the launch
 __device__ __forceinline__ void scale_down(longlong2 &x, int s, uint32_t dither) {
     if (s) {
@@ -159,7 +154,6 @@ __device__ __forceinline__ void scale_down(longlong2 &x, int s, uint32_t dither)
     }
 }
 __device__ __forceinline__ void scale_down(float2 &, int, uint32_t) {}
-__host__ __device__ constexpr uint32_t salt(int k) { return 0x9e3779b9u * (uint32_t)(2 * k + 1); }
 
 // -i eta, rounded by the dither
 __device__ __forceinline__ longlong2 seed_dithered(double2 e, const SeedScale &up, uint32_t d) {
@@ -314,10 +308,9 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
             } else {
                 const bool mult = r > 0;
                 const int shift = start ? 0 : u.rshift;  // a column that starts here has no Hadamards behind it
-                Sums<T, KB> sr, si;
-                sr.all = si.all = 0;
-#pragma unroll
-                for (int j = 0; j < KB; ++j) sr.bit[j] = si.bit[j] = 0;
+                constexpr int UP = 60 - kUnit + (kSumUnit - 60) / 2;  // a product's unit is 2^-60 at 60 - kUnit
+                using Part = typename T::Part;
+                Part pr[1 + KB] = {}, pi[1 + KB] = {};  // all products; signed by each of the thread's bits
                 // A loop over the thread's slots instead of unrolled registers: the vector is out of the
                 // registers meanwhile, which hold U checkpoint and factor reads in flight. The thread's bits lie
                 // in one half of the index (else, in narrow windows: `both`): the other half's factor is the same
@@ -352,7 +345,7 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
                 const uint32_t s0 = sslot<T>(tb0);
 #pragma unroll 1
                 for (int k0 = 0; k0 < NA; k0 += U) {
-                    Acc pu = 0, qu = 0;
+                    Part pu = {}, qu = {};
                     S av[U], vv[U];
                     const uint32_t ga = g0 + ((uint32_t)k0 << gsh), gv = both ? 0u : v0 + ((uint32_t)k0 << vsh);
                     const uint32_t sb = s0 ^ sslot<T>((uint32_t)k0 << low), sw = sgnw >> k0;
@@ -367,16 +360,15 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
                         A x = *sp;
                         const uint32_t dk = sizeof(A) == 16 ? (h0 ^ (0x9e3779b9u * (uint32_t)(k0 + k + 1))) | 64u : 0u;
                         if (sizeof(A) == 16) scale_down(x, shift, dk * 11u);
-                        constexpr int UP = 60 - kUnit + (kSumUnit - 60) / 2;  // prod's sum unit is 2^-60 at 60 - kUnit
-                        const Acc p = prod<0, UP>(av[k], x, dk);
-                        pu += p;
+                        const Part p = prod_part<0, UP>(av[k], x);
+                        add(pu, p, false);
 #pragma unroll
-                        for (int j = 0; j < LU; ++j) sr.bit[j] += (k >> j) & 1 ? -p : p;
+                        for (int j = 0; j < LU; ++j) add(pr[1 + j], p, (k >> j) & 1);
                         if (MIM) {
-                            const Acc q = prod<1, UP>(av[k], x, dk * 5u);
-                            qu += q;
+                            const Part q = prod_part<1, UP>(av[k], x);
+                            add(qu, q, false);
 #pragma unroll
-                            for (int j = 0; j < LU; ++j) si.bit[j] += (k >> j) & 1 ? -q : q;
+                            for (int j = 0; j < LU; ++j) add(pi[1 + j], q, (k >> j) & 1);
                         }
                         if (mult) {
                             S ov = ov0;
@@ -391,13 +383,22 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
                             *sp = x;
                         }
                     }
-                    sr.all += pu;
-                    if (MIM) si.all += qu;
+                    add(pr[0], pu, false);
+                    if (MIM) add(pi[0], qu, false);
 #pragma unroll
                     for (int j = LU; j < KB; ++j) {
-                        sr.bit[j] += (k0 >> j) & 1 ? -pu : pu;
-                        if (MIM) si.bit[j] += (k0 >> j) & 1 ? -qu : qu;
+                        add(pr[1 + j], pu, (k0 >> j) & 1);
+                        if (MIM) add(pi[1 + j], qu, (k0 >> j) & 1);
                     }
+                }
+                // the thread's sums are rounded once each: 2^(n - KB) roundings a sum instead of 2^n
+                Sums<T, KB> sr, si;
+                sr.all = rounded<UP>(pr[0], h0 ^ salt(160));
+                si.all = rounded<UP>(pi[0], h0 ^ salt(170));
+#pragma unroll
+                for (int j = 0; j < KB; ++j) {
+                    sr.bit[j] = rounded<UP>(pr[1 + j], h0 ^ salt(161 + j));
+                    si.bit[j] = rounded<UP>(pi[1 + j], h0 ^ salt(171 + j));
                 }
                 slots_of<T, KB>(smem, tb0, st, [&](int k, A *s) { b[k] = *s; });
                 // The run's rows, its parameters and (in the column's own run) <sigma_j>: each is one of the
