@@ -81,9 +81,11 @@ enum {
 
 /* amplitude precisions */
 enum {
-    QNG_C64 = 0,  /* complex64 amplitudes; float64 accumulation of inner products, assembly and solve */
+    QNG_C64 = 0,  /* complex64 amplitudes; inner products in float32 over the few amplitudes of a thread (a tile of
+                     the register form's passes), then in two float32 words or float64; float64 assembly and solve */
     QNG_C128 = 1  /* complex128 amplitudes, carried as float64 or as 64-bit fixed point with a resolution
-                     of 2^-58 or finer of the unit-norm state; float64 inner products, assembly and solve */
+                     of 2^-58 or finer of the unit-norm state; inner products in float64 or as 64-bit integers of
+                     2^-62; float64 assembly and solve */
 };
 
 /* One gate: param is the index of its angle in theta for the rotations (RX..RZ, CRX..CRP), which

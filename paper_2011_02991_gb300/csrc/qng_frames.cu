@@ -15,9 +15,9 @@
 // are exact and a product rounds at 2^-60, where float64 would round at 2^-53 of the component.
 // Products come from 32-bit halves in signed (balanced) form, x = hi 2^32 + lo: hi hi and the two
 // cross terms, six IMAD.WIDE for a sum of two products; lo lo (below 2^-62) is left out of the factors'
-// products and taken into the inner products'. Those sum 2^-60 units exactly in 64-bit integers, whatever
+// products and taken into the inner products'. Those sum 2^-62 units exactly in 64-bit integers, whatever
 // the order.
-// complex64 runs the same steps on float32 amplitudes.
+// complex64 runs the same steps on float32 amplitudes; its inner products leave the thread as two float32 words.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -518,8 +518,9 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
                 }
                 if (tpc >= 32) {
                     const int lane = threadIdx.x & 31, q = q0 + ((lane >> 2) & 7);
-                    const Acc xr = warp8(ar, lane);
-                    const Acc xi = MIM ? warp8(ai, lane) : Acc(0);
+                    const auto xr = warp8(ar, lane);
+                    auto xi = across(Acc(0));
+                    if (MIM) xi = warp8(ai, lane);
                     if (live && (lane & 3) == 0 && q < nrow) {
                         const int row = q < ipc ? ipf + q : P;
                         if (direct) {
@@ -534,10 +535,10 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
 #pragma unroll
                     for (int g = 0; g < 8; ++g) {
                         if (q0 + g >= nrow) break;
-                        Acc xr = ar[g], xi = MIM ? ai[g] : Acc(0);
+                        auto xr = across(ar[g]), xi = across(MIM ? ai[g] : Acc(0));
                         for (int s = tpc >> 1; s > 0; s >>= 1) {
-                            xr += shfl(xr, s);
-                            if (MIM) xi += shfl(xi, s);
+                            xr = xr + shfl(xr, s);
+                            if (MIM) xi = xi + shfl(xi, s);
                         }
                         if (live && tin == 0) put(col, q0 + g < ipc ? ipf + q0 + g : P, (double)xr, (double)xi);
                     }

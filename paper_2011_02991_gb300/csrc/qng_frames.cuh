@@ -153,18 +153,43 @@ __device__ __forceinline__ void halve(float2 &x, int s) {
 __device__ __forceinline__ ll shfl(ll v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ float shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 
+// A sum over threads of float32 partial sums, as the float32 nearest to it and what is left: 48 bits on the float32
+// pipe, which takes 64 times what the float64 pipe does.
+struct Two {
+    float s, e;
+    __device__ __forceinline__ explicit operator double() const { return (double)s + (double)e; }
+};
+__device__ __forceinline__ Two exact_sum(float a, float b) {  // s + e = a + b
+    const float s = a + b, t = s - a;
+    return Two{s, (a - (s - t)) + (b - t)};
+}
+__device__ __forceinline__ Two exact_product(float a, float b) {
+    const float p = a * b;
+    return Two{p, fmaf(a, b, -p)};
+}
+__device__ __forceinline__ Two operator+(Two a, Two b) {
+    const Two r = exact_sum(a.s, b.s);
+    return Two{r.s, r.e + (a.e + b.e)};
+}
+__device__ __forceinline__ Two shfl(Two v, int o) { return Two{shfl(v.s, o), shfl(v.e, o)}; }
+
+// the type that sums over threads are carried in
+__device__ __forceinline__ ll across(ll v) { return v; }
+__device__ __forceinline__ Two across(float v) { return Two{v, 0.0f}; }
+__device__ __forceinline__ ll pair_sum(ll a, ll b) { return a + b; }
+__device__ __forceinline__ Two pair_sum(float a, float b) { return exact_sum(a, b); }
+
 // Warp sums of 8 values: the lane returns the sum of a[(lane >> 2) & 7].
-template <typename T> __device__ __forceinline__ T warp8(const T (&a)[8], int lane) {
+template <typename T> __device__ __forceinline__ auto warp8(const T (&a)[8], int lane) {
     const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
-    T t[4], u[2];
+    decltype(across(a[0])) t[4], u[2];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) t[k] = (b4 ? a[4 + k] : a[k]) + shfl(b4 ? a[k] : a[4 + k], 16);
+    for (int k = 0; k < 4; ++k) t[k] = pair_sum(b4 ? a[4 + k] : a[k], shfl(b4 ? a[k] : a[4 + k], 16));
 #pragma unroll
     for (int k = 0; k < 2; ++k) u[k] = (b3 ? t[2 + k] : t[k]) + shfl(b3 ? t[k] : t[2 + k], 8);
-    T v = (b2 ? u[1] : u[0]) + shfl(b2 ? u[0] : u[1], 4);
-    v += shfl(v, 2);
-    v += shfl(v, 1);
-    return v;
+    auto v = (b2 ? u[1] : u[0]) + shfl(b2 ? u[0] : u[1], 4);
+    v = v + shfl(v, 2);
+    return v + shfl(v, 1);
 }
 
 // Hadamards (unnormalised) on the thread's bits hm, then `shift` halvings.

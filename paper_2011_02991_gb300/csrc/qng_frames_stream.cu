@@ -26,9 +26,10 @@ namespace frames {
 // the vector by 2^4), and as every rounding is unbiased (see hash) a unit of 2^-58 on each component moves an
 // inner product with a unit vector by no more.
 constexpr int kUnit = 58;
-// Inner products are sums of 2^-62: unit vectors, so no partial sum of products exceeds 1 in magnitude. What
-// their rounding leaves is a unit times 2^(n/2): at 22 qubits the gradient was 9.5e-15 off in units of 2^-60
-// and is 3.1e-15 in these, g 7.0e-15 and 5.6e-15 (float64 on the gate-by-gate passes: 2.2e-15 and 5.4e-15).
+// Inner products are sums of 2^-62: unit vectors, so no partial sum of products exceeds 1 in magnitude. A thread
+// keeps what lies below the unit as well and rounds its sum once; what that leaves is a unit times
+// 2^((n - KB)/2). 22 qubits, two-norm errors of gradient and g: 2.8e-15 and 4.4e-15 with every product rounded,
+// 2.0e-15 and 4.2e-15 so (float64 on the gate-by-gate passes: 2.1e-15 and 4.4e-15); 17.57 and 17.69 ms.
 constexpr int kSumUnit = 62;
 constexpr int kHalfThreads = 128;
 constexpr int kRows = 32;  // parameters of a run kept in shared memory
@@ -169,7 +170,8 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
     using S = typename T::S;
     using Acc = typename T::Acc;
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ Acc red[16][NT / 32][MIM ? 2 : 1];
+    using Red = typename T::Red;
+    __shared__ Red red[16][NT / 32][MIM ? 2 : 1];
     // the pass's steps and the parameters of its (first) run: read once, or each would wait on L2
     constexpr int kOpsMax = 48;
     __shared__ UOp ops_sh[kOpsMax];
@@ -422,11 +424,12 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
                                 ai[g] = g < 5 ? (neg ? -si.all : si.all) : Acc(0);
                             }
                         }
-                        const Acc xr = warp8(ar, lane);
-                        const Acc xi = MIM ? warp8(ai, lane) : Acc(0);
+                        const auto xr = warp8(ar, lane);
+                        auto xi = across(Acc(0));
+                        if (MIM) xi = warp8(ai, lane);
                         if ((lane & 3) == 0) {
-                            red[half * 8 + (lane >> 2)][wid][0] = xr;
-                            if (MIM) red[half * 8 + (lane >> 2)][wid][1] = xi;
+                            red[half * 8 + (lane >> 2)][wid][0] = (Red)xr;
+                            if (MIM) red[half * 8 + (lane >> 2)][wid][1] = (Red)xi;
                         }
                     }
                 }
@@ -435,10 +438,10 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
                     const int q = MIM ? x >> 1 : x, part = MIM ? x & 1 : 0, row = ipf + q;
                     SIp ip = {0, 0, 1, 0};
                     if (q < ipc) ip = r == ps.run0 && q < kRows ? ips_sh[q] : w.ip[rn.ip_begin + q];
-                    typename std::conditional<sizeof(A) == 16, ll, double>::type d = 0;
+                    Red d = 0;
                     for (int k = 0; k < NT / 32; ++k) {
                         const uint32_t g = gtile | spread(tbase<KB>(k * 32, low));
-                        const auto y = (typename std::conditional<sizeof(A) == 16, ll, double>::type)red[ip.src][k][part];
+                        const Red y = red[ip.src][k][part];
                         d += ((g & ip.z) != 0) != (ip.sgn < 0) ? -y : y;
                     }
                     ll v;
@@ -471,13 +474,14 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
 // complex64 sums in float32, the precision it is stored in. complex128 in fixed point: coefficients as
 // multiples of 2^(eexp - 62), sums as multiples of 2^(eexp - 61); the float64 pipe would take four times as
 // long (22 qubits, 43 terms: 3.4 ms). <E> and |eta|^2 in float64 and then fixed point (as the on-chip
-// kernel), complex64 in float32 over a thread's four amplitudes first. The next mask's
+// kernel), complex64 in two float32 over a thread's four amplitudes first. The next mask's
 // loads go out before a mask's products (20 qubits, 41 masks, complex64: 56 to 45 us, 344 MB of gathers from L2;
 // and float64 conversions and warp sums taken to once per thread and CTA).
 template <class T> struct Coef;
 template <> struct Coef<Fix> {
     using C = ll;
-    using S = double;  // a thread's share of <E> and |eta|^2
+    using S = double;   // a thread's share of |eta|^2
+    using S4 = double;  // of <E>, over four amplitudes
     static __device__ __forceinline__ C of(double c, int eexp) { return __double2ll_rn(scalbn(c, 62 - eexp)); }
     static __device__ __forceinline__ ll mul(ll c, ll x) {
         const int ch = hi_of(c), cl = lo_of(c), xh = hi_of(x), xl = lo_of(x);
@@ -493,6 +497,7 @@ template <> struct Coef<Fix> {
 template <> struct Coef<Flt> {
     using C = float;
     using S = float;
+    using S4 = Two;
     static __device__ __forceinline__ C of(double c, int) { return (float)c; }
     static __device__ __forceinline__ float mul(float c, float x) { return c * x; }
     static __device__ __forceinline__ float value(float h, int) { return h; }
@@ -580,7 +585,8 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
                 }
             }
         }
-        S e4 = 0, n4 = 0;  // a thread's four amplitudes
+        typename K::S4 e4 = {};  // a thread's four amplitudes
+        S n4 = 0;                // (an upper bound is all that is made of it)
 #pragma unroll
         for (int k = 0; k < NA; ++k) {
             const auto y = amp_at(v[m + 256 * k]);
@@ -589,11 +595,12 @@ template <class T> __global__ void __launch_bounds__(256) k_sheff(SWork w, int i
             o.x = hr;
             o.y = hi;
             eta[m + 256 * k] = o;
-            e4 += y.x * hr + y.y * hi;
+            if constexpr (sizeof(S) == 4) e4 = (e4 + exact_product(y.x, hr)) + exact_product(y.y, hi);
+            else e4 += y.x * hr + y.y * hi;
             const S ar = K::scaled(h[k].x, fs), ai = K::scaled(h[k].y, fs);
             n4 += ar * ar + ai * ai;
         }
-        e += e4;
+        e += (double)e4;
         n2 += n4;
     }
     red[threadIdx.x][0] = e;
