@@ -146,15 +146,23 @@ struct Builder {
         m.cval = fr[c].z.s > 0 ? m.ctrl : 0;
         open().push_back(m);
     }
-    void cnot(int c, int t) {
+    // CNOT c -> t; touched: the qubits that it and the CNOTs right after it share, through one another
+    void cnot(int c, int t, uint32_t touched) {
         if (fr[c].z.p == PZ && fr[t].x.p == PZ) { controlled_sign(c, t, kAxisX); return; }
-        diagonalise({{c, kAxisZ}, {t, kAxisZ}});
-        for (int q : {c, t})
-            if (fr[q].x.p == PY) {  // a diagonal S^dag of the open run turns the X image back to X
-                open().push_back(Member{2, -1, 1u << q, 0, 0, 1});
-                fr[q].x = conj_sdg(fr[q].x);
-                fr[q].z = conj_sdg(fr[q].z);
-            }
+        // Frames whose Z and X images are Z and X: for all of the CNOTs to come at once, so that a ladder is one
+        // index permutation behind one transition and at most one run of S^dag (a CNOT at a time, a ladder on n
+        // qubits cut n - 1 runs without a parameter: 12 qubits, 16 x [Ry, CNOT ladder], 192 runs for 32 now)
+        std::vector<std::pair<int, int>> req;
+        for (int q = 0; q < (int)fr.size(); ++q) if ((touched >> q) & 1) req.push_back({q, kAxisZ});
+        diagonalise(req);
+        for (auto &r : req) {
+            const int q = r.first;
+            if (fr[q].x.p != PY) continue;
+            // an S^dag turns the X image back to X: into the run before where nothing of the open one asks for it
+            if (!open().empty() || !sdg_before_open(q)) open().push_back(Member{2, -1, 1u << q, 0, 0, 1});
+            fr[q].x = conj_sdg(fr[q].x);
+            fr[q].z = conj_sdg(fr[q].z);
+        }
         if (!open().empty()) close();
         if (otau().empty() || !otau().back().perm) { otau().emplace_back(); otau().back().perm = true; }
         Lin &A = otau().back().map;
@@ -197,7 +205,18 @@ void walk_gates(const std::vector<qng_gate> &gates, const std::vector<uint64_t> 
             B.diagonalise({{g.q0, kAxisZ}, {g.q1, kAxisZ}});
             B.controlled_sign(g.q0, g.q1, kAxisZ);
             break;
-        case QNG_GATE_CNOT: B.cnot(g.q0, g.q1); break;
+        case QNG_GATE_CNOT: {
+            uint32_t touched = (1u << g.q0) | (1u << g.q1);
+            for (uint32_t before = 0; before != touched;) {
+                before = touched;
+                for (size_t k = gi + 1; k < gates.size() && gates[k].kind == QNG_GATE_CNOT; ++k) {
+                    const uint32_t m = (1u << gates[k].q0) | (1u << gates[k].q1);
+                    if (m & touched) touched |= m;
+                }
+            }
+            B.cnot(g.q0, g.q1, touched);
+            break;
+        }
         default: break;
         }
     }

@@ -3,6 +3,7 @@ executed in float64 by a host-only probe (tests/frames_probe.cu, linking the lib
 compared with the oracle: metric, its imaginary part, <sigma_j>, control probabilities, gradient and
 energy. Circuits of every gate kind in every order, so that frames of every kind meet rotations,
 CNOT networks, controlled and string rotations; 1 to 9 qubits, one to eight CTAs per vector."""
+import itertools
 import shutil
 import subprocess
 
@@ -78,8 +79,7 @@ def test_generalised(probe, oracle, seed):
 @pytest.mark.parametrize("cl", [0, 1, 2, 3])
 @pytest.mark.parametrize("kinds,ent", [((W.RY, W.RZ), W.CZ), ((W.RY, W.RX, W.RZ), W.CNOT), ((W.RX, W.RY), W.CNOT)])
 def test_layered(probe, oracle, kinds, ent, cl):
-    """Layered ansätze; every layer's rotations of one axis are one run (a CNOT ladder
-    right after rotations of another axis than Z is cut into more)."""
+    """Layered ansätze; every layer's rotations of one axis are one run."""
     n = 7
     c = W.layered_ansatz(n, 3, kinds, ent)
     rng = np.random.Generator(np.random.PCG64(3))
@@ -88,6 +88,20 @@ def test_layered(probe, oracle, kinds, ent, cl):
     check(probe, oracle, p, 3, cl)
     if kinds[-1] == W.RZ:
         assert d["runs"][0] <= 3 * len(kinds) + 1
+
+
+@pytest.mark.parametrize("ent", [W.CZ, W.CNOT])
+@pytest.mark.parametrize("kinds", [k for m in (1, 2, 3) for k in itertools.permutations((W.RX, W.RY, W.RZ), m)])
+def test_runs_per_layer(probe, oracle, kinds, ent):
+    """A layer costs one run per axis and at most one more, for the entangler's signs or S phases: a ladder is one
+    transition, whatever rotations it follows."""
+    n, layers = 6, 3
+    c = W.layered_ansatz(n, layers, kinds, ent)
+    rng = np.random.Generator(np.random.PCG64(5))
+    p = W.Problem("l", c, W.random_pauli_hamiltonian(n, 9, rng), W.uniform_theta(c.num_params, rng))
+    d = check(probe, oracle, p, 3)
+    assert d["runs"][0] <= layers * (len(kinds) + 1) + 1
+    check(probe, oracle, p, 3, 0, 5, 2)
 
 
 def test_z_runs_and_no_parameters(probe, oracle):
