@@ -469,20 +469,49 @@ qng_status plan_streaming(qng_ctx *c, int64_t scale_n) {
     return QNG_OK;
 }
 
+// Few instances: what counts is the latency of each one's longest walk, not how many walks the GPU holds.
+constexpr int kFewInstances = 8;
+
 // Index bits per thread of the diagonal-frame kernels. A single instance has few columns, and each one's
 // walk is a serial chain: 8 amplitudes a thread put twice the warps of 16 on it (11 qubits, general
-// circuit, complex128: columns 385 -> 233 us; 12 qubits, complex64: the same). A batch fills the GPU with
-// columns, where 16 need fewer exchanges (64 instances, complex64: 3.61 -> 1.84 ms). From 14 qubits on 16
-// keep the vector within 8 CTAs.
-int frames_kb(const qng_ctx *c) { return c->count == 1 && c->inst[0].n < 14 ? 3 : 4; }
+// circuit, complex128: columns 385 -> 233 us; 12 qubits, complex64: the same). A batch that fills the GPU with
+// columns does better with 16, which need fewer exchanges (64 instances of 6 to 14 qubits, complex64: 7.1 -> 4.5 ms),
+// unless its vectors are small, where a thread's chain is all there is (16 general instances of 3 to 7 qubits,
+// complex128: 800 -> 260 us with 8; 64 layered ones of 2 to 4: 930 -> 230 us). complex128 with 16 amplitudes has no
+// registers left for the products of a general run. 16 keep the largest vectors within 8 CTAs.
+int frames_kb(const qng_ctx *c) {
+    int n = 0;
+    bool general = false;
+    for (const HostInst &h : c->inst) {
+        n = std::max(n, h.n);
+        general = general || h.general;
+    }
+    if (c->precision == QNG_C128) {
+        if (general) return 3;
+        return n <= (c->count <= kFewInstances ? 14 : 12) ? 3 : 4;
+    }
+    if (c->count == 1) return n < 14 ? 3 : 4;
+    return n <= (general ? 12 : 10) ? 3 : 4;
+}
 
 // CTAs per vector (log2): as many as it takes to hold it at 2^kb amplitudes a thread and 512 threads a
-// CTA. A single complex128 instance, bound by instruction issue, spreads its walks over up to 4 SMs
-// (12 qubits: sweep 117 -> 86 us, columns 165 -> 148 us); complex64 ones lose more to the exchanges
-// between SMs than they gain (columns 82 -> 91 us).
+// CTA. complex128 instances, bound by instruction issue, spread their walks over up to 8 SMs while there are few
+// (12 qubits, 4 CTAs: sweep 117 -> 86 us, columns 165 -> 148 us; 14 qubits, 6 layers, 8 CTAs instead of 2: step 676 ->
+// 612 us, energy 235 -> 116; general circuits of 14 qubits 808 -> 428); complex64 ones lose more to the exchanges between
+// SMs than they gain (columns 82 -> 91 us).
 int frames_cl(const qng_ctx *c, int n, int kb) {
     const int need = std::max(0, n - (9 + kb));
-    return c->count == 1 && c->precision == QNG_C128 && n < 14 ? std::max(need, std::min(2, n - 10)) : need;
+    if (c->count > kFewInstances / 2 || c->precision != QNG_C128) return need;
+    return std::max(need, n >= 13 ? 3 : std::min(2, n - 10));
+}
+
+// CTA size of an instance's column kernel: room for the columns that start in a run, so that small vectors share a CTA
+// but none walks along empty (256 threads for every one cost 64 instances of 2 to 4 qubits 930 instead of 230 us).
+int frames_threads(const frames::Program &p, int tpc, int count) {
+    const int R = std::max<int>(1, (int)p.runs.size()), cols = std::max<int>(1, ((int)p.ips.size() + R - 1) / R);
+    int t = 64;
+    while (t < 256 && t < tpc * cols) t *= 2;
+    return std::max(tpc, count == 1 ? 64 : t);
 }
 
 // Programs, work lists and launch classes of the diagonal-frame path. False when a class's shared
@@ -543,9 +572,11 @@ bool plan_frames(qng_ctx *c) {
                 f.tab.push_back(frames::TabItem{b, r, first});
         f.inst.push_back(d);
         const int tpc = (N >> kb) >> d.cl;
-        // a batch packs small vectors into CTAs of 256 threads; one instance spreads over more CTAs
-        key[b] = {d.cl, std::max(tpc, c->count == 1 ? 64 : 256)};
+        key[b] = {d.cl, frames_threads(p, tpc, c->count)};
     }
+    if (c->count <= kFewInstances)  // one class per cluster size: launches side by side cost more than idle threads
+        for (auto &k : key)
+            for (const auto &o : key) if (o[0] == k[0]) k[1] = std::max(k[1], o[1]);
     std::vector<std::array<int, 2>> keys(key);
     std::sort(keys.begin(), keys.end(), [](const std::array<int, 2> &x, const std::array<int, 2> &y) { return x > y; });
     keys.erase(std::unique(keys.begin(), keys.end()), keys.end());
@@ -573,6 +604,7 @@ bool plan_frames(qng_ctx *c) {
             if (d.P > 0) items.push_back(It{frames::Item{b, d.R, 0, 0, 0, d.P, d.R, 0}, (d.R + 1.0), true});
             for (int r = 0; r < d.R; ++r) {
                 const frames::Run &rn = f.run[d.run_off + r];
+                cl.general = cl.general || !rn.simple;
                 std::vector<int32_t> list;
                 for (int q = 0; q < rn.ip_count; ++q) {
                     const int j = rn.ip_first + q;
@@ -607,6 +639,7 @@ bool plan_frames(qng_ctx *c) {
         fits = fits && cl.smem_col_im <= kMaxSmem && cl.smem_fwd <= kMaxSmem;
         f.cls.push_back(cl);
     }
+    for (const frames::Class &cl : f.cls) fits = fits && (!cl.general || frames::takes_general(c->precision, kb));
     return fits && 2 * (f.amps_ad + f.amps_v) * (int64_t)ab <= kFramesMax;
 }
 

@@ -351,16 +351,11 @@ template <class T> __global__ void __launch_bounds__(kHThreads) k_heff(FWork w, 
 // nearest is the same for the equal amplitudes of a structured state and adds up over them.
 constexpr int kSumUp = 1;
 
-// One run of the walk: products with the checkpoint, then (mult) the run's adjoint factors. scratch
-// (runs that are not simple): the products go to shared memory, stride apart.
-template <class T, int KB, int MIM>
+// One run of the walk: products with the checkpoint, f(k, re, im), then (mult) the run's adjoint factors.
+template <class T, int KB, int MIM, typename F>
 __device__ __forceinline__ void run_step(typename T::A (&b)[1 << KB], const typename T::S *a, const typename T::S *d,
-                                         uint32_t TC, bool mult, Sums<T, KB> &sr, Sums<T, KB> &si, typename T::A *scratch,
-                                         int stride, uint32_t h0) {
+                                         uint32_t TC, bool mult, uint32_t h0, F &&f) {
     constexpr int B = 4;  // loads in flight
-    sr.all = si.all = 0;
-#pragma unroll
-    for (int j = 0; j < KB; ++j) sr.bit[j] = si.bit[j] = 0;
 #pragma unroll
     for (int k0 = 0; k0 < (1 << KB); k0 += B) {
         typename T::S av[B], dv[B];
@@ -373,20 +368,27 @@ __device__ __forceinline__ void run_step(typename T::A (&b)[1 << KB], const type
         for (int k = 0; k < B; ++k) {
             const typename T::Acc p = prod<0, kSumUp>(av[k], b[k0 + k], h0 ^ salt(k0 + k));
             const typename T::Acc q = MIM ? prod<1, kSumUp>(av[k], b[k0 + k], h0 ^ salt(64 + k0 + k)) : typename T::Acc(0);
-            if (scratch) scratch[(k0 + k) * stride] = typename T::A{p, q};
-            sr.all += p;
-            if (MIM) si.all += q;
-#pragma unroll
-            for (int j = 0; j < KB; ++j) {
-                sr.bit[j] += ((k0 + k) >> j) & 1 ? -p : p;
-                if (MIM) si.bit[j] += ((k0 + k) >> j) & 1 ? -q : q;
-            }
+            f(k0 + k, p, q);
             if (mult) b[k0 + k] = mul<1>(b[k0 + k], dv[k]);
         }
     }
 }
 
-template <class T, int KB, int MIM>
+// A thread's products summed with a parameter's signs, over those that its control includes.
+template <class Acc, int NA> __device__ __forceinline__ Acc signed_sum(const Acc (&p)[NA], uint32_t incl, uint32_t sign) {
+    Acc v = 0;
+#pragma unroll
+    for (int k = 0; k < NA; ++k) {
+        const Acc x = (incl >> k) & 1 ? p[k] : Acc(0);
+        v += (sign >> k) & 1 ? -x : x;
+    }
+    return v;
+}
+
+// GEN = 1: instances with controlled and string rotations, whose parameters take the thread's products with signs
+// and controls of their own. A run that holds one keeps its products in registers and sums them once per parameter (runs
+// of such circuits have one or two).
+template <class T, int KB, int MIM, int GEN>
 __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int max_P) {
     constexpr int NA = 1 << KB;
     using A = typename T::A;
@@ -402,7 +404,6 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
     const int ltpc = nE - KB - cl, tpc = 1 << ltpc;  // threads of a column in this CTA
     const int sl = threadIdx.x >> ltpc, tin = threadIdx.x & (tpc - 1);
     const uint32_t boff = ((uint32_t)sl << (nE - cl)) * (uint32_t)sizeof(A);
-    A *buf = reinterpret_cast<A *>(smem + boff);
     // per-warp partial sums [slot][row][warp], rows 0..P-1 the parameters, row P <sigma_j>
     Red *red = reinterpret_cast<Red *>(reinterpret_cast<A *>(smem) + (size_t)blockDim.x * NA);
     const int nw = tpc >= 32 ? tpc / 32 : 1;
@@ -478,14 +479,52 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
         if (u.run >= 0) {
             const Run &rn = runs[u.run];
             const int64_t off = ((int64_t)u.run << nE) + p.t;
-            const bool simple = rn.simple;
-            if (!simple) vsync(cl > 0, tpc);
-            Sums<T, KB> sr, si;
-            run_step<T, KB, MIM>(b, reinterpret_cast<const S *>(w.a) + in.a_off + off,
-                             reinterpret_cast<const S *>(w.d) + in.d_off + off, TC, u.run > 0, sr, si,
-                             simple ? nullptr : buf + tin, tpc, h0);
+            const S *a = reinterpret_cast<const S *>(w.a) + in.a_off + off, *d = reinterpret_cast<const S *>(w.d) + in.d_off + off;
             const int ipc = rn.ip_count, ipf = rn.ip_first;
             const int nrow = ipc + (start ? 1 : 0);  // the column's own run: <sigma_j> as one more row
+            if (GEN && !rn.simple) {
+                Acc pr[NA], pi[NA];
+                run_step<T, KB, MIM>(b, a, d, TC, u.run > 0, h0, [&](int k, Acc p, Acc q) { pr[k] = p; pi[k] = q; });
+#pragma unroll 1
+                for (int q = 0; q < nrow; ++q) {
+                    uint32_t incl = 0xffffu, sign = 0;
+                    if (q < ipc) {
+                        const Ip &ip = ips[ipf + q];
+                        incl = (p.t & ip.ctrl) == ip.cval ? ip.incl16 : 0u;
+                        sign = ip.sign16 ^ (((__popc(p.t & ip.z) & 1) ^ (ip.sgn < 0)) ? 0xffffu : 0u);
+                    }
+                    auto xr = across(signed_sum<Acc, NA>(pr, incl, sign)), xi = across(Acc(0));
+                    if (MIM) xi = across(signed_sum<Acc, NA>(pi, incl, sign));
+                    for (int s = min(tpc, 32) >> 1; s > 0; s >>= 1) {
+                        xr = xr + shfl(xr, s);
+                        if (MIM) xi = xi + shfl(xi, s);
+                    }
+                    if (!live || (tin & 31) != 0) continue;
+                    const int row = q < ipc ? ipf + q : P;
+                    if (direct || tpc < 32) {
+                        put(col, row, (double)xr, (double)xi);
+                    } else {
+                        const size_t at = ((size_t)sl * (max_P + 1) + row) * nw + (tin >> 5);
+                        red[at] = (Red)xr;
+                        if (MIM) red[rows + at] = (Red)xi;
+                    }
+                }
+                start = false;
+                continue;
+            }
+            Sums<T, KB> sr, si;
+            sr.all = si.all = 0;
+#pragma unroll
+            for (int j = 0; j < KB; ++j) sr.bit[j] = si.bit[j] = 0;
+            run_step<T, KB, MIM>(b, a, d, TC, u.run > 0, h0, [&](int k, Acc p, Acc q) {
+                sr.all += p;
+                if (MIM) si.all += q;
+#pragma unroll
+                for (int j = 0; j < KB; ++j) {
+                    sr.bit[j] += (k >> j) & 1 ? -p : p;
+                    if (MIM) si.bit[j] += (k >> j) & 1 ? -q : q;
+                }
+            });
             for (int q0 = 0; q0 < nrow; q0 += 8) {
                 Acc ar[8], ai[8];
 #pragma unroll
@@ -495,20 +534,8 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
                     if (q < ipc) {
                         const Ip &ip = ips[ipf + q];
                         const uint32_t sgn = (__popc(p.t & ip.z) & 1) ^ (ip.sgn < 0);
-                        if (simple) {
-                            vr = pick<T, KB>(sr, ip.zreg);
-                            if (MIM) vi = pick<T, KB>(si, ip.zreg);
-                        } else if ((p.t & ip.ctrl) == ip.cval) {
-                            const uint32_t incl = ip.incl16, sign = ip.sign16;
-#pragma unroll 1
-                            for (int k = 0; k < (1 << KB); ++k) {
-                                const A x = buf[tin + k * tpc];
-                                if ((incl >> k) & 1) {
-                                    vr += ((sign >> k) & 1) ? -x.x : x.x;
-                                    if (MIM) vi += ((sign >> k) & 1) ? -x.y : x.y;
-                                }
-                            }
-                        }
+                        vr = pick<T, KB>(sr, ip.zreg);
+                        if (MIM) vi = pick<T, KB>(si, ip.zreg);
                         if (sgn) { vr = -vr; vi = -vi; }
                     } else if (q < nrow) {
                         vr = sr.all;
@@ -544,7 +571,6 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
                     }
                 }
             }
-            if (!simple) vsync(cl > 0, tpc);
         }
         start = false;
     }
@@ -577,10 +603,16 @@ __global__ void __launch_bounds__(512, 1) k_cols(FWork w, int first, int cl, int
 #define QNG_FRAMES(F)                                                                       \
     (precision == QNG_C128 ? (kb == 3 ? F(Fix, 3) : F(Fix, 4)) : (kb == 3 ? F(Flt, 3) : F(Flt, 4)))
 
+// takes_general: complex128 with 16 amplitudes a thread has no registers for a run's products (1.3 KB of spills)
+template <class T, int KB> constexpr int kGeneral = sizeof(typename T::A) == 16 && KB == 4 ? 0 : 1;
+
 template <class T, int KB> static cudaError_t prepare_t(size_t smem_fwd, size_t smem_col, size_t smem_col_im) {
     cudaError_t e = raise_smem_limit(reinterpret_cast<const void *>(k_fwd<T, KB>), smem_fwd);
-    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void *>(k_cols<T, KB, 0>), smem_col);
-    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void *>(k_cols<T, KB, 1>), smem_col_im);
+    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void *>(k_cols<T, KB, 0, 0>), smem_col);
+    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void *>(k_cols<T, KB, 1, 0>), smem_col_im);
+    constexpr int G = kGeneral<T, KB>;
+    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void *>(k_cols<T, KB, 0, G>), smem_col);
+    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void *>(k_cols<T, KB, 1, G>), smem_col_im);
     return e;
 }
 
@@ -613,7 +645,8 @@ cudaError_t launch_columns(const FWork &w, const Class &c, int precision, int fi
     if (num == 0) return cudaSuccess;
     const int kb = c.kb;
 #define QNG_F(T, KB)                                                                                             \
-    launch_next(w.chain, metric_im ? k_cols<T, KB, 1> : k_cols<T, KB, 0>, num << c.cl, c.threads,               \
+    launch_next(w.chain, c.general ? (metric_im ? k_cols<T, KB, 1, kGeneral<T, KB>> : k_cols<T, KB, 0, kGeneral<T, KB>>) \
+                                   : (metric_im ? k_cols<T, KB, 1, 0> : k_cols<T, KB, 0, 0>), num << c.cl, c.threads, \
                 metric_im ? c.smem_col_im : c.smem_col, 1u << c.cl, st, w, first, c.cl, c.max_P)
     return QNG_FRAMES(QNG_F);
 #undef QNG_F

@@ -127,6 +127,7 @@ struct Class {
     int threads = 0;                     // CTA size of the column kernel
     int fwd_threads = 0;                 // CTA size of the forward sweep
     int max_P = 0;
+    bool general = false;                // some run is not simple
     int first_inst = 0, num_inst = 0;    // into order
     int first_item = 0, num_item = 0;    // metric and gradient columns, longest first
     int first_met = 0, num_met = 0;
@@ -163,6 +164,8 @@ struct FWork {
 constexpr int kTabThreads = 128, kTabBits = 2, kTabAmps = 1 << kTabBits;
 constexpr int kHThreads = 64, kHSplit = 4;  // H psi: threads per CTA, threads per amplitude
 
+// The column kernel of that form takes runs that are not simple.
+inline bool takes_general(int precision, int kb) { return precision != QNG_C128 || kb == 3; }
 cudaError_t prepare(int precision, int kb, size_t smem_fwd, size_t smem_col, size_t smem_col_im);
 cudaError_t launch_tables(const FWork &w, int ntab, int kb, int precision, cudaStream_t st);
 cudaError_t launch_forward(const FWork &w, const Class &c, int precision, cudaStream_t st);

@@ -1,5 +1,5 @@
 """Inputs at the ends of what the entry points take: Hamiltonian coefficients near the ends of float64's range, more
-parameters than a launch grid's y dimension has tiles of the metric, more runs than it has blocks."""
+parameters than a launch grid's y dimension has tiles of the metric, more runs than it has blocks; and circuits on both sides of where a launch shape or a kernel changes."""
 import numpy as np
 import pytest
 import torch
@@ -105,3 +105,61 @@ def test_vanishing_imaginary_part(qng, n, path):
     ctx.sync()
     rms = float((G.imag ** 2).mean().sqrt())
     assert rms <= 1.5 * 0.25 * 0.29 * 2.0 ** -62 * np.sqrt(2.0 ** n / (16 if path == 2 else 1))
+
+
+def _layered(n, layers, kinds=(W.RY, W.RX), ent=W.CNOT):
+    return lambda seed: W.layered_ansatz(n, layers, kinds, ent)
+
+
+def _general(n, P):
+    return lambda seed: W.general_problem(n, P, seed).circuit
+
+
+def _random(n, gates):
+    return lambda seed: W.random_circuit(n, gates, np.random.Generator(np.random.PCG64([n, seed])))
+
+
+SHAPES = {
+    # gate by gate, or frames, by steps per parameter; one to eight qubits
+    "tiny": [_layered(1, 4), _layered(2, 5), _layered(3, 3), _random(4, 40)],
+    "small_frames": [_layered(2, 4, (W.RY, W.RZ), W.CZ), _layered(3, 3, (W.RY, W.RZ), W.CZ), _layered(7, 2, (W.RY, W.RZ), W.CZ)],
+    "small_general": [_general(3 + k % 6, 20 + k) for k in range(10)],
+    # 8 and 16 amplitudes a thread, CTAs of 64 to 512 threads, few instances and more
+    "general": [_general(5 + k, 24) for k in range(8)],
+    "general_more": [_general(4 + k, 20) for k in range(9)],
+    "ten": [_layered(10, 2, (W.RY, W.RZ), W.CZ), _layered(6, 3)],
+    "eleven": [_layered(11, 1, (W.RY, W.RZ), W.CZ), _random(5, 60)] + [_layered(4, 2)] * 7,
+    "thirteen": [_layered(13, 1), _layered(9, 2)],
+    "thirteen_general": [_general(13, 12)] + [_general(4 + k, 15) for k in range(8)],
+    "thirteen_more": [_layered(13, 1)] + [_layered(3 + k, 2) for k in range(8)],
+    # clusters of 8 CTAs
+    "one13": [_layered(13, 1)],
+    "one14": [_random(14, 40)],
+    "one14_general": [_general(14, 14)],
+    "one15": [_layered(15, 1, (W.RY, W.RZ), W.CZ)],
+    "one15_general": [_general(15, 9)],
+}
+
+
+@pytest.mark.parametrize("precision", [W.C64, W.C128])
+@pytest.mark.parametrize("name", sorted(SHAPES))
+def test_shapes(qng, oracle, name, precision):
+    """Metric, its imaginary part, gradient and energy of every instance against the oracle."""
+    probs = []
+    for k, make in enumerate(SHAPES[name]):
+        c = make(300 + k)
+        rng = np.random.Generator(np.random.PCG64([c.n, k]))
+        probs.append(W.Problem(name, c, W.random_pauli_hamiltonian(c.n, 6, rng), W.uniform_theta(c.num_params, rng), precision=precision))
+    ctx = qng.Context(probs if len(probs) > 1 else probs[0])
+    G = ctx.metric_complex(ctx.theta0())
+    g = ctx.metric(ctx.theta0())
+    grad, e = ctx.gradient(ctx.theta0())
+    ctx.sync()
+    tol = 1e-10 if precision == W.C128 else 2e-4
+    assert float((G.real - g).abs().max()) <= tol
+    for p, Gp, gr, en in zip(probs, ctx.split_metric(G), ctx.split_params(grad), e.cpu().numpy()):
+        ref = oracle.qng_step(p)
+        scale = np.abs(p.hamiltonian.coeffs).sum()
+        assert np.abs(Gp.cpu().numpy() - ref["G"]).max() <= tol / 4, p.n
+        assert np.abs(gr.cpu().numpy() - ref["grad"]).max() <= tol * scale, p.n
+        assert abs(en - ref["E"]) <= tol * scale, p.n
