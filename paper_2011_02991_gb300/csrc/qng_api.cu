@@ -643,6 +643,25 @@ bool plan_frames(qng_ctx *c) {
     return fits && 2 * (f.amps_ad + f.amps_v) * (int64_t)ab <= kFramesMax;
 }
 
+// Whether the diagonal-frame kernels beat the gate-by-gate ones. They do but for complex128 vectors of a few amplitudes,
+// where one thread's chain of 64-bit fixed-point steps is longer than a float64 rotation on a vector whose amplitudes
+// have a thread each: a step of the program costs about 1.6 parameters' rotations there, or, beyond as many fixed
+// gates as parameters, four fixed gates. Measured below 8 qubits (single instances, metric, frames / gate by gate in us):
+// 1 qubit, 40 rotations in 40 steps 164 / 104; 2 qubits, 400 in 400, 1343 / 782, 40 in 20, 97 / 109; 4 qubits, 240 in 210,
+// 569 / 513, 240 in 120, 390 / 458; general circuits of 3 and 6 qubits, 120 in 99 and 150 in 149, 394 / 350 and 465 /
+// 423; of 8 qubits 625 / 745. Batches (with 8 qubits too): 16 general instances of 3 to 7, 257 / 201.
+bool frames_faster(const qng_ctx *c) {
+    if (c->precision != QNG_C128) return true;
+    int64_t steps = 0, gates = 0;
+    for (int b = 0; b < c->count; ++b) {
+        const HostInst &h = c->inst[b];
+        if (h.n > (c->count == 1 ? 7 : 8)) return true;
+        steps += c->f.inst[b].fwd_cnt;
+        gates += 5 * h.P + 2 * std::max<int64_t>(0, (int64_t)h.gates.size() - 2 * h.P);
+    }
+    return gates >= 8 * steps;
+}
+
 // The default shapes of every qubit count of the context (no qng_set_tuning, qng_set_shape,
 // qng_set_forward_cluster and no shape kept by the autotuner).
 bool default_shapes(const qng_ctx *c) {
@@ -851,7 +870,7 @@ qng_status plan_as(qng_ctx *c) {
     // gate-by-gate kernels. The workspace has room for either.
     c->f = {};
     const bool frames_fit = !c->compact && plan_frames(c);
-    c->frames = frames_fit && default_shapes(c);
+    c->frames = frames_fit && default_shapes(c) && frames_faster(c);
 
     // workspace layout
     size_t off = 0;
