@@ -312,7 +312,7 @@ qng_status qng_last_launch_count(const qng_ctx *ctx, int64_t *launches);
  * leaves idle. The calling stream forks into these streams and joins them before the solve (graph
  * capture included). Results are bit-identical to the unchunked sweep.
  * The diagonal-frame kernels ignore the chunk count; batches on them run each launch class (one per
- * cluster size) on a stream of its own, whatever the setting.
+ * cluster and CTA size) on a stream of its own, and one after another with qng_set_pipeline(ctx, 1).
  * Batched contexts on gate-by-gate shapes can run each launch group's sweep and columns on a stream of
  * its own, most work first, so that the groups fill one another's tails (joined before the solve,
  * graph capture included). For those qng_set_pipeline(ctx, 0) does this for complex128 and runs

@@ -1397,8 +1397,11 @@ qng_status run_streaming(qng_ctx *c, int jobs, int64_t &launches) {
     return QNG_OK;
 }
 
-// The diagonal-frame launches up to the columns. A batch of several launch classes runs each class's
-// sweep and columns on a stream of its own, joined on the context's stream.
+// A batch of several launch classes runs each class's sweep and columns on a stream of its own, joined on the
+// context's stream, unless qng_set_pipeline(ctx, 1) asks for one after another.
+bool classes_apart(const qng_ctx *c) { return c->f.cls.size() > 1 && c->pipe_ready && c->pipe_req != 1; }
+
+// The diagonal-frame launches up to the columns.
 qng_status run_frames(qng_ctx *c, int jobs, const double *theta, int64_t &launches) {
     frames::FWork w = c->fwork(theta);
     const auto &f = c->f;
@@ -1408,7 +1411,7 @@ qng_status run_frames(qng_ctx *c, int jobs, const double *theta, int64_t &launch
     cudaError_t e = timed(c, 0, [&] { return frames::launch_tables(w, (int)f.tab.size(), c->fkb, c->precision, c->stream); });
     if (e != cudaSuccess) return cuda_status(e);
     launches += f.tab.empty() ? 0 : 1;
-    const bool side = f.cls.size() > 1 && c->pipe_ready;
+    const bool side = classes_apart(c);
     w.chain = !side;  // classes side by side: a waiting kernel would take another class's room
     if (side && (e = cudaEventRecord(c->pipe_ev0, c->stream)) != cudaSuccess) return cuda_status(e);
     for (size_t k = 0; k < f.cls.size(); ++k) {
@@ -1552,7 +1555,7 @@ qng_status run(qng_ctx *c, int jobs, const LaunchArgs &args) {
     }
     LaunchArgs a = args;
     a.jobs = jobs;
-    a.chain = (frames && !(c->f.cls.size() > 1 && c->pipe_ready)) || sframes;
+    a.chain = (frames && !classes_apart(c)) || sframes;
     if (need_cols && !S && !side_by_side) {
         for (const Group &g : c->groups) {
             if ((wm && wg ? g.num_work : (wm ? g.num_met : g.num_grad)) == 0) continue;

@@ -177,3 +177,26 @@ def test_sweep_on_sixteen_ctas(qng, oracle, fwd_threads):
     assert ctx.forward_cluster(12) == 4
     batch = qng.Context(W.config_batch(count=4))
     assert all(batch.forward_cluster(n) == batch.get_tuning(n)[0] for n in range(6, 15))
+
+
+@pytest.mark.parametrize("precision", [W.C64, W.C128])
+def test_batch_classes_in_turn(qng, precision):
+    """A batch of three launch classes: side by side (the default) and one after another give the same bits, and
+    so does a captured step."""
+    probs = [W.Problem("b", c, W.random_pauli_hamiltonian(c.n, 5, np.random.Generator(np.random.PCG64(k))),
+                       W.uniform_theta(c.num_params, np.random.Generator(np.random.PCG64(90 + k))), precision=precision)
+             for k, c in enumerate(W.layered_ansatz(n, 2) for n in (4, 6, 8, 9, 10, 11, 12, 13, 14, 5))]
+    with torch.cuda.stream(torch.cuda.Stream()):
+        ctx = qng.Context(probs)
+        out = []
+        for chunks in (0, 1, 2):
+            ctx.set_pipeline(chunks)
+            out.append({k: v.clone() for k, v in ctx.step(ctx.theta0()).items()})
+        ctx.set_pipeline(1)
+        cap = ctx.graph_capture(ctx.theta0())
+        ctx.graph_launch()
+        ctx.sync()
+        out.append(cap)
+        for o in out[1:]:
+            for k in o:
+                assert torch.equal(o[k], out[0][k]), k
