@@ -3,7 +3,8 @@ each chunk makes ready on streams of their own) against the unchunked sweep and 
 
 Column j of Algorithm 1's recurrence reads only the checkpoints psi_0..psi_j, and a chunk that
 restarts from checkpoint K carries that checkpoint exactly as the uninterrupted sweep carried it
-(renormalisation by 2^200 is exact), so every output is bit-identical to the unchunked sweep.
+(renormalisation by 2^200 is exact), so every output is bit-identical to the unchunked sweep. It is
+the gate-by-gate kernels' sweep: contexts take them through the least workspace or an explicit shape.
 """
 import numpy as np
 import pytest
@@ -14,6 +15,7 @@ from paper_2011_02991_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 TOL = {W.C128: 1e-10, W.C64: 2e-4}
+LEAST = 1  # a workspace limit that leaves the gate-by-gate kernels
 
 
 def rel(got, ref):
@@ -49,7 +51,7 @@ def test_chunk_counts_bit_identical(qng, oracle, precision):
     """12 qubits, P = 192: 2..8 chunks (boundaries every P/S parameters, P/S not whole for 5 and 7)
     give the unchunked step's outputs bit for bit, and the step matches the oracle."""
     p = W.config_rand12(precision=precision)
-    ctx = qng.Context(p, precision=precision)
+    ctx = qng.Context(p, precision=precision, workspace_limit=LEAST)
     th = ctx.theta0()
     ctx.set_pipeline(0)
     assert ctx.pipeline() == 0  # automatic: plain rotations run unchunked
@@ -80,7 +82,7 @@ def test_chunks_cut_z_runs_and_renormalisations(qng, chunks):
 def test_generalised_rotations_pipelined(qng, oracle):
     """Controlled and Pauli-string rotations (their own kernel instantiations) through 4 chunks."""
     p = W.general_problem(8, 150, 11, W.C128)
-    ctx = qng.Context(p, precision=W.C128)
+    ctx = qng.Context(p, precision=W.C128, workspace_limit=LEAST)
     th = ctx.theta0()
     ref = _step(ctx, 1, th)
     out = _step(ctx, 4, th)
@@ -93,7 +95,7 @@ def test_generalised_rotations_pipelined(qng, oracle):
 def test_metric_only_and_complex_metric_pipelined(qng):
     """qng_metric (no gradient column) and qng_metric_complex take the pipelined sweep too."""
     p = W.config_rand12()
-    ctx = qng.Context(p)
+    ctx = qng.Context(p, workspace_limit=LEAST)
     th = ctx.theta0()
     res = {}
     for chunks in (1, 4):
@@ -113,7 +115,7 @@ def test_graph_capture_and_descent_pipelined(qng):
     p = W.vqe_tfim(10, 8, seed=3)
     stream = torch.cuda.Stream()
     with torch.cuda.stream(stream):
-        ctx = qng.Context(p, stream=stream)
+        ctx = qng.Context(p, stream=stream, workspace_limit=LEAST)
         th = ctx.theta0()
         ref = _step(ctx, 4, th)
         out = ctx.graph_capture(th, 0.1, 1e-3)
@@ -200,3 +202,29 @@ def test_batch_classes_in_turn(qng, precision):
         for o in out[1:]:
             for k in o:
                 assert torch.equal(o[k], out[0][k]), k
+
+
+@pytest.mark.parametrize("precision", [W.C64, W.C128])
+def test_gate_by_gate_batch(qng, oracle, precision):
+    """An explicit CTA size takes the gate-by-gate kernels: persistent columns of several launch groups, in turn and
+    side by side, against the oracle and with the same bits either way."""
+    probs = W.config_batch(count=12, precision=precision)
+    ctx = qng.Context(probs)
+    before = ctx.step(ctx.theta0())
+    ctx.sync()
+    ctx.set_tuning(0, -1, 128)
+    ctx._alloc_workspace()
+    out = []
+    for chunks in (1, 2):
+        ctx.set_pipeline(chunks)
+        out.append({k: v.clone() for k, v in ctx.step(ctx.theta0()).items()})
+    ctx.sync()
+    tol = 1e-10 if precision == W.C128 else 2e-4
+    for k in out[0]:
+        assert torch.equal(out[0][k], out[1][k]), k
+    assert not torch.equal(out[0]["g"], before["g"])  # other kernels: other roundings
+    for p, g, gr, e in zip(probs, ctx.split_metric(out[0]["g"]), ctx.split_params(out[0]["grad"]), out[0]["energy"].cpu().numpy()):
+        ref = oracle.qng_step(p)
+        assert np.abs(g.cpu().numpy() - ref["g"]).max() <= tol * np.abs(ref["g"]).max()
+        assert np.abs(gr.cpu().numpy() - ref["grad"]).max() <= tol * np.abs(p.hamiltonian.coeffs).sum()
+        assert abs(e - ref["E"]) <= tol * np.abs(p.hamiltonian.coeffs).sum()

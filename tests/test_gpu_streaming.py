@@ -1,8 +1,8 @@
 """GPU parity of the streaming path (state vectors in HBM, tiled passes) against the CPU oracle.
 
 Small and medium instances are forced onto the streaming path and checked entry by entry; tiles of
-2^11 (complex128) or 2^12 (complex64) amplitudes make instances of 13-16 qubits span many tiles and
-many passes per column, with window qubits changing from pass to pass.
+2^11 amplitudes make instances of 13-16 qubits span many tiles and many passes per column, with window
+qubits changing from pass to pass. With the least workspace the same instances run on four registers.
 """
 import numpy as np
 import pytest
@@ -57,8 +57,8 @@ def test_streaming_small_configs(qng, oracle, precision):
 @pytest.mark.parametrize("precision", [W.C128, W.C64])
 @pytest.mark.parametrize("n,seed", [(6, 1), (9, 2), (12, 5), (13, 3), (15, 4), (17, 6)])
 def test_streaming_random_circuits(qng, oracle, n, seed, precision):
-    """Every gate kind, on instances that span 1 to 64 tiles (complex64 from 12 qubits on runs the
-    register-phase kernel: one tile at 12 qubits, 32 tiles over 152 CTAs at 17)."""
+    """Every gate kind: checkpoints of runs over 2 to 64 tiles from 13 (complex64) or 12 (complex128) qubits on, the
+    register form on one tile below."""
     p = W.random_problem(n, 50 + 4 * n, 10, 3000 + seed, precision)
     run_streaming(qng, oracle, p, precision)
 
@@ -79,10 +79,10 @@ def test_streaming_layered_14(qng, oracle, precision):
 
 @pytest.mark.parametrize("n,seed", [(12, 21), (14, 22)])
 def test_streaming_c64_diagonal_runs(qng, oracle, n, seed):
-    """Runs of 1-24 RZ steps with CZ / Z gates between them, some broken by a CNOT or H, at complex64
-    from 12 qubits: the register-phase kernel takes each run's inner products on its starting
-    registers and applies the run's rotations and signs as one composed factor per amplitude. Real
-    step and complex metric (Re and Im per step) against the oracle."""
+    """Runs of 1-24 RZ steps with CZ / Z gates between them, some broken by a CNOT or H, at complex64:
+    at 12 qubits the register-phase kernel takes each run's inner products on its starting registers and
+    applies the run's rotations and signs as one composed factor per amplitude, at 14 they are diagonal-frame
+    runs of many parameters. Real step and complex metric (Re and Im per step) against the oracle."""
     p = W.z_run_problem(n, 160, seed, W.C64)
     run_streaming(qng, oracle, p, W.C64)
     ctx = qng.Context(p, precision=W.C64, path=2)
@@ -113,8 +113,8 @@ def test_streaming_matches_onchip(qng):
 
 @pytest.mark.parametrize("seed", [11, 12])
 def test_streaming_c64_matches_onchip_c64(qng, seed):
-    """Complex64 at 12-14 qubits: the register-phase streaming kernel against the on-chip path, both
-    at complex64, on g, grad and <E> (within the complex64 tolerance of each other)."""
+    """Complex64 at 12-14 qubits: the streaming path (at 12 its register-phase kernel) against the on-chip
+    path, both at complex64, on g, grad and <E> (within the complex64 tolerance of each other)."""
     n = 12 + seed % 3
     p = W.random_problem(n, 140, 16, 4100 + seed, W.C64)
     a = qng.Context(p, path=1)
