@@ -192,10 +192,11 @@ qng_status qng_energy_backward(qng_ctx *ctx, const double *theta, const double *
 /* One natural-gradient step (Eq. 3 with a Tikhonov term): dtheta (device, sum P_b) solves
  * (g + lambda I) dtheta = -dt grad<E>, to float64 accuracy for both precisions. g and grad<E> are
  * computed first as in qng_metric and qng_gradient. The solve that runs depends on P (see
- * qng_solve_report): by default, for P from 48 to about 222 (where its factor fits
- * the shared memory of one cluster), a float32 Cholesky factorisation refined in
+ * qng_solve_report): by default, for P from 48 to about 222 (in batches to about 290: where its factor
+ * fits the shared memory of one cluster), a float32 Cholesky factorisation refined in
  * float64 (residuals of the float64 matrix), with a hand-over to a float64 Cholesky when the
- * refinement does not reach float64 accuracy; otherwise a float64 Cholesky factorisation, one
+ * refinement does not reach float64 accuracy; below 48 a float64 factorisation in one CTA's shared
+ * memory; otherwise a float64 Cholesky factorisation, one
  * cluster per instance when the rows fit in its shared memory (P up to about 330), else, for a
  * single instance, one launch per 16-column block with the factor in global memory, else one CTA
  * per instance. g_opt, grad_opt, energy_opt (device, may be NULL) also receive the metric, the
@@ -267,8 +268,9 @@ qng_status qng_set_tuning(qng_ctx *ctx, int min_qubits, int cluster_log2, int th
 /* Execution path: 0 automatic (on-chip for n <= 16 qubits, streaming above), 1 on-chip (every
  * state of an instance in the shared memory of one thread-block cluster, O(P) checkpoints in HBM),
  * 2 streaming (single instance only, states in HBM, tiled passes). By default the streaming path
- * keeps one checkpoint per run of commuting rotations (about P / n of them) plus as many column
- * slots as fill 32 MiB (at least 4), vectors of 2^n amplitudes, and every pass takes one run for
+ * keeps one checkpoint per run of commuting gates (a layer's rotations of one axis, and one more run a layer
+ * where the entangler needs signs or phases of its own) and column slots (2 to 32 of them up to 20 qubits,
+ * as many as fill 32 MiB; 4 beyond), vectors of 2^n amplitudes, and every pass takes one run for
  * several columns. Vectors beyond 4 GiB, instances whose checkpoints and slots would pass 96 GiB,
  * and n < 13 (complex64) or n < 12 (complex128) run on four registers instead: psi, a and b of
  * Algorithm 1 and a second b, the metric columns walking in pairs that share a; so do contexts whose

@@ -1262,7 +1262,6 @@ qng_status run_sframes(qng_ctx *c, int jobs, const double *theta, int64_t &launc
     w.n = h.n;
     w.P = h.P;
     w.R = (int32_t)p.runs.size();
-    w.kb = p.kb;
     w.tb = p.tb;
     w.low = p.low;
     w.hl = p.hl;
@@ -1301,7 +1300,7 @@ qng_status run_sframes(qng_ctx *c, int jobs, const double *theta, int64_t &launc
         w.chain = true;
     }
     e = timed(c, 7, [&] {
-        return frames::launch_stream_finish(w, (metric ? 1 : 0) | (grad ? 2 : 0) | (im ? 4 : 0), c->precision, c->stream);
+        return frames::launch_stream_finish(w, (metric ? 1 : 0) | (grad ? 2 : 0) | (im ? 4 : 0), c->stream);
     });
     if (e != cudaSuccess) return cuda_status(e);
     ++launches;

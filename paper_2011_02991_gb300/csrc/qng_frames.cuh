@@ -67,9 +67,10 @@ template <int CONJ> __device__ __forceinline__ float2 mul(float2 x, float2 d, ui
     return float2{fmaf(x.x, d.x, -x.y * s), fmaf(x.x, s, x.y * d.x)};
 }
 
-// Re (IM = 0) or Im (IM = 1) of conj(a) b for fixed-point vectors of unit 2^-(60 - UP), as a multiple of 2^-60 (v)
-// and what is left below it (f, kFracBits bits, never negative). Inner products are between vectors of norm 1 at
-// most, so sums stay within 1 in magnitude.
+// Re (IM = 0) or Im (IM = 1) of conj(a) b for fixed-point vectors of unit 2^-u, as a multiple v of
+// 2^-(2u - 60 + 2 UP) (2^-62 for both paths) and what is left below it (f, kFracBits bits, never negative). Inner
+// products are between vectors of norm 1 at most, so sums stay within 1 in magnitude. lo lo counts: at 2^12 amplitudes
+// and more a product is 2^-12 and less.
 struct Part {
     ll v;
     int f;
@@ -111,7 +112,8 @@ template <int IM, int UP> __device__ __forceinline__ ll prod(int4 a, longlong2 b
 }
 template <int IM, int UP> __device__ __forceinline__ float prod(float2 a, float2 b, uint32_t) { return prod_part<IM, UP>(a, b); }
 
-// Pseudo-random bits over the amplitudes: a thread's (hash of its index), xor a constant per amplitude.
+// Pseudo-random bits over the amplitudes: a thread's (hash of its index), xor a constant per amplitude. The hash is
+// the 32-bit mixer that Chris Wellons published as lowbias32 (public domain).
 __device__ __forceinline__ uint32_t hash(uint32_t x) {
     x = (x ^ (x >> 16)) * 0x7feb352du;
     x = (x ^ (x >> 15)) * 0x846ca68bu;

@@ -259,14 +259,14 @@ struct SWork {
     uint32_t *mask;           // 2^(n-hl) per run
     void *a;                  // checkpoints, natural order, 2^n per run
     void *b;                  // column slots, 2^n each
-    long long *acc;           // (P x P) sums of the metric, twice that with Im, in units of 2^-60
-    long long *sacc, *gacc;   // <sigma_j>; the gradient, units of 2^(etaexp - 60)
+    long long *acc;           // (P x P) sums of the metric, twice that with Im, in units of 2^-62
+    long long *sacc, *gacc;   // <sigma_j>, units of 2^-62; the gradient, units of 2^(etaexp - 62)
     unsigned long long *eacc; // as in FWork
     int32_t *etaexp;
     const double *theta;
     int32_t *status, *bad;
     double *pctrl, *sigma, *L, *Lim, *gradraw, *energy;
-    int32_t n, P, R, kb, tb, low, hl, nterms, eexp, hblocks;
+    int32_t n, P, R, tb, low, hl, nterms, eexp, hblocks;
 };
 
 cudaError_t prepare_stream(int precision, int tb);
@@ -278,7 +278,7 @@ cudaError_t launch_stream_walk(const SWork &w, const SPass &p, int pass, int col
 // H psi: slot `in` -> slot `out`, and <E>.
 cudaError_t launch_stream_hpsi(const SWork &w, int in, int out, int precision, cudaStream_t st);
 // Sums to float64: what = 1 metric, 2 gradient (bits), 4 with Im.
-cudaError_t launch_stream_finish(const SWork &w, int what, int precision, cudaStream_t st);
+cudaError_t launch_stream_finish(const SWork &w, int what, cudaStream_t st);
 
 }  // namespace frames
 }  // namespace qng

@@ -36,11 +36,6 @@ SP conj_sdg(SP a) { return a.p == PX ? SP{PY, -a.s} : (a.p == PY ? SP{PX, a.s} :
 struct Lin {
     uint32_t img[kMaxQubits];
     Lin() { for (int b = 0; b < kMaxQubits; ++b) img[b] = 1u << b; }
-    uint32_t operator()(uint32_t m) const {
-        uint32_t r = 0;
-        for (int b = 0; b < kMaxQubits; ++b) if ((m >> b) & 1) r ^= img[b];
-        return r;
-    }
     // mask z' with parity(m & z') = parity(A m & z)
     uint32_t pull(uint32_t z) const {
         uint32_t r = 0;

@@ -698,8 +698,7 @@ cudaError_t launch_stream_hpsi(const SWork &w, int in, int out, int precision, c
     return launch_next(w.chain, precision == QNG_C128 ? k_sheff<Fix> : k_sheff<Flt>, w.hblocks, 256, 0, 1, st, w, in, out);
 }
 
-cudaError_t launch_stream_finish(const SWork &w, int what, int precision, cudaStream_t st) {
-    (void)precision;
+cudaError_t launch_stream_finish(const SWork &w, int what, cudaStream_t st) {
     if (w.P == 0) return cudaSuccess;
     const size_t n = (what & 1) ? (size_t)w.P * w.P : (size_t)w.P;
     return launch_next(w.chain, k_sfinish, (unsigned)((n + 255) / 256), 256, 0, 1, st, w, what);
