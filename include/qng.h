@@ -144,10 +144,10 @@ qng_status qng_get_offsets(const qng_ctx *ctx, int64_t *param_offset, int64_t *m
 /* Bytes of device workspace the context runs fastest with (a multiple of 256). */
 qng_status qng_workspace_size(const qng_ctx *ctx, size_t *bytes);
 
-/* The least workspace qng_set_workspace takes (a multiple of 256, at most qng_workspace_size). With less than
- * qng_workspace_size the gate-by-gate kernels run, which keep no checkpoint per run: four vectors of
- * 2^n amplitudes for a streaming instance (Algorithm 1's O(1) registers), however long its circuit; the
- * results differ by rounding. */
+/* The least workspace qng_set_workspace takes (a multiple of 256, at most qng_workspace_size): four vectors of
+ * 2^n amplitudes for a streaming instance (Algorithm 1's O(1) registers), however long its circuit, and
+ * one per parameter on chip, beside the tables. Where that does not hold one checkpoint per run, the
+ * gate-by-gate kernels run with less than qng_workspace_size; results differ by rounding. */
 qng_status qng_workspace_min(const qng_ctx *ctx, size_t *bytes);
 
 /* Hand the context a device workspace (256-byte aligned, >= qng_workspace_min bytes, owned by

@@ -119,7 +119,7 @@ struct qng_ctx {
     size_t o_io_theta = 0, o_io_dtheta = 0, o_io_g = 0, o_io_grad = 0, o_io_energy = 0;
     size_t ws_bytes = 0;      // bytes the current plan needs
     size_t ws_want = 0;       // bytes that the plan without a workspace limit needs
-    bool compact = false;     // planned without checkpoints of runs: the workspace is smaller than ws_want
+    bool compact = false;     // planned with no more than the gate-by-gate kernels take: the workspace is below ws_want
     size_t ws_cap = 0;        // bytes of the workspace the caller set
     unsigned char *ws = nullptr;
     cudaStream_t stream = nullptr;
@@ -869,7 +869,7 @@ qng_status plan_as(qng_ctx *c) {
     // The diagonal-frame kernels run at the default shapes; qng_set_shape and the like choose the
     // gate-by-gate kernels. The workspace has room for either.
     c->f = {};
-    const bool frames_fit = !c->compact && plan_frames(c);
+    const bool frames_fit = plan_frames(c);
     c->frames = frames_fit && default_shapes(c) && frames_faster(c);
 
     // workspace layout
@@ -927,7 +927,8 @@ qng_status plan_as(qng_ctx *c) {
         c->of_d = take(ab * (size_t)f.amps_ad);
         c->of_v = take(ab * (size_t)f.amps_v);
         c->of_eta = take(ab * (size_t)f.amps_v);
-        off = std::max(off, end);
+        if (c->compact && off > end) c->frames = false;  // no more room than the gate-by-gate kernels take
+        off = c->compact ? end : std::max(off, end);
     }
     c->ws_bytes = align256(off);
     c->prepared = false;
@@ -942,8 +943,9 @@ int solve_cluster_log2(int max_P) {
     return -1;
 }
 
-// The plan, and, where a workspace is set that its checkpoints of runs do not fit, the plan of the gate-by-gate
-// kernels: four registers of a streaming instance, one checkpoint per parameter on chip.
+// The plan, and, where a workspace is set that its checkpoints of runs do not fit, one that takes what the
+// gate-by-gate kernels do: four registers of a streaming instance, one checkpoint per parameter on chip (which holds
+// most circuits' runs and factor tables as well).
 qng_status plan(qng_ctx *c) {
     c->compact = false;
     qng_status s = plan_as(c);
@@ -1688,7 +1690,7 @@ qng_status qng_workspace_min(const qng_ctx *c, size_t *bytes) {
     if (!c || !bytes) return QNG_ERR_ARG;
     *bytes = c->ws_bytes;
     if (c->compact) return QNG_OK;
-    qng_ctx t;  // the settings alone, planned without checkpoints of runs
+    qng_ctx t;  // the settings alone, planned for the least
     t.precision = c->precision;
     t.count = c->count;
     t.inst = c->inst;

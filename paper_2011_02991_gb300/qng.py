@@ -165,7 +165,7 @@ class Context:
     are concatenated over instances; metrics are concatenated P_b x P_b blocks.
 
     The workspace is what the context runs fastest with; where the device has no room for that, or it is more
-    than ``workspace_limit`` bytes, the least one (qng_workspace_min), on which the gate-by-gate kernels run.
+    than ``workspace_limit`` bytes, the least one (qng_workspace_min).
     """
 
     def __init__(self, problems, precision: int | None = None, device=None, stream: torch.cuda.Stream | None = None,

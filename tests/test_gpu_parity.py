@@ -319,12 +319,15 @@ def test_z_runs_complex_metric_and_gradient_c64(qng, oracle):
     assert rel(gr.cpu(), ref["grad"]) <= TOL[W.C64]
 
 
-def check_complex(qng, oracle, probs, precision, shape=None, limit=None):
+def check_complex(qng, oracle, probs, precision, shape=None, explicit=False):
     """qng_metric_complex against the oracle's G (Eq. 4), Re and Im, every instance."""
     probs = probs if isinstance(probs, list) else [probs]
-    ctx = qng.Context(probs if len(probs) > 1 else probs[0], precision=precision, workspace_limit=limit)
+    ctx = qng.Context(probs if len(probs) > 1 else probs[0], precision=precision)
     if shape is not None:
         ctx.set_shape(*shape)
+    if explicit:  # the default shapes, set: the gate-by-gate kernels
+        for n in {p.n for p in probs}:
+            ctx.set_shape(n, *ctx.get_tuning(n))
     G, sg = ctx.metric_complex(ctx.theta0(), want_sigma=True)
     ctx.sync()
     Gs = ctx.split_metric(G) if len(probs) > 1 else [G.reshape(probs[0].P, probs[0].P)]
@@ -366,13 +369,13 @@ def test_metric_complex_renormalisation(qng, oracle):
     check_complex(qng, oracle, W.z_run_problem(7, 600, 6, W.C128, near_half_pi=True), W.C128, shape=(7, 0, 64, 64))
 
 
-@pytest.mark.parametrize("limit", [None, 1])
+@pytest.mark.parametrize("explicit", [False, True])
 @pytest.mark.parametrize("precision", [W.C64, W.C128])
-def test_metric_complex_batch(qng, oracle, precision, limit):
-    """A batch with several launch shapes: the diagonal-frame classes, and (least workspace) the gate-by-gate groups
+def test_metric_complex_batch(qng, oracle, precision, explicit):
+    """A batch with several launch shapes: the diagonal-frame classes, and (explicit shapes) the gate-by-gate groups
     through the persistent column launch."""
     probs = [p for p in W.config_batch(count=12, precision=precision)]
-    ctx = check_complex(qng, oracle, probs, precision, limit=limit)
+    ctx = check_complex(qng, oracle, probs, precision, explicit=explicit)
     # the real part is qng_metric's metric up to the grouping of the warp sums (4 steps per
     # reduction instead of 8), i.e. float32 rounding for complex64
     g = ctx.metric(ctx.theta0())
@@ -540,14 +543,17 @@ def test_generalised_rotations_larger(qng, oracle):
     check_problem(qng, oracle, p, W.C128)
 
 
-@pytest.mark.parametrize("limit", [None, 1])
+@pytest.mark.parametrize("explicit", [False, True])
 @pytest.mark.parametrize("precision", [W.C64, W.C128])
-def test_generalised_batch(qng, oracle, precision, limit):
-    """A batch mixing generalised and ordinary instances of 5..9 qubits: diagonal frames, and (least workspace) the
+def test_generalised_batch(qng, oracle, precision, explicit):
+    """A batch mixing generalised and ordinary instances of 5..9 qubits: diagonal frames, and (explicit shapes) the
     gate-by-gate kernels' persistent column launch."""
     probs = [W.general_problem(5 + b % 5, 20 + 4 * b, 800 + b, precision) if b % 2 == 0 else
              W.random_problem(5 + b % 5, 40 + 4 * b, 8, 820 + b, precision) for b in range(8)]
-    ctx = qng.Context(probs, precision=precision, workspace_limit=limit)
+    ctx = qng.Context(probs, precision=precision)
+    if explicit:
+        for n in {p.n for p in probs}:
+            ctx.set_shape(n, *ctx.get_tuning(n))
     out = ctx.step(ctx.theta0(), 0.1, 1e-3)
     ctx.sync()
     gs, grads = ctx.split_metric(out["g"]), ctx.split_params(out["grad"])

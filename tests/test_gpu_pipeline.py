@@ -4,7 +4,7 @@ each chunk makes ready on streams of their own) against the unchunked sweep and 
 Column j of Algorithm 1's recurrence reads only the checkpoints psi_0..psi_j, and a chunk that
 restarts from checkpoint K carries that checkpoint exactly as the uninterrupted sweep carried it
 (renormalisation by 2^200 is exact), so every output is bit-identical to the unchunked sweep. It is
-the gate-by-gate kernels' sweep: contexts take them through the least workspace or an explicit shape.
+the gate-by-gate kernels' sweep: contexts take them through an explicit shape.
 """
 import numpy as np
 import pytest
@@ -15,7 +15,13 @@ from paper_2011_02991_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 TOL = {W.C128: 1e-10, W.C64: 2e-4}
-LEAST = 1  # a workspace limit that leaves the gate-by-gate kernels
+
+
+def gate_by_gate(ctx):
+    """The default launch shapes, set explicitly: what chooses the gate-by-gate kernels."""
+    for n in {p.n for p in ctx.problems}:
+        ctx.set_shape(n, *ctx.get_tuning(n))
+    return ctx
 
 
 def rel(got, ref):
@@ -51,7 +57,7 @@ def test_chunk_counts_bit_identical(qng, oracle, precision):
     """12 qubits, P = 192: 2..8 chunks (boundaries every P/S parameters, P/S not whole for 5 and 7)
     give the unchunked step's outputs bit for bit, and the step matches the oracle."""
     p = W.config_rand12(precision=precision)
-    ctx = qng.Context(p, precision=precision, workspace_limit=LEAST)
+    ctx = gate_by_gate(qng.Context(p, precision=precision))
     th = ctx.theta0()
     ctx.set_pipeline(0)
     assert ctx.pipeline() == 0  # automatic: plain rotations run unchunked
@@ -82,7 +88,7 @@ def test_chunks_cut_z_runs_and_renormalisations(qng, chunks):
 def test_generalised_rotations_pipelined(qng, oracle):
     """Controlled and Pauli-string rotations (their own kernel instantiations) through 4 chunks."""
     p = W.general_problem(8, 150, 11, W.C128)
-    ctx = qng.Context(p, precision=W.C128, workspace_limit=LEAST)
+    ctx = gate_by_gate(qng.Context(p, precision=W.C128))
     th = ctx.theta0()
     ref = _step(ctx, 1, th)
     out = _step(ctx, 4, th)
@@ -95,7 +101,7 @@ def test_generalised_rotations_pipelined(qng, oracle):
 def test_metric_only_and_complex_metric_pipelined(qng):
     """qng_metric (no gradient column) and qng_metric_complex take the pipelined sweep too."""
     p = W.config_rand12()
-    ctx = qng.Context(p, workspace_limit=LEAST)
+    ctx = gate_by_gate(qng.Context(p))
     th = ctx.theta0()
     res = {}
     for chunks in (1, 4):
@@ -115,7 +121,7 @@ def test_graph_capture_and_descent_pipelined(qng):
     p = W.vqe_tfim(10, 8, seed=3)
     stream = torch.cuda.Stream()
     with torch.cuda.stream(stream):
-        ctx = qng.Context(p, stream=stream, workspace_limit=LEAST)
+        ctx = gate_by_gate(qng.Context(p, stream=stream))
         th = ctx.theta0()
         ref = _step(ctx, 4, th)
         out = ctx.graph_capture(th, 0.1, 1e-3)
@@ -206,14 +212,13 @@ def test_batch_classes_in_turn(qng, precision):
 
 @pytest.mark.parametrize("precision", [W.C64, W.C128])
 def test_gate_by_gate_batch(qng, oracle, precision):
-    """An explicit CTA size takes the gate-by-gate kernels: persistent columns of several launch groups, in turn and
+    """Explicit shapes take the gate-by-gate kernels: persistent columns of several launch groups, in turn and
     side by side, against the oracle and with the same bits either way."""
     probs = W.config_batch(count=12, precision=precision)
     ctx = qng.Context(probs)
     before = ctx.step(ctx.theta0())
     ctx.sync()
-    ctx.set_tuning(0, -1, 128)
-    ctx._alloc_workspace()
+    gate_by_gate(ctx)
     out = []
     for chunks in (1, 2):
         ctx.set_pipeline(chunks)

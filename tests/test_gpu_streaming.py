@@ -295,3 +295,29 @@ def test_workspace_limit(qng, n, precision):
         g = least.metric(least.theta0())
         least.sync()
         assert rel(g.cpu(), out[0][0].cpu()) <= 1e-11
+
+
+@pytest.mark.parametrize("precision", [W.C64, W.C128])
+def test_workspace_limit_on_chip(qng, oracle, precision):
+    """Many runs and few parameters: checkpoints of runs need more than those of parameters, and the least
+    workspace leaves the gate-by-gate kernels."""
+    n = 10
+    rows = [[W.RY, 0, -1, 0], [W.RX, 1, -1, 1]]
+    for k in range(80):
+        rows += [[W.H, 0, -1, -1], [W.CZ, 0, 1 + k % (n - 1), -1]]
+    rows += [[W.RY, 0, -1, 2], [W.RZ, 3, -1, 3]]
+    rng = np.random.Generator(np.random.PCG64(10))
+    p = W.Problem("few", W.Circuit(n, np.array(rows, dtype=np.int32)), W.random_pauli_hamiltonian(n, 8, rng),
+                  W.uniform_theta(4, rng), precision=precision)
+    ref = oracle.qng_step(p)
+    out, sizes = [], []
+    for limit in (None, LEAST):
+        ctx = qng.Context(p, workspace_limit=limit)
+        g = ctx.metric(ctx.theta0())
+        gr, en = ctx.gradient(ctx.theta0())
+        ctx.sync()
+        sizes.append(ctx.workspace.numel())
+        assert np.abs(g.cpu().numpy().reshape(4, 4) - ref["g"]).max() <= TOL[precision] / 4
+        assert np.abs(gr.cpu().numpy() - ref["grad"]).max() <= TOL[precision] * np.abs(p.hamiltonian.coeffs).sum()
+        assert abs(float(en[0]) - ref["E"]) <= TOL[precision] * np.abs(p.hamiltonian.coeffs).sum()
+    assert sizes[1] < sizes[0]
