@@ -67,6 +67,25 @@ template <int CONJ> __device__ __forceinline__ float2 mul(float2 x, float2 d, ui
     return float2{fmaf(x.x, d.x, -x.y * s), fmaf(x.x, s, x.y * d.x)};
 }
 
+// A sum over threads of float32 partial sums, as the float32 nearest to it and what is left: 48 bits on the float32
+// pipe, which takes 64 times what the float64 pipe does.
+struct Two {
+    float s, e;
+    __device__ __forceinline__ explicit operator double() const { return (double)s + (double)e; }
+};
+__device__ __forceinline__ Two exact_sum(float a, float b) {  // s + e = a + b
+    const float s = a + b, t = s - a;
+    return Two{s, (a - (s - t)) + (b - t)};
+}
+__device__ __forceinline__ Two exact_product(float a, float b) {
+    const float p = a * b;
+    return Two{p, fmaf(a, b, -p)};
+}
+__device__ __forceinline__ Two operator+(Two a, Two b) {
+    const Two r = exact_sum(a.s, b.s);
+    return Two{r.s, r.e + (a.e + b.e)};
+}
+
 // Re (IM = 0) or Im (IM = 1) of conj(a) b for fixed-point vectors of unit 2^-u, as a multiple v of
 // 2^-(2u - 60 + 2 UP) (2^-62 for both paths) and what is left below it (f, kFracBits bits, never negative). Inner
 // products are between vectors of norm 1 at most, so sums stay within 1 in magnitude. lo lo counts: at 2^12 amplitudes
@@ -100,12 +119,14 @@ __device__ __forceinline__ void add(Part &s, Part p, bool neg) {
     s.f += neg ? -p.f : p.f;
 }
 __device__ __forceinline__ void add(float &s, float p, bool neg) { s += neg ? -p : p; }
-// A thread's sum rounded by rnd, uniform below one unit.
-template <int UP> __device__ __forceinline__ ll rounded(Part s, uint32_t rnd) {
-    constexpr int F = kFracBits<UP>;
-    return s.v + ((s.f + (int)(rnd >> (32 - F))) >> F);
+__device__ __forceinline__ Part operator-(Part p) { return Part{-p.v, -p.f}; }
+__device__ __forceinline__ Part operator+(Part a, Part b) { return Part{a.v + b.v, a.f + b.f}; }
+// A sum rounded by rnd, uniform below one unit; DROP: low bits of f left out, so that adding to it stays in range.
+template <int UP, int DROP = 0> __device__ __forceinline__ ll rounded(Part s, uint32_t rnd) {
+    constexpr int F = kFracBits<UP> - DROP;
+    return s.v + (((s.f >> DROP) + (int)(rnd >> (32 - F))) >> F);
 }
-template <int UP> __device__ __forceinline__ float rounded(float s, uint32_t) { return s; }
+template <int UP, int DROP = 0> __device__ __forceinline__ double rounded(Two s, uint32_t) { return (double)s; }
 // One product, rounded by rnd.
 template <int IM, int UP> __device__ __forceinline__ ll prod(int4 a, longlong2 b, uint32_t rnd) {
     return rounded<UP>(prod_part<IM, UP>(a, b), rnd);
@@ -155,30 +176,15 @@ __device__ __forceinline__ void halve(float2 &x, int s) {
 __device__ __forceinline__ ll shfl(ll v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ float shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 
-// A sum over threads of float32 partial sums, as the float32 nearest to it and what is left: 48 bits on the float32
-// pipe, which takes 64 times what the float64 pipe does.
-struct Two {
-    float s, e;
-    __device__ __forceinline__ explicit operator double() const { return (double)s + (double)e; }
-};
-__device__ __forceinline__ Two exact_sum(float a, float b) {  // s + e = a + b
-    const float s = a + b, t = s - a;
-    return Two{s, (a - (s - t)) + (b - t)};
-}
-__device__ __forceinline__ Two exact_product(float a, float b) {
-    const float p = a * b;
-    return Two{p, fmaf(a, b, -p)};
-}
-__device__ __forceinline__ Two operator+(Two a, Two b) {
-    const Two r = exact_sum(a.s, b.s);
-    return Two{r.s, r.e + (a.e + b.e)};
-}
 __device__ __forceinline__ Two shfl(Two v, int o) { return Two{shfl(v.s, o), shfl(v.e, o)}; }
+__device__ __forceinline__ Part shfl(Part p, int o) { return Part{shfl(p.v, o), __shfl_xor_sync(0xffffffffu, p.f, o)}; }
 
 // the type that sums over threads are carried in
 __device__ __forceinline__ ll across(ll v) { return v; }
+__device__ __forceinline__ Part across(Part p) { return p; }
 __device__ __forceinline__ Two across(float v) { return Two{v, 0.0f}; }
 __device__ __forceinline__ ll pair_sum(ll a, ll b) { return a + b; }
+__device__ __forceinline__ Part pair_sum(Part a, Part b) { return a + b; }
 __device__ __forceinline__ Two pair_sum(float a, float b) { return exact_sum(a, b); }
 
 // Warp sums of 8 values: the lane returns the sum of a[(lane >> 2) & 7].

@@ -26,10 +26,11 @@ namespace frames {
 // the vector by 2^4), and as every rounding is unbiased (see hash) a unit of 2^-58 on each component moves an
 // inner product with a unit vector by no more.
 constexpr int kUnit = 58;
-// Inner products are sums of 2^-62: unit vectors, so no partial sum of products exceeds 1 in magnitude. A thread
-// keeps what lies below the unit as well and rounds its sum once; what that leaves is a unit times
-// 2^((n - KB)/2). 22 qubits, two-norm errors of gradient and g: 2.8e-15 and 4.4e-15 with every product rounded,
-// 2.0e-15 and 4.2e-15 so (float64 on the gate-by-gate passes: 2.1e-15 and 4.4e-15); 17.57 and 17.69 ms.
+// Inner products are sums of 2^-62: unit vectors, so no partial sum of products exceeds 1 in magnitude. What lies
+// below the unit is kept as well and a warp's sum rounded once; what that leaves is a unit times 2^((n - 9)/2).
+// 22 qubits, two-norm errors of gradient and g: 2.8e-15 and 4.4e-15 with every product rounded,
+// 2.0e-15 and 4.2e-15 so (float64 on the gate-by-gate passes: 2.1e-15 and 4.4e-15); 17.58 and 17.83 ms. 26 qubits,
+// gradient entries against the oracle: 7.0e-14, 1.3e-14 so (float64: 1.2e-14).
 constexpr int kSumUnit = 62;
 constexpr int kHalfThreads = 128;
 constexpr int kRows = 32;  // parameters of a run kept in shared memory
@@ -393,15 +394,6 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
                         if (MIM) add(pi[1 + j], qu, (k0 >> j) & 1);
                     }
                 }
-                // the thread's sums are rounded once each: 2^(n - KB) roundings a sum instead of 2^n
-                Sums<T, KB> sr, si;
-                sr.all = rounded<UP>(pr[0], h0 ^ salt(160));
-                si.all = rounded<UP>(pi[0], h0 ^ salt(170));
-#pragma unroll
-                for (int j = 0; j < KB; ++j) {
-                    sr.bit[j] = rounded<UP>(pr[1 + j], h0 ^ salt(161 + j));
-                    si.bit[j] = rounded<UP>(pi[1 + j], h0 ^ salt(171 + j));
-                }
                 slots_of<T, KB>(smem, tb0, st, [&](int k, A *s) { b[k] = *s; });
                 // The run's rows, its parameters and (in the column's own run) <sigma_j>: each is one of the
                 // warp's 16 sums, of the products as they are (0), signed by one of the thread's bits (1 + j)
@@ -410,26 +402,29 @@ __global__ void __launch_bounds__(NT, ctas_per_sm<T>(KB, NT)) k_stream(SWork w, 
                 const int ipc = rn.ip_count, ipf = rn.ip_first, nrow = ipc + (start ? 1 : 0);
                 const int lane = t & 31, wid = t >> 5;
                 {
-                    Acc ar[8], ai[8];
+                    // A warp's sums are rounded once each (512 products, whose parts below the unit add up to less
+                    // than 2^31): 2^(n - 9) roundings in all instead of 2^n
+                    Part ar[8], ai[8];
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
 #pragma unroll
                         for (int g = 0; g < 8; ++g) {
                             if (half == 0) {
-                                ar[g] = g == 0 ? sr.all : (g <= KB ? sr.bit[g <= KB && g > 0 ? g - 1 : 0] : Acc(0));
-                                ai[g] = g == 0 ? si.all : (g <= KB ? si.bit[g <= KB && g > 0 ? g - 1 : 0] : Acc(0));
+                                ar[g] = g <= KB ? pr[g <= KB ? g : 0] : Part{};
+                                ai[g] = g <= KB ? pi[g <= KB ? g : 0] : Part{};
                             } else {
                                 const bool neg = g < 5 && ((lane >> g) & 1);
-                                ar[g] = g < 5 ? (neg ? -sr.all : sr.all) : Acc(0);
-                                ai[g] = g < 5 ? (neg ? -si.all : si.all) : Acc(0);
+                                ar[g] = g < 5 ? (neg ? -pr[0] : pr[0]) : Part{};
+                                ai[g] = g < 5 ? (neg ? -pi[0] : pi[0]) : Part{};
                             }
                         }
                         const auto xr = warp8(ar, lane);
-                        auto xi = across(Acc(0));
+                        auto xi = across(Part{});
                         if (MIM) xi = warp8(ai, lane);
                         if ((lane & 3) == 0) {
-                            red[half * 8 + (lane >> 2)][wid][0] = (Red)xr;
-                            if (MIM) red[half * 8 + (lane >> 2)][wid][1] = (Red)xi;
+                            const int row = half * 8 + (lane >> 2);
+                            red[row][wid][0] = rounded<UP, 1>(xr, h0 ^ salt(160 + half));
+                            if (MIM) red[row][wid][1] = rounded<UP, 1>(xi, h0 ^ salt(162 + half));
                         }
                     }
                 }
