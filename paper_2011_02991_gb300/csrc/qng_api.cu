@@ -575,8 +575,12 @@ bool plan_frames(qng_ctx *c) {
         key[b] = {d.cl, frames_threads(p, tpc, c->count)};
     }
     if (c->count <= kFewInstances)  // one class per cluster size: launches side by side cost more than idle threads
-        for (auto &k : key)
-            for (const auto &o : key) if (o[0] == k[0]) k[1] = std::max(k[1], o[1]);
+        for (auto &k : key) {
+            int t = k[1];
+            for (const auto &o : key) if (o[0] == k[0]) t = std::max(t, o[1]);
+            // (where the rows of the largest P leave room for it)
+            if (((size_t)t << kb) * ab + 2 * sizeof(double) * (size_t)(c->max_P + 1) * (t / 32) <= kMaxSmem / 2) k[1] = t;
+        }
     std::vector<std::array<int, 2>> keys(key);
     std::sort(keys.begin(), keys.end(), [](const std::array<int, 2> &x, const std::array<int, 2> &y) { return x > y; });
     keys.erase(std::unique(keys.begin(), keys.end()), keys.end());
