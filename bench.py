@@ -37,9 +37,9 @@ METRIC = "QNG steps/s (g,∇E,Δθ) per config; HBM GB/s vs GB300 peak; max err 
 FP64_PEAK_TFLOPS = 2 * 2 * 152 * 2.07e9 / 1e12
 FP32_PEAK_TFLOPS = 128 * 2 * 152 * 2.07e9 / 1e12
 HBM_PEAK_GBS = 6669.2  # measured copy bandwidth of this GPU pool
-# DRAM bytes (read + write) per launch of the timed kernel, from an ncu capture of this build's kernel on
-# the workload; empty while no capture of the current kernels at these sizes exists.
-TRAFFIC: dict[str, float] = {}
+# DRAM bytes (read + write) per launch of the timed kernel, from an ncu capture of its kernel on the workload
+# (profiles/diagonal_frames.md: mean over 30 consecutive walk launches of a step); none for the others.
+TRAFFIC = {"rand28_p252_c64": 17539828634.0}
 
 
 def workloads():
@@ -70,7 +70,7 @@ def _c64(p):
 DESCRIPTION = {
     "rand12_p192_c128": "12 qubits, 8 x [Ry all, Rz all, CZ ladder] (P=192), 40 random Pauli strings "
                         "(weight 1-4, N(0,1) coefficients), theta ~ U[0,2pi), complex128, dt=0.1, lambda=1e-3",
-    "rand12_p192_c64": "as rand12_p192_c128 with complex64 amplitudes (float64 accumulation, assembly, solve)",
+    "rand12_p192_c64": "as rand12_p192_c128 with complex64 amplitudes (sums beyond float32 from the warp on; float64 assembly, solve)",
     "tfim4_p16_c128": "4 qubits, 2 x [Ry, Rz, CZ ladder] (P=16), open TFIM, complex128",
     "batch256_c64": "256 instances, n ~ U{6..14}, 2-10 Ry/Rz/CZ layers (P 24-280), 16-48 strings each, complex64",
     "batch256_c128": "the same 256 instances in complex128",
@@ -586,7 +586,7 @@ def run_ours(args, name, rank, world, local_rank):
     line = {
         "metric": METRIC, "value": value, "unit": "steps/s", "n_gpus": world, "steps": steps,
         "warmup": args.warmup, "ms_per_step": res["ms_total"] / steps, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "f64" if prec64 else "f32 (f64 accumulation, assembly, solve)",
+        "vs_baseline": None, "dtype": "f64" if prec64 else "f32 (sums beyond f32 from the warp on; f64 assembly, solve)",
         "data": "synthetic",
         "config": {"workload": f"{name}: {DESCRIPTION[name]}", "instances": cnt,
                    "n_qubits": sorted({p.n for p in problems}), "P_total": P_tot,
