@@ -141,7 +141,7 @@ struct Builder {
         m.cval = fr[c].z.s > 0 ? m.ctrl : 0;
         open().push_back(m);
     }
-    // CNOT c -> t; touched: the qubits that it and the CNOTs right after it share, through one another
+    // CNOT c -> t; touched: the qubits that its stretch of CNOTs joins it with
     void cnot(int c, int t, uint32_t touched) {
         if (fr[c].z.p == PZ && fr[t].x.p == PZ) { controlled_sign(c, t, kAxisX); return; }
         // Frames whose Z and X images are Z and X: for all of the CNOTs to come at once, so that a ladder is one
@@ -180,6 +180,8 @@ std::vector<std::pair<int, int>> string_req(uint64_t x, uint64_t z, int n) {
 
 // The circuit's gates, in order, into runs and transitions.
 void walk_gates(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks, int n, Builder &B) {
+    size_t stretch_end = 0;
+    uint32_t joined[kMaxQubits];
     for (size_t gi = 0; gi < gates.size(); ++gi) {
         const qng_gate &g = gates[gi];
         Frame *f = (g.q0 >= 0 && g.q0 < n) ? &B.fr[g.q0] : nullptr;
@@ -200,18 +202,16 @@ void walk_gates(const std::vector<qng_gate> &gates, const std::vector<uint64_t> 
             B.diagonalise({{g.q0, kAxisZ}, {g.q1, kAxisZ}});
             B.controlled_sign(g.q0, g.q1, kAxisZ);
             break;
-        case QNG_GATE_CNOT: {
-            uint32_t touched = (1u << g.q0) | (1u << g.q1);
-            for (uint32_t before = 0; before != touched;) {
-                before = touched;
-                for (size_t k = gi + 1; k < gates.size() && gates[k].kind == QNG_GATE_CNOT; ++k) {
-                    const uint32_t m = (1u << gates[k].q0) | (1u << gates[k].q1);
-                    if (m & touched) touched |= m;
+        case QNG_GATE_CNOT:
+            if (gi >= stretch_end) {  // the qubits that each one's stretch of CNOTs joins it with
+                for (int q = 0; q < n; ++q) joined[q] = 1u << q;
+                for (stretch_end = gi; stretch_end < gates.size() && gates[stretch_end].kind == QNG_GATE_CNOT; ++stretch_end) {
+                    const uint32_t m = joined[gates[stretch_end].q0] | joined[gates[stretch_end].q1];
+                    for (int q = 0; q < n; ++q) if ((m >> q) & 1) joined[q] = m;
                 }
             }
-            B.cnot(g.q0, g.q1, touched);
+            B.cnot(g.q0, g.q1, joined[g.q0]);
             break;
-        }
         default: break;
         }
     }
@@ -421,10 +421,10 @@ bool holds(const Window &W, int q) { return q < W.low || (q >= W.s && q < W.s + 
 
 // The atoms of the list (those not done) that a pass over window W can execute: in order, each one
 // whose pair qubit the window holds and that no skipped atom shares a qubit with.
-std::vector<int> executable(const std::vector<Atom> &at, const std::vector<uint8_t> &done, size_t from, const Window &W) {
+std::vector<int> executable(const std::vector<Atom> &at, const std::vector<uint8_t> &done, size_t from, const Window &W, int n) {
     std::vector<int> ex;
     uint32_t blocked = 0;
-    for (size_t k = from; k < at.size(); ++k) {
+    for (size_t k = from; k < at.size() && blocked != (1u << n) - 1u; ++k) {
         if (done[k]) continue;
         const Atom &a = at[k];
         if (a.kind == 2) {
@@ -464,7 +464,7 @@ void pack_passes(const std::vector<Atom> &at, bool back, bool fixed, const std::
         std::vector<int> best;
         Window W = wins[0];
         for (const Window &w : wins) {
-            std::vector<int> ex = executable(at, done, from, w);
+            std::vector<int> ex = executable(at, done, from, w, n);
             if (ex.size() > best.size()) { best = ex; W = w; }
         }
         SPass ps = {};

@@ -3,6 +3,7 @@ logic (validation, sizes, offsets, workspace layout) behaves. No kernel is launc
 import ctypes
 import os
 import re
+import time
 
 import numpy as np
 import pytest
@@ -184,6 +185,20 @@ def test_least_workspace(lib, n, layers, precision):
         assert lib.qng_set_workspace(h, ctypes.c_void_p(0x1000), least.value - 256, None) == 6
         again = ctypes.c_size_t()
         assert lib.qng_workspace_size(h, ctypes.byref(again)) == 0 and again.value == nb.value
+    lib.qng_destroy(h)
+
+
+@pytest.mark.parametrize("n", [10, 20])
+def test_long_stretches_plan_in_linear_time(lib, n):
+    """100 000 CNOTs between the first and the last rotations: under 5 s, hundreds of times what a pass over the
+    gates takes and a fraction of what a look ahead from every CNOT would."""
+    rng = np.random.Generator(np.random.PCG64(n))
+    gates = [(W.RY, q, -1, q) for q in range(n)]
+    gates += [(W.CNOT, int(a), int(a + 1 + b) % n, -1) for a, b in zip(rng.integers(0, n, 100000), rng.integers(0, n - 1, 100000))]
+    gates += [(W.RY, q, -1, n + q) for q in range(n)]
+    t = time.perf_counter()
+    st, h = _create(lib, n, gates, [(1.0, 1, 0)], W.C64)
+    assert st == 0 and time.perf_counter() - t < 5.0
     lib.qng_destroy(h)
 
 
