@@ -239,7 +239,8 @@ qng_status qng_autotune(qng_ctx *ctx, const double *theta, int reps, int64_t *re
 /* Launch shape of the gate-by-gate kernels for instances of n_qubits qubits (after defaults,
  * autotuning and qng_set_shape). An explicit shape, here, through qng_set_tuning or through
  * qng_set_forward_cluster, makes instances of that size run those kernels instead of the
- * diagonal-frame ones; restoring the defaults restores the diagonal-frame ones.
+ * diagonal-frame ones; restoring the defaults restores the diagonal-frame ones (complex128 circuits of
+ * fewer than 8 qubits and 1.6 parameters a step of their diagonal-frame program run gate by gate by default).
  * cluster_log2 = log2 of CTAs per state, threads = CTA size of the column kernel (64..256),
  * forward_threads = CTA size of the checkpoint sweep (64..512); any output pointer may be NULL.
  * qng_set_shape is the manual override (cluster_log2 -1, threads 0 and forward_threads 0 restore
