@@ -141,7 +141,7 @@ struct Builder {
         m.cval = fr[c].z.s > 0 ? m.ctrl : 0;
         open().push_back(m);
     }
-    // CNOT c -> t; touched: the qubits that its stretch of CNOTs joins it with
+    // CNOT c -> t; touched: the qubits that it and the CNOTs after it in its stretch join it with
     void cnot(int c, int t, uint32_t touched) {
         if (fr[c].z.p == PZ && fr[t].x.p == PZ) { controlled_sign(c, t, kAxisX); return; }
         // Frames whose Z and X images are Z and X: for all of the CNOTs to come at once, so that a ladder is one
@@ -180,8 +180,8 @@ std::vector<std::pair<int, int>> string_req(uint64_t x, uint64_t z, int n) {
 
 // The circuit's gates, in order, into runs and transitions.
 void walk_gates(const std::vector<qng_gate> &gates, const std::vector<uint64_t> &masks, int n, Builder &B) {
-    size_t stretch_end = 0;
-    uint32_t joined[kMaxQubits];
+    size_t stretch = 0, stretch_end = 0;
+    std::vector<uint32_t> touched;
     for (size_t gi = 0; gi < gates.size(); ++gi) {
         const qng_gate &g = gates[gi];
         Frame *f = (g.q0 >= 0 && g.q0 < n) ? &B.fr[g.q0] : nullptr;
@@ -203,14 +203,19 @@ void walk_gates(const std::vector<qng_gate> &gates, const std::vector<uint64_t> 
             B.controlled_sign(g.q0, g.q1, kAxisZ);
             break;
         case QNG_GATE_CNOT:
-            if (gi >= stretch_end) {  // the qubits that each one's stretch of CNOTs joins it with
+            if (gi >= stretch_end) {  // per CNOT, the qubits that it and those after it in the stretch join it with
+                uint32_t joined[kMaxQubits];
                 for (int q = 0; q < n; ++q) joined[q] = 1u << q;
-                for (stretch_end = gi; stretch_end < gates.size() && gates[stretch_end].kind == QNG_GATE_CNOT; ++stretch_end) {
-                    const uint32_t m = joined[gates[stretch_end].q0] | joined[gates[stretch_end].q1];
+                stretch = stretch_end = gi;
+                while (stretch_end < gates.size() && gates[stretch_end].kind == QNG_GATE_CNOT) ++stretch_end;
+                touched.resize(stretch_end - gi);
+                for (size_t k = stretch_end; k-- > gi;) {
+                    const uint32_t m = joined[gates[k].q0] | joined[gates[k].q1];
                     for (int q = 0; q < n; ++q) if ((m >> q) & 1) joined[q] = m;
+                    touched[k - gi] = m;
                 }
             }
-            B.cnot(g.q0, g.q1, joined[g.q0]);
+            B.cnot(g.q0, g.q1, touched[gi - stretch]);
             break;
         default: break;
         }
@@ -489,8 +494,10 @@ void pack_passes(const std::vector<Atom> &at, bool back, bool fixed, const std::
         for (size_t i = 0; i < best.size();) {
             const Atom &a = at[best[i]];
             if (a.kind == 0) {
-                uint32_t h = 0;  // over local bits
-                while (i < best.size() && at[best[i]].kind == 0) h ^= 1u << local(at[best[i++]].q);
+                // over local bits; two on one qubit (with nothing on it between them) are two steps, as either
+                // counts for the norm
+                uint32_t h = 0;
+                while (i < best.size() && at[best[i]].kind == 0 && !((h >> local(at[best[i]].q)) & 1)) h |= 1u << local(at[best[i++]].q);
                 std::vector<int> bl;
                 for (int b = 0; b < tb; ++b) if ((h >> b) & 1) { const int lo = block_of(b); if (!std::count(bl.begin(), bl.end(), lo)) bl.push_back(lo); }
                 // the current block first, block 0 next, the others last: runs, loads and stores want their

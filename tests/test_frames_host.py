@@ -131,6 +131,25 @@ def test_long_transitions(probe, oracle, n, layers):
     check(probe, oracle, p, 3, 0, 5, 2)
 
 
+@pytest.mark.parametrize("n,kb,tb,low", [(7, 3, 5, 2), (9, 3, 6, 3)])
+def test_stretch_with_a_sign(probe, oracle, n, kb, tb, low):
+    """A stretch of CNOTs that begins with one that is a sign in its frame: the qubit that this one alone touches gets
+    no Hadamard for the others, which a pass would meet next to a later one. (What a transition's Hadamards leave of
+    the norm is what the run after it takes, whichever of them a pass executes together.)"""
+    for top in (n - 1, n - 2, 3):
+        rows, k = [], 0
+        for kind in (W.RY, W.RZ):
+            rows += [[kind, q, -1, k + q] for q in range(n)]
+            k += n
+        rows += [[W.H, 1, -1, -1], [W.H, 2, -1, -1], [W.CNOT, top, 1, -1], [W.CNOT, 2, top, -1], [W.H, 1, -1, -1], [W.CNOT, 1, 0, -1]]
+        rows += [[W.RY, q, -1, k + q] for q in range(n)]
+        rng = np.random.Generator(np.random.PCG64(n))
+        p = W.Problem("sign", W.Circuit(n, np.array(rows, dtype=np.int32)), W.random_pauli_hamiltonian(n, 6, rng),
+                      W.uniform_theta(k + n, rng))
+        check(probe, oracle, p, kb)
+        check(probe, oracle, p, kb, 0, tb, low)
+
+
 @pytest.mark.parametrize("n,kb,tb,low", [(7, 3, 5, 2), (9, 3, 6, 3), (8, 3, 7, 3), (9, 4, 6, 1), (10, 3, 6, 3), (6, 4, 6, 2)])
 @pytest.mark.parametrize("seed", range(4))
 def test_streaming_passes(probe, oracle, n, kb, tb, low, seed):
